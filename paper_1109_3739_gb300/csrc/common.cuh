@@ -218,6 +218,20 @@ __device__ __forceinline__ int64_t lower_bound_col(const int32_t *j, int64_t s, 
   return s;
 }
 
+// a[i] <= x holds for exactly the first returned entries of the non-decreasing
+// a[0..n); a whole warp searches, 32 probes a step (every lane returns it)
+__device__ __forceinline__ int64_t warp_upper_bound(const int64_t *a, int64_t n, int64_t x) {
+  int64_t lo = 0, hi = n;
+  while (hi - lo > 32) {
+    const int64_t s = (hi - lo) >> 5;
+    const int c = __popc(__ballot_sync(FULL, __ldg(a + lo + (lane_id() + 1) * s - 1) <= x));
+    if (c < 32) hi = lo + (c + 1) * s - 1;
+    lo += c * s;
+  }
+  const int64_t p = lo + lane_id();
+  return lo + __popc(__ballot_sync(FULL, p < hi && __ldg(a + p) <= x));
+}
+
 template <typename T> __device__ __forceinline__ T load_val(const void *v, int64_t q) {
   return __ldg(reinterpret_cast<const T *>(v) + q);
 }

@@ -11,8 +11,9 @@
 // and the final step of SpAsgn, the elementwise product of A with the
 // structural negation of S*A*T plus R*B*Q: an entry (r, c) of A is in the
 // structure of S*A*T exactly when r is in I and c is in J, so the negation is
-// applied through the inverse index maps rpos/cpos, so neither S*A*T nor its
-// negation is ever materialised (Section 3.1).
+// applied through I and the inverse index map cpos, and neither S*A*T nor its
+// negation is ever materialised (Section 3.1).  Nor is R*B*Q, when B's rows
+// keep their order under J: its entries are B's, moved to rows I and columns J.
 #include "common.cuh"
 #include "internal.h"
 
@@ -328,87 +329,237 @@ __device__ void combine_val(const AsgnArgs &a, int64_t di, int64_t ai, int64_t x
   }
 }
 
-// count: output entries of row r go to Cp[r+1]
-__global__ void k_asgn_count(AsgnArgs a) {
-  const int lane = lane_id();
-  const int64_t wpb = blockDim.x >> 5;
-  for (int64_t r = blockIdx.x * wpb + (threadIdx.x >> 5); r < a.m; r += (int64_t)gridDim.x * wpb) {
-    const int64_t a0 = a.Ap[r], a1 = a.Ap[r + 1];
-    const int64_t x0 = a.Xp[r], x1 = a.Xp[r + 1];
-    int64_t cnt;
-    if (a.rpos[r] < 0) {
-      cnt = a1 - a0;  // r is not in I: R*B*Q's row is empty
-    } else if (!a.accumulate) {
-      long long kept = 0;
-      for (int64_t q = a0 + lane; q < a1; q += 32) kept += a.cpos[a.Aj[q]] < 0;
-      kept = warp_sum(kept);
-      cnt = kept + (x1 - x0);
-    } else {
-      long long both = 0;  // columns present in A(r,:) and in R*B*Q(r,:)
-      for (int64_t x = x0 + lane; x < x1; x += 32) {
-        const int c = a.Xj[x];
-        const int64_t at = lower_bound_col(a.Aj, a0, a1, c);
-        both += (at < a1 && a.Aj[at] == c);
-      }
-      both = warp_sum(both);
-      cnt = (a1 - a0) + (x1 - x0) - both;
-    }
-    if (lane == 0) a.Cp[r + 1] = cnt;
+// The merge runs over entries, not rows, so a hub row costs what its entries
+// cost (assigning 20,000 edges into a 16M-entry graph: 6.62 of 7.20 ms with one
+// lane walking each touched row, 0.23 of 0.30 ms so; its 270 MB of A and C
+// take 0.04 ms at the copy rate).  X = R*B*Q as the
+// entries of B moved to row I[i] and column J[c], in (row, column) order:
+// entry t of X goes in front of A's entry at[t] (the first of its row whose
+// column is not smaller).  A bit per entry of A says whether it is kept: an
+// assignment drops the entries of the I x J block, extend-add those that X
+// repeats (X's entry then carries the sum).  With K(q) the kept entries
+// before q, A's entry q goes to K(q) + |{t : at[t] <= q}| and X's entry t to
+// K(at[t]) + t.
+
+// lengths of X's rows into XB[row + 1], and whether X's entries, taken as they
+// lie in B, are in increasing column order inside every row: viol[0] counts
+// the entries whose column is not above that of the entry before, viol[1] how
+// many of those begin a row.  Indices out of range are skipped (dbg, or flag
+// set by the marking, reports them).
+__global__ void k_asgn_rows(AsgnX x, int64_t m, int64_t n, int64_t *XB, unsigned long long *viol, long long *dbg) {
+  unsigned long long all = 0, starts = 0;
+  auto col = [&](int64_t e) -> int {
+    const int c = x.j[e];
+    if (!HS_G(dbg, c >= 0 && c < x.nJ, 51, c)) return -1;
+    return x.J[c];
+  };
+  GRID_STRIDE(e, x.nnz) if (e > 0) all += col(e) <= col(e - 1);
+  GRID_STRIDE(i, x.rows) {
+    const int64_t b = x.p[i], e = x.p[i + 1];
+    const int r = x.I[i];
+    if (!HS_G(dbg, b >= 0 && b <= e && e <= x.nnz, 3, e)) continue;
+    if (e > b && r >= 0 && r < m) atomicAdd(reinterpret_cast<unsigned long long *>(XB + r + 1), (unsigned long long)(e - b));
+    if (e > b && b > 0) starts += col(b) <= col(b - 1);
+  }
+  all = warp_sum(all);
+  starts = warp_sum(starts);
+  if (lane_id() == 0) {
+    if (all) atomicAdd(viol, all);
+    if (starts) atomicAdd(viol + 1, starts);
   }
 }
 
-__global__ void k_asgn_fill(AsgnArgs a) {
-  const int lane = lane_id();
-  const int64_t wpb = blockDim.x >> 5;
-  for (int64_t r = blockIdx.x * wpb + (threadIdx.x >> 5); r < a.m; r += (int64_t)gridDim.x * wpb) {
+// at[t] and the source of each entry of X (src[t] = its place in X's arrays;
+// ~place when A has an entry there too, whose keep bit extend-add clears).
+// Thread per entry: the row by a search of X's offsets, the place by a search
+// of A's row.
+__global__ void k_asgn_place(AsgnX x, AsgnArgs a, const int64_t *XB, int64_t *at, int64_t *src, uint32_t *keep) {
+  GRID_STRIDE(e, x.nnz) {
+    int64_t lo = 0, hi = x.rows;  // last row that starts at or before e
+    while (hi - lo > 1) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (x.p[mid] <= e) lo = mid;
+      else hi = mid;
+    }
+    const int64_t r = x.I ? (int64_t)x.I[lo] : lo;
+    int c = x.j[e];
+    if (x.J) {
+      if (!HS_G(a.dbg, c >= 0 && c < x.nJ, 51, c)) continue;
+      c = x.J[c];
+    }
+    const int64_t t = r >= 0 && r < a.m ? XB[r] + (e - x.p[lo]) : -1;
+    if (t < 0 || t >= x.nnz) continue;  // a bad or repeated index: reported before at[] is used
     const int64_t a0 = a.Ap[r], a1 = a.Ap[r + 1];
-    const int64_t x0 = a.Xp[r], x1 = a.Xp[r + 1];
-    const int64_t o = a.Cp[r];
-    if (a.rpos[r] < 0) {  // copy the row
-      for (int64_t q = lane; q < a1 - a0; q += 32) {
-        a.Cj[o + q] = a.Aj[a0 + q];
-        copy_val(a.Cv, o + q, a.Av, a0 + q, a.vbytes);
-      }
-      continue;
-    }
-    if (lane != 0) continue;
-    // merge A(r,:) (minus the I x J block when assigning) with R*B*Q(r,:)
-    int64_t i = a0, x = x0, w = o;
-    while (true) {
-      if (!a.accumulate)
-        while (i < a1 && a.cpos[a.Aj[i]] >= 0) ++i;
-      const bool ha = i < a1, hx = x < x1;
-      if (!ha && !hx) break;
-      const int ca = ha ? a.Aj[i] : 0x7fffffff, cx = hx ? a.Xj[x] : 0x7fffffff;
-      if (ca < cx) {
-        a.Cj[w] = ca;
-        copy_val(a.Cv, w, a.Av, i, a.vbytes);
-        ++i;
-      } else if (cx < ca) {
-        a.Cj[w] = cx;
-        copy_val(a.Cv, w, a.Xv, x, a.vbytes);
-        ++x;
-      } else {  // only with accumulate
-        a.Cj[w] = ca;
-        combine_val(a, w, i, x);
-        ++i;
-        ++x;
-      }
-      ++w;
-    }
+    if (!HS_G(a.dbg, a0 >= 0 && a0 <= a1 && a1 <= a.nnzA, 3, a1)) continue;
+    const int64_t q = lower_bound_col(a.Aj, a0, a1, c);
+    const bool both = a.accumulate && q < a1 && a.Aj[q] == c;
+    at[t] = q;
+    src[t] = both ? ~e : e;
+    if (both) atomicAnd(keep + (q >> 5), ~(1u << (q & 31)));
   }
 }
 
-void launch_asgn_count(const AsgnArgs &a, cudaStream_t st) {
-  if (a.m > 0) {
-    count_launch();
-    k_asgn_count<<<grid1(a.m * 32), 256, 0, st>>>(a);
+// assignment: the entries of A inside the I x J block lose their keep bit.  A
+// warp per row of I; a row of more than ASGN_LONG entries by the whole block.
+constexpr int ASGN_LONG = 1024;
+__device__ __forceinline__ void asgn_drop(const AsgnArgs &a, int64_t a0, int64_t a1, int64_t step, int64_t first,
+                                          uint32_t *keep) {
+  constexpr int U = 4;
+  // words are aligned to 32 entries, lane l on bit l: one atomic per word
+  for (int64_t q0 = (a0 & ~(int64_t)31) + first; q0 - lane_id() < a1; q0 += U * step) {
+    int c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t q = q0 + u * step;
+      c[u] = q >= a0 && q < a1 ? a.Aj[q] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned gone = __ballot_sync(FULL, c[u] >= 0 && c[u] < a.n && a.cpos[c[u]] >= 0);
+      if (gone && lane_id() == 0) atomicAnd(keep + ((q0 + u * step) >> 5), ~gone);
+    }
   }
 }
-void launch_asgn_fill(const AsgnArgs &a, cudaStream_t st) {
-  if (a.m > 0) {
+__global__ void __launch_bounds__(256) k_asgn_drop(AsgnArgs a, const int32_t *I, int64_t nI, uint32_t *keep) {
+  __shared__ int s_long[8], s_n;
+  const int w = threadIdx.x >> 5;
+  for (int64_t i0 = (int64_t)blockIdx.x * 8; i0 < nI; i0 += (int64_t)gridDim.x * 8) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int64_t i = i0 + w;
+    const int r = i < nI ? I[i] : -1;
+    if (r >= 0 && r < a.m) {
+      const int64_t a0 = a.Ap[r], a1 = a.Ap[r + 1];
+      if (HS_G(a.dbg, a0 >= 0 && a0 <= a1 && a1 <= a.nnzA, 3, a1)) {
+        if (a1 - a0 <= ASGN_LONG) asgn_drop(a, a0, a1, 32, lane_id(), keep);
+        else if (lane_id() == 0) s_long[atomicAdd(&s_n, 1)] = r;
+      }
+    }
+    __syncthreads();
+    for (int k = 0; k < s_n; ++k) asgn_drop(a, a.Ap[s_long[k]], a.Ap[s_long[k] + 1], 256, threadIdx.x, keep);
+    __syncthreads();
+  }
+}
+
+// kept entries per word of 32 (bits past A's last entry do not count)
+__global__ void k_asgn_words(const uint32_t *keep, int64_t nnz, int64_t nw, int64_t *S) {
+  GRID_STRIDE(w, nw) {
+    const int64_t left = nnz - w * 32;
+    S[w] = __popc(left >= 32 ? keep[w] : keep[w] & ((1u << left) - 1u));
+  }
+}
+// K(q): kept entries of A before q (S: inclusive scan of the words' counts)
+__device__ __forceinline__ int64_t kept_before(const int64_t *S, const uint32_t *keep, int64_t q) {
+  const int64_t w = q >> 5;
+  const int b = (int)(q & 31);
+  return (w ? S[w - 1] : 0) + (b ? __popc(keep[w] & ((1u << b) - 1u)) : 0);
+}
+__global__ void k_asgn_offsets(AsgnArgs a, const int64_t *XB, const int64_t *S, const uint32_t *keep) {
+  const int64_t k0 = kept_before(S, keep, min(a.Ap[0], a.nnzA));
+  GRID_STRIDE(r, a.m + 1) {
+    const int64_t q = a.Ap[r];
+    a.Cp[r] = XB[r] + (HS_G(a.dbg, q >= 0 && q <= a.nnzA, 3, q) ? kept_before(S, keep, q) - k0 : 0);
+  }
+}
+
+// A's kept entries into C, a tile of consecutive entries per block: the
+// entries of X that fall inside the tile are found by two searches of at[]
+constexpr int ASGN_NT = 256, ASGN_PER = 8, ASGN_TILE = ASGN_NT * ASGN_PER;
+__global__ void __launch_bounds__(ASGN_NT) k_asgn_fill_a(AsgnArgs a, const int64_t *at, int64_t nx, const int64_t *S,
+                                                         const uint32_t *keep) {
+  __shared__ int64_t s_at[ASGN_TILE];
+  __shared__ int64_t s_lo, s_hi;
+  const int64_t first = a.Ap[0], last = min(a.Ap[a.m], a.nnzA);
+  const int64_t k0 = kept_before(S, keep, min(first, a.nnzA));
+  const int64_t q0 = (int64_t)blockIdx.x * ASGN_TILE;
+  const int w = threadIdx.x >> 5;
+  int c[ASGN_PER];
+#pragma unroll
+  for (int u = 0; u < ASGN_PER; ++u) {
+    const int64_t q = q0 + u * ASGN_NT + threadIdx.x;
+    c[u] = q >= first && q < last ? a.Aj[q] : 0;
+  }
+  if (w < 2) {  // entries of X at or before the tile's first and last entry
+    const int64_t key = w == 0 ? q0 : q0 + ASGN_TILE - 1;
+    const int64_t r = warp_upper_bound(at, nx, key);
+    if (lane_id() == 0) (w == 0 ? s_lo : s_hi) = r;
+  }
+  __syncthreads();
+  const int64_t lo = s_lo, hi = s_hi;
+  const bool staged = hi - lo <= ASGN_TILE;
+  if (staged)
+    for (int64_t t = lo + threadIdx.x; t < hi; t += ASGN_NT) s_at[t - lo] = at[t];
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < ASGN_PER; ++u) {
+    const int64_t q = q0 + u * ASGN_NT + threadIdx.x;
+    if (q < first || q >= last) continue;
+    const uint32_t kw = keep[q >> 5];
+    if (!((kw >> (q & 31)) & 1u)) continue;
+    int64_t l = lo, h = hi;  // |{t : at[t] <= q}|
+    while (l < h) {
+      const int64_t mid = (l + h) >> 1;
+      if ((staged ? s_at[mid - lo] : at[mid]) <= q) l = mid + 1;
+      else h = mid;
+    }
+    const int64_t kb = (q >> 5) ? S[(q >> 5) - 1] : 0;
+    const int64_t d = kb + __popc(kw & ((1u << (q & 31)) - 1u)) - k0 + l;
+    if (!HS_G(a.dbg, d >= 0 && d < a.nnzC, 86, d)) continue;
+    a.Cj[d] = c[u];
+    copy_val(a.Cv, d, a.Av, q, a.vbytes);
+  }
+}
+__global__ void k_asgn_fill_x(AsgnX x, AsgnArgs a, const int64_t *at, const int64_t *src, const int64_t *S,
+                              const uint32_t *keep) {
+  const int64_t k0 = kept_before(S, keep, min(a.Ap[0], a.nnzA));
+  GRID_STRIDE(t, x.nnz) {
+    const int64_t s = src[t], q = at[t];
+    const int64_t e = s < 0 ? ~s : s;
+    if (!HS_G(a.dbg, q >= 0 && q <= a.nnzA && e < x.nnz, 87, q)) continue;
+    const int64_t d = kept_before(S, keep, q) - k0 + t;
+    if (!HS_G(a.dbg, d >= 0 && d < a.nnzC, 86, d)) continue;
+    a.Cj[d] = x.J ? x.J[x.j[e]] : x.j[e];
+    if (s < 0) combine_val(a, d, q, e);
+    else copy_val(a.Cv, d, a.Xv, e, a.vbytes);
+  }
+}
+
+void launch_asgn_rows(const AsgnX &x, int64_t m, int64_t n, int64_t *XB, unsigned long long *viol, long long *dbg,
+                      cudaStream_t st) {
+  const int64_t work = x.nnz > x.rows ? x.nnz : x.rows;
+  if (work <= 0) return;
+  count_launch();
+  k_asgn_rows<<<grid1(work), 256, 0, st>>>(x, m, n, XB, viol, dbg);
+}
+void launch_asgn_keep(const AsgnX &x, const AsgnArgs &a, const int32_t *I, int64_t nI, const int64_t *XB, int64_t *at,
+                      int64_t *src, uint32_t *keep, int64_t *S, int64_t nw, cudaStream_t st) {
+  if (x.nnz > 0) {
     count_launch();
-    k_asgn_fill<<<grid1(a.m * 32), 256, 0, st>>>(a);
+    k_asgn_place<<<grid1(x.nnz), 256, 0, st>>>(x, a, XB, at, src, keep);
+  }
+  if (!a.accumulate && nI > 0) {
+    count_launch();
+    k_asgn_drop<<<grid1(nI * 32), 256, 0, st>>>(a, I, nI, keep);
+  }
+  if (nw > 0) {
+    count_launch();
+    k_asgn_words<<<grid1(nw), 256, 0, st>>>(keep, a.nnzA, nw, S);
+  }
+}
+void launch_asgn_offsets(const AsgnArgs &a, const int64_t *XB, const int64_t *S, const uint32_t *keep,
+                         cudaStream_t st) {
+  count_launch();
+  k_asgn_offsets<<<grid1(a.m + 1), 256, 0, st>>>(a, XB, S, keep);
+}
+void launch_asgn_fill(const AsgnX &x, const AsgnArgs &a, const int64_t *at, const int64_t *src, const int64_t *S,
+                      const uint32_t *keep, cudaStream_t st) {
+  if (a.m > 0 && a.nnzA > 0) {
+    count_launch();
+    k_asgn_fill_a<<<(unsigned)((a.nnzA + ASGN_TILE - 1) / ASGN_TILE), ASGN_NT, 0, st>>>(a, at, x.nnz, S, keep);
+  }
+  if (x.nnz > 0) {
+    count_launch();
+    k_asgn_fill_x<<<grid1(x.nnz), 256, 0, st>>>(x, a, at, src, S, keep);
   }
 }
 

@@ -372,19 +372,35 @@ void launch_iota_i64(int64_t *p, int64_t n, cudaStream_t st);
 void launch_add_i64(int64_t *p, int64_t n, int64_t add, cudaStream_t st);  // p[i] += add
 struct AsgnArgs {
   const int64_t *Ap; const int32_t *Aj; const void *Av;   // A (m x n)
-  const int64_t *Xp; const int32_t *Xj; const void *Xv;   // X = R*B*Q (m x n)
-  const int32_t *rpos;  // m: row in I or -1
+  const void *Xv;       // values of X's entries
   const int32_t *cpos;  // n: column in J or -1
-  int64_t m;
+  int64_t m, n;
+  int64_t nnzA;
   int vbytes;           // value width (0 for bool)
   int accumulate;
   int add_kind;         // semiring for extend-add collisions
   int dtype;
-  int64_t *Cp;          // counts then offsets
+  int64_t *Cp;          // offsets
+  int64_t nnzC;
   int32_t *Cj;
   void *Cv;
+  long long *dbg;
 };
-void launch_asgn_count(const AsgnArgs &a, cudaStream_t st);
-void launch_asgn_fill(const AsgnArgs &a, cudaStream_t st);
+// X = R*B*Q: B's entries in row I[i] and column J[c] (I, J null: X's own rows
+// and columns)
+struct AsgnX {
+  const int64_t *p;
+  const int32_t *j;
+  const int32_t *I, *J;
+  int64_t rows, nJ, nnz;
+};
+void launch_asgn_rows(const AsgnX &x, int64_t m, int64_t n, int64_t *XB, unsigned long long *viol, long long *dbg,
+                      cudaStream_t st);
+void launch_asgn_keep(const AsgnX &x, const AsgnArgs &a, const int32_t *I, int64_t nI, const int64_t *XB, int64_t *at,
+                      int64_t *src, uint32_t *keep, int64_t *S, int64_t nw, cudaStream_t st);
+void launch_asgn_offsets(const AsgnArgs &a, const int64_t *XB, const int64_t *S, const uint32_t *keep,
+                         cudaStream_t st);
+void launch_asgn_fill(const AsgnX &x, const AsgnArgs &a, const int64_t *at, const int64_t *src, const int64_t *S,
+                      const uint32_t *keep, cudaStream_t st);
 
 }  // namespace hs

@@ -1080,6 +1080,12 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
   return check_launch();
 }
 
+// C = A .* not(S*A*T) + R*B*Q (assignment) or A + R*B*Q (extend-add), merged
+// entry by entry (index.cu).  X = R*B*Q is B itself with its rows and columns
+// relabelled, as long as every row of B keeps its column order under J (which
+// the device checks); otherwise X is computed as the two products, which sort
+// it.  One host synchronisation, to learn nnz(C) and the outcome of the
+// checks (with the products: theirs, and one more).
 static int spasgn_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ,
                        const hs_mat *B, int accumulate, int add_sr, hs_mat *C, Mem &mem, Mem &outmem,
                        uint32_t flags) {
@@ -1088,87 +1094,127 @@ static int spasgn_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int3
   if (nI < 0 || nJ < 0 || B->m != nI || B->n != nJ || A->dtype != B->dtype) return HS_EINVAL;
   if ((nI > 0 && !I) || (nJ > 0 && !J)) return HS_EINVAL;
   if (accumulate && A->dtype != HS_BOOL && add_sr != HS_PLUS_TIMES && add_sr != HS_MIN_PLUS) return HS_EINVAL;
+  if (!dtype_ok(A->dtype) || A->m < 0 || A->n < 0 || A->nnz < 0 || B->nnz < 0) return HS_EINVAL;
   const int vb = vbytes_of(A->dtype);
+  if ((A->m > 0 && !A->ptr) || (B->m > 0 && !B->ptr)) return HS_EINVAL;
+  if ((A->nnz > 0 && (!A->idx || (vb && !A->val))) || (B->nnz > 0 && (!B->idx || (vb && !B->val)))) return HS_EINVAL;
   const int64_t m = A->m, n = A->n;
+  if (nI > 0x7fffffffLL || nJ > 0x7fffffffLL || n > 0x7fffffffLL) return HS_EINVAL;
+  if (m > 0x7fffffffLL) return HS_EUNSUPPORTED;
+  const int64_t nnzA = m > 0 ? A->nnz : 0, nx = nI > 0 ? B->nnz : 0;
+  const int64_t nw = (nnzA + 31) / 32;
+  struct Small {  // device counters, read back in one copy
+    int flag[2];
+    unsigned long long viol[2];
+    long long dbg[2];
+    int64_t nnz, xtot;
+  };
+  Small *sb = mem.tmp<Small>(1);
+  Small *hb = (Small *)pinned(sizeof(Small));
   int32_t *rpos = mem.tmp<int32_t>(m > 0 ? m : 1);
   int32_t *cpos = mem.tmp<int32_t>(n > 0 ? n : 1);
-  int *flag = mem.tmp<int>(2);
-  int *hflag = (int *)pinned(8);
-  if (mem.failed || !hflag) return HS_ENOMEM;
-  CK(cudaMemsetAsync(flag, 0, 8, st));
-  launch_fill_i32(rpos, m, -1, st);
-  launch_fill_i32(cpos, n, -1, st);
-  launch_mark_positions(I, nI, m, rpos, flag, st);
-  launch_mark_positions(J, nJ, n, cpos, flag, st);
-  CK(cudaMemcpyAsync(hflag, flag, 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (hflag[0] & 1) return HS_EINVAL;
-  if (hflag[0] & 2) return HS_EDUP;
-
-  // R = sparse(I, 1:mb, 1, ma, mb) and Q = sparse(1:nb, J, 1, nb, na)
-  int64_t *Rp = mem.tmp<int64_t>(m + 1);
-  int32_t *Rj = mem.tmp<int32_t>(nI > 0 ? nI : 1);
-  int64_t *Qp = mem.tmp<int64_t>(nJ + 1);
-  int64_t *scan_tmp = mem.tmp<int64_t>(scan_tmp_elems((m > n ? m : n) + 1));
-  if (mem.failed) return HS_ENOMEM;
-  {
-    PhaseTimer t("spasgn_build", st);
-    CK(cudaMemsetAsync(Rp, 0, sizeof(int64_t), st));
-    launch_rows_from_pos(rpos, m, Rp, st);
-    launch_scan_i64(Rp, m + 1, scan_tmp, st);
-    launch_fill_from_pos(rpos, m, Rp, Rj, st);
-    launch_iota_i64(Qp, nJ + 1, st);
-  }
-  hs_mat R{HS_CSR, HS_BOOL, m, nI, nI, 0, Rp, Rj, nullptr, nullptr};
-  hs_mat Q{HS_CSR, HS_BOOL, nJ, n, nJ, 0, Qp, const_cast<int32_t *>(J), nullptr, nullptr};
-  hs_mat RB, X;
-  memset(&RB, 0, sizeof(RB));
-  memset(&X, 0, sizeof(X));
-  // the products feed the merge, which needs canonical rows
-  const uint32_t pf = flags & ~(HS_FLAG_VALIDATE | HS_FLAG_UNSORTED | HS_FLAG_PRUNE_ZEROS);
-  int e = spgemm_impl(HS_SELECT2ND, &R, B, &RB, mem, mem, pf);
-  if (!e) e = spgemm_impl(HS_SELECT1ST, &RB, &Q, &X, mem, mem, pf);
-  free_mat(&RB, mem);
-  if (e) {
-    free_mat(&X, mem);
-    return e;
-  }
-  // C = A .* not(S*A*T) + R*B*Q  (or A + R*B*Q for extend-add)
+  int64_t *XB = mem.tmp<int64_t>((size_t)m + 1);
+  int64_t *S = mem.tmp<int64_t>((size_t)(nw > 0 ? nw : 1));
+  uint32_t *keep = mem.tmp<uint32_t>((size_t)nw + 1);  // (K(q) at A's end may look at the word past the last)
+  int64_t *at = mem.tmp<int64_t>((size_t)(nx > 0 ? nx : 1));
+  int64_t *src = mem.tmp<int64_t>((size_t)(nx > 0 ? nx : 1));
+  int64_t *scan_tmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(m + 1 > nw ? m + 1 : nw));
+  if (mem.failed || !hb) return HS_ENOMEM;
   memset(C, 0, sizeof(*C));
   C->fmt = HS_CSR;
   C->dtype = A->dtype;
   C->m = m;
   C->n = n;
   C->ptr = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(m + 1));
-  if (!C->ptr) {
-    free_mat(&X, mem);
-    return HS_ENOMEM;
-  }
-  AsgnArgs aa{A->ptr, A->idx, A->val, X.ptr, X.idx, X.val, rpos, cpos, m, vb, accumulate, add_sr, A->dtype,
-              C->ptr, nullptr, nullptr};
-  int64_t *hnnz = (int64_t *)pinned(8);
-  {
+  if (!C->ptr) return HS_ENOMEM;
+  AsgnArgs aa{A->ptr, A->idx, A->val, B->val, cpos, m, n, nnzA, vb, accumulate, add_sr, A->dtype,
+              C->ptr, 0, nullptr, nullptr, sb->dbg};
+  AsgnX x{B->ptr, B->idx, I, J, nI, nJ, nx};
+  // everything up to C's offsets (xb: X's row offsets)
+  auto offsets = [&](const int64_t *xb) -> int {
     PhaseTimer t("spasgn_merge", st);
-    CK(cudaMemsetAsync(C->ptr, 0, sizeof(int64_t), st));
-    launch_asgn_count(aa, st);
-    launch_scan_i64(C->ptr, m + 1, scan_tmp, st);
+    CK(cudaMemsetAsync(keep, 0xff, sizeof(uint32_t) * ((size_t)nw + 1), st));
+    launch_asgn_keep(x, aa, I, nI, xb, at, src, keep, S, nw, st);
+    launch_scan_i64(S, nw, scan_tmp, st);
+    if (m > 0) launch_asgn_offsets(aa, xb, S, keep, st);
+    else CK(cudaMemsetAsync(C->ptr, 0, sizeof(int64_t), st));
+    CK(cudaMemcpyAsync(&sb->nnz, C->ptr + m, 8, cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemcpyAsync(&sb->xtot, xb + m, 8, cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemcpyAsync(hb, sb, sizeof(Small), cudaMemcpyDeviceToHost, st));
+    if (int e = check_launch()) return e;
+    CK(cudaStreamSynchronize(st));
+    return HS_OK;
+  };
+  {
+    PhaseTimer t("spasgn_build", st);
+    CK(cudaMemsetAsync(sb, 0, sizeof(Small), st));
+    CK(cudaMemsetAsync(rpos, 0xff, sizeof(int32_t) * (size_t)m, st));
+    CK(cudaMemsetAsync(cpos, 0xff, sizeof(int32_t) * (size_t)n, st));
+    launch_mark_positions(I, nI, m, rpos, sb->flag, st);
+    launch_mark_positions(J, nJ, n, cpos, sb->flag, st);
+    CK(cudaMemsetAsync(XB, 0, sizeof(int64_t) * (size_t)(m + 1), st));
+    launch_asgn_rows(x, m, n, XB, sb->viol, sb->dbg, st);
+    launch_scan_i64(XB, m + 1, scan_tmp, st);
   }
-  CK(cudaMemcpyAsync(hnnz, C->ptr + m, 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  C->nnz = *hnnz;
+  // (a bad or repeated index of I or J is known only after this: until then
+  // such indices are skipped or land inside the buffers)
+  if (int e = offsets(XB)) return e;
+  if (hb->flag[0] & 1) return HS_EINVAL;
+  if (hb->flag[0] & 2) return HS_EDUP;
+  auto internal = [&]() {
+    snprintf(t_detail, sizeof(t_detail), "index check %lld failed at %lld", hb->dbg[0], hb->dbg[1]);
+    return HS_EINTERNAL;
+  };
+  if (hb->dbg[0]) return internal();
+  hs_mat X;
+  memset(&X, 0, sizeof(X));
+  struct Guard {
+    hs_mat &x;
+    Mem &m;
+    ~Guard() { free_mat(&x, m); }
+  } guard{X, mem};
+  if (hb->viol[0] != hb->viol[1] || hb->xtot != nx) {
+    // X by the products R*B and (R*B)*Q, R = sparse(I, 1:mb, 1, ma, mb) and
+    // Q = sparse(1:nb, J, 1, nb, na)
+    int64_t *Rp = mem.tmp<int64_t>(m + 1);
+    int32_t *Rj = mem.tmp<int32_t>(nI > 0 ? nI : 1);
+    int64_t *Qp = mem.tmp<int64_t>(nJ + 1);
+    if (mem.failed) return HS_ENOMEM;
+    {
+      PhaseTimer t("spasgn_build", st);
+      CK(cudaMemsetAsync(Rp, 0, sizeof(int64_t), st));
+      launch_rows_from_pos(rpos, m, Rp, st);
+      launch_scan_i64(Rp, m + 1, scan_tmp, st);
+      launch_fill_from_pos(rpos, m, Rp, Rj, st);
+      launch_iota_i64(Qp, nJ + 1, st);
+    }
+    hs_mat R{HS_CSR, HS_BOOL, m, nI, nI, 0, Rp, Rj, nullptr, nullptr};
+    hs_mat Q{HS_CSR, HS_BOOL, nJ, n, nJ, 0, Qp, const_cast<int32_t *>(J), nullptr, nullptr};
+    hs_mat RB;
+    memset(&RB, 0, sizeof(RB));
+    // the products feed the merge, which needs canonical rows
+    const uint32_t pf = flags & ~(HS_FLAG_VALIDATE | HS_FLAG_UNSORTED | HS_FLAG_PRUNE_ZEROS);
+    int e = spgemm_impl(HS_SELECT2ND, &R, B, &RB, mem, mem, pf);
+    if (!e) e = spgemm_impl(HS_SELECT1ST, &RB, &Q, &X, mem, mem, pf);
+    free_mat(&RB, mem);
+    if (e) return e;
+    if (X.nnz > nx) return HS_EINTERNAL;
+    aa.Xv = X.val;
+    x = AsgnX{X.ptr, X.idx, nullptr, nullptr, m, n, X.nnz};
+    if (int e2 = offsets(X.ptr)) return e2;
+    if (hb->dbg[0]) return internal();
+  }
+  C->nnz = hb->nnz;
   C->idx = (int32_t *)outmem.raw(sizeof(int32_t) * (size_t)C->nnz);
   if (vb) C->val = outmem.raw((size_t)vb * (size_t)C->nnz);
-  if (!C->idx || (vb && !C->val)) {
-    free_mat(&X, mem);
-    return HS_ENOMEM;
-  }
+  if (!C->idx || (vb && !C->val)) return HS_ENOMEM;
+  aa.nnzC = C->nnz;
   aa.Cj = C->idx;
   aa.Cv = C->val;
   {
     PhaseTimer t("spasgn_merge", st);
-    launch_asgn_fill(aa, st);
+    launch_asgn_fill(x, aa, at, src, S, keep, st);
   }
-  free_mat(&X, mem);
   return check_launch();
 }
 
