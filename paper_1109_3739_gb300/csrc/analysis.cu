@@ -223,37 +223,73 @@ void launch_keep_nonzero(const void *v, int dtype, int64_t n, int64_t *keep, cud
 }
 
 // ---------------------------------------------------- B segment index
-// One warp per B row.  Rows longer than min_len take the next table row and
-// record, for every segment g = 0..nseg, the offset of their first entry with
-// column >= g*SEG_W (nseg gives the row length).  Entry p fills the segments
-// after its predecessor's up to its own; the last entry fills the rest.
-__global__ void k_build_bci(RightOp B, int nseg, int min_len, int64_t max_rows, int32_t *bci_id, int32_t *bci,
-                            int *counter) {
-  const int lane = lane_id();
-  const int64_t wpb = blockDim.x >> 5;
-  const int64_t stride = (int64_t)nseg + 1;
-  for (int64_t k = blockIdx.x * wpb + (threadIdx.x >> 5); k < B.m; k += (int64_t)gridDim.x * wpb) {
-    const int64_t b0 = B.p[k], b1 = B.p[k + 1];
-    const int64_t len = b1 - b0;
-    int t = -1;
-    if (len > min_len && lane == 0) {
-      t = atomicAdd(counter, 1);
-      if (t >= max_rows) t = -1;
+// Rows longer than min_len take the next table row and record, for every
+// segment g = 0..nseg, the offset of their first entry with column >=
+// g*SEG_W (nseg gives the row length).  Entry p fills the segments after its
+// predecessor's up to its own; the last entry fills the rest.  A block takes
+// 256 rows: a thread per row looks at its length, then a warp writes each
+// longer row, and the whole block each row of more than BCI_LONG entries (a
+// hub row of 4e4 entries walked by one warp set the kernel's time).
+constexpr int BCI_NT = 256, BCI_LONG = 2048;
+__device__ __forceinline__ void bci_row(const RightOp &B, int64_t b0, int len, int nseg, int32_t *row, int first,
+                                        int step) {
+  constexpr int U = 4;
+  for (int q0 = first; q0 < len; q0 += U * step) {
+    int c[U], cp[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = q0 + u * step;
+      c[u] = q < len ? __ldg(B.j + b0 + q) : 0;
+      cp[u] = q > 0 && q < len ? __ldg(B.j + b0 + q - 1) : -1;
     }
-    t = __shfl_sync(FULL, t, 0);
-    if (lane == 0) bci_id[k] = t;
-    if (t < 0) continue;
-    int32_t *row = bci + (int64_t)t * stride;
-    for (int64_t q = lane; q < len; q += 32) {
-      if (!HS_G(B.dbg, b0 + q < B.nnz, 53, b0 + q)) break;
-      const int c = B.j[b0 + q];
-      if (!HS_G(B.dbg, c >= 0 && c < B.n, 54, c)) break;
-      const int g = c / SEG_W;
-      const int gp = q ? B.j[b0 + q - 1] / SEG_W : -1;
-      for (int x = gp + 1; x <= g && x <= nseg; ++x) row[x] = (int32_t)q;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = q0 + u * step;
+      if (q >= len) break;
+      if (!HS_G(B.dbg, c[u] >= 0 && c[u] < B.n, 54, c[u])) continue;
+      const int g = c[u] / SEG_W;
+      const int gp = q ? (cp[u] >= 0 ? cp[u] / SEG_W : g) : -1;
+      for (int x = gp + 1; x <= g && x <= nseg; ++x) row[x] = q;
       if (q == len - 1)
-        for (int x = g + 1; x <= nseg; ++x) row[x] = (int32_t)len;
+        for (int x = g + 1; x <= nseg; ++x) row[x] = len;
     }
+  }
+}
+__global__ void __launch_bounds__(BCI_NT) k_build_bci(RightOp B, int nseg, int min_len, int64_t max_rows,
+                                                      int32_t *bci_id, int32_t *bci, int *counter) {
+  __shared__ int s_row[BCI_NT], s_long[BCI_NT], s_n, s_nlong;  // row within the block's 256
+  __shared__ int s_t[BCI_NT];                                  // its table row
+  const int64_t stride = (int64_t)nseg + 1;
+  for (int64_t k0 = (int64_t)blockIdx.x * BCI_NT; k0 < B.m; k0 += (int64_t)gridDim.x * BCI_NT) {
+    if (threadIdx.x == 0) s_n = s_nlong = 0;
+    __syncthreads();
+    const int64_t k = k0 + threadIdx.x;
+    if (k < B.m) {
+      const int64_t b0 = B.p[k], len = B.p[k + 1] - b0;
+      int t = -1;
+      if (len > min_len && len <= 0x7fffffffLL && HS_G(B.dbg, b0 >= 0 && b0 + len <= B.nnz, 53, b0)) {
+        t = atomicAdd(counter, 1);
+        if (t >= max_rows) t = -1;
+      }
+      bci_id[k] = t;
+      s_t[threadIdx.x] = t;
+      if (t >= 0) {
+        if (len > BCI_LONG) s_long[atomicAdd(&s_nlong, 1)] = threadIdx.x;
+        else s_row[atomicAdd(&s_n, 1)] = threadIdx.x;
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x >> 5; i < s_n; i += BCI_NT / 32) {
+      const int x = s_row[i];
+      const int64_t b0 = B.p[k0 + x];
+      bci_row(B, b0, (int)(B.p[k0 + x + 1] - b0), nseg, bci + s_t[x] * stride, lane_id(), 32);
+    }
+    for (int i = 0; i < s_nlong; ++i) {
+      const int x = s_long[i];
+      const int64_t b0 = B.p[k0 + x];
+      bci_row(B, b0, (int)(B.p[k0 + x + 1] - b0), nseg, bci + s_t[x] * stride, threadIdx.x, BCI_NT);
+    }
+    __syncthreads();
   }
 }
 
@@ -261,7 +297,7 @@ void launch_build_bci(const RightOp &B, int nseg, int min_len, int64_t max_rows,
                       int *counter, cudaStream_t st) {
   if (B.m <= 0) return;
   count_launch();
-  k_build_bci<<<grid_for(B.m, 8, 16), 256, 0, st>>>(B, nseg, min_len, max_rows, bci_id, bci, counter);
+  k_build_bci<<<grid_for(B.m, BCI_NT, 8), BCI_NT, 0, st>>>(B, nseg, min_len, max_rows, bci_id, bci, counter);
 }
 
 // one warp: exclusive scan of the NKEYS counters into offsets and cursors
@@ -580,84 +616,214 @@ void launch_plan_parts(const RowSet &A, const int *list, int count, const int32_
                                                        poff, units);
 }
 
-// One warp per unit: its row's A entries 32 at a time, each entry's B
-// segment inside the part from the segment index (or a binary search of a B
-// row without one), the non-empty ones compacted by ballot into the unit's
-// slice with the running product count as their exclusive prefix.  The
-// searches of many units run at once, so their latency is hidden here
-// instead of sitting on the numeric kernel's path.
+// The B segments of the units.  A warp takes `group` consecutive units; those
+// of one row are filled together, from one pass over the row's A entries, 32
+// at a time: a lane holds an entry's B row and the end of its last segment,
+// and every unit of the row takes the entry's next segment up to the unit's
+// last column (from the segment index, whose offsets of neighbouring
+// segments share a cache line, or by a short search of a B row without one),
+// the non-empty ones compacted by ballot.  Bound by the instructions per
+// (entry, unit) and the latency of the entry -> B row -> index chain: one
+// warp per unit went through the entries and B offsets again for each of a
+// row's units, and scanned the products of its segments, which the unit
+// kernel now does as it copies them.  The searches of many units run at
+// once, so their latency is hidden here instead of sitting on the numeric
+// kernel's path.  A row with more than PAIR_LONG entries of A is left to
+// k_build_pairs_long: a block per unit, four entries per thread at a time
+// (the few units of a product with 1e5-entry rows of A would keep one warp
+// each busy long after the others are done).
+constexpr int PAIR_NT = 256, PAIR_U = 4, PAIR_GROUP = 8;
+template <int AB> struct PairVal {
+  using T = typename std::conditional<AB == 8, unsigned long long, unsigned>::type;
+};
+// evict-first: the pairs are read once, later; B and the segment index stay
+// in L2 for this kernel and the unit kernel after it
 template <int AB>
-__global__ void k_build_pairs(RowSet A, RightOp B, HeavyUnit *units, int64_t nunits, const int32_t *bci_id,
-                              const int32_t *bci, int nseg, int64_t *pstart, int32_t *ppre, void *paval) {
-  using VT = typename std::conditional<AB == 8, unsigned long long, unsigned>::type;
+__device__ __forceinline__ void pair_put(int64_t at, int64_t s0, int len, typename PairVal<AB>::T av, int64_t *pseg,
+                                         void *paval) {
+  __stcs(reinterpret_cast<long long *>(pseg) + at, (long long)pair_pack(s0, len));
+  if constexpr (AB > 0) __stcs(reinterpret_cast<typename PairVal<AB>::T *>(paval) + at, av);
+}
+__device__ __forceinline__ bool unit_ok(const RowSet &A, const HeavyUnit &u, int nseg, int64_t ui) {
+  return HS_G(A.dbg, u.row >= 0 && u.row < A.nslots && u.seg_lo >= 0 && u.seg_lo < u.seg_hi && u.seg_hi <= nseg, 75,
+              ui);
+}
+// B row of A entry q (false: none), and its row of the segment index
+__device__ __forceinline__ bool pair_row(const RowSet &A, const RightOp &B, int64_t q, const int32_t *bci_id,
+                                         int64_t &base, int64_t &end, int &t) {
+  if (!HS_G(A.dbg, q >= 0 && q < A.nnz, 1, q)) return false;
+  const int k = __ldg(A.j + q);
+  if (!HS_G(A.dbg, k >= 0 && k < B.m, 2, k)) return false;
+  base = __ldg(B.p + k);
+  end = __ldg(B.p + k + 1);
+  t = bci_id ? __ldg(bci_id + k) : -1;
+  return HS_G(A.dbg, base >= 0 && base <= end && end <= B.nnz, 3, end);
+}
+// first entry of the B row at or after s whose segment is >= seg
+__device__ __forceinline__ int64_t pair_end(const RightOp &B, int64_t base, int64_t s, int64_t end, int t, int seg,
+                                            const int32_t *bci, int64_t bstride) {
+  if (t >= 0) return base + __ldg(bci + (int64_t)t * bstride + seg);
+  const int64_t x = (int64_t)seg * SEG_W;
+  return x > 0x7fffffffLL ? end : gallop_lower_bound(B.j, s, end, (int)x);
+}
+
+template <int AB>
+__global__ void __launch_bounds__(PAIR_NT) k_build_pairs(RowSet A, RightOp B, HeavyUnit *units, int64_t nunits,
+                                                         const int32_t *bci_id, const int32_t *bci, int nseg,
+                                                         int64_t *pseg, void *paval, int group) {
+  using VT = typename PairVal<AB>::T;
   const int lane = lane_id();
-  const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t bstride = (int64_t)nseg + 1;
-  for (int64_t ui = wid; ui < nunits; ui += nw) {
-    const HeavyUnit u = units[ui];
-    if (!HS_G(A.dbg, u.row >= 0 && u.row < A.nslots && u.seg_lo >= 0 && u.seg_lo < u.seg_hi && u.seg_hi <= nseg,
-              75, ui))
-      continue;
-    const int64_t lo = (int64_t)u.seg_lo * SEG_W, hi = (int64_t)u.seg_hi * SEG_W;
-    const int64_t q0 = A.p[u.row], q1 = A.p[u.row + 1];
-    int out = 0;
-    long long prod = 0;
-    for (int64_t qb = q0; qb < q1; qb += 32) {
-      const int64_t q = qb + lane;
-      int64_t s0 = 0, s1 = 0;
-      VT av = 0;
-      if (q < q1 && HS_G(A.dbg, q >= 0 && q < A.nnz, 1, q)) {
-        const int k = __ldg(A.j + q);
-        if (HS_G(A.dbg, k >= 0 && k < B.m, 2, k)) {
-          const int64_t base = __ldg(B.p + k), end = __ldg(B.p + k + 1);
-          const int t = bci_id ? __ldg(bci_id + k) : -1;
-          s0 = s1 = base;  // an empty B row: an empty segment at its start
-          if (t >= 0) {
-            s0 = base + __ldg(bci + (int64_t)t * bstride + u.seg_lo);
-            s1 = base + __ldg(bci + (int64_t)t * bstride + u.seg_hi);
-          } else if (end > base) {
-            s0 = lower_bound_col(B.j, base, end, (int)lo);
-            s1 = hi > 0x7fffffffLL ? end : lower_bound_col(B.j, s0, end, (int)hi);
-          }
-          if (!HS_G(A.dbg, base <= s0 && s0 <= s1 && s1 <= end, 65, s1)) s0 = s1 = 0;
-          if constexpr (AB > 0)
-            if (s1 > s0) av = __ldg(reinterpret_cast<const VT *>(A.v) + q);
-        }
-      }
-      const int len = (int)(s1 - s0);
-      const unsigned m = __ballot_sync(FULL, len > 0);
-      const int incl = warp_incl_scan(len);
-      if (len > 0) {
-        const int64_t at = u.poff + out + __popc(m & ((1u << lane) - 1u));
-        // evict-first: the pairs are read once, later; B and the segment
-        // index stay in L2 for this kernel and the unit kernel after it
-        __stcs(reinterpret_cast<long long *>(pstart) + at, (long long)s0);
-        __stcs(ppre + at, (int32_t)(prod + incl - len));
-        if constexpr (AB > 0) __stcs(reinterpret_cast<VT *>(paval) + at, av);
-      }
-      out += __popc(m);
-      prod += __shfl_sync(FULL, incl, 31);
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g * group < nunits; g += nw) {
+    const int64_t ua = g * group;
+    const int cnt = (int)min((int64_t)group, nunits - ua);
+    // lane j holds unit ua + j: its row (-1: skipped), segments and the next
+    // free place of its slice
+    int row = -1, slo = 0, shi = 0;
+    int64_t at = 0, poff = 0;
+    if (lane < cnt) {
+      const HeavyUnit u = units[ua + lane];
+      if (unit_ok(A, u, nseg, ua + lane)) row = u.row;
+      slo = u.seg_lo;
+      shi = u.seg_hi;
+      at = poff = u.poff;
     }
-    if (lane == 0) {
-      units[ui].npairs = out;
-      units[ui].nprod = HS_G(A.dbg, prod < 0x7fffffffLL, 76, ui) ? (int32_t)prod : 0;
+    for (int j0 = 0; j0 < cnt;) {
+      const int r = __shfl_sync(FULL, row, j0);
+      const unsigned same = __ballot_sync(FULL, lane >= j0 && lane < cnt && row == r) >> j0;
+      const int run = __ffs(~same) - 1;  // consecutive units of row r (group <= 8, so ~same is not 0)
+      const int j1 = j0 + run;
+      const int64_t q0 = r >= 0 ? A.p[r] : 0, q1 = r >= 0 ? A.p[r + 1] : 0;
+      if (q1 - q0 <= PAIR_LONG) {
+        const int lo0 = __shfl_sync(FULL, slo, j0);
+        for (int64_t qb = q0; qb < q1; qb += 32) {
+          const int64_t q = qb + lane;
+          int64_t base = 0, end = 0, s = 0;
+          int t = -1;
+          VT av = 0;
+          if (q < q1 && pair_row(A, B, q, bci_id, base, end, t)) {
+            s = lo0 ? pair_end(B, base, base, end, t, lo0, bci, bstride) : base;
+            if (!HS_G(A.dbg, s >= base && s <= end, 65, s)) s = end;
+            if constexpr (AB > 0)
+              if (s < end) av = __ldg(reinterpret_cast<const VT *>(A.v) + q);
+          }
+          for (int j = j0; j < j1; ++j) {
+            const int hi = __shfl_sync(FULL, shi, j);
+            const int64_t to = __shfl_sync(FULL, at, j);
+            int64_t e = s;
+            if (s < end) {
+              e = pair_end(B, base, s, end, t, hi, bci, bstride);
+              if (!HS_G(A.dbg, e >= s && e <= end, 65, e)) e = s;
+            }
+            const unsigned m = __ballot_sync(FULL, e > s);
+            if (e > s) pair_put<AB>(to + __popc(m & ((1u << lane) - 1u)), s, (int)(e - s), av, pseg, paval);
+            if (lane == j) at += __popc(m);
+            s = e;
+          }
+        }
+        if (lane >= j0 && lane < j1) units[ua + lane].npairs = (int32_t)(at - poff);
+      }
+      j0 = j1;
     }
   }
 }
 
+template <int AB>
+__global__ void __launch_bounds__(PAIR_NT) k_build_pairs_long(RowSet A, RightOp B, HeavyUnit *units, int64_t nunits,
+                                                              const int32_t *bci_id, const int32_t *bci, int nseg,
+                                                              int64_t *pseg, void *paval) {
+  using VT = typename PairVal<AB>::T;
+  constexpr int NW = PAIR_NT / 32;
+  __shared__ int s_long[PAIR_NT], s_n;
+  __shared__ int s_w[NW];
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const int64_t bstride = (int64_t)nseg + 1;
+  // units are dealt to the blocks one by one (a hub row's units are
+  // neighbours): block b looks at units b, b + gridDim, ...
+  for (int64_t v0 = 0; v0 * gridDim.x < nunits; v0 += PAIR_NT) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int64_t mine = (v0 + threadIdx.x) * gridDim.x + blockIdx.x;
+    if (mine < nunits) {
+      const HeavyUnit u = units[mine];
+      if (unit_ok(A, u, nseg, mine) && A.p[u.row + 1] - A.p[u.row] > PAIR_LONG)
+        s_long[atomicAdd(&s_n, 1)] = threadIdx.x;
+    }
+    __syncthreads();
+    const int n = s_n;
+    for (int i = 0; i < n; ++i) {
+      const int64_t vi = (v0 + s_long[i]) * gridDim.x + blockIdx.x;
+      const HeavyUnit u = units[vi];
+      const int64_t q0 = A.p[u.row], q1 = A.p[u.row + 1];
+      int out = 0;
+      for (int64_t qb = q0; qb < q1; qb += PAIR_U * PAIR_NT) {
+        int64_t s[PAIR_U];
+        int len[PAIR_U];
+        VT av[PAIR_U];
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < PAIR_U; ++k) {
+          const int64_t q = qb + k * PAIR_NT + threadIdx.x;
+          int64_t base = 0, end = 0;
+          int t = -1;
+          s[k] = 0;
+          len[k] = 0;
+          av[k] = 0;
+          if (q < q1 && pair_row(A, B, q, bci_id, base, end, t) && base < end) {
+            s[k] = u.seg_lo ? pair_end(B, base, base, end, t, u.seg_lo, bci, bstride) : base;
+            const int64_t e = pair_end(B, base, s[k], end, t, u.seg_hi, bci, bstride);
+            if (HS_G(A.dbg, base <= s[k] && s[k] <= e && e <= end, 65, e)) len[k] = (int)(e - s[k]);
+            if constexpr (AB > 0)
+              if (len[k] > 0) av[k] = __ldg(reinterpret_cast<const VT *>(A.v) + q);
+          }
+          c += len[k] > 0;
+        }
+        const int incl = warp_incl_scan(c);
+        if (lane == 31) s_w[warp] = incl;
+        __syncthreads();
+        int before = incl - c, all = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          before += w < warp ? s_w[w] : 0;
+          all += s_w[w];
+        }
+        int64_t to = u.poff + out + before;
+#pragma unroll
+        for (int k = 0; k < PAIR_U; ++k)
+          if (len[k] > 0) pair_put<AB>(to++, s[k], len[k], av[k], pseg, paval);
+        out += all;
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) units[vi].npairs = out;
+    }
+    __syncthreads();
+  }
+}
+
 void launch_build_pairs(const RowSet &A, const RightOp &B, HeavyUnit *units, int64_t nunits, const int32_t *bci_id,
-                        const int32_t *bci, int nseg, int a_bytes, int64_t *pstart, int32_t *ppre, void *paval,
+                        const int32_t *bci, int nseg, int a_bytes, int has_long, int64_t *pseg, void *paval,
                         cudaStream_t st) {
   if (nunits <= 0) return;
-  count_launch();
-  const int g = grid_for(nunits, 8, 16);
-  if (a_bytes == 8)
-    k_build_pairs<8><<<g, 256, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pstart, ppre, paval);
-  else if (a_bytes == 4)
-    k_build_pairs<4><<<g, 256, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pstart, ppre, paval);
-  else
-    k_build_pairs<0><<<g, 256, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pstart, ppre, paval);
+  // consecutive units per warp: as many as leave every resident warp a group
+  const int64_t warps = (int64_t)sm_count() * 40;
+  int group = (int)(nunits / warps);
+  group = group < 1 ? 1 : (group > PAIR_GROUP ? PAIR_GROUP : group);
+  const int g = grid_for((nunits + group - 1) / group, PAIR_NT / 32, 16);
+  const int gl = grid_for(nunits, 1, 4);
+#define HS_PAIRS(AB)                                                                                              \
+  do {                                                                                                            \
+    count_launch();                                                                                               \
+    k_build_pairs<AB><<<g, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval, group);         \
+    if (has_long) {                                                                                               \
+      count_launch();                                                                                             \
+      k_build_pairs_long<AB><<<gl, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval);        \
+    }                                                                                                             \
+  } while (0)
+  if (a_bytes == 8) HS_PAIRS(8);
+  else if (a_bytes == 4) HS_PAIRS(4);
+  else HS_PAIRS(0);
+#undef HS_PAIRS
 }
 
 }  // namespace hs

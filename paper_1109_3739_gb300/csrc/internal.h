@@ -237,7 +237,7 @@ struct alignas(16) HeavyUnit {
   int64_t done;
   int64_t poff;    // the unit's slice of the pair arrays (room for every A entry of its row)
   int32_t npairs;  // A entries with products in the part (the slice's used length)
-  int32_t nprod;   // products in the part
+  int32_t pad;
   int64_t out;     // position in C of the part's first entry (C's row offset + done)
   int64_t lofs;    // position of the part's first column in the sorted-list pool
 };
@@ -262,12 +262,18 @@ void launch_plan_parts(const RowSet &A, const int *list, int count, const int32_
                        const int64_t *loff, const int64_t *Cp, int nseg, int caph, int span, const int64_t *off,
                        const int64_t *poff, HeavyUnit *units, cudaStream_t st);
 // Each unit's B segments: for every A entry of its row whose B row has
-// entries inside the part's columns, (segment start, exclusive prefix of the
-// products, the entry's value when the semiring reads it), compacted into the
-// unit's slice; sets npairs and nprod.  a_bytes: width of A's values to copy
-// (0: none).
+// entries inside the part's columns, (segment start and length in one word,
+// the entry's value when the semiring reads it), compacted into the unit's
+// slice; sets npairs.  A part spans at most 2^17 columns, so a length fits 24
+// bits.  a_bytes: width of A's values to copy (0: none); has_long: some row
+// of A holds more than PAIR_LONG entries.
+constexpr int PAIR_LONG = 1024;
+__host__ __device__ constexpr int64_t pair_pack(int64_t start, int len) { return start << 24 | (int64_t)len; }
+__host__ __device__ constexpr int64_t pair_start(int64_t x) { return x >> 24; }
+__host__ __device__ constexpr int pair_len(int64_t x) { return (int)(x & 0xffffff); }
+static_assert(HU_SPAN_SEGS * SEG_W < (1 << 24), "a segment's length fits its word");
 void launch_build_pairs(const RowSet &A, const RightOp &B, HeavyUnit *units, int64_t nunits, const int32_t *bci_id,
-                        const int32_t *bci, int nseg, int a_bytes, int64_t *pstart, int32_t *ppre, void *paval,
+                        const int32_t *bci, int nseg, int a_bytes, int has_long, int64_t *pseg, void *paval,
                         cudaStream_t st);
 
 // numeric_*.cu
@@ -296,9 +302,9 @@ struct NumArgs {
   int64_t nunits;
   int *udyn;              // the unit kernel's work counter
   int lists_partial;      // with units: some heavy rows have no list (the row kernel takes them)
-  const int64_t *pstart;  // units' B segments (launch_build_pairs)
-  const int32_t *ppre;
+  const int64_t *pseg;    // units' B segments (launch_build_pairs)
   const void *paval;
+  int pair_long;          // some row of A holds more than PAIR_LONG entries
   int pair_abytes;        // width of the left values the pairs carry (0: none)
   int unit_kb;            // the units' value capacity in KB (16 or 32): which unit kernel runs
 };

@@ -665,9 +665,9 @@ __global__ void __launch_bounds__(HV_NT, 2) k_num_heavy(NumArgs a) {
 // row's parts run on many SMs at once and no row's length sets the kernel's
 // tail.  Everything a unit reads that depends on other data has been laid out
 // before the kernel runs: the part's slice of the row's sorted column list
-// (written by the symbolic pass) and the part's B segments with their product
-// prefix and left value (launch_build_pairs, which does the segment searches
-// for all units in bulk).  A unit copies both into shared memory with
+// (written by the symbolic pass) and the part's B segments with their left
+// values (launch_build_pairs, which does the segment searches for all units
+// in bulk).  A unit copies both into shared memory with
 // cp.async, then: the list slice is written as C's columns and gives the
 // part's occupancy bitmap and word ranks; the products add their value at
 // rank(col) = wpre[word] + popcount(bits below col), spread evenly over the
@@ -679,6 +679,7 @@ constexpr int HU_NT = 256;
 constexpr int HU_WMAX = HU_SPAN_SEGS * SEG_W;
 constexpr int HU_WORDS = HU_WMAX / 32;
 constexpr int HU_PB = 256;  // B segments copied per batch
+static_assert(HU_PB == HU_NT, "a segment per thread in the batch's scan");
 // as unit_part_cap(): KB kilobytes of values, at least one segment's SEG_W outputs
 template <typename T, int KB> constexpr int unit_cap() {
   return vbytes<T>() == 0 ? 65536 : (KB * 1024 / vbytes<T>() > SEG_W ? KB * 1024 / vbytes<T>() : SEG_W);
@@ -691,8 +692,8 @@ template <typename T, int KB> struct UnitSmem {
   static constexpr size_t VBYTES = ((size_t)CAP * (vbytes<T>() > 4 ? vbytes<T>() : 4) + 32 + 15) & ~(size_t)15;
   alignas(16) unsigned char vals_raw[VBYTES];
   alignas(16) unsigned bitmap[HU_WORDS];  // all zero at every unit's start
-  alignas(16) int64_t sbeg[HU_PB + 4];   // B segment starts (+ copy room)
-  alignas(16) int excl[HU_PB + 8];       // their product prefix, then the batch's end
+  alignas(16) int64_t seg[HU_PB + 4];    // B segments as they were laid out (+ copy room), then their starts
+  int excl[HU_PB + 1];                   // their product prefix, then the batch's total
   alignas(16) unsigned char aval_raw[(HU_PB + 4) * (vbytes<T>() > 4 ? 8 : 4) + 16];
   uint16_t wpre[HU_WORDS];                // set bits before word w within the part
   int wtmp[33];
@@ -731,7 +732,7 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
     const bool ok = HS_G(dbg, u.seg_lo >= 0 && u.seg_lo < u.seg_hi && u.seg_hi <= nseg &&
                                   u.seg_hi - u.seg_lo <= HU_SPAN_SEGS, 72, u.seg_lo) &&
                     HS_G(dbg, u.pc > 0 && u.pc <= CAP, 73, u.pc) &&
-                    HS_G(dbg, u.npairs >= 0 && u.nprod >= 0 && u.out >= 0 && u.lofs >= 0, 77, u.npairs);
+                    HS_G(dbg, u.npairs >= 0 && u.out >= 0 && u.lofs >= 0, 77, u.npairs);
     if (ok) {
       const int lo = u.seg_lo * SEG_W;
       const int hi = (int)min((int64_t)u.seg_hi * SEG_W, n);
@@ -742,8 +743,7 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
         // the list slice and the first batch of B segments, copied at once
         const int nb0 = u.npairs < HU_PB ? u.npairs : HU_PB;
         const int lofb = async_copy16(sm.vals_raw, Lp, (int64_t)pc * 4, tid, HU_NT) >> 2;
-        const int sofb = async_copy16(sm.sbeg, a.pstart + u.poff, (int64_t)nb0 * 8, tid, HU_NT) >> 3;
-        const int eofb = async_copy16(sm.excl, a.ppre + u.poff, (int64_t)nb0 * 4, tid, HU_NT) >> 2;
+        const int sofb = async_copy16(sm.seg, a.pseg + u.poff, (int64_t)nb0 * 8, tid, HU_NT) >> 3;
         int aofb = 0;
         if constexpr (SR::needs_a)
           aofb = async_copy16(sm.aval_raw, reinterpret_cast<const T *>(a.paval) + u.poff,
@@ -768,23 +768,35 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
         HeavyAdd<SR> add_val{sm.bitmap, sm.wpre, vals, lo, (unsigned)(hi - lo), pc, a.err, dbg};
         for (int pb = 0; pb < u.npairs; pb += HU_PB) {
           const int nb = min(HU_PB, u.npairs - pb);
-          int so = sofb, eo = eofb, ao = aofb;
+          int so = sofb, ao = aofb;
           if (pb > 0) {  // the next batch (rows with many A entries)
             __syncthreads();
-            so = async_copy16(sm.sbeg, a.pstart + u.poff + pb, (int64_t)nb * 8, tid, HU_NT) >> 3;
-            eo = async_copy16(sm.excl, a.ppre + u.poff + pb, (int64_t)nb * 4, tid, HU_NT) >> 2;
+            so = async_copy16(sm.seg, a.pseg + u.poff + pb, (int64_t)nb * 8, tid, HU_NT) >> 3;
             if constexpr (SR::needs_a)
               ao = async_copy16(sm.aval_raw, reinterpret_cast<const T *>(a.paval) + u.poff + pb,
                                 (int64_t)nb * sizeof(T), tid, HU_NT) / (int)sizeof(T);
             async_copy_wait();
-            __syncthreads();  // every copy has landed (the batch end below may share a copied piece)
+            __syncthreads();
           }
-          int *ex = sm.excl + eo;
-          if (tid == 0) ex[nb] = pb + nb < u.npairs ? __ldg(a.ppre + u.poff + pb + nb) : u.nprod;
+          // a segment per thread: its start, and its products' prefix over the batch
+          const int64_t sg = tid < nb ? sm.seg[so + tid] : 0;
+          const int len = pair_len(sg);
+          const int incl = warp_incl_scan(len);
+          if (lane == 31) sm.wtmp[tid >> 5] = incl;
           __syncthreads();
-          const int base = ex[0];
-          cta_expand_staged<SR, 4, 32>(B, sm.sbeg + so, ex, reinterpret_cast<const T *>(sm.aval_raw) + ao, nb,
-                                       ex[nb] - base, add_val, base);
+          int before = incl - len, total = 0;
+#pragma unroll
+          for (int w = 0; w < HU_NT / 32; ++w) {
+            const int x = sm.wtmp[w];
+            before += w < (tid >> 5) ? x : 0;
+            total += x;
+          }
+          sm.seg[tid] = pair_start(sg);  // (every thread has read its word)
+          sm.excl[tid] = before;
+          if (tid == 0) sm.excl[nb] = total;  // (thread nb writes the same value: its segment is empty)
+          __syncthreads();
+          cta_expand_staged<SR, 4, 32>(B, sm.seg, sm.excl, reinterpret_cast<const T *>(sm.aval_raw) + ao, nb, total,
+                                       add_val);
         }
         __syncthreads();
         // values in column order; the part's bitmap words cleared for the next unit

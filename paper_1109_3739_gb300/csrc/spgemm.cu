@@ -472,6 +472,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   int key_off[NKEYS + 1];
   memcpy(key_off, hb->key_off, sizeof(key_off));
   const int nhist = hb->nhist;
+  const int pair_long = hb->stats[2] > (unsigned long long)PAIR_LONG;  // (read before hb is copied to again)
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
 
   // A entries whose B row is empty make no products.  When they are most of
@@ -670,12 +671,10 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
 
   // ---- numeric
   // heavy bin: units, planned from the segment counts of the rows with lists
-  // and, for semirings with values, each unit's B segments (start, product
-  // prefix, left value) laid out by launch_build_pairs once the segment
-  // index exists (below)
+  // and, for semirings with values, each unit's B segments (place and left
+  // value) laid out by launch_build_pairs once the segment index exists (below)
   HeavyUnit *units = nullptr;
-  int64_t *pstart = nullptr;
-  int32_t *ppre = nullptr;
+  int64_t *pseg = nullptr;
   void *paval = nullptr;
   const int64_t nunits = pcnt ? hb->nunits : 0;
   const int64_t npcap = pcnt ? hb->npcap : 0;
@@ -684,10 +683,9 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   if (nheavy > 0 && nunits > 0) {
     units = mem.tmp<HeavyUnit>((size_t)nunits);
     if (units && vb) {  // 16 bytes of slack each: the units copy their slices in 16-byte pieces
-      pstart = (int64_t *)mem.tmp<char>((size_t)npcap * 8 + 16);
-      ppre = (int32_t *)mem.tmp<char>((size_t)npcap * 4 + 16);
+      pseg = (int64_t *)mem.tmp<char>((size_t)npcap * 8 + 16);
       paval = a_bytes ? (void *)mem.tmp<char>((size_t)npcap * a_bytes + 16) : nullptr;
-      if (!pstart || !ppre || (a_bytes && !paval)) units = nullptr;
+      if (!pseg || (a_bytes && !paval)) units = nullptr;
     }
     mem.failed = false;  // optional, as above
     if (units) {
@@ -712,7 +710,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     if (int e = build_bci()) return e;
   if (units && vb) {
     PhaseTimer t("heavy_pairs", st);
-    launch_build_pairs(rs, rb, units, nunits, bci_id, bci, nseg, a_bytes, pstart, ppre, paval, st);
+    launch_build_pairs(rs, rb, units, nunits, bci_id, bci, nseg, a_bytes, pair_long, pseg, paval, st);
     if (int e = phase_check("heavy_pairs", st, sb->dbg)) return e;
   }
   NumArgs na{rs, rb,   f,    nullptr, 0,    Cp,    C->idx, C->val, hslot,
@@ -722,10 +720,10 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   na.nunits = units ? nunits : 0;
   na.udyn = &sb->dyn[2];
   na.lists_partial = lists_partial ? 1 : 0;
-  na.pstart = pstart;
-  na.ppre = ppre;
+  na.pseg = pseg;
   na.paval = paval;
   na.pair_abytes = a_bytes;
+  na.pair_long = pair_long;
   na.unit_kb = bins.unit_kb;
   const char *names[NUM_KINDS] = {"numeric_tiny",   "numeric_warp_s", "numeric_warp",   "numeric_mid_s",
                                   "numeric_mid",    "numeric_large_s", "numeric_large", "numeric_sort_xs",
@@ -1273,10 +1271,10 @@ int hs_plan_execute(const hs_plan *P, const void *A_val, const void *B_val, void
   na.Cv = C_val;
   CK(cudaMemsetAsync(P->dyn, 0, 2 * sizeof(int), st));  // the heavy rows' and units' counters
   // the heavy units' B segments carry A's values: laid out again from the new ones
-  if (na.units && na.pstart && na.nunits > 0)
+  if (na.units && na.pseg && na.nunits > 0)
     launch_build_pairs(na.A, na.B, const_cast<HeavyUnit *>(na.units), na.nunits, na.bci_id, na.bci, na.nseg,
-                       na.pair_abytes, const_cast<int64_t *>(na.pstart), const_cast<int32_t *>(na.ppre),
-                       const_cast<void *>(na.paval), st);
+                       na.pair_abytes, na.pair_long, const_cast<int64_t *>(na.pseg), const_cast<void *>(na.paval),
+                       st);
   for (int kind = 0; kind < NUM_KINDS; ++kind) {
     if (P->count[kind] <= 0) continue;
     na.list = P->list + P->off[kind];
