@@ -38,103 +38,145 @@ static int grid_for(int64_t items, int per_block, int max_per_sm) {
   return (int)(g < 1 ? 1 : g);
 }
 
-// ------------------------------------------------------------------ flops
-// stats[0] += total flops, stats[1] = max row flops, stats[2] = max row nnz
-// of A, stats[3] += min(f, n) over rows of the symbolic heavy bin
-__global__ void k_flops(RowSet A, RightOp B, int64_t *f, int *key_cnt, unsigned long long *stats, BinCfg bins) {
-  __shared__ int hist[NKEYS];
-  __shared__ unsigned long long blk_tot, blk_max, blk_amax, blk_heavy;
-  for (int i = threadIdx.x; i < NKEYS; i += blockDim.x) hist[i] = 0;
-  if (threadIdx.x == 0) blk_tot = blk_max = blk_amax = blk_heavy = 0;
+// ------------------------------------------------------- tiles and last block
+// Inclusive scan of NT*PER values held PER to a thread, value u of thread x at
+// position u*NT + x; s_tot holds PER*NT/32 words (64).  Returns the total.
+// One barrier; the caller separates two uses of s_tot.
+constexpr int TL_NT = 256, TL_PER = 8, TL_TILE = TL_NT * TL_PER, TL_NW = TL_NT / 32;
+static_assert(TL_PER * TL_NW == 64, "two warp totals per lane");
+__device__ __forceinline__ long long tile_scan(long long (&v)[TL_PER], long long *s_tot) {
+  const int lane = lane_id(), w = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    v[u] = warp_incl_scan(v[u]);
+    if (lane == 31) s_tot[u * TL_NW + w] = v[u];
+  }
   __syncthreads();
+  const long long x0 = s_tot[lane], x1 = s_tot[lane + 32];
+  const long long i0 = warp_incl_scan(x0), t0 = __shfl_sync(FULL, i0, 31);
+  const long long i1 = warp_incl_scan(x1) + t0;
+  const long long e0 = i0 - x0, e1 = i1 - x1;
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) v[u] += __shfl_sync(FULL, u < 4 ? e0 : e1, (u * TL_NW + w) & 31);
+  return __shfl_sync(FULL, i1, 31);
+}
+// True in every thread of the block that finishes last (its reads then see
+// what all blocks wrote before).
+__device__ __forceinline__ bool last_block(int *ticket, int *s_flag) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) *s_flag = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!*s_flag) return false;
+  __threadfence();
+  return true;
+}
+// one warp: exclusive scan of the NKEYS counters into offsets and cursors
+__device__ __forceinline__ void key_offsets(const int *cnt, int *off, int *cur) {
   const int lane = lane_id();
-  const int64_t wpb = blockDim.x >> 5;
-  unsigned long long my_tot = 0, my_max = 0, my_amax = 0, my_heavy = 0;
-  for (int64_t r = blockIdx.x * wpb + (threadIdx.x >> 5); r < A.nslots; r += (int64_t)gridDim.x * wpb) {
-    const int64_t q0 = A.p[r], q1 = A.p[r + 1];
-    long long s = 0;
-    for (int64_t q = q0 + lane; q < q1; q += 32) {
-      if (!HS_G(A.dbg, q >= 0 && q < A.nnz, 50, q)) break;
-      const int k = A.j[q];
-      if (HS_G(A.dbg, k >= 0 && k < B.m, 51, k)) s += B.p[k + 1] - B.p[k];
-    }
-    s = warp_sum(s);
-    if (lane == 0) {
-      f[r] = s;
-      const int key = sym_key(s, bins);
-      if (key) atomicAdd(hist + key, 1);
-      if (key >= KEY_HEAVY) my_heavy += (unsigned long long)min((int64_t)s, B.n);
-      my_tot += (unsigned long long)s;
-      my_max = max(my_max, (unsigned long long)s);
-      my_amax = max(my_amax, (unsigned long long)(q1 - q0));
-    }
-  }
-  if (lane == 0) {
-    atomicAdd(&blk_tot, my_tot);
-    atomicMax(&blk_max, my_max);
-    atomicMax(&blk_amax, my_amax);
-    atomicAdd(&blk_heavy, my_heavy);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < NKEYS; i += blockDim.x)
-    if (hist[i]) atomicAdd(key_cnt + i, hist[i]);
-  if (threadIdx.x == 0) {
-    atomicAdd(stats + 0, blk_tot);
-    atomicMax(stats + 1, blk_max);
-    atomicMax(stats + 2, blk_amax);
-    atomicAdd(stats + 3, blk_heavy);
-  }
+  const int a = __ldcg(cnt + 2 * lane), b = __ldcg(cnt + 2 * lane + 1);
+  const int incl = warp_incl_scan(a + b);
+  const int ex = incl - a - b;
+  off[2 * lane] = ex;
+  off[2 * lane + 1] = ex + a;
+  cur[2 * lane] = ex;
+  cur[2 * lane + 1] = ex + a;
+  if (lane == 31) off[NKEYS] = incl;
 }
+static_assert(NKEYS == 64, "key_offsets assumes 64 keys");
 
-void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, int *key_cnt, unsigned long long *stats,
-                  const BinCfg &bins, cudaStream_t st) {
-  if (A.nslots == 0) return;
-  count_launch();
-  k_flops<<<grid_for(A.nslots, 8, 16), 256, 0, st>>>(A, B, f, key_cnt, stats, bins);
-}
-
-// ------------------------------------------------ flat products per entry
-// The same counts, computed per A entry instead of per row, so that no row
-// is walked by one warp: s[q - lo] = nnz(B(A.j[q], :)) for q in [lo, hi) =
-// [A.p[0], A.p[nslots]); zeros[0] counts the entries whose B row is empty
-// (they make no product).  After an inclusive scan S of s, a row's count is
-// S[q1 - 1 - lo] - S[q0 - 1 - lo].
-__global__ void k_entry_flops(RowSet A, RightOp B, int64_t *s, unsigned long long *zeros) {
-  // offsets are trusted only as far as s's length (A.nnz entries)
-  const int64_t lo = A.p[0], hi = min(A.p[A.nslots], lo + A.nnz);
+// ------------------------------------------------------------------ flops
+// f[r] = sum over the row's entries of nnz(B(A.j[q], :)), f zeroed before.
+// A block takes TL_TILE consecutive entries of A, so that a hub row costs what
+// its entries cost: their counts are scanned in shared memory and every row
+// that has entries in the tile takes the difference of two scanned values (a
+// row that crosses a tile's border adds its parts by atomics).  The rows at
+// the tile's ends are found by a search of the offsets while the entries are
+// on their way.  One read of A's columns and B's offsets and no array of
+// counts per entry, which was written and passed over four times: the whole
+// analysis of R-MAT scale 20 (8.2M entries) 0.22 -> 0.10 ms, of a 128^3
+// Galerkin product (10.4M entries) 0.26 -> 0.14 ms; bound by the latency of
+// column -> offset, not by its 0.2 GB.  zeros counts the entries
+// whose B row is empty (they make no product).
+__global__ void __launch_bounds__(TL_NT) k_entry_flops(RowSet A, RightOp B, int64_t *f, unsigned long long *zeros) {
+  __shared__ long long S[TL_TILE], s_tot[64];
+  __shared__ int64_t s_row[2];
+  // offsets are trusted only inside A's arrays
+  const int64_t lo = max(A.p[0], (int64_t)0), hi = min(A.p[A.nslots], A.nnz);
+  const int64_t t0 = lo + (int64_t)blockIdx.x * TL_TILE, t1 = min(t0 + TL_TILE, hi);
+  if (t0 >= hi) return;
+  long long v[TL_PER];
   int z = 0;
-  for (int64_t q = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < hi;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int k = A.j[q];
-    const int64_t v = HS_G(A.dbg, k >= 0 && k < B.m, 52, k) ? B.p[k + 1] - B.p[k] : 0;
-    s[q - lo] = v;
-    z += v == 0;
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t q = t0 + u * TL_NT + threadIdx.x;
+    const int k = q < t1 ? A.j[q] : -1;
+    v[u] = 0;
+    if (q < t1 && HS_G(A.dbg, k >= 0 && k < B.m, 52, k)) v[u] = B.p[k + 1] - B.p[k];
+    z += q < t1 && v[u] == 0;
   }
+  if (threadIdx.x < 64) {  // the rows that hold the tile's first and last entry
+    const int which = threadIdx.x >> 5;
+    const int64_t r = warp_upper_bound(A.p, A.nslots + 1, which ? t1 - 1 : t0) - 1;
+    if (lane_id() == 0) s_row[which] = r;
+  }
+  tile_scan(v, s_tot);
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) S[u * TL_NT + threadIdx.x] = v[u];
   z = warp_sum(z);
   if (lane_id() == 0 && z) atomicAdd(zeros, (unsigned long long)z);
+  __syncthreads();
+  const int64_t r0 = max(s_row[0], (int64_t)0), r1 = min(s_row[1], A.nslots - 1);
+  auto put = [&](int64_t r) {
+    const int64_t q0 = A.p[r], q1 = A.p[r + 1];
+    const int64_t a = max(q0, t0), b = min(q1, t1);
+    if (a >= b) return;
+    const long long x = S[b - 1 - t0] - (a > t0 ? S[a - 1 - t0] : 0);
+    if (q0 >= t0 && q1 <= t1) f[r] = x;
+    else atomicAdd(reinterpret_cast<unsigned long long *>(f + r), (unsigned long long)x);
+  };
+  if (r1 - r0 < 8 * TL_TILE) {
+    for (int64_t r = r0 + threadIdx.x; r <= r1; r += TL_NT) put(r);
+  } else {  // far more rows than entries (most are empty): every entry looks for its row, its first entry reports it
+    for (int64_t q = t0 + threadIdx.x; q < t1; q += TL_NT) {
+      int64_t l = r0, h = r1 + 1;  // last row that starts at or before q
+      while (h - l > 1) {
+        const int64_t mid = (l + h) >> 1;
+        if (A.p[mid] <= q) l = mid;
+        else h = mid;
+      }
+      if (max(A.p[l], t0) == q) put(l);
+    }
+  }
+}
+void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, unsigned long long *zeros, cudaStream_t st) {
+  if (A.nslots == 0 || A.nnz == 0) return;
+  count_launch();
+  k_entry_flops<<<(unsigned)((A.nnz + TL_TILE - 1) / TL_TILE), TL_NT, 0, st>>>(A, B, f, zeros);
 }
 
-// thread per row: f from the scanned entry counts, then the row's key and
-// the statistics k_flops gathers
-__global__ void k_row_flops(RowSet A, const int64_t *S, int64_t *f, int *key_cnt, unsigned long long *stats,
-                            BinCfg bins, int64_t bn) {
-  __shared__ int hist[NKEYS];
+// Rows per key, and (the last block) the keys' offsets.  stats[0] += total
+// flops, stats[1] = max row flops, stats[2] = max row nnz of A, stats[3] +=
+// min(f, n) over rows of the symbolic heavy bin.  Cnt (CSR only): the output
+// counts, all set to zero here.
+__global__ void __launch_bounds__(TL_NT) k_row_keys(RowSet A, const int64_t *f, int64_t *cnt, BinCounters c,
+                                                    unsigned long long *stats, BinCfg bins, int64_t bn) {
+  __shared__ int hist[NKEYS], s_last;
   for (int i = threadIdx.x; i < NKEYS; i += blockDim.x) hist[i] = 0;
   __syncthreads();
-  const int64_t lo = A.p[0], len = min(A.p[A.nslots] - lo, A.nnz);
   unsigned long long my_tot = 0, my_max = 0, my_amax = 0, my_heavy = 0;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < A.nslots;
        r += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q0 = min(max(A.p[r] - lo, (int64_t)0), len), q1 = min(max(A.p[r + 1] - lo, (int64_t)0), len);
-    const int64_t fr = q1 > q0 ? S[q1 - 1] - (q0 > 0 ? S[q0 - 1] : 0) : 0;
-    f[r] = fr;
+    const int64_t fr = f[r];
+    if (cnt) cnt[r + 1] = 0;
     const int key = sym_key(fr, bins);
     if (key) atomicAdd(hist + key, 1);
     if (key >= KEY_HEAVY) my_heavy += (unsigned long long)min(fr, bn);
     my_tot += (unsigned long long)fr;
     my_max = max(my_max, (unsigned long long)fr);
-    my_amax = max(my_amax, (unsigned long long)(q1 - q0));
+    my_amax = max(my_amax, (unsigned long long)max(A.p[r + 1] - A.p[r], (int64_t)0));
   }
+  if (cnt && blockIdx.x == 0 && threadIdx.x == 0) cnt[0] = 0;
   my_tot = warp_sum(my_tot);
   my_heavy = warp_sum(my_heavy);
   my_max = warp_max(my_max);
@@ -147,30 +189,26 @@ __global__ void k_row_flops(RowSet A, const int64_t *S, int64_t *f, int *key_cnt
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NKEYS; i += blockDim.x)
-    if (hist[i]) atomicAdd(key_cnt + i, hist[i]);
+    if (hist[i]) atomicAdd(c.cnt + i, hist[i]);
+  if (last_block(c.ticket, &s_last) && threadIdx.x < 32) key_offsets(c.cnt, c.off, c.cur);
 }
-
-void launch_entry_flops(const RowSet &A, const RightOp &B, int64_t *s, unsigned long long *zeros,
-                        cudaStream_t st) {
-  if (A.nslots == 0 || A.nnz == 0) return;
-  count_launch();
-  k_entry_flops<<<grid_for(A.nnz, 256, 8), 256, 0, st>>>(A, B, s, zeros);
-}
-void launch_row_flops(const RowSet &A, const int64_t *S, int64_t *f, int *key_cnt, unsigned long long *stats,
-                      const BinCfg &bins, int64_t bn, cudaStream_t st) {
+void launch_row_keys(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCounters &c, unsigned long long *stats,
+                     const BinCfg &bins, int64_t bn, cudaStream_t st) {
   if (A.nslots == 0) return;
   count_launch();
-  k_row_flops<<<grid_for(A.nslots, 256, 8), 256, 0, st>>>(A, S, f, key_cnt, stats, bins, bn);
+  k_row_keys<<<grid_for(A.nslots, TL_NT, 4), TL_NT, 0, st>>>(A, f, cnt, c, stats, bins, bn);
 }
 
 // Dropping the A entries whose B row is empty (their products are none, so
-// C is unchanged): keep[q - lo] = 1 where s > 0, recovered from the scanned
-// counts; after an inclusive scan K of keep, entry q goes to K[q - lo] - 1
-// and row r starts at K[A.p[r] - 1 - lo].
-__global__ void k_keep_flags(RowSet A, const int64_t *S, int64_t *keep) {
-  const int64_t n = min(A.p[A.nslots] - A.p[0], A.nnz);
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-    keep[x] = (S[x] - (x > 0 ? S[x - 1] : 0)) > 0;
+// C is unchanged): keep[q - lo] = 1 where nnz(B(A.j[q], :)) > 0; after an
+// inclusive scan K of keep, entry q goes to K[q - lo] - 1 and row r starts at
+// K[A.p[r] - 1 - lo].
+__global__ void k_keep_flags(RowSet A, RightOp B, int64_t *keep) {
+  const int64_t lo = A.p[0], n = min(A.p[A.nslots] - lo, A.nnz);
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+    const int k = A.j[lo + x];
+    keep[x] = HS_G(A.dbg, k >= 0 && k < B.m, 52, k) && B.p[k + 1] != B.p[k];
+  }
 }
 __global__ void k_compact_entries(RowSet A, const int64_t *K, int32_t *j2, void *v2, int vb) {
   const int64_t lo = A.p[0], n = min(A.p[A.nslots] - lo, A.nnz);
@@ -197,10 +235,10 @@ void launch_compact_by_keep(const RowSet &A, const int64_t *K, int32_t *j2, void
   count_launch();
   k_compact_offsets<<<grid_for(A.nslots + 1, 256, 8), 256, 0, st>>>(A, K, p2);
 }
-void launch_compact_a(const RowSet &A, const int64_t *S, int64_t *keep, int64_t *scan_tmp, int32_t *j2, void *v2,
+void launch_compact_a(const RowSet &A, const RightOp &B, int64_t *keep, int64_t *scan_tmp, int32_t *j2, void *v2,
                       int vb, int64_t *p2, cudaStream_t st) {
   count_launch();
-  k_keep_flags<<<grid_for(A.nnz, 256, 8), 256, 0, st>>>(A, S, keep);
+  k_keep_flags<<<grid_for(A.nnz, 256, 8), 256, 0, st>>>(A, B, keep);
   launch_scan_i64(keep, A.nnz, scan_tmp, st);
   launch_compact_by_keep(A, keep, j2, v2, vb, p2, st);
 }
@@ -300,54 +338,61 @@ void launch_build_bci(const RightOp &B, int nseg, int min_len, int64_t max_rows,
   k_build_bci<<<grid_for(B.m, BCI_NT, 8), BCI_NT, 0, st>>>(B, nseg, min_len, max_rows, bci_id, bci, counter);
 }
 
-// one warp: exclusive scan of the NKEYS counters into offsets and cursors
-__global__ void k_key_offsets(const int *cnt, int *off, int *cur) {
-  const int lane = lane_id();
-  const int a = cnt[2 * lane], b = cnt[2 * lane + 1];
-  const int incl = warp_incl_scan(a + b);
-  const int ex = incl - a - b;
-  off[2 * lane] = ex;
-  off[2 * lane + 1] = ex + a;
-  cur[2 * lane] = ex;
-  cur[2 * lane + 1] = ex + a;
-  if (lane == 31) off[NKEYS] = incl;
-}
-static_assert(NKEYS == 64, "k_key_offsets assumes 64 keys");
-
-void launch_key_offsets(const int *key_cnt, int *key_off, int *key_cur, cudaStream_t st) {
-  count_launch();
-  k_key_offsets<<<1, 32, 0, st>>>(key_cnt, key_off, key_cur);
-}
-
-// append row r to the list of its key; lanes with equal keys share one atomic
-__device__ __forceinline__ void append_row(int key, int r, int *key_cur, int *list, int64_t cap, long long *dbg) {
-  const unsigned act = __activemask();
-  const unsigned grp = __match_any_sync(act, key);
-  const int leader = __ffs(grp) - 1;
-  int base = 0;
-  if (lane_id() == leader) base = atomicAdd(key_cur + key, __popc(grp));
-  base = __shfl_sync(grp, base, leader);
-  const int64_t at = base + __popc(grp & ((1u << lane_id()) - 1));
-  if (HS_G(dbg, at >= 0 && at < cap, 52, at)) list[at] = r;
+// The tile's rows (row u*TL_NT + x of the tile with key key[u] of thread x;
+// key 0: none) appended to the lists of their keys: counted per key in shared
+// memory, one atomic per key and block.  s_cnt: NKEYS zeroed counters; two
+// barriers.
+__device__ __forceinline__ void append_tile(const int (&key)[TL_PER], int64_t r0, int *s_cnt, int *key_cur, int *list,
+                                            int64_t cap, long long *dbg) {
+  int at[TL_PER];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const unsigned grp = __match_any_sync(FULL, key[u]);
+    const int leader = __ffs(grp) - 1;
+    int base = 0;
+    if (lane_id() == leader && key[u]) base = atomicAdd(s_cnt + key[u], __popc(grp));
+    at[u] = __shfl_sync(FULL, base, leader) + __popc(grp & ((1u << lane_id()) - 1));
+  }
+  __syncthreads();
+  if (threadIdx.x < NKEYS && s_cnt[threadIdx.x]) s_cnt[threadIdx.x] = atomicAdd(key_cur + threadIdx.x, s_cnt[threadIdx.x]);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    if (!key[u]) continue;
+    const int64_t x = (int64_t)s_cnt[key[u]] + at[u];
+    if (HS_G(dbg, x >= 0 && x < cap, 52, x)) list[x] = (int)(r0 + u * TL_NT + threadIdx.x);
+  }
 }
 
-__global__ void k_scatter_sym(RowSet A, const int64_t *f, int *key_cur, int *list, int32_t *hslot, int *nhist,
-                              BinCfg bins) {
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < A.nslots;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t fr = f[r];
-    const int key = sym_key(fr, bins);
-    if (key) append_row(key, (int)r, key_cur, list, A.nslots, A.dbg);
+__global__ void __launch_bounds__(TL_NT) k_scatter_sym(RowSet A, const int64_t *f, int *key_cur, int *list,
+                                                       int32_t *hslot, int *nhist, BinCfg bins) {
+  __shared__ int s_cnt[NKEYS], s_h;
+  if (threadIdx.x < NKEYS) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x == NKEYS) s_h = 0;
+  __syncthreads();
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
+  int key[TL_PER], slot[TL_PER];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    const int64_t fr = r < A.nslots ? f[r] : 0;
+    key[u] = sym_key(fr, bins);
     // rows that may need column parts in the numeric pass (every row of the
     // bitmap kernel) get a histogram slot
     const bool h = fr > bins.sym_heavy_from;
-    const unsigned act = __activemask();
-    const unsigned hm = __ballot_sync(act, h);
+    const unsigned hm = __ballot_sync(FULL, h);
     int base = 0;
-    const int leader = __ffs(act) - 1;
-    if (lane_id() == leader && hm) base = atomicAdd(nhist, __popc(hm));
-    base = __shfl_sync(act, base, leader);
-    hslot[r] = h ? base + __popc(hm & ((1u << lane_id()) - 1)) : -1;
+    if (lane_id() == 0 && hm) base = atomicAdd(&s_h, __popc(hm));
+    base = __shfl_sync(FULL, base, 0);
+    slot[u] = h ? base + __popc(hm & ((1u << lane_id()) - 1)) : -1;
+  }
+  append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
+  if (threadIdx.x == 0 && s_h) s_h = atomicAdd(nhist, s_h);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    if (r < A.nslots) hslot[r] = slot[u] >= 0 ? s_h + slot[u] : -1;
   }
 }
 
@@ -355,98 +400,190 @@ void launch_scatter_sym(const RowSet &A, const int64_t *f, int *key_cur, int *li
                         const BinCfg &bins, cudaStream_t st) {
   if (A.nslots == 0) return;
   count_launch();
-  k_scatter_sym<<<grid_for(A.nslots, 256, 8), 256, 0, st>>>(A, f, key_cur, list, hslot, nhist, bins);
+  k_scatter_sym<<<(unsigned)((A.nslots + TL_TILE - 1) / TL_TILE), TL_NT, 0, st>>>(A, f, key_cur, list, hslot, nhist,
+                                                                                 bins);
 }
 
-__device__ __forceinline__ int64_t out_count(const RowSet &A, const int64_t *Cp, int64_t r) {
-  const int64_t o = A.ids ? A.ids[r] : r;
-  return Cp[o + 1] - Cp[o];
+// ------------------------------------------- C's offsets and numeric bins
+// Two kernels: the first counts the rows of every numeric key and sums the
+// output counts of each tile of rows, and its last block turns both into
+// offsets; the second scans each tile's counts from its offset into C's row
+// offsets and, as it holds the counts, appends its rows to their lists.  (A
+// scan of three to five kernels, a pass for the keys and a third for the
+// lists made 18 launches of a 4096-row product; it now makes 10, 225 -> 187 us.)  For DCSR the rows
+// of the lists are not those of the scan: the lists are written by a kernel of
+// their own in between.
+__device__ __forceinline__ int64_t raw_count(const RowSet &A, const int64_t *cnt, int64_t slot) {
+  const int64_t o = A.ids ? (int64_t)A.ids[slot] : slot;
+  return HS_G(A.dbg, o >= 0 && o < A.m, 30, o) ? cnt[o + 1] : 0;
 }
-
-__global__ void k_num_count(RowSet A, const int64_t *f, const int64_t *Cp, BinCfg bins, int *key_cnt) {
-  __shared__ int hist[NKEYS];
-  for (int i = threadIdx.x; i < NKEYS; i += blockDim.x) hist[i] = 0;
+__global__ void __launch_bounds__(TL_NT) k_num_count(RowSet A, const int64_t *f, const int64_t *cnt, BinCfg bins,
+                                                     BinCounters c, int64_t *tsum, int64_t tiles, long long *nnz) {
+  __shared__ int hist[NKEYS], s_last;
+  __shared__ long long s_w[64];
+  for (int i = threadIdx.x; i < NKEYS; i += TL_NT) hist[i] = 0;
   __syncthreads();
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < A.nslots;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    const int key = num_key(f[r], out_count(A, Cp, r), bins);
-    if (key) atomicAdd(hist + key, 1);
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
+  long long sum = 0;
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    const int64_t n = r < A.m ? cnt[r + 1] : 0;
+    sum += n;
+    if (r < A.nslots) {
+      const int key = num_key(f[r], A.ids ? raw_count(A, cnt, r) : n, bins);
+      if (key) atomicAdd(hist + key, 1);
+    }
   }
+  sum = warp_sum(sum);
+  if (lane_id() == 0) s_w[threadIdx.x >> 5] = sum;
   __syncthreads();
-  for (int i = threadIdx.x; i < NKEYS; i += blockDim.x)
-    if (hist[i]) atomicAdd(key_cnt + i, hist[i]);
-}
-
-void launch_num_count(const RowSet &A, const int64_t *f, const int64_t *Cp, const BinCfg &bins, int *key_cnt,
-                      cudaStream_t st) {
-  if (A.nslots == 0) return;
-  count_launch();
-  k_num_count<<<grid_for(A.nslots, 256, 8), 256, 0, st>>>(A, f, Cp, bins, key_cnt);
-}
-
-__global__ void k_scatter_num(RowSet A, const int64_t *f, const int64_t *Cp, BinCfg bins, int *key_cur,
-                              int *list) {
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < A.nslots;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    const int key = num_key(f[r], out_count(A, Cp, r), bins);
-    if (key) append_row(key, (int)r, key_cur, list, A.nslots, A.dbg);
+  if (threadIdx.x == 0) {
+    long long t = 0;
+    for (int w = 0; w < TL_NW; ++w) t += s_w[w];
+    tsum[blockIdx.x] = t;
   }
+  for (int i = threadIdx.x; i < NKEYS; i += TL_NT)
+    if (hist[i]) atomicAdd(c.cnt + i, hist[i]);
+  if (!last_block(c.ticket, &s_last)) return;
+  if (threadIdx.x < 32) key_offsets(c.cnt, c.off, c.cur);
+  // exclusive scan of the tile sums, in place
+  long long run = 0;
+  for (int64_t b = 0; b < tiles; b += TL_TILE) {
+    long long v[TL_PER], x[TL_PER];
+#pragma unroll
+    for (int u = 0; u < TL_PER; ++u) {
+      const int64_t i = b + u * TL_NT + threadIdx.x;
+      v[u] = x[u] = i < tiles ? __ldcg(tsum + i) : 0;
+    }
+    __syncthreads();  // s_w: the previous use is over
+    const long long t = tile_scan(v, s_w);
+#pragma unroll
+    for (int u = 0; u < TL_PER; ++u) {
+      const int64_t i = b + u * TL_NT + threadIdx.x;
+      if (i < tiles) tsum[i] = run + v[u] - x[u];
+    }
+    run += t;
+  }
+  if (threadIdx.x == 0) *nnz = run;
 }
-
-void launch_scatter_num(const RowSet &A, const int64_t *f, const int64_t *Cp, const BinCfg &bins, int *key_cur,
-                        int *list, cudaStream_t st) {
-  if (A.nslots == 0) return;
+template <bool LISTS>
+__global__ void __launch_bounds__(TL_NT) k_num_offsets(RowSet A, const int64_t *f, int64_t *cnt, BinCfg bins,
+                                                       int *key_cur, const int64_t *tsum, int *list) {
+  __shared__ int s_cnt[NKEYS];
+  __shared__ long long s_tot[64];
+  if (threadIdx.x < NKEYS) s_cnt[threadIdx.x] = 0;
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
+  long long v[TL_PER];
+  int key[TL_PER];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    v[u] = r < A.m ? cnt[r + 1] : 0;
+    key[u] = 0;
+    if constexpr (LISTS)
+      if (r < A.nslots) key[u] = num_key(f[r], v[u], bins);
+  }
+  tile_scan(v, s_tot);
+  const int64_t base = tsum[blockIdx.x];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    if (r < A.m) cnt[r + 1] = base + v[u];
+  }
+  if constexpr (LISTS) append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
+}
+__global__ void __launch_bounds__(TL_NT) k_num_lists(RowSet A, const int64_t *f, const int64_t *cnt, BinCfg bins,
+                                                     int *key_cur, int *list) {
+  __shared__ int s_cnt[NKEYS];
+  if (threadIdx.x < NKEYS) s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
+  int key[TL_PER];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t r = r0 + u * TL_NT + threadIdx.x;
+    key[u] = r < A.nslots ? num_key(f[r], raw_count(A, cnt, r), bins) : 0;
+  }
+  append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
+}
+void launch_num_bins(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCfg &bins, const BinCounters &c,
+                     int64_t *tsum, long long *nnz, int *list, cudaStream_t st) {
+  const int64_t rows = A.m > A.nslots ? A.m : A.nslots;
+  if (rows <= 0) return;
+  const int64_t tiles = (rows + TL_TILE - 1) / TL_TILE;
   count_launch();
-  k_scatter_num<<<grid_for(A.nslots, 256, 8), 256, 0, st>>>(A, f, Cp, bins, key_cur, list);
+  k_num_count<<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c, tsum, tiles, nnz);
+  if (A.ids) {
+    count_launch();
+    k_num_lists<<<(unsigned)((A.nslots + TL_TILE - 1) / TL_TILE), TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, list);
+    count_launch();
+    k_num_offsets<false><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, tsum, list);
+  } else {
+    count_launch();
+    k_num_offsets<true><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, tsum, list);
+  }
 }
 
 // ------------------------------------------------------------------- scan
-// Inclusive prefix sum of an int64 array, in place: tiles of SCAN_TILE
-// elements are scanned by one CTA each; the tile totals are scanned
-// recursively and added back.
-constexpr int SCAN_NT = 256, SCAN_PER = 8, SCAN_TILE = SCAN_NT * SCAN_PER;
-
-__global__ void k_scan_tiles(int64_t *a, int64_t n, int64_t *tot) {
-  __shared__ long long wsum[SCAN_NT / 32 + 1];
-  const int64_t base = blockIdx.x * (int64_t)SCAN_TILE + threadIdx.x * SCAN_PER;
-  long long v[SCAN_PER];
+// Inclusive prefix sum of an int64 array, in place, by two kernels: the sums
+// of tiles of TL_TILE elements, then every tile's scan from the sum of the
+// tiles before it.  Each block of the second kernel adds those sums itself
+// (an array of up to 2^12 tiles, 8.4e6 elements, is a few coalesced reads
+// from L2); for longer arrays they are scanned by a recursion.
+constexpr int64_t SCAN_FLAT = 1 << 12;
+__global__ void __launch_bounds__(TL_NT) k_scan_sums(const int64_t *a, int64_t n, int64_t *tot) {
+  __shared__ long long s_w[TL_NW];
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
   long long s = 0;
 #pragma unroll
-  for (int i = 0; i < SCAN_PER; ++i) {
-    v[i] = (base + i < n) ? a[base + i] : 0;
-    s += v[i];
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t i = r0 + u * TL_NT + threadIdx.x;
+    s += i < n ? a[i] : 0;
   }
-  long long incl = warp_incl_scan(s);
-  if (lane_id() == 31) wsum[threadIdx.x >> 5] = incl;
+  s = warp_sum(s);
+  if (lane_id() == 0) s_w[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    long long w = threadIdx.x < SCAN_NT / 32 ? wsum[threadIdx.x] : 0;
-    long long wi = warp_incl_scan(w);
-    if (threadIdx.x < SCAN_NT / 32) wsum[threadIdx.x] = wi - w;
-    if (threadIdx.x == 31) wsum[SCAN_NT / 32] = wi;
+  if (threadIdx.x == 0) {
+    long long t = 0;
+    for (int w = 0; w < TL_NW; ++w) t += s_w[w];
+    tot[blockIdx.x] = t;
   }
-  __syncthreads();
-  long long run = incl - s + wsum[threadIdx.x >> 5];
-#pragma unroll
-  for (int i = 0; i < SCAN_PER; ++i) {
-    run += v[i];
-    if (base + i < n) a[base + i] = run;
-  }
-  if (threadIdx.x == 0 && tot) tot[blockIdx.x] = wsum[SCAN_NT / 32];
 }
-
-__global__ void k_scan_add(int64_t *a, int64_t n, const int64_t *tot) {
-  if (blockIdx.x == 0) return;
-  const int64_t add = tot[blockIdx.x - 1];
-  const int64_t base = blockIdx.x * (int64_t)SCAN_TILE;
-  for (int i = threadIdx.x; i < SCAN_TILE; i += blockDim.x)
-    if (base + i < n) a[base + i] += add;
+// tot: the tiles' sums (flat) or their inclusive scan; null: a single tile
+__global__ void __launch_bounds__(TL_NT) k_scan_apply(int64_t *a, int64_t n, const int64_t *tot, bool flat) {
+  __shared__ long long s_tot[64], s_w[TL_NW];
+  const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
+  long long v[TL_PER];
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t i = r0 + u * TL_NT + threadIdx.x;
+    v[u] = i < n ? a[i] : 0;
+  }
+  long long base = 0;
+  if (tot && flat) {
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += TL_NT) base += tot[i];
+    base = warp_sum(base);
+    if (lane_id() == 0) s_w[threadIdx.x >> 5] = base;
+  } else if (tot && blockIdx.x) {
+    base = tot[blockIdx.x - 1];
+  }
+  tile_scan(v, s_tot);  // (its barrier also publishes s_w)
+  if (tot && flat) {
+    base = 0;
+    for (int w = 0; w < TL_NW; ++w) base += s_w[w];
+  }
+#pragma unroll
+  for (int u = 0; u < TL_PER; ++u) {
+    const int64_t i = r0 + u * TL_NT + threadIdx.x;
+    if (i < n) a[i] = base + v[u];
+  }
 }
 
 int64_t scan_tmp_elems(int64_t n) {
   int64_t t = 0;
-  while (n > SCAN_TILE) {
-    n = (n + SCAN_TILE - 1) / SCAN_TILE;
+  while (n > TL_TILE) {
+    n = (n + TL_TILE - 1) / TL_TILE;
     t += n;
   }
   return t + 1;
@@ -454,17 +591,14 @@ int64_t scan_tmp_elems(int64_t n) {
 
 void launch_scan_i64(int64_t *a, int64_t n, int64_t *tmp, cudaStream_t st) {
   if (n <= 0) return;
-  const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  if (tiles == 1) {
+  const int64_t tiles = (n + TL_TILE - 1) / TL_TILE;
+  if (tiles > 1) {
     count_launch();
-    k_scan_tiles<<<1, SCAN_NT, 0, st>>>(a, n, nullptr);
-    return;
+    k_scan_sums<<<(unsigned)tiles, TL_NT, 0, st>>>(a, n, tmp);
+    if (tiles > SCAN_FLAT) launch_scan_i64(tmp, tiles, tmp + tiles, st);
   }
   count_launch();
-  k_scan_tiles<<<(unsigned)tiles, SCAN_NT, 0, st>>>(a, n, tmp);
-  launch_scan_i64(tmp, tiles, tmp + tiles, st);
-  count_launch();
-  k_scan_add<<<(unsigned)tiles, SCAN_NT, 0, st>>>(a, n, tmp);
+  k_scan_apply<<<(unsigned)tiles, TL_NT, 0, st>>>(a, n, tiles > 1 ? tmp : nullptr, tiles <= SCAN_FLAT);
 }
 
 // -------------------------------------------------------------- validation
@@ -708,17 +842,26 @@ __global__ void __launch_bounds__(PAIR_NT) k_build_pairs(RowSet A, RightOp B, He
             if constexpr (AB > 0)
               if (s < end) av = __ldg(reinterpret_cast<const VT *>(A.v) + q);
           }
-          for (int j = j0; j < j1; ++j) {
-            const int hi = __shfl_sync(FULL, shi, j);
-            const int64_t to = __shfl_sync(FULL, at, j);
+          // the index's offsets for all units of the run first: their loads are in flight together
+          int off[PAIR_GROUP];
+#pragma unroll
+          for (int i = 0; i < PAIR_GROUP; ++i) {
+            const int hi = __shfl_sync(FULL, shi, (j0 + i) & 31);
+            off[i] = i < run && t >= 0 ? __ldg(bci + (int64_t)t * bstride + hi) : 0;
+          }
+#pragma unroll
+          for (int i = 0; i < PAIR_GROUP; ++i) {
+            if (i >= run) break;
+            const int hi = __shfl_sync(FULL, shi, j0 + i);
+            const int64_t to = __shfl_sync(FULL, at, j0 + i);
             int64_t e = s;
             if (s < end) {
-              e = pair_end(B, base, s, end, t, hi, bci, bstride);
+              e = t >= 0 ? base + off[i] : pair_end(B, base, s, end, -1, hi, bci, bstride);
               if (!HS_G(A.dbg, e >= s && e <= end, 65, e)) e = s;
             }
             const unsigned m = __ballot_sync(FULL, e > s);
             if (e > s) pair_put<AB>(to + __popc(m & ((1u << lane) - 1u)), s, (int)(e - s), av, pseg, paval);
-            if (lane == j) at += __popc(m);
+            if (lane == j0 + i) at += __popc(m);
             s = e;
           }
         }

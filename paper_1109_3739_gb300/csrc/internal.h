@@ -82,33 +82,39 @@ struct BinCfg {
 };
 // Symbolic bins.  Every row that may end in the numeric heavy bin (c >
 // cap_large needs f > cap_large) takes the bitmap kernel, which also writes
-// the row's sorted column list for the numeric pass.
+// the row's sorted column list.  Both key functions are chains of selects,
+// weakest condition first, without a branch: the kernels that call them for
+// eight rows a thread between warp-wide operations must not diverge (with
+// early returns a lane was seen to fall behind its warp past a barrier).
 __host__ __device__ inline int sym_key(int64_t f, const BinCfg &b) {
-  if (f <= 0) return 0;
-  if (f <= F_TINY) return KEY_TINY;
-  if (b.spa) return KEY_SPA;
-  if (f <= F_WARP) return KEY_WARP;
-  if (f <= b.sym_mid_s_max) return KEY_MID_S;
-  if (f <= F_MID && f <= b.sym_heavy_from) return KEY_MID;
-  if (f <= F_LARGE && f <= b.sym_heavy_from) return KEY_LARGE;
-  return heavy_key(f);
+  int k = heavy_key(f | 1);
+  k = f <= F_LARGE && f <= b.sym_heavy_from ? KEY_LARGE : k;
+  k = f <= F_MID && f <= b.sym_heavy_from ? KEY_MID : k;
+  k = f <= b.sym_mid_s_max ? KEY_MID_S : k;
+  k = f <= F_WARP ? KEY_WARP : k;
+  k = b.spa ? KEY_SPA : k;
+  k = f <= F_TINY ? KEY_TINY : k;
+  return f <= 0 ? 0 : k;
 }
 // Numeric bins: the smaller tiers take smaller tables, so more of their rows
 // are in flight on an SM at once.
 __host__ __device__ inline int num_key(int64_t f, int64_t c, const BinCfg &b) {
-  if (c <= 0) return 0;
-  if (f <= F_TINY) return KEY_TINY;
-  if (b.spa) return KEY_SPA;
-  if (f <= b.sort_max && c * 100 >= f * b.sort_pct)
-    return f <= F_SORT_XS ? KEY_SORT_XS : (f <= F_SORT_S ? KEY_SORT_S : (f <= F_SORT_M ? KEY_SORT_M : KEY_SORT));
-  if (f <= b.warp_s_max) return KEY_WARP_S;
-  if (f <= F_WARP) return KEY_WARP;
-  if (c > b.num_heavy_from && f > b.sym_heavy_from) return heavy_key(f);  // a sorted list exists
-  if (c <= b.mid_s_max) return KEY_MID_S;
-  if (c <= CAP_MID) return KEY_MID;
-  if (c <= b.large_s_max) return KEY_LARGE_S;
-  if (c <= b.cap_large) return KEY_LARGE;
-  return heavy_key(f);
+  const int heavy = heavy_key(f | 1);
+  int k = heavy;
+  k = c <= b.cap_large ? KEY_LARGE : k;
+  k = c <= b.large_s_max ? KEY_LARGE_S : k;
+  k = c <= CAP_MID ? KEY_MID : k;
+  k = c <= b.mid_s_max ? KEY_MID_S : k;
+  k = c > b.num_heavy_from && f > b.sym_heavy_from ? heavy : k;  // a sorted list exists
+  k = f <= F_WARP ? KEY_WARP : k;
+  k = f <= b.warp_s_max ? KEY_WARP_S : k;
+  int s = f <= F_SORT_M ? KEY_SORT_M : KEY_SORT;
+  s = f <= F_SORT_S ? KEY_SORT_S : s;
+  s = f <= F_SORT_XS ? KEY_SORT_XS : s;
+  k = f <= b.sort_max && c * 100 >= f * b.sort_pct ? s : k;
+  k = b.spa ? KEY_SPA : k;
+  k = f <= F_TINY ? KEY_TINY : k;
+  return c <= 0 ? 0 : k;
 }
 // the default thresholds for a value width, clamped tuning values otherwise
 BinCfg bin_config(int value_bytes);
@@ -160,31 +166,35 @@ template <class K> inline void set_smem_attr(K kernel, size_t bytes) {
 
 // --------------------------------------------------------------- launchers
 // analysis.cu
-// stats[0] total flops, [1] max row flops, [2] max row nnz of A, [3] sum of
-// min(f, n) over the rows of the symbolic heavy bin (their list pool bound)
-void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, int *key_cnt, unsigned long long *stats,
-                  const BinCfg &bins, cudaStream_t st);
-// per-entry product counts (s over A's entries, zeros: entries with an
-// empty B row), the row counts and keys from their inclusive scan S, and the
-// copy of A without the zero entries (p2: nslots+1 offsets from 0)
-void launch_entry_flops(const RowSet &A, const RightOp &B, int64_t *s, unsigned long long *zeros, cudaStream_t st);
-void launch_row_flops(const RowSet &A, const int64_t *S, int64_t *f, int *key_cnt, unsigned long long *stats,
-                      const BinCfg &bins, int64_t bn, cudaStream_t st);
-void launch_compact_a(const RowSet &A, const int64_t *S, int64_t *keep, int64_t *scan_tmp, int32_t *j2, void *v2,
+// a binning's device counters: rows per key, the keys' list offsets and write
+// cursors, and a ticket that finds the last block (counts and ticket zeroed
+// before each binning)
+struct BinCounters {
+  int *cnt, *off, *cur, *ticket;
+};
+// products per row (f zeroed before) and the A entries with an empty B row;
+// then the rows' symbolic keys, their offsets, and stats[0] total flops, [1]
+// max row flops, [2] max row nnz of A, [3] sum of min(f, n) over the rows of
+// the symbolic heavy bin (their list pool bound).  cnt: C's counts, set to
+// zero on the way (CSR), or null
+void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, unsigned long long *zeros, cudaStream_t st);
+void launch_row_keys(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCounters &c, unsigned long long *stats,
+                     const BinCfg &bins, int64_t bn, cudaStream_t st);
+// the copy of A without the entries whose B row is empty (p2: nslots+1 offsets from 0)
+void launch_compact_a(const RowSet &A, const RightOp &B, int64_t *keep, int64_t *scan_tmp, int32_t *j2, void *v2,
                       int vb, int64_t *p2, cudaStream_t st);
 // entries of a CSR whose value is not zero (dtype F64, F32, I32 or I64):
 // keep flags, then (after their inclusive scan) the compacted copy
 void launch_keep_nonzero(const void *v, int dtype, int64_t n, int64_t *keep, cudaStream_t st);
 void launch_compact_by_keep(const RowSet &A, const int64_t *K, int32_t *j2, void *v2, int vb, int64_t *p2,
                             cudaStream_t st);
-void launch_key_offsets(const int *key_cnt, int *key_off, int *key_cur, cudaStream_t st);
 // rows with more than cap_large products get a column-segment histogram slot
 void launch_scatter_sym(const RowSet &A, const int64_t *f, int *key_cur, int *list, int32_t *hslot,
                         int *nhist, const BinCfg &bins, cudaStream_t st);
-void launch_num_count(const RowSet &A, const int64_t *f, const int64_t *Cp, const BinCfg &bins, int *key_cnt,
-                      cudaStream_t st);
-void launch_scatter_num(const RowSet &A, const int64_t *f, const int64_t *Cp, const BinCfg &bins, int *key_cur,
-                        int *list, cudaStream_t st);
+// the counts cnt[1..m] into offsets (cnt[0] is zero), nnz(C), and the rows'
+// lists by numeric key; tsum: scan_tmp_elems(max(m, nslots)) words
+void launch_num_bins(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCfg &bins, const BinCounters &c,
+                     int64_t *tsum, long long *nnz, int *list, cudaStream_t st);
 void launch_scan_i64(int64_t *a, int64_t n, int64_t *tmp, cudaStream_t st);  // inclusive, in place
 int64_t scan_tmp_elems(int64_t n);
 // B segment index: for every B row longer than `min_len`, the offset (within

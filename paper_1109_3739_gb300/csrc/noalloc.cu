@@ -74,13 +74,15 @@ struct Arena {
 };
 
 struct NaBlock {  // device counters, read back to host memory
-  int key_cnt[NKEYS];
+  int key_cnt[2][NKEYS];  // symbolic, numeric
   int key_off[NKEYS + 1];
   int key_cur[NKEYS];
   int dyn[2];
   int nhist;
   int err;
-  int pad[2];
+  int ticket[2];
+  int pad;
+  unsigned long long zeros;
   unsigned long long stats[4];
   long long nnz;
   long long dbg[2];
@@ -178,7 +180,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   int64_t *f = ar.take<int64_t>(nslots);
   int *list = ar.take<int>(nslots);
   int32_t *hslot = ar.take<int32_t>(nslots);
-  int64_t *scan_tmp = ar.take<int64_t>(scan_tmp_elems(m + 1));
+  int64_t *scan_tmp = ar.take<int64_t>(scan_tmp_elems(m > nslots ? m : nslots));
   if (ar.over) return HS_ESCRATCH;
   static thread_local NaBlock hb;  // host copy (ordinary memory)
 
@@ -186,8 +188,11 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   RowSet rs{A->ptr, A->idx, A->val, A->fmt == HS_DCSR ? A->ids : nullptr, nslots, A->nnz, m, sb->dbg};
   RightOp rb{B->ptr, B->idx, B->val, n, B->m, B->nnz, sb->dbg};
   NA_CK(cudaMemsetAsync(sb, 0, sizeof(NaBlock), st));
-  launch_flops(rs, rb, f, sb->key_cnt, sb->stats, bins, st);
-  launch_key_offsets(sb->key_cnt, sb->key_off, sb->key_cur, st);
+  NA_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nslots, st));
+  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0]};
+  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1]};
+  launch_flops(rs, rb, f, &sb->zeros, st);
+  launch_row_keys(rs, f, nullptr, sym_c, sb->stats, bins, n, st);
   launch_scatter_sym(rs, f, sb->key_cur, list, hslot, &sb->nhist, bins, st);
   if (int e = check_last()) return e;
   NA_CK(cudaMemcpyAsync(&hb, sb, sizeof(NaBlock), cudaMemcpyDeviceToHost, st));
@@ -225,12 +230,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   launch_sym_heavy(sa, st);
   if (int e = check_last()) return e;
 
-  launch_scan_i64(Cp, m + 1, scan_tmp, st);
-  NA_CK(cudaMemsetAsync(sb->key_cnt, 0, sizeof(int) * NKEYS, st));
-  launch_num_count(rs, f, Cp, numeric_bins(bins, n), sb->key_cnt, st);
-  launch_key_offsets(sb->key_cnt, sb->key_off, sb->key_cur, st);
-  launch_scatter_num(rs, f, Cp, numeric_bins(bins, n), sb->key_cur, list, st);
-  NA_CK(cudaMemcpyAsync(&sb->nnz, Cp + m, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
+  launch_num_bins(rs, f, Cp, numeric_bins(bins, n), num_c, scan_tmp, &sb->nnz, list, st);
   if (int e = check_last()) return e;
   NA_CK(cudaMemcpyAsync(&hb, sb, sizeof(NaBlock), cudaMemcpyDeviceToHost, st));
   NA_CK(cudaStreamSynchronize(st));

@@ -233,13 +233,14 @@ static void free_mat(hs_mat *M, Mem &mem) {
 
 // ----------------------------------------------------------------- SpGEMM
 struct SmallBlock {  // device counters, read back in one copy
-  int key_cnt[NKEYS];
+  int key_cnt[2][NKEYS];  // symbolic, numeric
   int key_off[NKEYS + 1];
   int key_cur[NKEYS];
   int dyn[3];  // symbolic heavy rows, numeric heavy rows, numeric heavy units
   int nhist;
   int err;
   int valflag;
+  int ticket[2];
   int pad;
   unsigned long long stats[4];
   unsigned long long lpool;  // heavy rows' column lists: pool entries handed out
@@ -404,14 +405,16 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   int64_t *Cp = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(m + 1));
   if (!Cp) return HS_ENOMEM;
   C->ptr = Cp;
-  CK(cudaMemsetAsync(Cp, 0, sizeof(int64_t) * (size_t)(m + 1), st));
+  const bool none = nslots == 0 || A->nnz == 0 || B->nnz == 0 || n == 0;
+  if (none || A->fmt == HS_DCSR)  // (a CSR product's counts are cleared as its rows are binned)
+    CK(cudaMemsetAsync(Cp, 0, sizeof(int64_t) * (size_t)(m + 1), st));
   if (plan) {
     plan->sr = sr;
     plan->out_dt = out_dt;
     plan->a_nnz = A->nnz;
     plan->b_nnz = B->nnz;
   }
-  if (nslots == 0 || A->nnz == 0 || B->nnz == 0 || n == 0) {
+  if (none) {
     if (place) {  // nothing to write
       C->idx = place->idx;
       C->val = place->val;
@@ -427,39 +430,30 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   }
 
   const BinCfg bins = product_bins(bin_config(vb), n, vb);
-  int64_t *f = mem.tmp<int64_t>(nslots);
+  // the counters and, behind them, the rows' product counts: cleared together
+  const size_t sb_bytes = (sizeof(SmallBlock) + 15) & ~(size_t)15;
+  char *zeroed = mem.tmp<char>(sb_bytes + sizeof(int64_t) * (size_t)nslots);
+  SmallBlock *sb = (SmallBlock *)zeroed;
+  int64_t *f = zeroed ? (int64_t *)(zeroed + sb_bytes) : nullptr;
   int *list = mem.tmp<int>(nslots);
   int32_t *hslot = mem.tmp<int32_t>(nslots);
-  SmallBlock *sb = mem.tmp<SmallBlock>(1);
+  int64_t *scan_tmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(m > nslots ? m : nslots));
   if (mem.failed) return HS_ENOMEM;
   RowSet rs{A->ptr, A->idx, A->val, A->fmt == HS_DCSR ? A->ids : nullptr, nslots, A->nnz, m, sb->dbg};
   RightOp rb{B->ptr, B->idx, B->val, n, B->m, B->nnz, sb->dbg};
   SmallBlock *hb = (SmallBlock *)pinned(sizeof(SmallBlock));
   if (!hb) return HS_ECUDA;
-  CK(cudaMemsetAsync(sb, 0, sizeof(SmallBlock), st));
-
-  // product counts per A entry and their scan: every row's count without a
-  // warp walking the row (optional scratch; without it, one warp per row)
-  int64_t *es = (int64_t *)mem.raw(sizeof(int64_t) * (size_t)A->nnz);
-  int64_t *es_tmp = es ? (int64_t *)mem.raw(sizeof(int64_t) * (size_t)scan_tmp_elems(A->nnz)) : nullptr;
-  if (es) mem.scratch.push_back({es, sizeof(int64_t) * (size_t)A->nnz});
-  if (es_tmp) mem.scratch.push_back({es_tmp, sizeof(int64_t) * (size_t)scan_tmp_elems(A->nnz)});
-  mem.failed = false;
-  const bool flat = es && es_tmp;
+  CK(cudaMemsetAsync(zeroed, 0, sb_bytes + sizeof(int64_t) * (size_t)nslots, st));
+  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0]};
+  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1]};
   {
     PhaseTimer t("analysis", st);
     if (flags & HS_FLAG_VALIDATE) {
       launch_validate(A->ptr, A->idx, nslots, A->n, &sb->valflag, st);
       launch_validate(B->ptr, B->idx, B->m, B->n, &sb->valflag, st);
     }
-    if (flat) {
-      launch_entry_flops(rs, rb, es, &sb->zeros, st);
-      launch_scan_i64(es, A->nnz, es_tmp, st);
-      launch_row_flops(rs, es, f, sb->key_cnt, sb->stats, bins, B->n, st);
-    } else {
-      launch_flops(rs, rb, f, sb->key_cnt, sb->stats, bins, st);
-    }
-    launch_key_offsets(sb->key_cnt, sb->key_off, sb->key_cur, st);
+    launch_flops(rs, rb, f, &sb->zeros, st);
+    launch_row_keys(rs, f, rs.ids ? nullptr : Cp, sym_c, sb->stats, bins, n, st);
     launch_scatter_sym(rs, f, sb->key_cur, list, hslot, &sb->nhist, bins, st);
   }
   if (int e = phase_check("analysis", st, sb->dbg)) return e;
@@ -481,16 +475,17 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   // counts, bins and results, and a long row of A with few products no longer
   // costs a walk over all its entries.  Not for plans, whose execute reads A's
   // values in place.
-  if (flat && !plan && A->nnz >= (1 << 20) && hb->zeros * 2 > (unsigned long long)A->nnz) {
+  if (!plan && A->nnz >= (1 << 20) && hb->zeros * 2 > (unsigned long long)A->nnz) {
     const int64_t kept = A->nnz - (int64_t)hb->zeros;
     const int va = A->val ? vbytes_of(A->dtype) : 0;
     int64_t *keep = mem.tmp<int64_t>((size_t)A->nnz);
     int32_t *j2 = mem.tmp<int32_t>((size_t)(kept > 0 ? kept : 1));
     void *v2 = va ? (void *)mem.tmp<char>((size_t)va * (size_t)(kept > 0 ? kept : 1)) : nullptr;
     int64_t *p2 = mem.tmp<int64_t>((size_t)nslots + 1);
+    int64_t *ktmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(A->nnz));
     if (!mem.failed) {
       PhaseTimer t("compact_a", st);
-      launch_compact_a(rs, es, keep, es_tmp, j2, v2, va, p2, st);
+      launch_compact_a(rs, rb, keep, ktmp, j2, v2, va, p2, st);
       rs.p = p2;
       rs.j = j2;
       rs.v = v2;
@@ -606,16 +601,9 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   }
 
   // ---- offsets and numeric bins
-  int64_t *scan_tmp = mem.tmp<int64_t>(scan_tmp_elems(m + 1));
-  if (!scan_tmp) return HS_ENOMEM;
   {
     PhaseTimer t("scan_bin", st);
-    launch_scan_i64(Cp, m + 1, scan_tmp, st);
-    CK(cudaMemsetAsync(sb->key_cnt, 0, sizeof(int) * NKEYS, st));
-    launch_num_count(rs, f, Cp, numeric_bins(bins, n), sb->key_cnt, st);
-    launch_key_offsets(sb->key_cnt, sb->key_off, sb->key_cur, st);
-    launch_scatter_num(rs, f, Cp, numeric_bins(bins, n), sb->key_cur, list, st);
-    CK(cudaMemcpyAsync(&sb->nnz, Cp + m, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
+    launch_num_bins(rs, f, Cp, numeric_bins(bins, n), num_c, scan_tmp, &sb->nnz, list, st);
   }
   // numeric heavy rows that have a sorted column list run as units (column
   // parts spread over the SMs): their parts are counted now, so that the
