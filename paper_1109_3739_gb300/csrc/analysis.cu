@@ -6,6 +6,9 @@
 // products are left out of every bin, so no later kernel does work for empty
 // rows: the dimension-independent work list of the doubly compressed format
 // (Section 2.2), built on the fly.
+#include <mutex>
+#include <vector>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -29,6 +32,37 @@ void launch_sm_count_init() {
 int sm_count() {
   launch_sm_count_init();
   return g_sms;
+}
+
+int kernel_fit(const void *kernel, int threads, size_t smem) {
+  struct Fit {
+    const void *kernel;
+    int dev, threads, ctas;
+    size_t smem;
+  };
+  static std::mutex mu;
+  static std::vector<Fit> fits;  // one per kernel, size and device: a few dozen
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> g(mu);
+  size_t limit = 0;  // the limit set so far (never lowered: other sizes of the kernel may need it)
+  for (const Fit &f : fits) {
+    if (f.kernel != kernel || f.dev != dev) continue;
+    if (f.threads == threads && f.smem == smem) return f.ctas;
+    if (f.smem > limit) limit = f.smem;
+  }
+  if (e == cudaSuccess && smem > limit && smem > 0)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int n = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem);
+  if (e != cudaSuccess) {
+    attr_error() = e;
+    cudaGetLastError();
+    return 1;
+  }
+  if (n < 1) n = 1;
+  fits.push_back(Fit{kernel, dev, threads, n, smem});
+  return n;
 }
 
 static int grid_for(int64_t items, int per_block, int max_per_sm) {

@@ -438,7 +438,7 @@ template <class SR> size_t bp_smem() {
 
 template <class SR> static int bp_launch(BpArgs &a, int grid, cudaStream_t st) {
   auto k = k_batch_persist<SR>;
-  set_smem_attr(k, bp_smem<SR>());
+  fit_per_sm(k, BP_NT, bp_smem<SR>());  // (sets its shared memory limit)
   count_launch();
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
@@ -454,11 +454,9 @@ template <class SR> static int bp_launch(BpArgs &a, int grid, cudaStream_t st) {
 }
 
 template <class SR> static int bp_grid() {
-  int per = 0;
-  auto k = k_batch_persist<SR>;
-  set_smem_attr(k, bp_smem<SR>());
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BP_NT, bp_smem<SR>()) != cudaSuccess || per < 1) {
-    cudaGetLastError();
+  const int per = fit_per_sm(k_batch_persist<SR>, BP_NT, bp_smem<SR>());
+  if (attr_error() != cudaSuccess) {
+    attr_error() = cudaSuccess;
     return 0;
   }
   return per * sm_count();

@@ -156,12 +156,15 @@ struct RightOp {
 void count_launch();
 unsigned long long launch_total();
 
-// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) with the failure kept for
-// the driver to report (launchers return void)
+// A kernel's dynamic shared memory limit raised to `smem` bytes, and how many
+// of its CTAs of `threads` threads then fit an SM (at least 1).  Both are
+// asked of the runtime once per kernel, size and device: asking at every
+// launch took a third of the launch's own time.  A failure is kept in
+// attr_error() for the driver to report (launchers return void).
 cudaError_t &attr_error();
-template <class K> inline void set_smem_attr(K kernel, size_t bytes) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) attr_error() = e;
+int kernel_fit(const void *kernel, int threads, size_t smem);
+template <class K> inline int fit_per_sm(K kernel, int threads, size_t smem) {
+  return kernel_fit((const void *)kernel, threads, smem);
 }
 
 // --------------------------------------------------------------- launchers

@@ -821,16 +821,6 @@ inline int ngrid_cap(int items, int per_block, int per_sm) {
   int cap = sm_count() * per_sm;
   return g < cap ? (g < 1 ? 1 : g) : cap;
 }
-// CTAs that fit one SM for this kernel, block size and dynamic shared memory
-template <class K> int fit_per_sm(K kernel, int threads, size_t smem) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    n = 1;
-  }
-  return n < 1 ? 1 : n;
-}
-
 // ------------------------------------------------------------- sort tiers
 // Rows with 32 < f <= F_SORT whose output count is close to their product
 // count: one warp per row sorts the row's products (sort_row), one kernel
@@ -871,7 +861,6 @@ template <class SR, int K> void launch_num_sort(const NumArgs &a, cudaStream_t s
   using T = typename SR::val_t;
   const size_t bytes = SortSmemLayout<T, K>::per_warp * NSORT_WPB;
   auto k = k_num_sort<SR, K>;
-  set_smem_attr(k, bytes);
   count_launch();
   k<<<ngrid_cap(a.count, NSORT_WPB, fit_per_sm(k, NSORT_WPB * 32, bytes)), NSORT_WPB * 32, bytes, st>>>(a);
 }
@@ -980,7 +969,6 @@ template <class SR> void launch_num_spa(const NumArgs &a, cudaStream_t st) {
   using T = typename SR::val_t;
   const size_t bytes = SpaLayout<T>::per_warp * NSPA_WPB;
   auto k = k_num_spa<SR>;
-  set_smem_attr(k, bytes);
   count_launch();
   k<<<ngrid_cap(a.count, NSPA_WPB, fit_per_sm(k, NSPA_WPB * 32, bytes)), NSPA_WPB * 32, bytes, st>>>(a);
 }
@@ -989,7 +977,6 @@ template <class SR, int SLOTS, int CAP> void launch_num_warp(const NumArgs &a, c
   using T = typename SR::val_t;
   const size_t bytes = WarpNumSmem<T, SLOTS, CAP>::per_warp * NWARP_WPB;
   auto k = k_num_warp<SR, SLOTS, CAP>;
-  set_smem_attr(k, bytes);
   count_launch();
   k<<<ngrid_cap(a.count, NWARP_WPB, fit_per_sm(k, NWARP_WPB * 32, bytes)), NWARP_WPB * 32, bytes, st>>>(a);
 }
@@ -998,7 +985,6 @@ template <class SR, int SLOTS, int CAP, int NT> void launch_num_cta(const NumArg
   using T = typename SR::val_t;
   using L = CtaNumLayout<T, SLOTS, CAP>;
   auto k = k_num_cta<SR, SLOTS, CAP, NT>;
-  set_smem_attr(k, L::bytes);
   count_launch();
   k<<<ngrid_cap(a.count, 1, fit_per_sm(k, NT, L::bytes)), NT, L::bytes, st>>>(a);
 }
@@ -1007,7 +993,6 @@ template <class SR, int KB> void launch_num_units(const NumArgs &a, cudaStream_t
   using T = typename SR::val_t;
   const size_t ub = sizeof(UnitSmem<T, KB>);
   auto ku = k_num_units<SR, KB>;
-  set_smem_attr(ku, ub);
   count_launch();
   const int items = a.nunits < (1 << 30) ? (int)a.nunits : (1 << 30);
   ku<<<ngrid_cap(items, 1, fit_per_sm(ku, HU_NT, ub)), HU_NT, ub, st>>>(a);
@@ -1042,9 +1027,9 @@ template <class SR> void launch_numeric_sr(int kind, const NumArgs &a, cudaStrea
       }
       if (!a.units || a.lists_partial) {  // rows without a list: one CTA per row
         const size_t bytes = sizeof(HeavySmem<T>);
-        set_smem_attr(k_num_heavy<SR>, bytes);
+        const int fit = fit_per_sm(k_num_heavy<SR>, HV_NT, bytes);
         count_launch();
-        k_num_heavy<SR><<<ngrid_cap(a.count, 1, 2), HV_NT, bytes, st>>>(a);
+        k_num_heavy<SR><<<ngrid_cap(a.count, 1, fit < 2 ? fit : 2), HV_NT, bytes, st>>>(a);
       }
       break;
     }

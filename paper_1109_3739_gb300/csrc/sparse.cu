@@ -450,7 +450,7 @@ static void sp_pass_one(const uint64_t *Kin, const int32_t *I, const int32_t *J,
                         unsigned long long *status, int *ticket, int64_t ntiles, uint64_t *Kout, void *Vout,
                         int *flag, int spin_limit, long long withhold, cudaStream_t st) {
   constexpr size_t smem = sp_scatter_smem<VB>();
-  set_smem_attr(k_sp_onesweep<FIRST, VB>, smem);
+  fit_per_sm(k_sp_onesweep<FIRST, VB>, SP_NT, smem);  // (sets its shared memory limit)
   count_launch();
   k_sp_onesweep<FIRST, VB><<<sp_grid(ntiles), SP_NT, smem, st>>>(Kin, I, J, Vin, nnz, nbj, m, n, pass, ghist,
                                                                  status, ticket, Kout, Vout, flag, spin_limit,
@@ -490,7 +490,7 @@ void launch_sp_emit(int op, const uint64_t *K, const void *V, int64_t nnz, int n
   if (ntiles <= 0) return;
   count_launch();
 #define SP_EM(O)                                                                                       \
-  set_smem_attr(k_sp_emit<O>, sp_emit_smem<O>());                                                      \
+  fit_per_sm(k_sp_emit<O>, SP_NT, sp_emit_smem<O>());                                                      \
   k_sp_emit<O><<<sp_grid(ntiles), SP_NT, sp_emit_smem<O>(), st>>>(K, V, nnz, nbj, theads_incl, Cidx, Cval, \
                                                                   rowcnt, longlist, nlong)
   switch (op) {

@@ -105,6 +105,12 @@ struct Mem {
   };
   std::vector<Blk> scratch;
   bool failed = false;
+  // temporaries of at most SMALL bytes are cut from blocks of CHUNK bytes: a
+  // call of the caller's allocator costs some 5 us, and a small operation
+  // would make a dozen of them for a few KB each
+  static constexpr size_t SMALL = 256 << 10, CHUNK = 1 << 20;
+  char *chunk = nullptr;
+  size_t chunk_left = 0;
 
   void *raw(size_t bytes) {
     if (bytes == 0) bytes = 16;
@@ -126,8 +132,23 @@ struct Mem {
     else if (!al || !al->alloc) cudaFreeAsync(p, st);
   }
   template <typename T> T *tmp(size_t count) {
-    T *p = (T *)raw(sizeof(T) * count);
-    if (p) scratch.push_back({p, sizeof(T) * count});
+    const size_t bytes = sizeof(T) * count;
+    if (bytes <= SMALL) {
+      const size_t room = ((bytes ? bytes : 1) + 255) & ~(size_t)255;
+      if (room > chunk_left) {
+        chunk_left = 0;
+        chunk = (char *)raw(CHUNK);
+        if (!chunk) return nullptr;
+        scratch.push_back({chunk, CHUNK});
+        chunk_left = CHUNK;
+      }
+      T *p = (T *)chunk;
+      chunk += room;
+      chunk_left -= room;
+      return p;
+    }
+    T *p = (T *)raw(bytes);
+    if (p) scratch.push_back({p, bytes});
     return p;
   }
   ~Mem() {

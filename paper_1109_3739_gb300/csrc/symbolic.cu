@@ -447,20 +447,9 @@ void launch_sym_tiny(const SymArgs &a, cudaStream_t st) {
   count_launch();
   k_sym_tiny<<<grid_cap(a.count, TINY_WPB, 8), TINY_WPB * 32, 0, st>>>(a);
 }
-// CTAs that fit one SM for this kernel, block size and dynamic shared memory
-template <class K> static int fit_per_sm(K kernel, int threads, size_t smem) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    n = 1;
-  }
-  return n < 1 ? 1 : n;
-}
-
 template <int SLOTS> static void launch_sym_warp_slots(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
   const size_t bytes = sizeof(int) * WARP_WPB * SLOTS;
-  set_smem_attr(k_sym_warp<SLOTS>, bytes);
   count_launch();
   k_sym_warp<SLOTS><<<grid_cap(a.count, WARP_WPB, fit_per_sm(k_sym_warp<SLOTS>, WARP_WPB * 32, bytes)),
                       WARP_WPB * 32, bytes, st>>>(a);
@@ -475,7 +464,6 @@ void launch_sym_spa(const SymArgs &a, cudaStream_t st) {
 template <int SLOTS, int NT> static void launch_sym_cta(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
   const size_t bytes = sizeof(SymCtaSmem<SLOTS>);
-  set_smem_attr(k_sym_cta<SLOTS, NT>, bytes);
   count_launch();
   k_sym_cta<SLOTS, NT><<<grid_cap(a.count, 1, fit_per_sm(k_sym_cta<SLOTS, NT>, NT, bytes)), NT, bytes, st>>>(a);
 }
@@ -489,7 +477,6 @@ void launch_sym_heavy(const SymArgs &a, cudaStream_t st) {
   const int64_t words = (a.B.n + 31) / 32;
   const size_t bytes = offsetof(SymHeavySmem, bitmap) +
                        sizeof(unsigned) * (size_t)(words < SH_COLS / 32 ? words : SH_COLS / 32);
-  set_smem_attr(k_sym_heavy, sizeof(SymHeavySmem));
   count_launch();
   k_sym_heavy<<<grid_cap(a.count, 1, fit_per_sm(k_sym_heavy, SH_NT, bytes)), SH_NT, bytes, st>>>(a);
 }
