@@ -407,7 +407,12 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
       const int c = (int)(a.Cp[r + 1] - cb);
       const int fr = a.fw[r];
       int kmn = 0, kmx = 0;
-      const int got = sort_expand<SR>(A, B, A.p[r], A.p[r + 1], BPW_F, s_col, s_val, &kmn, &kmx);
+      RowAhead<SR> x;
+      x.r = r;
+      x.range(A);
+      x.entries(A);
+      x.segments(B);
+      const int got = sort_expand<SR>(A, B, x, BPW_F, s_col, s_val, &kmn, &kmx);
       if (got != fr || fr > ((BPW_FS / 2) << g)) {
         if (lane == 0) atomicExch(&ctr->kerr, 12);
       } else if (HS_G(dbg, cb + c <= a.cap, 81, cb + c)) {

@@ -411,6 +411,235 @@ __device__ __forceinline__ void warp_products(const DevCsr &A, const DevCsr &B, 
   }
 }
 
+// position of the (r + 1)-th set bit of m (r < popc(m))
+__device__ __forceinline__ int nth_bit(unsigned m, int r) {
+  int pos = 0;
+#pragma unroll
+  for (int w = 16; w >= 1; w >>= 1) {
+    const int c = __popc((m >> pos) & ((1u << w) - 1u));
+    if (c <= r) {
+      r -= c;
+      pos += w;
+    }
+  }
+  return pos;
+}
+
+// warp_expand for the kernels that give a row to a warp.  The short segments
+// are moved to the lowest lanes (empty ones drop out) and a round's segment
+// starts are or-ed into one word (__reduce_or_sync), so that a lane's segment
+// is the number of starts at or below it instead of a search over the length
+// scan; the check against B's size is made once per segment.  (R-MAT scale
+// 20: warp rows of the symbolic pass 0.36 -> 0.30 ms, a batch of random
+// products 1.53 -> 1.38 ms.  In the kernels that give a row to a block, which
+// hold more registers, the search measured faster: rows of 1024 to 4096
+// products 1.52 against 1.58 ms, the bitmap kernel 23.8 against 24.2 ms.)
+// visit and the result as for warp_expand; a segment outside B (a failed
+// check) makes no products.
+template <class SR, int U = 2, int SB = 4, class Visit>
+__device__ __forceinline__ int warp_expand_row(const DevCsr &B, int64_t s, int len, typename SR::val_t a,
+                                            Visit &visit) {
+  using T = typename SR::val_t;
+  using VisitT = std::decay_t<Visit>;
+  const int lane = lane_id();
+  if (len > 0 && !HS_G(B.dbg, s >= 0 && s + len <= B.nnz, 4, s)) len = 0;
+  const int incl = warp_incl_scan(len);
+  const int total = __shfl_sync(FULL, incl, 31);
+  const int ex_full = incl - len;
+  // long segments: the whole warp on one segment, U entries per lane per
+  // step (all loads of a step issued before the first visit); a last step of
+  // fewer than U * 32 entries runs only the sub-steps it has
+  const unsigned long_all = __ballot_sync(FULL, len >= 32);
+  for (unsigned longm = long_all; longm; longm &= longm - 1) {
+    const int l = __ffs(longm) - 1;
+    const int64_t sl = __shfl_sync(FULL, s, l);
+    const int ll = __shfl_sync(FULL, len, l);
+    const int el = __shfl_sync(FULL, ex_full, l);
+    const T al = shfl_val<T>(a, l);
+    const int32_t *bj = B.j + sl;
+    const T *bv = reinterpret_cast<const T *>(B.v) + sl;
+    for (int o0 = 0; o0 < ll; o0 += 32 * U) {
+      const int off = o0 + lane;
+      int c[U];
+      T b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool ok = off + 32 * u < ll;
+        c[u] = ok ? __ldg(bj + off + 32 * u) : 0;
+        b[u] = T{};
+        if constexpr (SR::needs_b)
+          if (ok) b[u] = __ldg(bv + off + 32 * u);
+      }
+      if constexpr (two_stage<VisitT>::value) {
+        typename VisitT::State st[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (off + 32 * u < ll) st[u] = visit.prep(c[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (o0 + 32 * u >= ll) break;
+          if (off + 32 * u >= ll) continue;
+          if constexpr (SR::has_val) visit.commit(st[u], SR::mul(al, b[u]));
+          else visit.commit(st[u], NoVal{});
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (o0 + 32 * u >= ll) break;
+          if (off + 32 * u >= ll) continue;
+          if constexpr (SR::has_val) visit(c[u], SR::mul(al, b[u]), el + off + 32 * u);
+          else visit(c[u], NoVal{}, el + off + 32 * u);
+        }
+      }
+    }
+  }
+  // short segments: one product per lane, SB rounds of 32 at a time
+  const unsigned shortm = __ballot_sync(FULL, len > 0 && len < 32);
+  if (!shortm) return total;
+  const int ns = __popc(shortm);
+  int fex = ex_full;  // the segment's first product in the order of all segments
+  int sex = ex_full;  // and among the short ones
+  if (long_all) {
+    const int slen = len < 32 ? len : 0;
+    sex = warp_incl_scan(slen) - slen;
+  }
+  if (shortm & (shortm + 1)) {  // gaps: the short segments move to lanes 0 .. ns-1
+    const int src = nth_bit(shortm, lane < ns ? lane : 0);
+    s = __shfl_sync(FULL, s, src);
+    a = shfl_val<T>(a, src);
+    fex = __shfl_sync(FULL, fex, src);
+    sex = __shfl_sync(FULL, sex, src);
+    len = __shfl_sync(FULL, len, src);
+  }
+  const int stotal = __shfl_sync(FULL, sex + len, ns - 1);
+  const int64_t place = s - sex;  // product p of the segment lies at place + p
+  const unsigned le = 0xffffffffu >> (31 - lane);
+  int before = 0;  // segments that start before the round
+  for (int base = 0; base < stotal; base += 32 * SB) {
+    int col[SB], pidx[SB];
+    T pv[SB];
+    bool ok[SB];
+#pragma unroll
+    for (int u = 0; u < SB; ++u) {
+      ok[u] = false;
+      col[u] = 0;
+      pidx[u] = 0;
+      pv[u] = T{};
+      if (base + 32 * u < stotal) {  // warp-uniform: the shuffles below see every lane
+        const int p = base + 32 * u + lane;
+        const unsigned at = (unsigned)(sex - (base + 32 * u));
+        const unsigned starts = __reduce_or_sync(FULL, lane < ns && at < 32u ? 1u << at : 0u);
+        const int src = before + __popc(starts & le) - 1;
+        before += __popc(starts);
+        const int64_t pos = __shfl_sync(FULL, place, src) + p;
+        const T aa = shfl_val<T>(a, src);
+        if constexpr (!two_stage<VisitT>::value) {
+          pidx[u] = p;
+          if (long_all) pidx[u] += __shfl_sync(FULL, fex - sex, src);
+        }
+        if (p < stotal) {
+          ok[u] = true;
+          col[u] = __ldg(B.j + pos);
+          if constexpr (SR::has_val) {
+            T b{};
+            if constexpr (SR::needs_b) b = load_val<T>(B.v, pos);
+            pv[u] = SR::mul(aa, b);
+          }
+        }
+      }
+    }
+    if constexpr (two_stage<VisitT>::value) {
+      typename VisitT::State st[SB];
+#pragma unroll
+      for (int u = 0; u < SB; ++u)
+        if (ok[u]) st[u] = visit.prep(col[u]);
+#pragma unroll
+      for (int u = 0; u < SB; ++u)
+        if (ok[u]) visit.commit(st[u], pv[u]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < SB; ++u)
+        if (ok[u]) visit(col[u], pv[u], pidx[u]);
+    }
+  }
+  return total;
+}
+
+// The row a warp will take next, looked up in steps while it works on the
+// present one: row id, its range of A, and for the first 32 entries of A
+// their columns (with A's values) and B offsets.  Row kernels with one warp
+// per row are a chain of five dependent loads before the first product; each
+// step is issued one stage of the present row ahead of the next, so that only
+// B's entries themselves are waited for.
+template <class SR> struct RowAhead {
+  using T = typename SR::val_t;
+  int r = -1;
+  int64_t q0 = 0, q1 = 0;
+  int k = -1;
+  T a{};
+  int64_t s = 0;
+  int len = 0;
+  __device__ __forceinline__ void row(const DevCsr &A, const int *list, int idx, int count) {
+    r = idx < count ? __ldg(list + idx) : -1;
+    if (r >= 0 && !HS_G(A.dbg, r < A.rows, 35, r)) r = -1;
+  }
+  __device__ __forceinline__ void range(const DevCsr &A) {
+    q0 = q1 = 0;
+    if (r >= 0) {
+      q0 = __ldg(A.p + r);
+      q1 = __ldg(A.p + r + 1);
+    }
+  }
+  __device__ __forceinline__ void entries(const DevCsr &A) {
+    const int64_t q = q0 + lane_id();
+    k = -1;
+    if (q < q1 && HS_G(A.dbg, q >= 0 && q < A.nnz, 1, q)) {
+      k = __ldg(A.j + q);
+      if constexpr (SR::needs_a) a = load_val<T>(A.v, q);
+    }
+  }
+  __device__ __forceinline__ void segments(const DevCsr &B) {
+    s = 0;
+    len = 0;
+    if (q0 + lane_id() >= q1) return;
+    if (!HS_G(B.dbg, k >= 0 && k < B.rows, 2, k)) return;
+    s = __ldg(B.p + k);
+    const int64_t e = __ldg(B.p + k + 1);
+    if (HS_G(B.dbg, s >= 0 && s <= e && e <= B.nnz, 3, e)) len = (int)(e - s);
+  }
+  __device__ __forceinline__ void all(const DevCsr &A, const DevCsr &B, const int *list, int idx, int count) {
+    row(A, list, idx, count);
+    range(A);
+    entries(A);
+    segments(B);
+  }
+};
+
+// Every product of the row held by `x`: its first 32 entries as looked up,
+// the others as they come.  Returns their number.
+template <class SR, class Visit>
+__device__ __forceinline__ int warp_products_of(const DevCsr &A, const DevCsr &B, const RowAhead<SR> &x, Visit &visit) {
+  using T = typename SR::val_t;
+  int64_t s = x.s;
+  int len = x.len, total = 0;
+  T a = x.a;
+  for (int64_t qb = x.q0;;) {
+    const int done = total;
+    auto at = [&](int col, T v, int p) { visit(col, v, done + p); };
+    total += warp_expand_row<SR>(B, s, len, a, at);
+    qb += 32;
+    if (qb >= x.q1) return total;
+    const int64_t q = qb + lane_id();
+    int64_t e = 0;
+    s = 0;
+    if (q < x.q1) {
+      entry_segment(A, B, q, false, 0, 0, s, e);
+      if constexpr (SR::needs_a) a = load_val<T>(A.v, q);
+    }
+    len = (int)(e - s);
+  }
+}
+
 // Ask for [p, p + bytes) to be brought into L2 ahead of its reads (bulk
 // prefetch, no completion to wait for).  The range is narrowed to 16-byte
 // boundaries, so it never leaves the buffer, and issued in pieces of at most

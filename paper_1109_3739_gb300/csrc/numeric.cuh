@@ -50,30 +50,26 @@ __global__ void __launch_bounds__(NTINY_WPB * 32, 4) k_num_tiny(NumArgs a) {
   const int w = threadIdx.x >> 5, lane = lane_id();
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
   T *Cv = reinterpret_cast<T *>(a.Cv);
-  for (int idx = blockIdx.x * NTINY_WPB + w; idx < a.count; idx += gridDim.x * NTINY_WPB) {
-    const int r = a.list[idx];
-    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
-    const int64_t q0 = A.p[r], q1 = A.p[r + 1];
-    int nprod = 0;
-    for (int64_t qb = q0; qb < q1; qb += 32) {
-      const int64_t q = qb + lane;
-      int64_t s = 0, e = 0;
-      T av{};
-      if (q < q1) {
-        entry_segment(A, B, q, false, 0, 0, s, e);
-        if constexpr (SR::needs_a) av = load_val<T>(A.v, q);
+  const int step = gridDim.x * NTINY_WPB;
+  int idx = blockIdx.x * NTINY_WPB + w;
+  RowAhead<SR> x, nx;
+  x.all(A, B, a.list, idx, a.count);
+  for (; idx < a.count; idx += step) {
+    nx.row(A, a.list, idx + step, a.count);
+    const int64_t o = x.r >= 0 ? nout_row(a.A, x.r) : 0;
+    const int64_t base = a.Cp[o], end = a.Cp[o + 1];
+    auto put = [&](int col, T v, int p) {
+      if (HS_G(a.A.dbg, p < 32, 40, p)) {
+        scol[w][p] = col;
+        if constexpr (SR::has_val) sval[w][p] = v;
       }
-      auto put = [&](int col, T v, int p) {
-        if (HS_G(a.A.dbg, nprod + p < 32, 40, nprod + p)) {
-          scol[w][nprod + p] = col;
-          if constexpr (SR::has_val) sval[w][nprod + p] = v;
-        }
-      };
-      nprod += warp_expand<SR>(B, s, (int)(e - s), av, put);
-    }
+    };
+    const int nprod = x.r >= 0 ? warp_products_of<SR>(A, B, x, put) : 0;
+    nx.range(A);
     __syncwarp();
     const bool have = lane < nprod;
     const int col = have ? scol[w][lane] : 0;
+    nx.entries(A);
     const unsigned act = __ballot_sync(FULL, have);
     unsigned grp = 0;
     if (have) grp = __match_any_sync(act, col);
@@ -86,18 +82,18 @@ __global__ void __launch_bounds__(NTINY_WPB * 32, 4) k_num_tiny(NumArgs a) {
       }
     }
     const unsigned leaders = __ballot_sync(FULL, lead);
-    const int64_t o = nout_row(a.A, r);
-    const int64_t base = a.Cp[o];
+    nx.segments(B);
     if (lead) {
       int rank = 0;
       for (unsigned m = leaders; m; m &= m - 1) rank += scol[w][__ffs(m) - 1] < col;
-      if (HS_G(a.A.dbg, base + rank < a.Cp[o + 1], 41, base + rank)) {
+      if (HS_G(a.A.dbg, base + rank < end, 41, base + rank)) {
         a.Cj[base + rank] = col;
         if constexpr (SR::has_val) Cv[base + rank] = acc;
       }
     }
-    if (lane == 0 && (int64_t)__popc(leaders) != a.Cp[o + 1] - base) atomicExch(a.err, 3);
+    if (lane == 0 && x.r >= 0 && (int64_t)__popc(leaders) != end - base) atomicExch(a.err, 3);
     __syncwarp();
+    x = nx;
   }
 }
 
@@ -128,12 +124,15 @@ __global__ void __launch_bounds__(NWARP_WPB * 32, 4) k_num_warp(NumArgs a) {
   EmitScratch *es = reinterpret_cast<EmitScratch *>(base + L::region0 + L::compact);
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
   T *Cv = reinterpret_cast<T *>(a.Cv);
-  for (int idx = blockIdx.x * NWARP_WPB + w; idx < a.count; idx += gridDim.x * NWARP_WPB) {
-    const int r = a.list[idx];
-    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
-    const int64_t o = nout_row(a.A, r);
+  const int step = gridDim.x * NWARP_WPB;
+  int idx = blockIdx.x * NWARP_WPB + w;
+  RowAhead<SR> x, nx;
+  x.all(A, B, a.list, idx, a.count);
+  for (; idx < a.count; idx += step) {
+    nx.row(A, a.list, idx + step, a.count);
+    const int64_t o = x.r >= 0 ? nout_row(a.A, x.r) : 0;
     const int64_t cb = a.Cp[o];
-    const int c = (int)(a.Cp[o + 1] - cb);
+    const int c = x.r >= 0 ? (int)(a.Cp[o + 1] - cb) : 0;
     const int slots = max(64, min(NWARP_SLOTS, next_pow2(2 * min(c, NWARP_CAP))));
     const unsigned mask = slots - 1;
     for (int s = lane; s < slots; s += 32) {
@@ -141,13 +140,18 @@ __global__ void __launch_bounds__(NWARP_WPB * 32, 4) k_num_warp(NumArgs a) {
       if constexpr (SR::has_val) vals[s] = SR::identity();
     }
     __syncwarp();
-    warp_products<SR>(A, B, A.p[r], A.p[r + 1],
-                      [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
+    nx.range(A);
+    auto put = [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); };
+    if (x.r >= 0) warp_products_of<SR>(A, B, x, put);
+    nx.entries(A);
     __syncwarp();
-    group_sort_emit<WarpGroup, T, SR::has_val>(keys, vals, slots, c, ck, cv, base, nullptr, es, a.Cj + cb,
-                                               SR::has_val ? Cv + cb : nullptr, a.err, NWARP_CAP, a.A.dbg,
-                                               a.unsorted);
+    nx.segments(B);
+    if (x.r >= 0)
+      group_sort_emit<WarpGroup, T, SR::has_val>(keys, vals, slots, c, ck, cv, base, nullptr, es, a.Cj + cb,
+                                                 SR::has_val ? Cv + cb : nullptr, a.err, NWARP_CAP, a.A.dbg,
+                                                 a.unsorted);
     __syncwarp();
+    x = nx;
   }
 }
 
@@ -843,17 +847,32 @@ __global__ void __launch_bounds__(NSORT_WPB * 32, K >= 32 ? 6 : 8) k_num_sort(Nu
   T *s_val = reinterpret_cast<T *>(smem_raw + (size_t)w * L::per_warp + L::col_bytes);
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
   T *Cv = reinterpret_cast<T *>(a.Cv);
-  for (int idx = blockIdx.x * NSORT_WPB + w; idx < a.count; idx += gridDim.x * NSORT_WPB) {
-    const int r = a.list[idx];
-    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
-    const int64_t o = nout_row(a.A, r);
+  const int step = gridDim.x * NSORT_WPB;
+  int idx = blockIdx.x * NSORT_WPB + w;
+  RowAhead<SR> x, nx;
+  x.all(A, B, a.list, idx, a.count);
+  for (; idx < a.count; idx += step) {
+    nx.row(A, a.list, idx + step, a.count);
+    const int64_t o = x.r >= 0 ? nout_row(a.A, x.r) : 0;
     const int64_t cb = a.Cp[o];
-    const int c = (int)(a.Cp[o + 1] - cb);
-    const int64_t F = a.f[r];
-    T *out_v = SR::has_val ? Cv + cb : nullptr;
-    sort_row<SR, K, (K <= SORT_WIDE_K)>(A, B, A.p[r], A.p[r + 1], F <= 32 * K ? (int)F : -1, c, s_col, s_val,
-                                        a.Cj + cb, out_v, a.err);
+    const int c = x.r >= 0 ? (int)(a.Cp[o + 1] - cb) : 0;
+    const int64_t F = x.r >= 0 ? a.f[x.r] : 0;
+    int kmn = 0, kmx = 0;
+    const int got = x.r >= 0 ? sort_expand<SR>(A, B, x, 32 * K, s_col, s_val, &kmn, &kmx) : 0;
+    nx.range(A);
+    nx.entries(A);
+    if (got != F || F > 32 * K) {
+      if (lane_id() == 0) atomicExch(a.err, 12);
+    } else if (K == 4 && F <= 64) {  // half the keys: 21 instead of 28 stages, of two keys a lane instead of four
+      sort_finish<SR, 2, true>(got, c, kmn, kmx, s_col, s_val, a.Cj + cb, SR::has_val ? Cv + cb : nullptr, a.err,
+                               a.A.dbg);
+    } else {
+      sort_finish<SR, K, (K <= SORT_WIDE_K)>(got, c, kmn, kmx, s_col, s_val, a.Cj + cb, SR::has_val ? Cv + cb : nullptr,
+                                             a.err, a.A.dbg);
+    }
+    nx.segments(B);
     __syncwarp();
+    x = nx;
   }
 }
 

@@ -107,40 +107,29 @@ template <int K, typename KT> __device__ __forceinline__ void warp_bitonic(KT (&
   }
 }
 
-// The products of A entries [q0, q1) by one warp, in product order, to
+// The products of the row held by x by one warp, in product order, to
 // shared memory (columns at s_col[sr_pad(p)], values at s_val[p], at most
 // nmax of them); returns their number (warp-uniform) and the least and
 // greatest column in *kmn, *kmx.  Shared by every register width, so a kernel
 // that sorts rows of several widths holds one copy of the expansion.
 template <class SR>
-__device__ __forceinline__ int sort_expand(const DevCsr &A, const DevCsr &B, int64_t q0, int64_t q1, int nmax,
+__device__ __forceinline__ int sort_expand(const DevCsr &A, const DevCsr &B, const RowAhead<SR> &x, int nmax,
                                            int *s_col, typename SR::val_t *s_val, int *kmn_out, int *kmx_out) {
   using T = typename SR::val_t;
-  const int lane = lane_id();
-  int base = 0, kmn = 0x7fffffff, kmx = -1;
-  for (int64_t qb = q0; qb < q1; qb += 32) {
-    const int64_t q = qb + lane;
-    int64_t s = 0, e = 0;
-    T av{};
-    if (q < q1) {
-      entry_segment(A, B, q, false, 0, 0, s, e);
-      if constexpr (SR::needs_a) av = load_val<T>(A.v, q);
+  int kmn = 0x7fffffff, kmx = -1;
+  auto put = [&](int col, T v, int p) {
+    if (HS_G(A.dbg, p >= 0 && p < nmax, 90, p)) {
+      s_col[sr_pad(p)] = col;
+      if constexpr (SR::has_val) s_val[p] = v;
     }
-    auto put = [&](int col, T v, int p) {
-      const int at = base + p;
-      if (HS_G(A.dbg, at >= 0 && at < nmax, 90, at)) {
-        s_col[sr_pad(at)] = col;
-        if constexpr (SR::has_val) s_val[at] = v;
-      }
-      kmn = min(kmn, col);
-      kmx = max(kmx, col);
-    };
-    base += warp_expand<SR>(B, s, (int)(e - s), av, put);
-  }
+    kmn = min(kmn, col);
+    kmx = max(kmx, col);
+  };
+  const int got = warp_products_of<SR>(A, B, x, put);
   __syncwarp();
   *kmn_out = warp_min(kmn);
   *kmx_out = warp_max(kmx);
-  return base;
+  return got;
 }
 
 // Sort and fold a row whose F products (F <= 32*K) sort_expand laid out,
@@ -169,41 +158,39 @@ __device__ __forceinline__ void sort_finish(int F, int c, int kmn, int kmx, int 
 #pragma unroll
     for (int i = 0; i < K; ++i) s_col[sr_pad(lane * K + i)] = (int)key[i];
     __syncwarp();
-    // 3. runs of equal columns folded in sorted order, 32 elements a round
-    // (lane l takes element 32*i + l): a run's sum is complete at its last
-    // element, which writes it at the run's rank among the row's columns
+    // 3. runs of equal columns, 32 elements a round (lane l takes element
+    // 32*i + l): the lane at a run's head walks the run in sorted (so product)
+    // order and writes its sum at the run's rank among the row's columns.
+    // These rows hardly repeat a column, so a walk is a step or none; a
+    // segmented scan of every round took five shuffle-and-add steps of two
+    // words each whatever the runs.
     const unsigned le = 0xffffffffu >> (31 - lane);  // lanes <= this one
     int outb = 0;
-    T carry = sr_identity<SR>();
+    uint32_t last = 0;  // the previous round's last key
     for (int i = 0; i * 32 < F; ++i) {
       const int e = i * 32 + lane;
       const bool valid = e < F;
       const uint32_t kk = valid ? (uint32_t)s_col[sr_pad(e)] : 0xffffffffu;
-      const uint32_t kp = (valid && e > 0) ? (uint32_t)s_col[sr_pad(e - 1)] : 0xffffffffu;
-      const uint32_t kn = (e + 1 < F) ? (uint32_t)s_col[sr_pad(e + 1)] : 0xffffffffu;
+      uint32_t kp = __shfl_up_sync(FULL, kk, 1);
+      if (lane == 0) kp = last;
+      last = __shfl_sync(FULL, kk, 31);
       const bool head = valid && (e == 0 || (kk >> PB) != (kp >> PB));
-      const bool tail = valid && (e + 1 >= F || (kn >> PB) != (kk >> PB));
       const unsigned hm = __ballot_sync(FULL, head);
       const int pos = outb + __popc(hm & le) - 1;
-      T v{};
-      if constexpr (SR::has_val) {
-        v = valid ? s_val[kk & (N - 1)] : SR::identity();
-        bool fl = head;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const T y = shfl_up_val<T>(v, d);
-          const bool g = __shfl_up_sync(FULL, (int)fl, d) != 0;
-          if (lane >= d) {
-            if (!fl) v = SR::add(y, v);
-            fl = fl || g;
+      if (head) {
+        T v{};
+        if constexpr (SR::has_val) {
+          v = s_val[kk & (N - 1)];
+          for (int j = e + 1; j < F; ++j) {
+            const uint32_t kj = (uint32_t)s_col[sr_pad(j)];
+            if ((kj >> PB) != (kk >> PB)) break;
+            v = SR::add(v, s_val[kj & (N - 1)]);
           }
         }
-        if (!fl && valid) v = SR::add(carry, v);  // continues the previous round's last run
-        carry = shfl_val<T>(v, 31);
-      }
-      if (tail && HS_G(dbg, pos >= 0 && pos < c, 91, pos)) {
-        __stcs(out_j + pos, (int)(kk >> PB) + kmn);
-        if constexpr (SR::has_val) __stcs(out_v + pos, v);
+        if (HS_G(dbg, pos >= 0 && pos < c, 91, pos)) {
+          __stcs(out_j + pos, (int)(kk >> PB) + kmn);
+          if constexpr (SR::has_val) __stcs(out_v + pos, v);
+        }
       }
       outb += __popc(hm);
     }
@@ -277,22 +264,6 @@ __device__ __forceinline__ void sort_finish(int F, int c, int kmn, int kmx, int 
     if constexpr (SR::has_val) __stcs(out_v + outi, acc);
   }
   if (total != c && lane == 0) atomicExch(err, 13);
-}
-
-// Row r of C (A entries [q0, q1), F products, c outputs) by one warp, for
-// F <= 32*K.  s_col holds sr_pad_len(32*K) ints, s_val 32*K values.  A
-// product count other than F sets *err.
-template <class SR, int K, bool WIDE>
-__device__ __forceinline__ void sort_row(const DevCsr &A, const DevCsr &B, int64_t q0, int64_t q1, int F, int c,
-                                         int *s_col, typename SR::val_t *s_val, int32_t *out_j,
-                                         typename SR::val_t *out_v, int *err) {
-  int kmn = 0, kmx = 0;
-  const int got = sort_expand<SR>(A, B, q0, q1, 32 * K, s_col, s_val, &kmn, &kmx);
-  if (got != F || F < 0 || F > 32 * K) {
-    if (lane_id() == 0) atomicExch(err, 12);
-    return;
-  }
-  sort_finish<SR, K, WIDE>(F, c, kmn, kmx, s_col, s_val, out_j, out_v, err, A.dbg);
 }
 
 }  // namespace hs

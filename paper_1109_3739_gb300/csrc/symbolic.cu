@@ -40,23 +40,21 @@ __global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny(SymArgs a) {
   __shared__ int scol[TINY_WPB][32];
   const int w = threadIdx.x >> 5, lane = lane_id();
   const DevCsr A = dev_a(a.A), B = dev_b(a.B);
-  for (int idx = blockIdx.x * TINY_WPB + w; idx < a.count; idx += gridDim.x * TINY_WPB) {
-    const int r = a.list[idx];
-    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
-    const int64_t q0 = A.p[r], q1 = A.p[r + 1];
-    int nprod = 0;
-    for (int64_t qb = q0; qb < q1; qb += 32) {
-      const int64_t q = qb + lane;
-      int64_t s = 0, e = 0;
-      if (q < q1) entry_segment(A, B, q, false, 0, 0, s, e);
-      auto put = [&](int col, NoVal, int p) {
-        if (HS_G(a.A.dbg, nprod + p < 32, 34, nprod + p)) scol[w][nprod + p] = col;
-      };
-      nprod += warp_expand<StructSR>(B, s, (int)(e - s), NoVal{}, put);
-    }
+  const int step = gridDim.x * TINY_WPB;
+  int idx = blockIdx.x * TINY_WPB + w;
+  RowAhead<StructSR> x, nx;
+  x.all(A, B, a.list, idx, a.count);
+  for (; idx < a.count; idx += step) {
+    nx.row(A, a.list, idx + step, a.count);
+    auto put = [&](int col, NoVal, int p) {
+      if (HS_G(a.A.dbg, p < 32, 34, p)) scol[w][p] = col;
+    };
+    const int nprod = x.r >= 0 ? warp_products_of<StructSR>(A, B, x, put) : 0;
+    nx.range(A);
     __syncwarp();
     const bool have = lane < nprod && lane < 32;
     const int col = have ? scol[w][lane] : 0;
+    nx.entries(A);
     const unsigned act = __ballot_sync(FULL, have);
     bool first = false;
     if (have) {
@@ -64,11 +62,13 @@ __global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny(SymArgs a) {
       first = lane == __ffs(grp) - 1;
     }
     const int cnt = __popc(__ballot_sync(FULL, first));
-    if (lane == 0) {
-      put_count(a, out_row(a.A, r), cnt);
+    nx.segments(B);
+    if (lane == 0 && x.r >= 0) {
+      put_count(a, out_row(a.A, x.r), cnt);
       if (nprod > 32) atomicExch(a.err, 2);
     }
     __syncwarp();
+    x = nx;
   }
 }
 
@@ -83,19 +83,28 @@ __global__ void __launch_bounds__(WARP_WPB * 32, 4) k_sym_warp(SymArgs a) {
   const int w = threadIdx.x >> 5, lane = lane_id();
   int *keys = tables + w * SLOTS;
   const DevCsr A = dev_a(a.A), B = dev_b(a.B);
-  for (int idx = blockIdx.x * WARP_WPB + w; idx < a.count; idx += gridDim.x * WARP_WPB) {
-    const int r = a.list[idx];
-    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
-    const int slots = max(64, min(SLOTS, next_pow2(2 * (int)a.f[r])));
+  const int step = gridDim.x * WARP_WPB;
+  int idx = blockIdx.x * WARP_WPB + w;
+  RowAhead<StructSR> x, nx;
+  x.all(A, B, a.list, idx, a.count);
+  int fr = x.r >= 0 ? (int)a.f[x.r] : 0;
+  for (; idx < a.count; idx += step) {
+    nx.row(A, a.list, idx + step, a.count);
+    const int slots = max(64, min(SLOTS, next_pow2(2 * fr)));
     for (int s = lane; s < slots; s += 32) keys[s] = EMPTY;
     __syncwarp();
     int cnt = 0;
     const unsigned mask = slots - 1;
-    warp_products<StructSR>(A, B, A.p[r], A.p[r + 1],
-                            [&](int col, NoVal, int) { cnt += hash_insert_key(keys, mask, col); });
+    nx.range(A);
+    fr = nx.r >= 0 ? (int)__ldg(a.f + nx.r) : 0;
+    auto put = [&](int col, NoVal, int) { cnt += hash_insert_key(keys, mask, col); };
+    if (x.r >= 0) warp_products_of<StructSR>(A, B, x, put);
+    nx.entries(A);
     cnt = warp_sum(cnt);
-    if (lane == 0) put_count(a, out_row(a.A, r), cnt);
+    nx.segments(B);
+    if (lane == 0 && x.r >= 0) put_count(a, out_row(a.A, x.r), cnt);
     __syncwarp();
+    x = nx;
   }
 }
 
