@@ -14,6 +14,8 @@
 // applied through I and the inverse index map cpos, and neither S*A*T nor its
 // negation is ever materialised (Section 3.1).  Nor is R*B*Q, when B's rows
 // keep their order under J: its entries are B's, moved to rows I and columns J.
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -28,6 +30,11 @@ static int grid1(int64_t n, int nt = 256) {
 
 #define GRID_STRIDE(i, n) \
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
+
+__device__ __forceinline__ void copy_val(void *dst, int64_t at, const void *src, int64_t q, int vb) {
+  if (vb == 8) reinterpret_cast<uint64_t *>(dst)[at] = reinterpret_cast<const uint64_t *>(src)[q];
+  else if (vb == 4) reinterpret_cast<uint32_t *>(dst)[at] = reinterpret_cast<const uint32_t *>(src)[q];
+}
 
 __global__ void k_iota_i64(int64_t *p, int64_t n) { GRID_STRIDE(i, n) p[i] = i; }
 
@@ -116,14 +123,324 @@ void launch_sort_short_rows(const int64_t *ptr, int32_t *j, int64_t rows, cudaSt
 // B = A(I, J) without forming R*A: the rows I[t] of A are laid end to end
 // (gathered entry g of output row t is entry A.p[I[t]] + g - G[t] of A,
 // G the scanned row lengths), every gathered entry (t, c, v) becomes one
-// tuple (t, p, v) for each p with J[p] == c (Q's row c), and the tuples are
-// sorted by (t, p) -- or, when J is strictly increasing, written in place,
-// already in order.
+// tuple (t, p, v) for each p with J[p] == c (Q's row c).  When J repeats no
+// index, that is at most one tuple: Q is J's inverse map, the tuples lie row
+// by row, in order when J is increasing, else each row is sorted.  When J
+// repeats indices the tuples are sorted by (t, p).
 
-// G[t + 1] = length of row I[t] (G[0] is zero)
-__global__ void k_gather_len(const int64_t *Ap, const int32_t *I, int64_t nI, int64_t *G) {
-  GRID_STRIDE(t, nI) G[t + 1] = Ap[I[t] + 1] - Ap[I[t]];
+// First look at A, I and J: flag bit 1: an index out of range, bit 2: J
+// repeats an index, bit 4: J not strictly increasing; pos[J[p]] = p (filled
+// with -1 before); G[t + 1] = length of row I[t] (0 for a bad index), the
+// longest in *lmax.
+__global__ void k_spref_begin(const int64_t *Ap, int64_t m, int64_t n, const int32_t *I, int64_t nI, const int32_t *J,
+                              int64_t nJ, int32_t *pos, int64_t *G, int *flag, unsigned long long *lmax) {
+  int bad = 0;
+  unsigned long long mx = 0;
+  GRID_STRIDE(p, nJ) {
+    const int32_t c = J[p];
+    if (c < 0 || c >= n) bad |= 1;
+    else if (atomicExch(pos + c, (int32_t)p) != -1) bad |= 2;
+    if (p + 1 < nJ && c >= J[p + 1]) bad |= 4;
+  }
+  GRID_STRIDE(t, nI) {
+    const int32_t r = I[t];
+    int64_t len = 0;
+    if (r < 0 || r >= m) bad |= 1;
+    else len = max(Ap[r + 1] - Ap[r], (int64_t)0);
+    G[t + 1] = len;
+    if (t == 0) G[0] = 0;
+    mx = max(mx, (unsigned long long)len);
+  }
+  bad = __reduce_or_sync(FULL, bad);
+  mx = warp_max(mx);
+  if (lane_id() == 0) {
+    if (bad) atomicOr(flag, bad);
+    if (mx) atomicMax(lmax, mx);
+  }
 }
+void launch_spref_begin(const int64_t *Ap, int64_t m, int64_t n, const int32_t *I, int64_t nI, const int32_t *J,
+                        int64_t nJ, int32_t *pos, int64_t *G, int *flag, unsigned long long *lmax, cudaStream_t st) {
+  const int64_t work = nI > nJ ? nI : nJ;
+  if (work <= 0) return;
+  count_launch();
+  k_spref_begin<<<grid1(work), 256, 0, st>>>(Ap, m, n, I, nI, J, nJ, pos, G, flag, lmax);
+}
+
+// ---- J without repetitions: an entry makes at most one tuple.  A block takes
+// 2048 gathered entries, finds the output rows they lie in by a search of G
+// and notes for each entry its column p in B (-1: none) and its value, a bit
+// per entry and the kept entries per word of 32; after a scan of the words'
+// counts, K(g) = kept entries before g is an entry's place among the kept.
+constexpr int SG_NT = 256, SG_PER = 8, SG_TILE = SG_NT * SG_PER;
+__global__ void __launch_bounds__(SG_NT) k_spref_gather(SprefArgs a) {
+  __shared__ int64_t s_g[SG_TILE], s_row[2];
+  const int64_t g0 = (int64_t)blockIdx.x * SG_TILE, g1 = min(g0 + SG_TILE, a.total);
+  if (threadIdx.x < 64) {
+    const int64_t r = warp_upper_bound(a.G, a.nI + 1, threadIdx.x < 32 ? g0 : g1 - 1) - 1;
+    if (lane_id() == 0) s_row[threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
+  const int64_t r0 = s_row[0], r1 = s_row[1];
+  const bool staged = r1 - r0 < SG_TILE;
+  if (staged)
+    for (int64_t r = r0 + threadIdx.x; r <= r1; r += SG_NT) s_g[r - r0] = a.G[r];
+  __syncthreads();
+  int64_t q[SG_PER];
+  int c[SG_PER], p[SG_PER];
+#pragma unroll
+  for (int u = 0; u < SG_PER; ++u) {
+    const int64_t g = g0 + u * SG_NT + threadIdx.x;
+    q[u] = -1;
+    if (g >= g1) continue;
+    int64_t l = r0, h = r1 + 1;  // last row that starts at or before g
+    while (h - l > 1) {
+      const int64_t mid = (l + h) >> 1;
+      if ((staged ? s_g[mid - r0] : a.G[mid]) <= g) l = mid;
+      else h = mid;
+    }
+    q[u] = a.Ap[a.I[l]] + (g - (staged ? s_g[l - r0] : a.G[l]));
+  }
+#pragma unroll
+  for (int u = 0; u < SG_PER; ++u) c[u] = q[u] >= 0 ? a.Aj[q[u]] : -1;
+#pragma unroll
+  for (int u = 0; u < SG_PER; ++u) p[u] = c[u] >= 0 && c[u] < a.n ? __ldg(a.pos + c[u]) : -1;
+#pragma unroll
+  for (int u = 0; u < SG_PER; ++u) {
+    const int64_t g = g0 + u * SG_NT + threadIdx.x;
+    const unsigned m = __ballot_sync(FULL, p[u] >= 0);
+    if (g < g1) a.P[g] = p[u];
+    if (p[u] >= 0) copy_val(a.V, g, a.Av, q[u], a.vb);
+    if (lane_id() == 0 && g < g1) {
+      a.keep[g >> 5] = m;
+      a.S[g >> 5] = __popc(m);
+    }
+  }
+}
+// the kept entries in order: B's entries as they stand when J is increasing
+__global__ void __launch_bounds__(256) k_spref_emit(SprefArgs a, int32_t *Bj, void *Bv) {
+  GRID_STRIDE(g, a.total) {
+    const uint32_t kw = a.keep[g >> 5];
+    if (!((kw >> (g & 31)) & 1u)) continue;
+    const int64_t d = ((g >> 5) ? a.S[(g >> 5) - 1] : 0) + __popc(kw & ((1u << (g & 31)) - 1u));
+    Bj[d] = a.P[g];
+    copy_val(Bv, d, a.V, g, a.vb);
+  }
+}
+__global__ void k_spref_offsets(SprefArgs a, int64_t *Bp) {
+  GRID_STRIDE(t, a.nI + 1) {
+    const int64_t g = a.G[t], w = g >> 5;
+    const int b = (int)(g & 31);
+    Bp[t] = (w ? a.S[w - 1] : 0) + (b ? __popc(a.keep[w] & ((1u << b) - 1u)) : 0);
+  }
+}
+
+// ---- rows into increasing order of p, for a J in any order.  The tuples of a
+// row lie together already, so only rows are sorted, by their length: eight
+// lanes a row of at most 8, a warp up to SR_WARP (ranks counted directly), a
+// block up to SR_CTA (buckets in shared memory), and longer ones through a
+// bitmap of B's columns (rank = set bits before p).  Every tuple is read and
+// written once; a radix sort of all (row, p) keys took five passes.
+constexpr int SR_WARP = 256, SR_CTA = 2048;
+template <typename T> struct SprefRowArgs {
+  const int64_t *Bp;
+  int64_t nI, nJ;
+  const int32_t *P;  // kept tuples, row by row
+  const T *V;
+  int32_t *Bj;
+  T *Bv;
+  int *count;        // rows left to the block kernel, to the bitmap kernel; their work counters; error
+  int32_t *list;     // 2 * nI
+  long long *dbg;
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_spref_rows(SprefRowArgs<T> a) {
+  constexpr bool HAS_VAL = !std::is_same<T, NoVal>::value;
+  const int lane = lane_id(), sub = lane >> 3, l = lane & 7;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; t0 < a.nI; t0 += nw * 4) {
+    const int64_t t = t0 + sub;
+    const int64_t b = t < a.nI ? a.Bp[t] : 0;
+    const int64_t c = t < a.nI ? a.Bp[t + 1] - b : 0;
+    {
+      const bool mine = c <= 8 && l < c;
+      const int32_t p = mine ? a.P[b + l] : 0x7fffffff;
+      T v{};
+      if constexpr (HAS_VAL)
+        if (mine) v = a.V[b + l];
+      int rank = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) rank += __shfl_sync(FULL, p, (sub << 3) + j) < p;
+      if (mine) {
+        a.Bj[b + rank] = p;
+        if constexpr (HAS_VAL) a.Bv[b + rank] = v;
+      }
+    }
+    // longer rows: the whole warp, one row after the other
+    for (unsigned more = __ballot_sync(FULL, l == 0 && c > 8); more; more &= more - 1) {
+      const int src = __ffs(more) - 1;
+      const int64_t rb = __shfl_sync(FULL, b, src), rc = __shfl_sync(FULL, c, src);
+      if (rc > SR_WARP) {
+        if (lane == 0) {
+          const int kind = rc > SR_CTA;
+          a.list[kind * a.nI + atomicAdd(a.count + kind, 1)] = (int32_t)(t0 + (src >> 3));
+        }
+        continue;
+      }
+      const int n = (int)rc;
+      for (int e0 = 0; e0 < n; e0 += 64) {  // two of the row's tuples per lane
+        const int ea = e0 + lane, eb = ea + 32;
+        const int32_t pa = ea < n ? a.P[rb + ea] : 0x7fffffff, pb = eb < n ? a.P[rb + eb] : 0x7fffffff;
+        int ra = 0, rk = 0;
+        for (int x0 = 0; x0 < n; x0 += 32) {
+          const int32_t px = x0 + lane < n ? a.P[rb + x0 + lane] : 0x7fffffff;
+          const int lim = min(32, n - x0);
+          for (int j = 0; j < lim; ++j) {
+            const int32_t y = __shfl_sync(FULL, px, j);
+            ra += y < pa;
+            rk += y < pb;
+          }
+        }
+        if (ea < n) {
+          a.Bj[rb + ra] = pa;
+          if constexpr (HAS_VAL) a.Bv[rb + ra] = a.V[rb + ea];
+        }
+        if (eb < n) {
+          a.Bj[rb + rk] = pb;
+          if constexpr (HAS_VAL) a.Bv[rb + rk] = a.V[rb + eb];
+        }
+      }
+    }
+  }
+}
+template <typename T> struct SprefCtaSmem {
+  static constexpr size_t vb = std::is_same<T, NoVal>::value ? 0 : sizeof(T);
+  static constexpr size_t arr = (size_t)SR_CTA * (4 + vb);          // keys and values
+  static constexpr size_t work = (size_t)SR_CTA * (12 + vb) + 16;   // group_sort_emit's work
+  static constexpr size_t bytes = 2 * arr + work;
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_spref_rows_cta(SprefRowArgs<T> a) {
+  constexpr bool HAS_VAL = !std::is_same<T, NoVal>::value;
+  using L = SprefCtaSmem<T>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ EmitScratch es;
+  __shared__ int s_item, wtmp[33];
+  T *v0 = reinterpret_cast<T *>(smem), *v1 = reinterpret_cast<T *>(smem + L::arr);
+  int *k0 = reinterpret_cast<int *>(smem + SR_CTA * L::vb), *k1 = reinterpret_cast<int *>(smem + L::arr + SR_CTA * L::vb);
+  const int count = a.count[0];
+  while (true) {
+    if (threadIdx.x == 0) s_item = atomicAdd(a.count + 2, 1);
+    __syncthreads();
+    const int i = s_item;
+    if (i >= count) break;
+    const int64_t t = a.list[i];
+    const int64_t b = a.Bp[t];
+    const int c = (int)(a.Bp[t + 1] - b);
+    for (int e = threadIdx.x; e < c; e += 256) {
+      k0[e] = a.P[b + e];
+      if constexpr (HAS_VAL) v0[e] = a.V[b + e];
+    }
+    __syncthreads();
+    group_sort_emit<CtaGroup, T, HAS_VAL>(k0, v0, c, c, k1, v1, smem + 2 * L::arr, wtmp, &es, a.Bj + b,
+                                          HAS_VAL ? a.Bv + b : nullptr, a.count + 4, SR_CTA, a.dbg);
+    __syncthreads();
+  }
+}
+constexpr int SR_NT = 1024, SR_WORDS = BITMAP_COLS / 32, SR_GROUPS = SR_WORDS / 32;
+struct SprefBitSmem {
+  unsigned bits[SR_WORDS];  // B's columns of the chunk
+  uint16_t pre[SR_WORDS];   // set bits before the word in its group of 32 words
+  int base[SR_GROUPS];      // set bits before the group
+  int wtmp[33];
+  int item;
+};
+template <typename T>
+__global__ void __launch_bounds__(SR_NT) k_spref_rows_bits(SprefRowArgs<T> a) {
+  constexpr bool HAS_VAL = !std::is_same<T, NoVal>::value;
+  extern __shared__ __align__(16) unsigned char smem[];
+  SprefBitSmem &sm = *reinterpret_cast<SprefBitSmem *>(smem);
+  const int count = a.count[1], tid = threadIdx.x;
+  while (true) {
+    if (tid == 0) sm.item = atomicAdd(a.count + 3, 1);
+    __syncthreads();
+    const int i = sm.item;
+    if (i >= count) break;
+    const int64_t t = a.list[a.nI + i];
+    const int64_t b = a.Bp[t], c = a.Bp[t + 1] - b;
+    int64_t done = 0;  // entries with smaller columns than the chunk's
+    for (int64_t lo = 0; lo < a.nJ; lo += BITMAP_COLS) {
+      const int groups = (int)((min(a.nJ - lo, (int64_t)BITMAP_COLS) + 1023) >> 10);
+      for (int w = tid; w < groups * 32; w += SR_NT) sm.bits[w] = 0u;
+      __syncthreads();
+      for (int64_t e = tid; e < c; e += SR_NT) {
+        const int64_t x = a.P[b + e] - lo;
+        if (x >= 0 && x < BITMAP_COLS) atomicOr(sm.bits + (x >> 5), 1u << (x & 31));
+      }
+      __syncthreads();
+      for (int g = tid >> 5; g < groups; g += SR_NT / 32) {  // a warp per group, a word per lane
+        const int w = g * 32 + lane_id();
+        const int n1 = __popc(sm.bits[w]);
+        const int incl = warp_incl_scan(n1);
+        sm.pre[w] = (uint16_t)(incl - n1);
+        if (lane_id() == 31) sm.base[g] = incl;
+      }
+      __syncthreads();
+      const int tot = group_excl_scan<CtaGroup>(sm.base, groups, sm.wtmp);
+      for (int64_t e = tid; e < c; e += SR_NT) {
+        const int32_t p = a.P[b + e];
+        const int64_t x = p - lo;
+        if (x < 0 || x >= BITMAP_COLS) continue;
+        const int w = (int)(x >> 5);
+        const int64_t r = done + sm.base[w >> 5] + sm.pre[w] + __popc(sm.bits[w] & ((1u << (x & 31)) - 1u));
+        if (!HS_G(a.dbg, r < c, 88, r)) continue;
+        a.Bj[b + r] = p;
+        if constexpr (HAS_VAL) a.Bv[b + r] = a.V[b + e];
+      }
+      done += tot;
+      __syncthreads();
+    }
+  }
+}
+
+void launch_spref_gather(const SprefArgs &a, cudaStream_t st) {
+  if (a.total <= 0) return;
+  count_launch();
+  k_spref_gather<<<(unsigned)((a.total + SG_TILE - 1) / SG_TILE), SG_NT, 0, st>>>(a);
+}
+void launch_spref_emit(const SprefArgs &a, int64_t *Bp, int32_t *Bj, void *Bv, cudaStream_t st) {
+  count_launch();
+  k_spref_offsets<<<grid1(a.nI + 1), 256, 0, st>>>(a, Bp);
+  if (a.total <= 0) return;
+  count_launch();
+  k_spref_emit<<<grid1(a.total), 256, 0, st>>>(a, Bj, Bv);
+}
+template <typename T>
+static void spref_rows(const int64_t *Bp, int64_t nI, int64_t nJ, const int32_t *P, const void *V, int32_t *Bj,
+                       void *Bv, int64_t lmax, int *count, int32_t *list, long long *dbg, cudaStream_t st) {
+  const SprefRowArgs<T> a{Bp, nI, nJ, P, reinterpret_cast<const T *>(V), Bj, reinterpret_cast<T *>(Bv), count, list, dbg};
+  count_launch();
+  k_spref_rows<T><<<grid1(nI * 8), 256, 0, st>>>(a);
+  if (lmax > SR_WARP) {
+    const int fit = fit_per_sm(k_spref_rows_cta<T>, 256, SprefCtaSmem<T>::bytes);
+    count_launch();
+    k_spref_rows_cta<T><<<sm_count() * fit, 256, SprefCtaSmem<T>::bytes, st>>>(a);
+  }
+  if (lmax > SR_CTA) {
+    fit_per_sm(k_spref_rows_bits<T>, SR_NT, sizeof(SprefBitSmem));
+    count_launch();
+    k_spref_rows_bits<T><<<sm_count(), SR_NT, sizeof(SprefBitSmem), st>>>(a);
+  }
+}
+void launch_spref_rows(int vb, const int64_t *Bp, int64_t nI, int64_t nJ, const int32_t *P, const void *V, int32_t *Bj,
+                       void *Bv, int64_t lmax, int *count, int32_t *list, long long *dbg, cudaStream_t st) {
+  if (nI <= 0) return;
+  if (vb == 8) spref_rows<unsigned long long>(Bp, nI, nJ, P, V, Bj, Bv, lmax, count, list, dbg, st);
+  else if (vb == 4) spref_rows<uint32_t>(Bp, nI, nJ, P, V, Bj, Bv, lmax, count, list, dbg, st);
+  else spref_rows<NoVal>(Bp, nI, nJ, P, V, Bj, Bv, lmax, count, list, dbg, st);
+}
+
+// ---- J with repetitions: every tuple (t, p) of an entry is laid out and the
+// tuples are sorted
 // inc[G[t]] += 1 for every row starting inside [0, total): after an
 // inclusive scan, inc[g] - 1 is the output row of gathered entry g
 __global__ void k_row_starts(const int64_t *G, int64_t nI, int64_t total, int64_t *inc) {
@@ -146,10 +463,6 @@ __global__ void k_gather_w(GatherArgs a, int64_t *W) {
     W[g] = (c >= 0 && c < a.ncols) ? a.Qp[c + 1] - a.Qp[c] : 0;
   }
 }
-__device__ __forceinline__ void copy_val(void *dst, int64_t at, const void *src, int64_t q, int vb) {
-  if (vb == 8) reinterpret_cast<uint64_t *>(dst)[at] = reinterpret_cast<const uint64_t *>(src)[q];
-  else if (vb == 4) reinterpret_cast<uint32_t *>(dst)[at] = reinterpret_cast<const uint32_t *>(src)[q];
-}
 // the tuples, entry g's at [W[g-1], W[g]) of the scanned counts
 __global__ void k_gather_fill(GatherArgs a, const int64_t *W, int32_t *ti, int32_t *pj, void *tv) {
   GRID_STRIDE(g, a.total) {
@@ -164,36 +477,6 @@ __global__ void k_gather_fill(GatherArgs a, const int64_t *W, int32_t *ti, int32
       copy_val(tv, at, a.Av, q, a.vb);
     }
   }
-}
-// J strictly increasing: each entry makes at most one tuple and a row's
-// tuples come out in increasing p, so they are B's entries as they stand
-__global__ void k_gather_direct(GatherArgs a, const int64_t *W, int32_t *Bj, void *Bv) {
-  GRID_STRIDE(g, a.total) {
-    const int64_t before = g > 0 ? W[g - 1] : 0;
-    if (W[g] == before) continue;
-    int64_t t, q;
-    int c;
-    gather_entry(a, g, t, q, c);
-    Bj[before] = a.Qj[a.Qp[c]];
-    copy_val(Bv, before, a.Av, q, a.vb);
-  }
-}
-// B's offsets from the scanned tuple counts: Bp[t] = W[G[t] - 1]
-__global__ void k_gather_offsets(const int64_t *G, int64_t nI, const int64_t *W, int64_t *Bp) {
-  GRID_STRIDE(t, nI + 1) {
-    const int64_t g = G[t];
-    Bp[t] = g > 0 ? W[g - 1] : 0;
-  }
-}
-// flag bit 4: J not strictly increasing
-__global__ void k_check_increasing(const int32_t *X, int64_t n, int *flag) {
-  GRID_STRIDE(i, n - 1) if (X[i] >= X[i + 1]) atomicOr(flag, 4);
-}
-
-void launch_gather_len(const int64_t *Ap, const int32_t *I, int64_t nI, int64_t *G, cudaStream_t st) {
-  if (nI <= 0) return;
-  count_launch();
-  k_gather_len<<<grid1(nI), 256, 0, st>>>(Ap, I, nI, G);
 }
 void launch_row_starts(const int64_t *G, int64_t nI, int64_t total, int64_t *inc, cudaStream_t st) {
   if (nI <= 0 || total <= 0) return;
@@ -210,35 +493,6 @@ void launch_gather_fill(const GatherArgs &a, const int64_t *W, int32_t *ti, int3
   count_launch();
   k_gather_fill<<<grid1(a.total), 256, 0, st>>>(a, W, ti, pj, tv);
 }
-void launch_gather_direct(const GatherArgs &a, const int64_t *W, int32_t *Bj, void *Bv, cudaStream_t st) {
-  if (a.total <= 0) return;
-  count_launch();
-  k_gather_direct<<<grid1(a.total), 256, 0, st>>>(a, W, Bj, Bv);
-}
-void launch_gather_offsets(const int64_t *G, int64_t nI, const int64_t *W, int64_t *Bp, cudaStream_t st) {
-  count_launch();
-  k_gather_offsets<<<grid1(nI + 1), 256, 0, st>>>(G, nI, W, Bp);
-}
-void launch_check_increasing(const int32_t *X, int64_t n, int *flag, cudaStream_t st) {
-  if (n <= 1) return;
-  count_launch();
-  k_check_increasing<<<grid1(n - 1), 256, 0, st>>>(X, n, flag);
-}
-
-// flag bit 1: an index outside [0, bound)
-__global__ void k_check_range(const int32_t *X, int64_t n, int64_t bound, int *flag) {
-  GRID_STRIDE(i, n) {
-    const int32_t v = X[i];
-    if (v < 0 || v >= bound) atomicOr(flag, 1);
-  }
-}
-void launch_check_range(const int32_t *X, int64_t n, int64_t bound, int *flag, cudaStream_t st) {
-  if (n > 0) {
-    count_launch();
-    k_check_range<<<grid1(n), 256, 0, st>>>(X, n, bound, flag);
-  }
-}
-
 // pos[X[i]] = i (pos pre-filled with -1) for indices inside [0, bound);
 // flag bit 1: an index out of range (skipped), bit 2: a repeated index.
 __global__ void k_mark_positions(const int32_t *X, int64_t n, int64_t bound, int32_t *pos, int *flag) {

@@ -337,7 +337,6 @@ void launch_max_count(const int64_t *cnt, int64_t n, unsigned long long *out, cu
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t st);
 void launch_build_Q_fill(const int32_t *J, int64_t nJ, int64_t *Qcur, int32_t *Qj, cudaStream_t st);
 void launch_sort_short_rows(const int64_t *ptr, int32_t *j, int64_t rows, cudaStream_t st);
-void launch_check_range(const int32_t *X, int64_t n, int64_t bound, int *flag, cudaStream_t st);
 // pos[X[i]] = i for in-range X[i] (bit 1 of flag: out of range; bit 2: repeated)
 void launch_mark_positions(const int32_t *X, int64_t n, int64_t bound, int32_t *pos, int *flag, cudaStream_t st);
 void launch_fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t st);
@@ -355,13 +354,34 @@ struct GatherArgs {
   int64_t total;       // gathered entries
   int64_t ncols;       // columns of A: a column id outside [0, ncols) makes no tuple
 };
-void launch_gather_len(const int64_t *Ap, const int32_t *I, int64_t nI, int64_t *G, cudaStream_t st);
+void launch_spref_begin(const int64_t *Ap, int64_t m, int64_t n, const int32_t *I, int64_t nI, const int32_t *J,
+                        int64_t nJ, int32_t *pos, int64_t *G, int *flag, unsigned long long *lmax, cudaStream_t st);
+// J without repetitions: the gathered entries' columns in B, values, keep
+// bits and kept entries per word; then B (J increasing) or its rows' tuples in
+// A's order, and the rows sorted (lmax: entries of a row at most; count: 5
+// zeroed ints, [4] an error code; list: 2 * nI)
+struct SprefArgs {
+  const int64_t *Ap;
+  const int32_t *Aj;
+  const void *Av;
+  int vb;
+  const int32_t *I;
+  int64_t nI, n;
+  const int64_t *G;    // nI + 1 gathered offsets
+  int64_t total;       // gathered entries
+  const int32_t *pos;  // n: place in J or -1
+  int32_t *P;          // total
+  void *V;             // total
+  uint32_t *keep;      // a bit per gathered entry
+  int64_t *S;          // kept entries per word, then their inclusive scan
+};
+void launch_spref_gather(const SprefArgs &a, cudaStream_t st);
+void launch_spref_emit(const SprefArgs &a, int64_t *Bp, int32_t *Bj, void *Bv, cudaStream_t st);
+void launch_spref_rows(int vb, const int64_t *Bp, int64_t nI, int64_t nJ, const int32_t *P, const void *V, int32_t *Bj,
+                       void *Bv, int64_t lmax, int *count, int32_t *list, long long *dbg, cudaStream_t st);
 void launch_row_starts(const int64_t *G, int64_t nI, int64_t total, int64_t *inc, cudaStream_t st);
 void launch_gather_w(const GatherArgs &a, int64_t *W, cudaStream_t st);
 void launch_gather_fill(const GatherArgs &a, const int64_t *W, int32_t *ti, int32_t *pj, void *tv, cudaStream_t st);
-void launch_gather_direct(const GatherArgs &a, const int64_t *W, int32_t *Bj, void *Bv, cudaStream_t st);
-void launch_gather_offsets(const int64_t *G, int64_t nI, const int64_t *W, int64_t *Bp, cudaStream_t st);
-void launch_check_increasing(const int32_t *X, int64_t n, int *flag, cudaStream_t st);
 
 // sparse.cu: sparse(i, j, v, m, n) by a stable radix sort of (row, column)
 // keys.  Tiles of sp_tiles(nnz); look-back status of 256 words per tile.

@@ -832,11 +832,13 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
                        int dtype, int sr, hs_mat *C, Mem &mem, Mem &outmem, uint32_t flags);
 
 // B = A(I, J) (Section 3.1's SpRef), the triple product R*A*Q evaluated
-// without forming R*A: the rows I[t] are gathered end to end, each gathered
-// entry (t, c, v) yields (t, p, v) for every p with J[p] == c (Q's row c),
-// and the tuples are ordered by (t, p) with the radix sort of sparse(); when
-// J is strictly increasing they are in order already and are written out
-// directly.  Four host synchronisations (three with a strictly increasing J).
+// without forming R*A: the rows I[t] are gathered end to end and each gathered
+// entry (t, c, v) yields (t, p, v) for every p with J[p] == c (Q's row c).
+// When J repeats no index, Q is the inverse map of J: an entry yields one
+// tuple or none, the tuples lie row by row, and only the rows are sorted (not
+// even those when J is increasing); two host synchronisations.  When J
+// repeats indices the tuples are ordered by (t, p) with the radix sort of
+// sparse(); five host synchronisations.
 static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ, hs_mat *Bout,
                       Mem &mem, Mem &outmem, uint32_t flags) {
   cudaStream_t st = mem.st;
@@ -847,46 +849,115 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
   if (A->dtype != HS_BOOL && A->nnz > 0 && !A->val) return HS_EINVAL;
   const int vb = A->dtype == HS_BOOL ? 0 : vbytes_of(A->dtype);
   const int64_t n = A->n;
-  int *flag = mem.tmp<int>(2);
-  unsigned long long *qmax = mem.tmp<unsigned long long>(1);
-  int64_t *hbuf = (int64_t *)pinned(32);
-  int64_t *Qp = mem.tmp<int64_t>(n + 1);
-  int64_t *Qcur = mem.tmp<int64_t>(n + 1);
-  int32_t *Qj = mem.tmp<int32_t>(nJ > 0 ? nJ : 1);
+  struct Small {  // device counters, read back in one copy
+    int flag[2];
+    int count[5];
+    int pad;
+    unsigned long long lmax, qmax;
+    int64_t total;
+    long long dbg[2];
+  };
+  Small *sb = mem.tmp<Small>(1);
+  Small *hb = (Small *)pinned(sizeof(Small));
+  int32_t *pos = mem.tmp<int32_t>(n > 0 ? n : 1);
   int64_t *G = mem.tmp<int64_t>(nI + 1);
   int64_t *scan_tmp = mem.tmp<int64_t>(scan_tmp_elems((n + 1) > (nI + 1) ? (n + 1) : (nI + 1)));
-  if (mem.failed || !hbuf) return HS_ENOMEM;
-  // index ranges are always checked, and before any kernel uses I or J as
-  // an address: they index A's rows, Q's rows and the gathered offsets (the
-  // row counts of Q skip out-of-range ids, so they run alongside)
-  CK(cudaMemsetAsync(flag, 0, 8, st));
-  CK(cudaMemsetAsync(qmax, 0, 8, st));
-  CK(cudaMemsetAsync(Qp, 0, sizeof(int64_t) * (size_t)(n + 1), st));
-  launch_check_range(I, nI, A->m, flag, st);
-  launch_check_range(J, nJ, n, flag, st);
-  launch_check_increasing(J, nJ, flag, st);
-  if (flags & HS_FLAG_VALIDATE) launch_validate(A->ptr, A->idx, A->m, A->n, flag + 1, st);
-  launch_build_Q_count(J, nJ, n, Qp, st);
-  launch_max_count(Qp, n + 1, qmax, st);
-  CK(cudaMemcpyAsync(hbuf, flag, 8, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(hbuf + 1, qmax, 8, cudaMemcpyDeviceToHost, st));
+  if (mem.failed || !hb) return HS_ENOMEM;
+  // index ranges are always checked, and before any kernel uses I or J as an
+  // address of its own (the look itself skips bad ones)
+  {
+    PhaseTimer t("spref_gather", st);
+    CK(cudaMemsetAsync(sb, 0, sizeof(Small), st));
+    CK(cudaMemsetAsync(pos, 0xff, sizeof(int32_t) * (size_t)n, st));
+    if (nI == 0) CK(cudaMemsetAsync(G, 0, sizeof(int64_t), st));
+    launch_spref_begin(A->ptr, A->m, n, I, nI, J, nJ, pos, G, sb->flag, &sb->lmax, st);
+    if (flags & HS_FLAG_VALIDATE) launch_validate(A->ptr, A->idx, A->m, A->n, &sb->flag[1], st);
+    launch_scan_i64(G, nI + 1, scan_tmp, st);
+    CK(cudaMemcpyAsync(&sb->total, G + nI, 8, cudaMemcpyDeviceToDevice, st));
+  }
+  CK(cudaMemcpyAsync(hb, sb, sizeof(Small), cudaMemcpyDeviceToHost, st));
+  if (int e = check_launch()) return e;
   CK(cudaStreamSynchronize(st));
-  const int fl = ((int *)hbuf)[0], vf = ((int *)hbuf)[1];
+  const int fl = hb->flag[0], vf = hb->flag[1];
   if (fl & 1) return HS_EINVAL;
   if (vf & 5) return HS_EINVAL;
   if (vf & 2) return HS_ENONCANON;
-  const bool increasing = !(fl & 4);
-  const int64_t qrow_max = hbuf[1];
+  const bool repeats = fl & 2, increasing = !(fl & 4);
+  const int64_t total = hb->total, lmax = (int64_t)hb->lmax;
+
+  auto out = [&](int64_t nnz) {
+    memset(Bout, 0, sizeof(*Bout));
+    Bout->fmt = HS_CSR;
+    Bout->dtype = A->dtype;
+    Bout->m = nI;
+    Bout->n = nJ;
+    Bout->nnz = nnz;
+    Bout->ptr = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(nI + 1));
+    Bout->idx = (int32_t *)outmem.raw(sizeof(int32_t) * (size_t)(nnz > 0 ? nnz : 1));
+    Bout->val = vb ? outmem.raw((size_t)vb * (size_t)(nnz > 0 ? nnz : 1)) : nullptr;
+    return Bout->ptr && Bout->idx && (!vb || Bout->val);
+  };
+  auto empty_out = [&]() -> int {
+    if (!out(0)) return HS_ENOMEM;
+    CK(cudaMemsetAsync(Bout->ptr, 0, sizeof(int64_t) * (size_t)(nI + 1), st));
+    return check_launch();
+  };
+  if (total == 0 || nJ == 0) return empty_out();
+
+  if (!repeats) {
+    const int64_t nw = (total + 31) / 32;
+    int32_t *P = mem.tmp<int32_t>((size_t)total);
+    void *V = vb ? (void *)mem.tmp<char>((size_t)vb * (size_t)total) : nullptr;
+    uint32_t *keep = mem.tmp<uint32_t>((size_t)nw + 1);
+    int64_t *S = mem.tmp<int64_t>((size_t)nw);
+    int64_t *stmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(nw));
+    if (mem.failed) return HS_ENOMEM;
+    const SprefArgs a{A->ptr, A->idx, A->val, vb, I, nI, n, G, total, pos, P, V, keep, S};
+    {
+      PhaseTimer t("spref_gather", st);
+      launch_spref_gather(a, st);
+      launch_scan_i64(S, nw, stmp, st);
+    }
+    CK(cudaMemcpyAsync(&hb->total, S + nw - 1, 8, cudaMemcpyDeviceToHost, st));
+    if (int e = check_launch()) return e;
+    CK(cudaStreamSynchronize(st));
+    const int64_t ntup = hb->total;
+    if (ntup == 0) return empty_out();
+    if (!increasing && ntup > 0x7fffffffLL) return HS_EUNSUPPORTED;
+    if (!out(ntup)) return HS_ENOMEM;
+    PhaseTimer t("spref_emit", st);
+    if (increasing) {
+      launch_spref_emit(a, Bout->ptr, Bout->idx, Bout->val, st);
+      return check_launch();
+    }
+    int32_t *tp = mem.tmp<int32_t>((size_t)ntup);
+    void *tv = vb ? (void *)mem.tmp<char>((size_t)vb * (size_t)ntup) : nullptr;
+    int32_t *list = mem.tmp<int32_t>((size_t)(2 * nI));
+    if (mem.failed) return HS_ENOMEM;
+    launch_spref_emit(a, Bout->ptr, tp, tv, st);
+    launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
+    return check_launch();
+  }
+
   // Q = sparse(J, 1:len(J), 1, n, len(J)): row k holds every p with J[p] == k,
   // increasing.  Short rows (at most 32 repetitions of an index): counted,
   // filled by atomics and sorted in place; otherwise built by the stable
   // radix sort of sparse() itself
+  int64_t *Qp = mem.tmp<int64_t>(n + 1);
+  int64_t *Qcur = mem.tmp<int64_t>(n + 1);
+  int32_t *Qj = mem.tmp<int32_t>(nJ);
+  if (mem.failed) return HS_ENOMEM;
+  CK(cudaMemsetAsync(Qp, 0, sizeof(int64_t) * (size_t)(n + 1), st));
+  launch_build_Q_count(J, nJ, n, Qp, st);
+  launch_max_count(Qp, n + 1, &sb->qmax, st);
+  CK(cudaMemcpyAsync(&hb->qmax, &sb->qmax, 8, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
   struct QGuard {
     hs_mat q{};
     Mem &m;
     ~QGuard() { free_mat(&q, m); }
   } qg{hs_mat{}, mem};
-  if (qrow_max <= 32) {
+  if (hb->qmax <= 32) {
     PhaseTimer t("spref_build", st);
     launch_scan_i64(Qp, n + 1, scan_tmp, st);
     CK(cudaMemcpyAsync(Qcur, Qp, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyDeviceToDevice, st));
@@ -900,32 +971,6 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     Qp = qg.q.ptr;
     Qj = qg.q.idx;
   }
-  {
-    PhaseTimer t("spref_gather", st);
-    CK(cudaMemsetAsync(G, 0, sizeof(int64_t) * (size_t)(nI + 1), st));
-    launch_gather_len(A->ptr, I, nI, G, st);
-    launch_scan_i64(G, nI + 1, scan_tmp, st);
-  }
-  CK(cudaMemcpyAsync(hbuf, G + nI, 8, cudaMemcpyDeviceToHost, st));
-  if (int e = check_launch()) return e;
-  CK(cudaStreamSynchronize(st));
-  const int64_t total = hbuf[0];
-
-  auto empty_out = [&]() {
-    memset(Bout, 0, sizeof(*Bout));
-    Bout->fmt = HS_CSR;
-    Bout->dtype = A->dtype;
-    Bout->m = nI;
-    Bout->n = nJ;
-    Bout->ptr = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(nI + 1));
-    Bout->idx = (int32_t *)outmem.raw(4);
-    Bout->val = vb ? outmem.raw((size_t)vb) : nullptr;
-    if (!Bout->ptr || !Bout->idx || (vb && !Bout->val)) return HS_ENOMEM;
-    CK(cudaMemsetAsync(Bout->ptr, 0, sizeof(int64_t) * (size_t)(nI + 1), st));
-    return check_launch();
-  };
-  if (total == 0 || nJ == 0) return empty_out();
-
   int64_t *inc = mem.tmp<int64_t>((size_t)total);
   int64_t *W = mem.tmp<int64_t>((size_t)total);
   int64_t *scan_g = mem.tmp<int64_t>(scan_tmp_elems(total));
@@ -939,28 +984,11 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     launch_gather_w(ga, W, st);
     launch_scan_i64(W, total, scan_g, st);
   }
-  CK(cudaMemcpyAsync(hbuf, W + total - 1, 8, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&hb->total, W + total - 1, 8, cudaMemcpyDeviceToHost, st));
   if (int e = check_launch()) return e;
   CK(cudaStreamSynchronize(st));
-  const int64_t ntup = hbuf[0];
+  const int64_t ntup = hb->total;
   if (ntup == 0) return empty_out();
-
-  if (increasing) {
-    memset(Bout, 0, sizeof(*Bout));
-    Bout->fmt = HS_CSR;
-    Bout->dtype = A->dtype;
-    Bout->m = nI;
-    Bout->n = nJ;
-    Bout->nnz = ntup;
-    Bout->ptr = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(nI + 1));
-    Bout->idx = (int32_t *)outmem.raw(sizeof(int32_t) * (size_t)ntup);
-    Bout->val = vb ? outmem.raw((size_t)vb * (size_t)ntup) : nullptr;
-    if (!Bout->ptr || !Bout->idx || (vb && !Bout->val)) return HS_ENOMEM;
-    PhaseTimer t("spref_emit", st);
-    launch_gather_offsets(G, nI, W, Bout->ptr, st);
-    launch_gather_direct(ga, W, Bout->idx, Bout->val, st);
-    return check_launch();
-  }
   if (ntup > 0x7fffffffLL) return HS_EUNSUPPORTED;
   int32_t *ti = mem.tmp<int32_t>((size_t)ntup);
   int32_t *pj = mem.tmp<int32_t>((size_t)ntup);
