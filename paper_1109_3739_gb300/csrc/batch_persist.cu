@@ -182,6 +182,8 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
   // ---- 2. distinct columns per row
   {
     int *ckeys = reinterpret_cast<int *>(smem_raw);  // CTA set
+    // the sets are bitmaps of all columns where those fit the tables' room
+    const bool cbits = n <= 32 * BPC_SYM, wbits = n <= 32 * BPW_SYM;
     auto &cex = *reinterpret_cast<CtaExpandSmem<NoVal, BP_CH> *>(smem_raw + BPC_SYM * 4);
     while (true) {
       if (tid == 0) s_item = atomicAdd(&ctr->sym_c, 1);
@@ -190,7 +192,9 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
       if (i >= nc_rows) break;
       const int r = a.clist[i];
       const int cslots = max(64, min(BPC_SYM, next_pow2(2 * a.fw[r])));  // load at most one half
-      for (int s = tid; s < cslots; s += BP_NT) ckeys[s] = EMPTY;
+      if (cbits) bitmap_clear<CtaGroup>(ckeys, (int)n);
+      else
+        for (int s = tid; s < cslots; s += BP_NT) ckeys[s] = EMPTY;
       if (tid < BP_NBUCK) s_cnt_b[tid] = 0;
       if (tid == 0) {
         s_count = 0;
@@ -221,7 +225,8 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
       const int64_t span = (int64_t)s_kmax - kmin + 1;
       int cnt = 0;
       cta_products<Struct, BP_CH>(A, B, A.p[r], A.p[r + 1], false, 0, 0, cex, s_wtmp, [&](int col, NoVal, int) {
-        if (hash_insert_key(ckeys, cslots - 1, col)) {
+        if (cbits ? HS_G(dbg, col >= 0 && col < n, 33, col) && bitmap_insert(ckeys, col)
+                  : hash_insert_key(ckeys, cslots - 1, col)) {
           ++cnt;
           const int bkt = (int)(((int64_t)(col - kmin) * BP_NBUCK) / span);
           if (HS_G(dbg, bkt >= 0 && bkt < BP_NBUCK, 82, col)) atomicAdd(&s_cnt_b[bkt], 1);
@@ -267,12 +272,26 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
           off = nw_pre[t];
         }
       const int r = wl[i - off];
-      const int slots = max(64, min(BPW_SYM, next_pow2(2 * a.fw[r])));  // load at most one half
-      for (int s = lane; s < slots; s += 32) wkeys[s] = EMPTY;
-      __syncwarp();
+      RowAhead<Struct> x;
+      x.r = r;
+      x.range(A);
+      x.entries(A);
+      x.segments(B);
       int cnt = 0;
-      warp_products<Struct>(A, B, A.p[r], A.p[r + 1],
-                            [&](int col, NoVal, int) { cnt += hash_insert_key(wkeys, slots - 1, col); });
+      if (wbits) {
+        bitmap_clear<WarpGroup>(wkeys, (int)n);
+        __syncwarp();
+        auto put = [&](int col, NoVal, int) {
+          if (HS_G(dbg, col >= 0 && col < n, 33, col)) cnt += bitmap_insert(wkeys, col);
+        };
+        warp_products_of<Struct>(A, B, x, put);
+      } else {
+        const int slots = max(64, min(BPW_SYM, next_pow2(2 * a.fw[r])));  // load at most one half
+        for (int s = lane; s < slots; s += 32) wkeys[s] = EMPTY;
+        __syncwarp();
+        auto put = [&](int col, NoVal, int) { cnt += hash_insert_key(wkeys, slots - 1, col); };
+        warp_products_of<Struct>(A, B, x, put);
+      }
       cnt = warp_sum(cnt);
       if (lane == 0) a.Cp[r + 1] = cnt;
       __syncwarp();

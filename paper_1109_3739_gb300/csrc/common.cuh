@@ -848,6 +848,18 @@ __device__ __forceinline__ int hash_insert_key(int *keys, unsigned mask, int key
   return 0;
 }
 
+// Symbolic insert into a bitmap of all columns (when they fit the table's
+// room): one atomic whose answer says whether the column was new, no probes.
+__device__ __forceinline__ int bitmap_insert(int *words, int col) {
+  const unsigned bit = 1u << (col & 31);
+  return (atomicOr(reinterpret_cast<unsigned *>(words) + (col >> 5), bit) & bit) == 0u;
+}
+// the words of a bitmap of n columns, rounded up to 16-byte pieces, cleared by a group
+template <class G> __device__ __forceinline__ void bitmap_clear(int *words, int n) {
+  int4 *w4 = reinterpret_cast<int4 *>(words);
+  for (int i = G::rank(); i < (n + 127) >> 7; i += G::size()) w4[i] = make_int4(0, 0, 0, 0);
+}
+
 // Numeric insert: fold v into the slot of key.  The table is sized from the
 // symbolic count (at least twice the row's distinct keys), so it cannot fill;
 // should it ever, the probe gives up after visiting every slot and raises

@@ -107,6 +107,37 @@ template <int K, typename KT> __device__ __forceinline__ void warp_bitonic(KT (&
   }
 }
 
+// The same network for few keys a lane, fully unrolled (no loop, and a
+// descending block compares the other way round instead of holding its keys
+// complemented): K = 2 is 21 stages in some 170 instructions.
+template <int K, typename KT> __device__ __forceinline__ void warp_bitonic_flat(KT (&key)[K]) {
+  constexpr int N = 32 * K;
+  const int lane = lane_id();
+  bitonic_in_lane<K>(key);
+#pragma unroll
+  for (int size = K; size <= N; size <<= 1) {
+    const bool desc = ((lane * K) & size) != 0;
+#pragma unroll
+    for (int stride = size >> 1; stride >= K; stride >>= 1) {
+      const bool small = ((lane & (stride / K)) == 0) != desc;
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const KT o = __shfl_xor_sync(FULL, key[i], stride / K);
+        key[i] = small ? min(key[i], o) : max(key[i], o);
+      }
+    }
+#pragma unroll
+    for (int stride = K >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        if ((i & stride) == 0) {
+          const KT lo = min(key[i], key[i | stride]), hi = max(key[i], key[i | stride]);
+          key[i] = desc ? hi : lo;
+          key[i | stride] = desc ? lo : hi;
+        }
+  }
+}
+
 // The products of the row held by x by one warp, in product order, to
 // shared memory (columns at s_col[sr_pad(p)], values at s_val[p], at most
 // nmax of them); returns their number (warp-uniform) and the least and
@@ -153,7 +184,8 @@ __device__ __forceinline__ void sort_finish(int F, int c, int kmn, int kmx, int 
       const int e = lane * K + i;
       key[i] = e < F ? (((uint32_t)(s_col[sr_pad(e)] - kmn)) << PB) | (uint32_t)e : 0xffffffffu;
     }
-    warp_bitonic<K>(key);
+    if constexpr (K <= 4) warp_bitonic_flat<K>(key);
+    else warp_bitonic<K>(key);
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < K; ++i) s_col[sr_pad(lane * K + i)] = (int)key[i];

@@ -75,29 +75,40 @@ __global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny(SymArgs a) {
 // --------------------------------------------------------------- warp
 // one warp per row, a private table of 2f slots (at most SLOTS): rows of at
 // most 512 products (1024 slots) and, in their own launch, of 513..1024
-// products (2048 slots)
+// products (2048 slots).  BITS: B's columns fit the table's room as a bitmap
+// (32 columns a slot), which replaces the hash set: one atomic a product
+// instead of hash, probe and compare-and-swap.
 constexpr int WARP_WPB = 8;
-template <int SLOTS>
+template <int SLOTS, bool BITS>
 __global__ void __launch_bounds__(WARP_WPB * 32, 4) k_sym_warp(SymArgs a) {
   extern __shared__ __align__(16) int tables[];
   const int w = threadIdx.x >> 5, lane = lane_id();
   int *keys = tables + w * SLOTS;
   const DevCsr A = dev_a(a.A), B = dev_b(a.B);
+  const int n = (int)a.B.n;
   const int step = gridDim.x * WARP_WPB;
   int idx = blockIdx.x * WARP_WPB + w;
   RowAhead<StructSR> x, nx;
   x.all(A, B, a.list, idx, a.count);
-  int fr = x.r >= 0 ? (int)a.f[x.r] : 0;
+  int fr = !BITS && x.r >= 0 ? (int)a.f[x.r] : 0;
   for (; idx < a.count; idx += step) {
     nx.row(A, a.list, idx + step, a.count);
     const int slots = max(64, min(SLOTS, next_pow2(2 * fr)));
-    for (int s = lane; s < slots; s += 32) keys[s] = EMPTY;
+    if constexpr (BITS) bitmap_clear<WarpGroup>(keys, n);
+    else
+      for (int s = lane; s < slots; s += 32) keys[s] = EMPTY;
     __syncwarp();
     int cnt = 0;
     const unsigned mask = slots - 1;
     nx.range(A);
-    fr = nx.r >= 0 ? (int)__ldg(a.f + nx.r) : 0;
-    auto put = [&](int col, NoVal, int) { cnt += hash_insert_key(keys, mask, col); };
+    if constexpr (!BITS) fr = nx.r >= 0 ? (int)__ldg(a.f + nx.r) : 0;
+    auto put = [&](int col, NoVal, int) {
+      if constexpr (BITS) {
+        if (HS_G(a.A.dbg, col >= 0 && col < n, 33, col)) cnt += bitmap_insert(keys, col);
+      } else {
+        cnt += hash_insert_key(keys, mask, col);
+      }
+    };
     if (x.r >= 0) warp_products_of<StructSR>(A, B, x, put);
     nx.entries(A);
     cnt = warp_sum(cnt);
@@ -147,28 +158,37 @@ constexpr int CH = 1024;   // A entries per expansion round (heavy)
 constexpr int CHM = 256;   // the same for the hash kernels: smaller staging, more CTAs per SM
 
 template <int SLOTS> struct SymCtaSmem {
-  int keys[SLOTS];
+  alignas(16) int keys[SLOTS];
   CtaExpandSmem<NoVal, CHM> ex;
   int wtmp[33];
   int total;
 };
 
-template <int SLOTS, int NT>
-__global__ void __launch_bounds__(NT) k_sym_cta(SymArgs a) {
+template <int SLOTS, int NT, bool BITS>  // BITS: as for k_sym_warp; 1536 threads an SM, as its shared memory allows
+__global__ void __launch_bounds__(NT, 1536 / NT) k_sym_cta(SymArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto &sm = *reinterpret_cast<SymCtaSmem<SLOTS> *>(smem_raw);
   const DevCsr A = dev_a(a.A), B = dev_b(a.B);
+  const int n = (int)a.B.n;
   for (int idx = blockIdx.x; idx < a.count; idx += gridDim.x) {
     const int r = a.list[idx];
     if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 35, r)) continue;
     const int slots = max(64, min(SLOTS, next_pow2(2 * (int)a.f[r])));
     const unsigned mask = slots - 1;
-    for (int s = threadIdx.x; s < slots; s += blockDim.x) sm.keys[s] = EMPTY;
+    if constexpr (BITS) bitmap_clear<CtaGroup>(sm.keys, n);
+    else
+      for (int s = threadIdx.x; s < slots; s += blockDim.x) sm.keys[s] = EMPTY;
     if (threadIdx.x == 0) sm.total = 0;
     __syncthreads();
     int cnt = 0;
     cta_products<StructSR, CHM>(A, B, A.p[r], A.p[r + 1], false, 0, 0, sm.ex, sm.wtmp,
-                                [&](int col, NoVal, int) { cnt += hash_insert_key(sm.keys, mask, col); });
+                                [&](int col, NoVal, int) {
+                                  if constexpr (BITS) {
+                                    if (HS_G(a.A.dbg, col >= 0 && col < n, 33, col)) cnt += bitmap_insert(sm.keys, col);
+                                  } else {
+                                    cnt += hash_insert_key(sm.keys, mask, col);
+                                  }
+                                });
     cnt = warp_sum(cnt);
     if (lane_id() == 0 && cnt) atomicAdd(&sm.total, cnt);
     __syncthreads();
@@ -456,12 +476,21 @@ void launch_sym_tiny(const SymArgs &a, cudaStream_t st) {
   count_launch();
   k_sym_tiny<<<grid_cap(a.count, TINY_WPB, 8), TINY_WPB * 32, 0, st>>>(a);
 }
+// A table of `slots` words holds a bitmap of all of B's columns up to 32 a
+// slot; on both sides of the line the kernel needs the same shared memory, so
+// the line lies where the room ends.
+static bool fits_bitmap(const SymArgs &a, int64_t slots) { return a.B.n <= 32 * slots; }
+template <int SLOTS, bool BITS> static void launch_sym_warp_as(const SymArgs &a, cudaStream_t st) {
+  const size_t bytes = sizeof(int) * WARP_WPB * SLOTS;
+  auto k = k_sym_warp<SLOTS, BITS>;
+  const int fit = fit_per_sm(k, WARP_WPB * 32, bytes);
+  count_launch();
+  k<<<grid_cap(a.count, WARP_WPB, fit), WARP_WPB * 32, bytes, st>>>(a);
+}
 template <int SLOTS> static void launch_sym_warp_slots(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
-  const size_t bytes = sizeof(int) * WARP_WPB * SLOTS;
-  count_launch();
-  k_sym_warp<SLOTS><<<grid_cap(a.count, WARP_WPB, fit_per_sm(k_sym_warp<SLOTS>, WARP_WPB * 32, bytes)),
-                      WARP_WPB * 32, bytes, st>>>(a);
+  if (fits_bitmap(a, SLOTS)) launch_sym_warp_as<SLOTS, true>(a, st);
+  else launch_sym_warp_as<SLOTS, false>(a, st);
 }
 void launch_sym_warp(const SymArgs &a, cudaStream_t st) { launch_sym_warp_slots<2 * F_WARP>(a, st); }
 void launch_sym_spa(const SymArgs &a, cudaStream_t st) {
@@ -470,11 +499,17 @@ void launch_sym_spa(const SymArgs &a, cudaStream_t st) {
   k_sym_spa<<<grid_cap(a.count, SPA_WPB, fit_per_sm(k_sym_spa, SPA_WPB * 32, 0)), SPA_WPB * 32, 0, st>>>(a);
 }
 
+template <int SLOTS, int NT, bool BITS> static void launch_sym_cta_as(const SymArgs &a, cudaStream_t st) {
+  const size_t bytes = sizeof(SymCtaSmem<SLOTS>);
+  auto k = k_sym_cta<SLOTS, NT, BITS>;
+  const int fit = fit_per_sm(k, NT, bytes);
+  count_launch();
+  k<<<grid_cap(a.count, 1, fit), NT, bytes, st>>>(a);
+}
 template <int SLOTS, int NT> static void launch_sym_cta(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
-  const size_t bytes = sizeof(SymCtaSmem<SLOTS>);
-  count_launch();
-  k_sym_cta<SLOTS, NT><<<grid_cap(a.count, 1, fit_per_sm(k_sym_cta<SLOTS, NT>, NT, bytes)), NT, bytes, st>>>(a);
+  if (fits_bitmap(a, SLOTS)) launch_sym_cta_as<SLOTS, NT, true>(a, st);
+  else launch_sym_cta_as<SLOTS, NT, false>(a, st);
 }
 // table capacity 2f: mid rows have f <= 4096, large rows f <= min(16384, cap_large) = 8192 at most
 void launch_sym_mid_s(const SymArgs &a, cudaStream_t st) { launch_sym_warp_slots<2 * F_MID_S>(a, st); }
