@@ -191,14 +191,17 @@ void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, unsigned long l
 
 // Rows per key, and (the last block) the keys' offsets.  stats[0] += total
 // flops, stats[1] = max row flops, stats[2] = max row nnz of A, stats[3] +=
-// min(f, n) over rows of the symbolic heavy bin.  Cnt (CSR only): the output
+// min(f, n) over rows of the symbolic heavy bin, stats[4] += products of the
+// tiny rows.  cnt (CSR only): the output
 // counts, all set to zero here.
 __global__ void __launch_bounds__(TL_NT) k_row_keys(RowSet A, const int64_t *f, int64_t *cnt, BinCounters c,
                                                     unsigned long long *stats, BinCfg bins, int64_t bn) {
   __shared__ int hist[NKEYS], s_last;
+  __shared__ unsigned long long s_stats[5];  // (a block's atomics on the four words; one per warp took most of the kernel)
   for (int i = threadIdx.x; i < NKEYS; i += blockDim.x) hist[i] = 0;
+  if (threadIdx.x < 5) s_stats[threadIdx.x] = 0;
   __syncthreads();
-  unsigned long long my_tot = 0, my_max = 0, my_amax = 0, my_heavy = 0;
+  unsigned long long my_tot = 0, my_max = 0, my_amax = 0, my_heavy = 0, my_tiny = 0;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < A.nslots;
        r += (int64_t)gridDim.x * blockDim.x) {
     const int64_t fr = f[r];
@@ -206,6 +209,7 @@ __global__ void __launch_bounds__(TL_NT) k_row_keys(RowSet A, const int64_t *f, 
     const int key = sym_key(fr, bins);
     if (key) atomicAdd(hist + key, 1);
     if (key >= KEY_HEAVY) my_heavy += (unsigned long long)min(fr, bn);
+    if (key == KEY_TINY) my_tiny += (unsigned long long)fr;
     my_tot += (unsigned long long)fr;
     my_max = max(my_max, (unsigned long long)fr);
     my_amax = max(my_amax, (unsigned long long)max(A.p[r + 1] - A.p[r], (int64_t)0));
@@ -213,17 +217,23 @@ __global__ void __launch_bounds__(TL_NT) k_row_keys(RowSet A, const int64_t *f, 
   if (cnt && blockIdx.x == 0 && threadIdx.x == 0) cnt[0] = 0;
   my_tot = warp_sum(my_tot);
   my_heavy = warp_sum(my_heavy);
+  my_tiny = warp_sum(my_tiny);
   my_max = warp_max(my_max);
   my_amax = warp_max(my_amax);
   if (lane_id() == 0) {
-    if (my_tot) atomicAdd(stats + 0, my_tot);
-    atomicMax(stats + 1, my_max);
-    atomicMax(stats + 2, my_amax);
-    if (my_heavy) atomicAdd(stats + 3, my_heavy);
+    if (my_tot) atomicAdd(s_stats + 0, my_tot);
+    atomicMax(s_stats + 1, my_max);
+    atomicMax(s_stats + 2, my_amax);
+    if (my_heavy) atomicAdd(s_stats + 3, my_heavy);
+    if (my_tiny) atomicAdd(s_stats + 4, my_tiny);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NKEYS; i += blockDim.x)
     if (hist[i]) atomicAdd(c.cnt + i, hist[i]);
+  if (threadIdx.x < 5 && s_stats[threadIdx.x]) {
+    if (threadIdx.x == 1 || threadIdx.x == 2) atomicMax(stats + threadIdx.x, s_stats[threadIdx.x]);
+    else atomicAdd(stats + threadIdx.x, s_stats[threadIdx.x]);
+  }
   if (last_block(c.ticket, &s_last) && threadIdx.x < 32) key_offsets(c.cnt, c.off, c.cur);
 }
 void launch_row_keys(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCounters &c, unsigned long long *stats,
@@ -465,7 +475,7 @@ __global__ void __launch_bounds__(TL_NT) k_num_count(RowSet A, const int64_t *f,
     const int64_t n = r < A.m ? cnt[r + 1] : 0;
     sum += n;
     if (r < A.nslots) {
-      const int key = num_key(f[r], A.ids ? raw_count(A, cnt, r) : n, bins);
+      const int key = hub_key(num_key(f[r], A.ids ? raw_count(A, cnt, r) : n, bins), A.p[r + 1] - A.p[r]);
       if (key) atomicAdd(hist + key, 1);
     }
   }
@@ -516,7 +526,7 @@ __global__ void __launch_bounds__(TL_NT) k_num_offsets(RowSet A, const int64_t *
     v[u] = r < A.m ? cnt[r + 1] : 0;
     key[u] = 0;
     if constexpr (LISTS)
-      if (r < A.nslots) key[u] = num_key(f[r], v[u], bins);
+      if (r < A.nslots) key[u] = hub_key(num_key(f[r], v[u], bins), A.p[r + 1] - A.p[r]);
   }
   tile_scan(v, s_tot);
   const int64_t base = tsum[blockIdx.x];
@@ -537,7 +547,7 @@ __global__ void __launch_bounds__(TL_NT) k_num_lists(RowSet A, const int64_t *f,
 #pragma unroll
   for (int u = 0; u < TL_PER; ++u) {
     const int64_t r = r0 + u * TL_NT + threadIdx.x;
-    key[u] = r < A.nslots ? num_key(f[r], raw_count(A, cnt, r), bins) : 0;
+    key[u] = r < A.nslots ? hub_key(num_key(f[r], raw_count(A, cnt, r), bins), A.p[r + 1] - A.p[r]) : 0;
   }
   append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
 }

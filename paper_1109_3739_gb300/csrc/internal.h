@@ -116,6 +116,22 @@ __host__ __device__ inline int num_key(int64_t f, int64_t c, const BinCfg &b) {
   k = f <= F_TINY ? KEY_TINY : k;
   return c <= 0 ? 0 : k;
 }
+// Tiny rows (at most 32 products) are taken several to a warp when they are
+// many and small: below 8 products on average a warp holds four rows or more;
+// a list that gives every warp of the GPU but a few rows is a matter of
+// latency, which the kernel for single rows hides better.
+inline bool tiny_group_pays(int64_t rows, unsigned long long products) {
+  return rows >= 65536 && products <= 8ull * (unsigned long long)rows;
+}
+// A row whose key is a warp's or a small block's, but which has more than
+// HUB_ENTRIES entries of A, goes to the kernel of 1024 threads: its time is
+// not its products' but the rounds of entries that are looked up (3.5e4
+// entries with one product each: 0.52 ms as the last row of the kernel of 256
+// threads, 137 rounds of 3.8 us, whatever else ran beside it).
+constexpr int64_t HUB_ENTRIES = 4096;
+__host__ __device__ inline int hub_key(int key, int64_t entries) {
+  return entries > HUB_ENTRIES && key > KEY_TINY && key < KEY_SPA ? KEY_LARGE : key;
+}
 // the default thresholds for a value width, clamped tuning values otherwise
 BinCfg bin_config(int value_bytes);
 // the thresholds of a product whose B has ncols columns (value_bytes: C's
@@ -178,7 +194,8 @@ struct BinCounters {
 // products per row (f zeroed before) and the A entries with an empty B row;
 // then the rows' symbolic keys, their offsets, and stats[0] total flops, [1]
 // max row flops, [2] max row nnz of A, [3] sum of min(f, n) over the rows of
-// the symbolic heavy bin (their list pool bound).  cnt: C's counts, set to
+// the symbolic heavy bin (their list pool bound), [4] products of the tiny
+// rows.  cnt: C's counts, set to
 // zero on the way (CSR), or null
 void launch_flops(const RowSet &A, const RightOp &B, int64_t *f, unsigned long long *zeros, cudaStream_t st);
 void launch_row_keys(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCounters &c, unsigned long long *stats,
@@ -227,6 +244,7 @@ struct SymArgs {
   int64_t *loff;           // per row slot: start of its list in the pool (-1 none)
   unsigned long long *lpool;  // pool cursor (entries handed out)
   int64_t lcap;
+  int tiny_group;          // tiny rows several to a warp
 };
 void launch_sym_tiny(const SymArgs &a, cudaStream_t st);
 void launch_sym_warp(const SymArgs &a, cudaStream_t st);
@@ -320,6 +338,7 @@ struct NumArgs {
   int pair_long;          // some row of A holds more than PAIR_LONG entries
   int pair_abytes;        // width of the left values the pairs carry (0: none)
   int unit_kb;            // the units' value capacity in KB (16 or 32): which unit kernel runs
+  int tiny_group;         // tiny rows several to a warp
 };
 // kind: 0 tiny, 1 warp_s, 2 warp, 3 mid_s, 4 mid, 5 large_s, 6 large,
 // 7 sort_xs, 8 sort_s, 9 sort_m, 10 sort, 11 spa, 12 heavy (bin key

@@ -83,7 +83,7 @@ struct NaBlock {  // device counters, read back to host memory
   int ticket[2];
   int pad;
   unsigned long long zeros;
-  unsigned long long stats[4];
+  unsigned long long stats[5];
   long long nnz;
   long long dbg[2];
 };
@@ -201,6 +201,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   int key_off[NKEYS + 1];
   memcpy(key_off, hb.key_off, sizeof(key_off));
   const int nhist = hb.nhist;
+  const int tiny_group = tiny_group_pays(key_off[KEY_TINY + 1] - key_off[KEY_TINY], hb.stats[4]);
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
   uint32_t *hist = nullptr;
   if (nhist > 0) {
@@ -209,7 +210,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
     NA_CK(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)nhist * nseg, st));
   }
 
-  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, nullptr, nullptr, nullptr, 0};
+  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, nullptr, nullptr, nullptr, 0, tiny_group};
   auto sym_bin = [&](int k0, int k1) {
     sa.list = list + key_off[k0];
     sa.count = key_off[k1] - key_off[k0];
@@ -250,6 +251,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   }
   NumArgs na{rs,   rb,   f,    nullptr,     0,        Cp,   C->idx, C->val,  hslot,
              hist, nseg, &sb->dyn[1], &sb->err, gcur, gend, nullptr, nullptr, nullptr, nullptr};
+  na.tiny_group = tiny_group;
   for (int kind = 0; kind < NUM_KINDS; ++kind) {
     const int k0 = KEY_TINY + kind, k1 = kind == NUM_KINDS - 1 ? NKEYS : k0 + 1;
     na.list = list + key_off[k0];

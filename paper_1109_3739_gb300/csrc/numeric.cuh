@@ -2,8 +2,9 @@
 //
 // Each bin runs the row-wise form of Algorithm 1 (C(i,:) += A(i,k)*B(k,:))
 // into the accumulator that fits its rows:
-//   tiny  (f <= 32)        one warp; products sit one per lane; lanes with
-//                          equal columns (__match_any_sync) are folded by the
+//   tiny  (f <= 32)        several rows to a warp; products sit one per lane;
+//                          lanes with equal columns of one row
+//                          (__match_any_sync) are folded by the
 //                          lowest lane in product order, and each distinct
 //                          column's rank among the row's columns is its output
 //                          position;
@@ -97,6 +98,85 @@ __global__ void __launch_bounds__(NTINY_WPB * 32, 4) k_num_tiny(NumArgs a) {
   }
 }
 
+// the same rows, several to a warp at a time (tiny_group): for long lists of
+// rows of few products (tiny_group_pays)
+template <class SR>
+__global__ void __launch_bounds__(NTINY_WPB * 32, 4) k_num_tiny_group(NumArgs a) {
+  using T = typename SR::val_t;
+  __shared__ int scol[NTINY_WPB][32];
+  __shared__ T sval[NTINY_WPB][32];
+  const int w = threadIdx.x >> 5, lane = lane_id();
+  const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
+  T *Cv = reinterpret_cast<T *>(a.Cv);
+  const int per = (a.count + gridDim.x * NTINY_WPB - 1) / (gridDim.x * NTINY_WPB);
+  const int64_t first = (int64_t)(blockIdx.x * NTINY_WPB + w) * per;
+  const int end = (int)min(first + per, (int64_t)a.count);
+  int idx = (int)min(first, (int64_t)a.count);
+  TinyWindow win;
+  win.ids(A, a.list, idx, end, 0);
+  win.ranges(A, a.f, 0);
+  while (idx < end) {
+    TinyGroup<SR> g = tiny_group<SR>(A, B, a.list, idx, end, a.f, win);
+    if (g.rows == 0) {  // more than 32 entries of A for at most 32 products
+      RowAhead<SR> x;
+      x.all(A, B, a.list, idx, end);
+      auto put = [&](int col, T v, int p) {
+        if (HS_G(a.A.dbg, p < 32, 40, p)) {
+          scol[w][p] = col;
+          if constexpr (SR::has_val) sval[w][p] = v;
+        }
+      };
+      const int nprod = x.r >= 0 ? warp_products_of<SR>(A, B, x, put) : 0;
+      __syncwarp();
+      g.rows = 1;
+      const int from = win.slide(1);
+      win.ids(A, a.list, idx + 1, end, from);
+      win.ranges(A, a.f, from);
+      g.nprod = min(nprod, 32);
+      g.r = lane == 0 ? x.r : -1;
+      g.mask = lane == 0 && g.nprod ? 0xffffffffu >> (32 - g.nprod) : 0u;
+      g.row = 0;
+      g.col = lane < g.nprod ? scol[w][lane] : 0;
+      if constexpr (SR::has_val) g.v = lane < g.nprod ? sval[w][lane] : T{};
+      __syncwarp();
+    }
+    const bool have = lane < g.nprod;
+    int64_t base = 0, cend = 0;  // lane l < rows: its row's place in C
+    if (lane < g.rows && g.r >= 0) {
+      const int64_t o = nout_row(a.A, g.r);
+      base = a.Cp[o];
+      cend = a.Cp[o + 1];
+    }
+    scol[w][lane] = g.col;
+    if constexpr (SR::has_val) sval[w][lane] = g.v;
+    __syncwarp();
+    // a lane without a product matches nobody's (row, column)
+    const unsigned long long key = have ? ((unsigned long long)(unsigned)g.row << 32) | (unsigned)g.col
+                                        : ~0ull - (unsigned)lane;
+    const unsigned grp = __match_any_sync(FULL, key);
+    const bool lead = have && lane == __ffs(grp) - 1;
+    const unsigned leaders = __ballot_sync(FULL, lead);
+    if (lane < g.rows && g.r >= 0 && (int64_t)__popc(leaders & g.mask) != cend - base) atomicExch(a.err, 3);
+    const unsigned mine = __shfl_sync(FULL, g.mask, g.row) & leaders;
+    const int64_t rb = __shfl_sync(FULL, base, g.row), re = __shfl_sync(FULL, cend, g.row);
+    if (lead) {
+      T acc{};
+      if constexpr (SR::has_val) {  // the column's products in product order
+        acc = g.v;
+        for (unsigned m = grp & (grp - 1); m; m &= m - 1) acc = SR::add(acc, sval[w][__ffs(m) - 1]);
+      }
+      int rank = 0;
+      for (unsigned m = mine; m; m &= m - 1) rank += scol[w][__ffs(m) - 1] < g.col;
+      if (HS_G(a.A.dbg, rb + rank < re, 41, rb + rank)) {
+        a.Cj[rb + rank] = g.col;
+        if constexpr (SR::has_val) Cv[rb + rank] = acc;
+      }
+    }
+    __syncwarp();
+    idx += g.rows;
+  }
+}
+
 // --------------------------------------------------------------- warp
 constexpr int NWARP_WPB = 4;
 
@@ -156,18 +236,20 @@ __global__ void __launch_bounds__(NWARP_WPB * 32, 4) k_num_warp(NumArgs a) {
 }
 
 // ---------------------------------------------------- mid / large / heavy
-// A entries per expansion round: the mid kernel stages fewer so that more of
-// its CTAs fit an SM (rows in flight hide each other's latency)
-template <int CAP> constexpr int nch() { return CAP >= 8192 ? 1024 : 256; }
+// A entries per expansion round: the smaller kernels stage fewer so that more
+// of their CTAs fit an SM (rows in flight hide each other's latency); the
+// kernel of 1024 threads, which also takes the rows with very many entries, an
+// entry per thread
+constexpr int nch(int nt) { return nt >= 1024 ? 1024 : 256; }
 
-template <typename T, int SLOTS, int CAP> struct CtaNumLayout {
+template <typename T, int SLOTS, int CAP, int NT> struct CtaNumLayout {
   static constexpr size_t table_bytes = (size_t)SLOTS * (4 + vbytes<T>());
   static constexpr size_t work_bytes =
       ((((size_t)(CAP + 2 * CAP) * 4 + 7) & ~(size_t)7)) + (size_t)CAP * vbytes<T>();
   static constexpr size_t region0 = ((table_bytes > work_bytes ? table_bytes : work_bytes) + 15) & ~(size_t)15;
   static constexpr size_t compact = (((size_t)CAP * (4 + vbytes<T>())) + 15) & ~(size_t)15;
   static constexpr size_t ex_off = region0 + compact;
-  static constexpr size_t tail_off = ex_off + ((sizeof(CtaExpandSmem<T, nch<CAP>()>) + 15) & ~(size_t)15);
+  static constexpr size_t tail_off = ex_off + ((sizeof(CtaExpandSmem<T, nch(NT)>) + 15) & ~(size_t)15);
   struct Tail {
     EmitScratch es;
     int wtmp[33];
@@ -181,13 +263,13 @@ template <typename T, int SLOTS, int CAP> struct CtaNumLayout {
 template <class SR, int SLOTS, int CAP, int NT>
 __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
   using T = typename SR::val_t;
-  using L = CtaNumLayout<T, SLOTS, CAP>;
+  using L = CtaNumLayout<T, SLOTS, CAP, NT>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int *keys = reinterpret_cast<int *>(smem_raw);
   T *vals = reinterpret_cast<T *>(smem_raw + (size_t)SLOTS * 4);
   int *ck = reinterpret_cast<int *>(smem_raw + L::region0);
   T *cv = reinterpret_cast<T *>(smem_raw + L::region0 + (size_t)CAP * 4);
-  auto &ex = *reinterpret_cast<CtaExpandSmem<T, nch<CAP>()> *>(smem_raw + L::ex_off);
+  auto &ex = *reinterpret_cast<CtaExpandSmem<T, nch(NT)> *>(smem_raw + L::ex_off);
   auto &tl = *reinterpret_cast<typename L::Tail *>(smem_raw + L::tail_off);
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
   T *Cv = reinterpret_cast<T *>(a.Cv);
@@ -204,7 +286,7 @@ __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
       if constexpr (SR::has_val) vals[s] = SR::identity();
     }
     __syncthreads();
-    cta_products<SR, nch<CAP>()>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
+    cta_products<SR, nch(NT)>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
                           [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
     const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
     if (lofs >= 0) {
@@ -1002,7 +1084,7 @@ template <class SR, int SLOTS, int CAP> void launch_num_warp(const NumArgs &a, c
 
 template <class SR, int SLOTS, int CAP, int NT> void launch_num_cta(const NumArgs &a, cudaStream_t st) {
   using T = typename SR::val_t;
-  using L = CtaNumLayout<T, SLOTS, CAP>;
+  using L = CtaNumLayout<T, SLOTS, CAP, NT>;
   auto k = k_num_cta<SR, SLOTS, CAP, NT>;
   count_launch();
   k<<<ngrid_cap(a.count, 1, fit_per_sm(k, NT, L::bytes)), NT, L::bytes, st>>>(a);
@@ -1022,10 +1104,13 @@ template <class SR> void launch_numeric_sr(int kind, const NumArgs &a, cudaStrea
   if (a.count <= 0) return;
   constexpr int CAPL = cap_large<T>();
   switch (kind) {
-    case 0:
+    case 0: {
+      auto k = a.tiny_group ? k_num_tiny_group<SR> : k_num_tiny<SR>;
+      const int fit = fit_per_sm(k, NTINY_WPB * 32, 0);
       count_launch();
-      k_num_tiny<SR><<<ngrid_cap(a.count, NTINY_WPB, 8), NTINY_WPB * 32, 0, st>>>(a);
+      k<<<ngrid_cap(a.count, NTINY_WPB, fit), NTINY_WPB * 32, 0, st>>>(a);
       break;
+    }
     case 1: launch_num_warp<SR, 2 * F_WARP_S, F_WARP_S>(a, st); break;
     case 2: launch_num_warp<SR, 2 * F_WARP, F_WARP>(a, st); break;
     case 3: launch_num_cta<SR, 2 * CAP_MID_S, CAP_MID_S, 256>(a, st); break;

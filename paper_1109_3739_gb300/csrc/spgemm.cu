@@ -263,7 +263,7 @@ struct SmallBlock {  // device counters, read back in one copy
   int valflag;
   int ticket[2];
   int pad;
-  unsigned long long stats[4];
+  unsigned long long stats[5];
   unsigned long long lpool;  // heavy rows' column lists: pool entries handed out
   int bci_cnt;               // B segment index rows handed out
   int pad2;
@@ -487,6 +487,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   int key_off[NKEYS + 1];
   memcpy(key_off, hb->key_off, sizeof(key_off));
   const int nhist = hb->nhist;
+  const int tiny_group = tiny_group_pays(key_off[KEY_TINY + 1] - key_off[KEY_TINY], hb->stats[4]);
   const int pair_long = hb->stats[2] > (unsigned long long)PAIR_LONG;  // (read before hb is copied to again)
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
 
@@ -591,7 +592,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   };
 
   // ---- symbolic
-  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, glist, loff, &sb->lpool, lcap};
+  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, glist, loff, &sb->lpool, lcap, tiny_group};
   auto sym_bin = [&](int k0, int k1) {
     sa.list = list + key_off[k0];
     sa.count = key_off[k1] - key_off[k0];
@@ -734,6 +735,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   na.pair_abytes = a_bytes;
   na.pair_long = pair_long;
   na.unit_kb = bins.unit_kb;
+  na.tiny_group = tiny_group;
   const char *names[NUM_KINDS] = {"numeric_tiny",   "numeric_warp_s", "numeric_warp",   "numeric_mid_s",
                                   "numeric_mid",    "numeric_large_s", "numeric_large", "numeric_sort_xs",
                                   "numeric_sort_s", "numeric_sort_m",  "numeric_sort",  "numeric_spa",

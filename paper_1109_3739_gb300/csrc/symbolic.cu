@@ -3,8 +3,8 @@
 // The row-wise form of Algorithm 1 with the sparse accumulator of Figure 1
 // reduced to its occupancy part: each row's distinct output columns are
 // counted by the accumulator its bin selects.
-//   tiny  (f <= 32)    one warp, one product per lane, equal columns found
-//                      with __match_any_sync;
+//   tiny  (f <= 32)    several rows to a warp, one product per lane, equal
+//                      columns of a row found with __match_any_sync;
 //   warp  (f <= 512)   one warp, private shared-memory hash set;
 //   mid   (f <= 1024, and f <= 4096)
 //                      one CTA, shared hash set of 2f slots (at most 2048,
@@ -69,6 +69,52 @@ __global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny(SymArgs a) {
     }
     __syncwarp();
     x = nx;
+  }
+}
+
+// the same rows, several to a warp at a time (tiny_group): for long lists of
+// rows of few products (tiny_group_pays)
+__global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny_group(SymArgs a) {
+  __shared__ int scol[TINY_WPB][32];
+  const int w = threadIdx.x >> 5, lane = lane_id();
+  const DevCsr A = dev_a(a.A), B = dev_b(a.B);
+  const int per = (a.count + gridDim.x * TINY_WPB - 1) / (gridDim.x * TINY_WPB);
+  const int64_t first = (int64_t)(blockIdx.x * TINY_WPB + w) * per;
+  const int end = (int)min(first + per, (int64_t)a.count);
+  int idx = (int)min(first, (int64_t)a.count);
+  TinyWindow win;
+  win.ids(A, a.list, idx, end, 0);
+  win.ranges(A, a.f, 0);
+  while (idx < end) {
+    TinyGroup<StructSR> g = tiny_group<StructSR>(A, B, a.list, idx, end, a.f, win);
+    if (g.rows == 0) {  // more than 32 entries of A for at most 32 products
+      RowAhead<StructSR> x;
+      x.all(A, B, a.list, idx, end);
+      auto put = [&](int col, NoVal, int p) {
+        if (HS_G(a.A.dbg, p < 32, 34, p)) scol[w][p] = col;
+      };
+      const int nprod = x.r >= 0 ? warp_products_of<StructSR>(A, B, x, put) : 0;
+      __syncwarp();
+      g.rows = 1;
+      const int from = win.slide(1);
+      win.ids(A, a.list, idx + 1, end, from);
+      win.ranges(A, a.f, from);
+      g.nprod = min(nprod, 32);
+      g.r = lane == 0 ? x.r : -1;
+      g.mask = lane == 0 && g.nprod ? 0xffffffffu >> (32 - g.nprod) : 0u;
+      g.row = 0;
+      g.col = lane < g.nprod ? scol[w][lane] : 0;
+      if (lane == 0 && nprod > 32) atomicExch(a.err, 2);
+      __syncwarp();
+    }
+    const bool have = lane < g.nprod;
+    // a lane without a product matches nobody's (row, column)
+    const unsigned long long key = have ? ((unsigned long long)(unsigned)g.row << 32) | (unsigned)g.col
+                                        : ~0ull - (unsigned)lane;
+    const unsigned grp = __match_any_sync(FULL, key);
+    const unsigned lead = __ballot_sync(FULL, have && lane == __ffs(grp) - 1);
+    if (lane < g.rows && g.r >= 0) put_count(a, out_row(a.A, g.r), __popc(lead & g.mask));
+    idx += g.rows;
   }
 }
 
@@ -473,8 +519,10 @@ static int grid_cap(int items, int per_block, int per_sm) {
 
 void launch_sym_tiny(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
+  auto k = a.tiny_group ? k_sym_tiny_group : k_sym_tiny;
+  const int fit = fit_per_sm(k, TINY_WPB * 32, 0);
   count_launch();
-  k_sym_tiny<<<grid_cap(a.count, TINY_WPB, 8), TINY_WPB * 32, 0, st>>>(a);
+  k<<<grid_cap(a.count, TINY_WPB, fit), TINY_WPB * 32, 0, st>>>(a);
 }
 // A table of `slots` words holds a bitmap of all of B's columns up to 32 a
 // slot; on both sides of the line the kernel needs the same shared memory, so
@@ -492,7 +540,11 @@ template <int SLOTS> static void launch_sym_warp_slots(const SymArgs &a, cudaStr
   if (fits_bitmap(a, SLOTS)) launch_sym_warp_as<SLOTS, true>(a, st);
   else launch_sym_warp_as<SLOTS, false>(a, st);
 }
-void launch_sym_warp(const SymArgs &a, cudaStream_t st) { launch_sym_warp_slots<2 * F_WARP>(a, st); }
+// (up to 2^16 columns the short rows take the larger table for its bitmap)
+void launch_sym_warp(const SymArgs &a, cudaStream_t st) {
+  if (!fits_bitmap(a, 2 * F_WARP) && fits_bitmap(a, 2 * F_MID_S)) launch_sym_warp_slots<2 * F_MID_S>(a, st);
+  else launch_sym_warp_slots<2 * F_WARP>(a, st);
+}
 void launch_sym_spa(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
   count_launch();

@@ -72,11 +72,14 @@ def test_tiny_rows_together(sr, dt, seed):
     rows, empty = [], np.nonzero(blen == 0)[0]
     for i in range(m):
         w = I.draws(seed, 41, 64 * i, 64)
-        pick = np.unique((w[: 1 + int(w[60] % 14)] % np.uint64(k)).astype(np.int64))
+        pick = np.unique((w[: 1 + int(w[60] % (20 if i % 17 == 0 else 5))] % np.uint64(k)).astype(np.int64))
         pick = pick[np.cumsum(blen[pick]) <= 32]
         if i % 97 == 0:
             pick = np.unique(np.concatenate([pick, empty]))  # more than 32 entries, most of them idle
         rows.append(pick if i % 11 else pick[:0])
-    rowptr = np.concatenate([[0], np.cumsum([len(r) for r in rows])])
-    A = csr(m, k, rowptr, np.concatenate(rows), I.random_values(int(rowptr[-1]), dt, seed + 9, kind="signed"), dt)
-    product(A, B, f"tiny {sr}", sr)
+    assert np.mean([blen[r].sum() for r in rows if blen[r].sum()]) < 8
+    for copies in (1, 40):  # a short list of such rows (one to a warp) and a long one (several to a warp)
+        long = rows * copies
+        rowptr = np.concatenate([[0], np.cumsum([len(r) for r in long])])
+        vals = I.random_values(int(rowptr[-1]), dt, seed + 9, kind="signed")
+        product(csr(m * copies, k, rowptr, np.concatenate(long), vals, dt), B, f"tiny {sr} x{copies}", sr)
