@@ -37,14 +37,16 @@ constexpr int EMPTY = -1;
 // ----------------------------------------------------------------- semirings
 enum SrKind { PLUS_TIMES = 0, OR_AND = 1, MIN_PLUS = 2, SELECT2ND = 3, SELECT1ST = 4 };
 
+// Minimum of floats by one integer atomic: floats without their sign bit order
+// like integers, those with it the other way round among unsigned numbers, and
+// any of them lies below any float without one (a compare-and-swap loop took
+// two shared accesses and a branch per attempt).  A NaN is never the smaller
+// value and changes nothing; -0 lies below +0.
 __device__ __forceinline__ void atomic_min_f32(float *p, float v) {
-  unsigned *ip = reinterpret_cast<unsigned *>(p);
-  unsigned old = *reinterpret_cast<volatile unsigned *>(ip);
-  while (__uint_as_float(old) > v) {
-    unsigned prev = atomicCAS(ip, old, __float_as_uint(v));
-    if (prev == old) break;
-    old = prev;
-  }
+  const int b = __float_as_int(v);
+  if (v != v) return;
+  if (b >= 0) atomicMin(reinterpret_cast<int *>(p), b);
+  else atomicMax(reinterpret_cast<unsigned *>(p), (unsigned)b);
 }
 
 // A semiring over value type T.  mul() is applied to one stored pair,
@@ -926,7 +928,8 @@ __device__ __forceinline__ int64_t gallop_lower_bound(const int32_t *j, int64_t 
 // round are cut into one contiguous range per warp, and each warp deals its
 // range one product per lane (warp_expand).  Per-row product counts must stay
 // below 2^31.  All threads of the CTA must call this together.
-template <class SR, int CH, int U = 2, class Visit>
+// SU: entries a thread looks up at a time (column, then B's offsets).
+template <class SR, int CH, int U = 2, int SU = 1, class Visit>
 __device__ __forceinline__ void cta_products(const DevCsr &A, const DevCsr &B, int64_t q0, int64_t q1, bool restrict_cols,
                              int lo, int hi, CtaExpandSmem<typename SR::val_t, CH> &sm, int *wtmp,
                              Visit &&visit) {
@@ -934,12 +937,37 @@ __device__ __forceinline__ void cta_products(const DevCsr &A, const DevCsr &B, i
   const int tid = threadIdx.x;
   for (int64_t c0 = q0; c0 < q1; c0 += CH) {
     const int n = (int)min((int64_t)CH, q1 - c0);
-    for (int e = tid; e < n; e += blockDim.x) {
-      int64_t s = 0, en = 0;
-      entry_segment(A, B, c0 + e, restrict_cols, lo, hi, s, en);
-      if constexpr (SR::needs_a) sm.aval[e] = load_val<T>(A.v, c0 + e);
-      sm.excl[e] = (int)(en - s);
-      sm.sbeg[e] = s;
+    for (int e0 = tid; e0 < n; e0 += SU * blockDim.x) {
+      int k[SU];
+      int64_t s[SU], en[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * blockDim.x;
+        k[u] = -1;
+        if (e < n && HS_G(A.dbg, c0 + e >= 0 && c0 + e < A.nnz, 1, c0 + e)) k[u] = __ldg(A.j + c0 + e);
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * blockDim.x;
+        s[u] = en[u] = 0;
+        if (e < n && HS_G(A.dbg, k[u] >= 0 && k[u] < B.rows, 2, k[u])) {
+          s[u] = __ldg(B.p + k[u]);
+          en[u] = __ldg(B.p + k[u] + 1);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * blockDim.x;
+        if (e >= n) break;
+        if (!HS_G(A.dbg, s[u] >= 0 && s[u] <= en[u] && en[u] <= B.nnz, 3, en[u])) s[u] = en[u] = 0;
+        if (restrict_cols && s[u] < en[u]) {
+          s[u] = lower_bound_col(B.j, s[u], en[u], lo);
+          en[u] = lower_bound_col(B.j, s[u], en[u], hi);
+        }
+        if constexpr (SR::needs_a) sm.aval[e] = load_val<T>(A.v, c0 + e);
+        sm.excl[e] = (int)(en[u] - s[u]);
+        sm.sbeg[e] = s[u];
+      }
     }
     if (tid == 0) sm.excl[n] = 0;  // scanned with the entries, it becomes the round's total
     __syncthreads();

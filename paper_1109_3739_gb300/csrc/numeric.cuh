@@ -236,20 +236,24 @@ __global__ void __launch_bounds__(NWARP_WPB * 32, 4) k_num_warp(NumArgs a) {
 }
 
 // ---------------------------------------------------- mid / large / heavy
-// A entries per expansion round: the smaller kernels stage fewer so that more
-// of their CTAs fit an SM (rows in flight hide each other's latency); the
-// kernel of 1024 threads, which also takes the rows with very many entries, an
-// entry per thread
-constexpr int nch(int nt) { return nt >= 1024 ? 1024 : 256; }
+// A entries per expansion round and per thread.  A round costs the latency of
+// its look-ups and barriers (3.8 us for 256 entries with a product each), so
+// rows of many short segments want long rounds: the smallest kernel's staging
+// of 1024 entries leaves room for the three CTAs an SM that its registers
+// allow (rows of 35,000 entries and 1000 outputs 204 -> 115 us), and the
+// kernel of 1024 threads, which takes the longest rows, has an entry per
+// thread.  In the others it would cost a CTA (R-MAT scale 20, rows of up to
+// 2048 outputs: 3.15 against 2.56 ms).
+constexpr int num_ch(int cap, int nt) { return cap <= CAP_MID_S || nt >= 1024 ? 1024 : 256; }
 
-template <typename T, int SLOTS, int CAP, int NT> struct CtaNumLayout {
+template <typename T, int SLOTS, int CAP, int CH> struct CtaNumLayout {
   static constexpr size_t table_bytes = (size_t)SLOTS * (4 + vbytes<T>());
   static constexpr size_t work_bytes =
       ((((size_t)(CAP + 2 * CAP) * 4 + 7) & ~(size_t)7)) + (size_t)CAP * vbytes<T>();
   static constexpr size_t region0 = ((table_bytes > work_bytes ? table_bytes : work_bytes) + 15) & ~(size_t)15;
   static constexpr size_t compact = (((size_t)CAP * (4 + vbytes<T>())) + 15) & ~(size_t)15;
   static constexpr size_t ex_off = region0 + compact;
-  static constexpr size_t tail_off = ex_off + ((sizeof(CtaExpandSmem<T, nch(NT)>) + 15) & ~(size_t)15);
+  static constexpr size_t tail_off = ex_off + ((sizeof(CtaExpandSmem<T, CH>) + 15) & ~(size_t)15);
   struct Tail {
     EmitScratch es;
     int wtmp[33];
@@ -263,13 +267,13 @@ template <typename T, int SLOTS, int CAP, int NT> struct CtaNumLayout {
 template <class SR, int SLOTS, int CAP, int NT>
 __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
   using T = typename SR::val_t;
-  using L = CtaNumLayout<T, SLOTS, CAP, NT>;
+  using L = CtaNumLayout<T, SLOTS, CAP, num_ch(CAP, NT)>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int *keys = reinterpret_cast<int *>(smem_raw);
   T *vals = reinterpret_cast<T *>(smem_raw + (size_t)SLOTS * 4);
   int *ck = reinterpret_cast<int *>(smem_raw + L::region0);
   T *cv = reinterpret_cast<T *>(smem_raw + L::region0 + (size_t)CAP * 4);
-  auto &ex = *reinterpret_cast<CtaExpandSmem<T, nch(NT)> *>(smem_raw + L::ex_off);
+  auto &ex = *reinterpret_cast<CtaExpandSmem<T, num_ch(CAP, NT)> *>(smem_raw + L::ex_off);
   auto &tl = *reinterpret_cast<typename L::Tail *>(smem_raw + L::tail_off);
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
   T *Cv = reinterpret_cast<T *>(a.Cv);
@@ -286,7 +290,7 @@ __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
       if constexpr (SR::has_val) vals[s] = SR::identity();
     }
     __syncthreads();
-    cta_products<SR, nch(NT)>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
+    cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
                           [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
     const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
     if (lofs >= 0) {
@@ -1084,7 +1088,7 @@ template <class SR, int SLOTS, int CAP> void launch_num_warp(const NumArgs &a, c
 
 template <class SR, int SLOTS, int CAP, int NT> void launch_num_cta(const NumArgs &a, cudaStream_t st) {
   using T = typename SR::val_t;
-  using L = CtaNumLayout<T, SLOTS, CAP, NT>;
+  using L = CtaNumLayout<T, SLOTS, CAP, num_ch(CAP, NT)>;
   auto k = k_num_cta<SR, SLOTS, CAP, NT>;
   count_launch();
   k<<<ngrid_cap(a.count, 1, fit_per_sm(k, NT, L::bytes)), NT, L::bytes, st>>>(a);
