@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -214,6 +215,100 @@ static void *pinned(size_t bytes) {
   return bytes <= 8192 ? t_pin.p : nullptr;
 }
 
+// Streams beside the caller's, for bins that run at the same time: a few per
+// host thread and device, made on first use and destroyed with the thread.
+// They never outlive a call's work: every call that used one lets the caller's
+// stream wait for it before it returns.
+constexpr int FAN_SIDES = 3, FAN_DEVICES = 64;
+struct SideStreams {
+  struct Dev {
+    cudaStream_t s[FAN_SIDES];
+    cudaEvent_t fork, join[FAN_SIDES];
+    bool ok;
+  };
+  Dev *dev[FAN_DEVICES] = {nullptr};
+  ~SideStreams() {
+    for (Dev *d : dev) {
+      if (!d) continue;
+      for (int i = 0; i < FAN_SIDES; ++i) {
+        if (d->s[i]) cudaStreamDestroy(d->s[i]);
+        if (d->join[i]) cudaEventDestroy(d->join[i]);
+      }
+      if (d->fork) cudaEventDestroy(d->fork);
+      delete d;
+    }
+  }
+  Dev *get() {
+    int id = 0;
+    if (cudaGetDevice(&id) != cudaSuccess || id < 0 || id >= FAN_DEVICES) return nullptr;
+    if (!dev[id]) {
+      Dev *d = new (std::nothrow) Dev();
+      if (!d) return nullptr;
+      d->ok = cudaEventCreateWithFlags(&d->fork, cudaEventDisableTiming) == cudaSuccess;
+      for (int i = 0; i < FAN_SIDES; ++i)
+        d->ok = d->ok && cudaStreamCreateWithFlags(&d->s[i], cudaStreamNonBlocking) == cudaSuccess &&
+                cudaEventCreateWithFlags(&d->join[i], cudaEventDisableTiming) == cudaSuccess;
+      cudaGetLastError();
+      dev[id] = d;
+    }
+    return dev[id]->ok ? dev[id] : nullptr;
+  }
+};
+static thread_local SideStreams t_sides;
+
+// The bins of a pass over four streams: the caller's (group 0) and three
+// beside it.  Bins of one pass work on different rows, and the larger ones end
+// in tails of a few blocks (a row of very many entries or products), which the
+// others fill (a contraction's two products 2.44 -> 1.76 ms, a narrow frontier
+// product 1.43 -> 0.93 ms, a batch of random products 6.44 -> 6.15 ms).  All of
+// a pass's work starts after what the caller's stream holds and the caller's
+// stream goes on after all of it, so nothing else changes (stream capture
+// included).  In a product of more than FAN_PRODUCTS products the tails are
+// nothing and the bins only take each other's cache (6.0e9 products: 72.4
+// against 72.2 ms; 6e8: 4.6 against 4.8 ms): its bins run one by one.
+constexpr unsigned long long FAN_PRODUCTS = 1ull << 31;
+struct Fan {
+  cudaStream_t main;
+  SideStreams::Dev *d = nullptr;
+  bool used[FAN_SIDES] = {false};
+  bool failed = false;
+  // groups: bit g set when group g has work; with one group nothing is forked
+  Fan(cudaStream_t st, unsigned groups) : main(st) {
+    if ((groups & (groups - 1)) == 0) return;
+    d = t_sides.get();
+    if (d && cudaEventRecord(d->fork, main) != cudaSuccess) {
+      cudaGetLastError();
+      d = nullptr;
+    }
+  }
+  cudaStream_t stream(int group) {
+    if (!d || group == 0) return main;
+    const int i = group - 1;
+    if (!used[i]) {
+      if (cudaStreamWaitEvent(d->s[i], d->fork, 0) != cudaSuccess) failed = true;
+      used[i] = true;
+    }
+    return d->s[i];
+  }
+  int join() {
+    for (int i = 0; i < FAN_SIDES; ++i) {
+      if (!used[i]) continue;
+      used[i] = false;
+      if (cudaEventRecord(d->join[i], d->s[i]) != cudaSuccess || cudaStreamWaitEvent(main, d->join[i], 0) != cudaSuccess)
+        failed = true;
+    }
+    if (!failed) return HS_OK;
+    // the side streams' work must end before the caller's buffers are touched again
+    if (d)
+      for (int i = 0; i < FAN_SIDES; ++i) cudaStreamSynchronize(d->s[i]);
+    cudaGetLastError();
+    return HS_ECUDA;
+  }
+  ~Fan() { join(); }
+};
+// numeric kinds: heavy rows, large, mid, and the rows of a warp
+static int num_group(int kind) { return kind == NUM_KINDS - 1 ? 1 : kind == 5 || kind == 6 ? 2 : kind == 3 || kind == 4 ? 3 : 0; }
+
 #define CK(call)                          \
   do {                                    \
     cudaError_t e_ = (call);              \
@@ -383,6 +478,7 @@ struct hs_plan {
   long long *dbg = nullptr;
   hs_allocator al{};
   bool has_al = false;
+  bool side_by_side = false;  // the bins run beside each other (hs::Fan)
   std::vector<hs::Mem::Blk> blocks;
 };
 
@@ -488,6 +584,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   memcpy(key_off, hb->key_off, sizeof(key_off));
   const int nhist = hb->nhist;
   const int tiny_group = tiny_group_pays(key_off[KEY_TINY + 1] - key_off[KEY_TINY], hb->stats[4]);
+  const bool side_by_side = hb->stats[0] <= FAN_PRODUCTS;
   const int pair_long = hb->stats[2] > (unsigned long long)PAIR_LONG;  // (read before hb is copied to again)
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
 
@@ -557,69 +654,65 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
 
   // the B segment index: for every B row longer than min_len, the offset of
   // its first entry in each SEG_W-column segment (the table kept within an
-  // eighth of the free memory, at most 4 GiB); built once, on first need
+  // eighth of the free memory, at most 4 GiB): its room is taken here, the
+  // numeric pass fills it
   int32_t *bci_id = nullptr, *bci = nullptr;
-  bool bci_done = false;
-  auto build_bci = [&]() -> int {
-    if (bci_done || B->nnz <= 0) return HS_OK;
-    bci_done = true;
+  int64_t bci_min_len = 32, bci_rows = 0;
+  auto alloc_bci = [&]() {
+    if (B->nnz <= 0) return;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
       const size_t budget = free_b / 8 < ((size_t)4 << 30) ? free_b / 8 : ((size_t)4 << 30);
-      const int64_t stride = (int64_t)nseg + 1;
-      const int64_t row_bytes = stride * 4;
-      int64_t min_len = 32;
+      const int64_t row_bytes = ((int64_t)nseg + 1) * 4;
       const int64_t need = (B->nnz * row_bytes + (int64_t)budget - 1) / (int64_t)(budget ? budget : 1);
-      if (need > min_len) min_len = need;
-      int64_t max_rows = B->nnz / (min_len + 1);
-      if (max_rows > (int64_t)(budget / row_bytes)) max_rows = (int64_t)(budget / row_bytes);
-      if (max_rows > 0 && min_len < 0x7fffffff) {
+      if (need > bci_min_len) bci_min_len = need;
+      bci_rows = B->nnz / (bci_min_len + 1);
+      if (bci_rows > (int64_t)(budget / row_bytes)) bci_rows = (int64_t)(budget / row_bytes);
+      if (bci_rows > 0 && bci_min_len < 0x7fffffff) {
         bci_id = (int32_t *)mem.raw(sizeof(int32_t) * (size_t)B->m);
-        bci = bci_id ? (int32_t *)mem.raw((size_t)max_rows * (size_t)row_bytes) : nullptr;
+        bci = bci_id ? (int32_t *)mem.raw((size_t)bci_rows * (size_t)row_bytes) : nullptr;
         if (bci_id) mem.scratch.push_back({bci_id, sizeof(int32_t) * (size_t)B->m});
-        if (bci) mem.scratch.push_back({bci, (size_t)max_rows * (size_t)row_bytes});
+        if (bci) mem.scratch.push_back({bci, (size_t)bci_rows * (size_t)row_bytes});
         mem.failed = false;  // optional: without it the part ends are searched
         if (!bci) bci_id = nullptr;
-        else {
-          PhaseTimer t("bci", st);
-          launch_build_bci(rb, nseg, (int)min_len, max_rows, bci_id, bci, &sb->bci_cnt, st);
-          if (int e = phase_check("bci", st, sb->dbg)) return e;
-        }
       }
     }
     cudaGetLastError();
-    return HS_OK;
   };
 
   // ---- symbolic
   SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, glist, loff, &sb->lpool, lcap, tiny_group};
-  auto sym_bin = [&](int k0, int k1) {
-    sa.list = list + key_off[k0];
-    sa.count = key_off[k1] - key_off[k0];
-  };
   {
+    struct SymBin {
+      const char *name;
+      int k0, k1, group;
+      void (*launch)(const SymArgs &, cudaStream_t);
+    };
+    // the longest first; the rows of a warp stay on the caller's stream
+    const SymBin bins_[] = {{"symbolic_heavy", KEY_HEAVY, NKEYS, 1, launch_sym_heavy},
+                            {"symbolic_large", KEY_LARGE, KEY_LARGE + 1, 2, launch_sym_large},
+                            {"symbolic_mid", KEY_MID, KEY_MID + 1, 2, launch_sym_mid},
+                            {"symbolic_mid_s", KEY_MID_S, KEY_MID_S + 1, 3, launch_sym_mid_s},
+                            {"symbolic_tiny", KEY_TINY, KEY_TINY + 1, 0, launch_sym_tiny},
+                            {"symbolic_warp", KEY_WARP, KEY_WARP + 1, 0, launch_sym_warp},
+                            {"symbolic_spa", KEY_SPA, KEY_SPA + 1, 0, launch_sym_spa}};
+    unsigned groups = 0;
+    for (const SymBin &x : bins_)
+      if (side_by_side && key_off[x.k1] > key_off[x.k0]) groups |= 1u << x.group;
     PhaseTimer t("symbolic", st);
-    sym_bin(KEY_TINY, KEY_TINY + 1);
-    { PhaseTimer t2("symbolic_tiny", st, sa.count > 0); launch_sym_tiny(sa, st); }
-    if (int e = phase_check("symbolic_tiny", st, sb->dbg)) return e;
-    sym_bin(KEY_WARP, KEY_WARP + 1);
-    { PhaseTimer t2("symbolic_warp", st, sa.count > 0); launch_sym_warp(sa, st); }
-    if (int e = phase_check("symbolic_warp", st, sb->dbg)) return e;
-    sym_bin(KEY_MID_S, KEY_MID_S + 1);
-    { PhaseTimer t2("symbolic_mid_s", st, sa.count > 0); launch_sym_mid_s(sa, st); }
-    if (int e = phase_check("symbolic_mid_s", st, sb->dbg)) return e;
-    sym_bin(KEY_MID, KEY_MID + 1);
-    { PhaseTimer t2("symbolic_mid", st, sa.count > 0); launch_sym_mid(sa, st); }
-    if (int e = phase_check("symbolic_mid", st, sb->dbg)) return e;
-    sym_bin(KEY_LARGE, KEY_LARGE + 1);
-    { PhaseTimer t2("symbolic_large", st, sa.count > 0); launch_sym_large(sa, st); }
-    if (int e = phase_check("symbolic_large", st, sb->dbg)) return e;
-    sym_bin(KEY_SPA, KEY_SPA + 1);
-    { PhaseTimer t2("symbolic_spa", st, sa.count > 0); launch_sym_spa(sa, st); }
-    if (int e = phase_check("symbolic_spa", st, sb->dbg)) return e;
-    sym_bin(KEY_HEAVY, NKEYS);
-    { PhaseTimer t2("symbolic_heavy", st, sa.count > 0); launch_sym_heavy(sa, st); }
-    if (int e = phase_check("symbolic_heavy", st, sb->dbg)) return e;
+    Fan fan(st, groups);
+    for (const SymBin &x : bins_) {
+      sa.list = list + key_off[x.k0];
+      sa.count = key_off[x.k1] - key_off[x.k0];
+      if (sa.count <= 0) continue;
+      const cudaStream_t bst = fan.stream(x.group);
+      {
+        PhaseTimer t2(x.name, bst);
+        x.launch(sa, bst);
+      }
+      if (int e = phase_check(x.name, bst, sb->dbg)) return e;
+    }
+    if (int e = fan.join()) return e;
   }
 
   // ---- offsets and numeric bins
@@ -714,14 +807,25 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     gend = mem.tmp<int32_t>((size_t)A->nnz);
     if (!gcur || !gend) return HS_ENOMEM;
   }
-  // heavy bin: the B segment index (built before the symbolic pass when
-  // symbolic units used it)
-  if (key_off[NKEYS] > key_off[KEY_HEAVY])
-    if (int e = build_bci()) return e;
+  unsigned groups = 0;
+  for (int kind = 0; kind < NUM_KINDS; ++kind) {
+    const int k0 = KEY_TINY + kind, k1 = kind == NUM_KINDS - 1 ? NKEYS : k0 + 1;
+    if (side_by_side && key_off[k1] > key_off[k0]) groups |= 1u << num_group(kind);
+  }
+  if (nheavy > 0) alloc_bci();  // (every allocation before the streams part: they are ordered on the caller's)
+  std::unique_ptr<PhaseTimer> t_num(new PhaseTimer("numeric", st));
+  Fan fan(st, groups);
+  // heavy bin: the B segment index, and the units' B segments
+  const cudaStream_t hst = nheavy > 0 ? fan.stream(num_group(NUM_KINDS - 1)) : st;
+  if (bci) {
+    PhaseTimer t("bci", hst);
+    launch_build_bci(rb, nseg, (int)bci_min_len, bci_rows, bci_id, bci, &sb->bci_cnt, hst);
+    if (int e = phase_check("bci", hst, sb->dbg)) return e;
+  }
   if (units && vb) {
-    PhaseTimer t("heavy_pairs", st);
-    launch_build_pairs(rs, rb, units, nunits, bci_id, bci, nseg, a_bytes, pair_long, pseg, paval, st);
-    if (int e = phase_check("heavy_pairs", st, sb->dbg)) return e;
+    PhaseTimer t("heavy_pairs", hst);
+    launch_build_pairs(rs, rb, units, nunits, bci_id, bci, nseg, a_bytes, pair_long, pseg, paval, hst);
+    if (int e = phase_check("heavy_pairs", hst, sb->dbg)) return e;
   }
   NumArgs na{rs, rb,   f,    nullptr, 0,    Cp,    C->idx, C->val, hslot,
              hist, nseg, &sb->dyn[1], &sb->err, gcur, gend, glist, loff, bci_id, bci};
@@ -741,23 +845,25 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
                                   "numeric_sort_s", "numeric_sort_m",  "numeric_sort",  "numeric_spa",
                                   "numeric_heavy"};
   static_assert(KEY_TINY + NUM_KINDS - 1 == KEY_HEAVY, "one key per numeric kind before the heavy keys");
-  {
-    PhaseTimer t("numeric", st);
-    for (int kind = 0; kind < NUM_KINDS; ++kind) {
-      const int k0 = KEY_TINY + kind, k1 = kind == NUM_KINDS - 1 ? NKEYS : k0 + 1;
-      na.list = list + key_off[k0];
-      na.count = key_off[k1] - key_off[k0];
-      if (plan) {
-        plan->off[kind] = key_off[k0];
-        plan->count[kind] = na.count;
-      }
-      {
-        PhaseTimer t2(names[kind], st, na.count > 0);
-        if (na.count > 0 && !launch_num(sr, out_dt, kind, na, st)) return HS_EINVAL;
-      }
-      if (int e = phase_check(names[kind], st, sb->dbg)) return e;
+  for (int i = 0; i < NUM_KINDS; ++i) {
+    const int kind = NUM_KINDS - 1 - i;  // the longest first
+    const int k0 = KEY_TINY + kind, k1 = kind == NUM_KINDS - 1 ? NKEYS : k0 + 1;
+    na.list = list + key_off[k0];
+    na.count = key_off[k1] - key_off[k0];
+    if (plan) {
+      plan->off[kind] = key_off[k0];
+      plan->count[kind] = na.count;
     }
+    if (na.count <= 0) continue;
+    const cudaStream_t bst = fan.stream(num_group(kind));
+    {
+      PhaseTimer t2(names[kind], bst);
+      if (!launch_num(sr, out_dt, kind, na, bst)) return HS_EINVAL;
+    }
+    if (int e = phase_check(names[kind], bst, sb->dbg)) return e;
   }
+  if (int e = fan.join()) return e;
+  t_num.reset();
   if (flags & HS_FLAG_VALIDATE) {
     CK(cudaMemcpyAsync(hb, sb, sizeof(SmallBlock), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -813,6 +919,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   if (plan) {  // the plan takes over every scratch buffer
     plan->c_nnz = nnz;
     plan->na = na;
+    plan->side_by_side = side_by_side;
     plan->list = list;
     plan->dyn = &sb->dyn[1];
     plan->err = &sb->err;
@@ -1309,17 +1416,23 @@ int hs_plan_execute(const hs_plan *P, const void *A_val, const void *B_val, void
   na.B.v = B_val;
   na.Cv = C_val;
   CK(cudaMemsetAsync(P->dyn, 0, 2 * sizeof(int), st));  // the heavy rows' and units' counters
+  unsigned groups = 0;
+  for (int kind = 0; kind < NUM_KINDS; ++kind)
+    if (P->side_by_side && P->count[kind] > 0) groups |= 1u << num_group(kind);
+  Fan fan(st, groups);
   // the heavy units' B segments carry A's values: laid out again from the new ones
   if (na.units && na.pseg && na.nunits > 0)
     launch_build_pairs(na.A, na.B, const_cast<HeavyUnit *>(na.units), na.nunits, na.bci_id, na.bci, na.nseg,
                        na.pair_abytes, na.pair_long, const_cast<int64_t *>(na.pseg), const_cast<void *>(na.paval),
-                       st);
-  for (int kind = 0; kind < NUM_KINDS; ++kind) {
+                       fan.stream(num_group(NUM_KINDS - 1)));
+  for (int i = 0; i < NUM_KINDS; ++i) {
+    const int kind = NUM_KINDS - 1 - i;
     if (P->count[kind] <= 0) continue;
     na.list = P->list + P->off[kind];
     na.count = P->count[kind];
-    if (!launch_num(P->sr, P->out_dt, kind, na, st)) return HS_EINVAL;
+    if (!launch_num(P->sr, P->out_dt, kind, na, fan.stream(num_group(kind)))) return HS_EINVAL;
   }
+  if (int e = fan.join()) return e;
   return check_launch();
 }
 
