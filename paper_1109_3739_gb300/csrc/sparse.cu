@@ -32,7 +32,11 @@ constexpr int SP_MAX_PASSES = 8;
 constexpr unsigned long long SP_INCL = 1ull << 63, SP_AGG = 1ull << 62;
 constexpr int SP_SPIN_LIMIT = 1 << 18;  // polls of one status word before giving up (well under a second)
 int sp_spin_limit() { return SP_SPIN_LIMIT; }
-static_assert(SP_NT == SP_RADIX, "one thread per digit in the per-tile digit scan");
+constexpr int SP_LOOK = 8;  // status words a look-back asks for at a time
+// the sorting pass: eight tuples a thread, so that two blocks of 16 warps fit
+// an SM's registers (sixteen a thread left it with 24 warps)
+constexpr int OS_NT = 512, OS_IPT = SP_TILE / OS_NT, OS_WARPS = OS_NT / 32;
+static_assert(OS_IPT % 2 == 0 && SP_RADIX % 32 == 0 && SP_RADIX <= OS_NT, "two ranks a register, a thread per digit");
 
 template <bool FIRST>
 __device__ __forceinline__ uint64_t sp_key(const uint64_t *K, const int32_t *I, const int32_t *J, int64_t t,
@@ -68,7 +72,7 @@ template <int VB> struct SpVal { using T = uint32_t; };
 template <> struct SpVal<8> { using T = uint64_t; };
 
 template <int VB> constexpr size_t sp_scatter_smem() {
-  return (size_t)SP_TILE * 8 + (size_t)SP_TILE * (VB ? VB : 0) + sizeof(int) * SP_WARPS * SP_RADIX +
+  return (size_t)SP_TILE * 8 + (size_t)SP_TILE * (VB ? VB : 0) + sizeof(int) * OS_WARPS * SP_RADIX +
          sizeof(int) * SP_RADIX + sizeof(long long) * SP_RADIX;
 }
 
@@ -81,11 +85,24 @@ __device__ __forceinline__ void sp_st(unsigned long long *p, unsigned long long 
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// lanes of `act` that hold the same digit: one ballot per bit (a match
+// instruction looks for every distinct digit in turn)
+__device__ __forceinline__ unsigned sp_peers(unsigned act, int d) {
+  unsigned p = act;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const bool one = (d >> b) & 1;
+    const unsigned m = __ballot_sync(FULL, one);
+    p &= one ? m : ~m;
+  }
+  return p;
+}
+
 // one stable pass.  ghist: this pass's 256 digit totals; status: tiles x 256
 // look-back words (zeroed once per call); ticket: tiles are numbered in the
 // order the CTAs start, so every tile a CTA waits for has started before it.
 template <bool FIRST, int VB>
-__global__ void __launch_bounds__(SP_NT, 3) k_sp_onesweep(const uint64_t *Kin, const int32_t *I, const int32_t *J,
+__global__ void __launch_bounds__(OS_NT, 2) k_sp_onesweep(const uint64_t *Kin, const int32_t *I, const int32_t *J,
                                                        const void *Vin, int64_t nnz, int nbj, int64_t m,
                                                        int64_t n, int pass, const unsigned long long *ghist,
                                                        unsigned long long *status, int *ticket, uint64_t *Kout,
@@ -95,58 +112,61 @@ __global__ void __launch_bounds__(SP_NT, 3) k_sp_onesweep(const uint64_t *Kin, c
   uint64_t *skey = reinterpret_cast<uint64_t *>(sp_smem);
   VT *sval = reinterpret_cast<VT *>(sp_smem + (size_t)SP_TILE * 8);
   int *wcnt = reinterpret_cast<int *>(sp_smem + (size_t)SP_TILE * 8 + (size_t)SP_TILE * VB);  // [warp][digit]
-  int *start = wcnt + SP_WARPS * SP_RADIX;
+  int *start = wcnt + OS_WARPS * SP_RADIX;
   long long *goff = reinterpret_cast<long long *>(start + SP_RADIX);
-  __shared__ int wsum[SP_WARPS];
+  __shared__ int wsum[OS_WARPS];
   __shared__ int tile_s;
 
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int shift = 8 * pass;
-  for (int x = threadIdx.x; x < SP_WARPS * SP_RADIX; x += SP_NT) wcnt[x] = 0;
+  for (int x = threadIdx.x; x < OS_WARPS * SP_RADIX; x += OS_NT) wcnt[x] = 0;
   if (threadIdx.x == 0) tile_s = atomicAdd(ticket, 1);
   __syncthreads();
   const int64_t tile = tile_s;
   const int64_t t0 = tile * SP_TILE;
   const int nt = (int)(nnz - t0 < SP_TILE ? nnz - t0 : SP_TILE);
   const unsigned lt = (1u << lane) - 1u;
-  uint64_t k[SP_IPT];
-  VT v[SP_IPT];
-  unsigned r2[SP_IPT / 2];  // ranks inside the warp's digit group (< 512), two per register
-  // warp w ranks the tile's items w*512 .. w*512+511 in order, 32 at a time;
-  // every load is issued before the first ranking step
+  uint64_t k[OS_IPT];
+  VT v[OS_IPT];
+  unsigned r2[OS_IPT / 2];  // ranks inside the warp's digit group (< 512), two per register
+  // warp w ranks the tile's items w*256 .. w*256+255 in order, 32 at a time;
+  // every key is asked for before the first ranking step
 #pragma unroll
-  for (int it = 0; it < SP_IPT; ++it) {
-    const int e = w * (SP_IPT * 32) + it * 32 + lane;
+  for (int it = 0; it < OS_IPT; ++it) {
+    const int e = w * (OS_IPT * 32) + it * 32 + lane;
     k[it] = 0;
-    v[it] = 0;
-    if (e < nt) {
-      k[it] = sp_key<FIRST>(Kin, I, J, t0 + e, nbj, m, n, flag);
-      if (VB) v[it] = reinterpret_cast<const VT *>(Vin)[t0 + e];
-    }
+    if (e < nt) k[it] = sp_key<FIRST>(Kin, I, J, t0 + e, nbj, m, n, flag);
   }
 #pragma unroll
-  for (int it = 0; it < SP_IPT; ++it) {
-    const int e = w * (SP_IPT * 32) + it * 32 + lane;
+  for (int it = 0; it < OS_IPT; ++it) {
+    const int e = w * (OS_IPT * 32) + it * 32 + lane;
     const bool ok = e < nt;
     if (!(it & 1)) r2[it >> 1] = 0;
     const unsigned act = __ballot_sync(FULL, ok);
-    if (ok) {
-      const int d = (int)((k[it] >> shift) & (SP_RADIX - 1));
-      const unsigned peers = __match_any_sync(act, d);
-      const int base = wcnt[w * SP_RADIX + d];
-      r2[it >> 1] |= (unsigned)(base + __popc(peers & lt)) << (16 * (it & 1));
-      __syncwarp(act);
-      if (lane == 31 - __clz(peers)) wcnt[w * SP_RADIX + d] = base + __popc(peers);
-    }
+    const int d = (int)((k[it] >> shift) & (SP_RADIX - 1));
+    const unsigned peers = sp_peers(act, d);
+    const int base = wcnt[w * SP_RADIX + d];
+    r2[it >> 1] |= (unsigned)(base + __popc(peers & lt)) << (16 * (it & 1));
     __syncwarp();
+    if (ok && lane == 31 - __clz(peers)) wcnt[w * SP_RADIX + d] = base + __popc(peers);
+    __syncwarp();
+  }
+  // the values are asked for now, when the ranking's registers are free again,
+  // and arrive while the digits are counted
+#pragma unroll
+  for (int it = 0; it < OS_IPT; ++it) {
+    const int e = w * (OS_IPT * 32) + it * 32 + lane;
+    v[it] = 0;
+    if (VB && e < nt) v[it] = reinterpret_cast<const VT *>(Vin)[t0 + e];
   }
   __syncthreads();
   // thread d: the warps' offsets inside the tile's run of digit d, the tile's
   // count of d, published at once so that later tiles can go on
   const int d = threadIdx.x;
+  const bool digit = d < SP_RADIX;  // (whole warps)
   int tot = 0;
 #pragma unroll
-  for (int ww = 0; ww < SP_WARPS; ++ww) {
+  for (int ww = 0; ww < (digit ? OS_WARPS : 0); ++ww) {
     const int c = wcnt[ww * SP_RADIX + d];
     wcnt[ww * SP_RADIX + d] = tot;
     tot += c;
@@ -156,16 +176,16 @@ __global__ void __launch_bounds__(SP_NT, 3) k_sp_onesweep(const uint64_t *Kin, c
   // (a tile equal to `withhold` never publishes: the failure-detection
   // tests use it so that the next tile's bounded wait runs out)
   const bool publish = tile != withhold;
-  if (publish) {
+  if (publish && digit) {
     if (tile == 0) sp_st(my, SP_INCL | tag | (unsigned)tot);
     else sp_st(my, SP_AGG | tag | (unsigned)tot);
   }
   // tile start of each digit (exclusive scan over the digits) and the digit's
   // start in the whole output (exclusive scan of this pass's totals)
   const int incl = warp_incl_scan(tot);
-  const long long gh = (long long)ghist[d];
+  const long long gh = digit ? (long long)ghist[d] : 0;
   const long long gincl = warp_incl_scan(gh);
-  __shared__ long long gsum[SP_WARPS];
+  __shared__ long long gsum[OS_WARPS];
   if (lane == 31) {
     wsum[w] = incl;
     gsum[w] = gincl;
@@ -174,38 +194,17 @@ __global__ void __launch_bounds__(SP_NT, 3) k_sp_onesweep(const uint64_t *Kin, c
   int before = 0;
   long long gbefore = 0;
 #pragma unroll
-  for (int ww = 0; ww < SP_WARPS; ++ww) {
+  for (int ww = 0; ww < OS_WARPS; ++ww) {
     before += ww < w ? wsum[ww] : 0;
     gbefore += ww < w ? gsum[ww] : 0;
   }
-  start[d] = before + incl - tot;
-  // decoupled look-back over the tiles before this one
-  long long excl = 0;
-  if (tile > 0) {
-    for (int64_t j = tile - 1; j >= 0; --j) {
-      const unsigned long long *q = status + j * SP_RADIX + d;
-      unsigned long long x = 0;
-      int spin = 0;
-      for (;;) {
-        x = sp_ld(q);
-        if ((x & (0xffffull << 32)) == tag && (x & (SP_INCL | SP_AGG))) break;
-        if (++spin > spin_limit) {  // never expected: the host reports HS_ETIMEDOUT
-          atomicOr(flag, 2);
-          x = SP_INCL | tag;
-          break;
-        }
-        if (spin > 32) __nanosleep(64);
-      }
-      excl += (long long)(x & 0xffffffffull);
-      if (x & SP_INCL) break;
-    }
-    if (publish) sp_st(my, SP_INCL | tag | (unsigned)(excl + tot));
-  }
-  goff[d] = gbefore + gincl - gh + excl;
+  if (digit) start[d] = before + incl - tot;
   __syncthreads();
+  // the tile in digit order to shared memory, which frees the registers that
+  // the look-back would otherwise have to carry along
 #pragma unroll
-  for (int it = 0; it < SP_IPT; ++it) {
-    const int e = w * (SP_IPT * 32) + it * 32 + lane;
+  for (int it = 0; it < OS_IPT; ++it) {
+    const int e = w * (OS_IPT * 32) + it * 32 + lane;
     if (e < nt) {
       const int dd = (int)((k[it] >> shift) & (SP_RADIX - 1));
       const int pos = start[dd] + wcnt[w * SP_RADIX + dd] + (int)((r2[it >> 1] >> (16 * (it & 1))) & 0xffffu);
@@ -213,8 +212,39 @@ __global__ void __launch_bounds__(SP_NT, 3) k_sp_onesweep(const uint64_t *Kin, c
       if (VB) sval[pos] = v[it];
     }
   }
+  // decoupled look-back over the tiles before this one, SP_LOOK of them asked
+  // at a time: tiles that start together find only counts, no prefixes, before
+  // them, and a round trip to L2 for each in turn was most of a tile's time
+  long long excl = 0;
+  if (tile > 0 && digit) {
+    bool done = false;
+    for (int64_t j = tile - 1; j >= 0 && !done; j -= SP_LOOK) {
+      unsigned long long x[SP_LOOK];
+#pragma unroll
+      for (int u = 0; u < SP_LOOK; ++u) x[u] = j - u >= 0 ? sp_ld(status + (j - u) * SP_RADIX + d) : 0ull;
+#pragma unroll
+      for (int u = 0; u < SP_LOOK; ++u) {
+        if (done || j - u < 0) continue;
+        const unsigned long long *q = status + (j - u) * SP_RADIX + d;
+        int spin = 0;
+        while ((x[u] & (0xffffull << 32)) != tag || !(x[u] & (SP_INCL | SP_AGG))) {
+          if (++spin > spin_limit) {  // never expected: the host reports HS_ETIMEDOUT
+            atomicOr(flag, 2);
+            x[u] = SP_INCL | tag;
+            break;
+          }
+          if (spin > 32) __nanosleep(64);
+          x[u] = sp_ld(q);
+        }
+        excl += (long long)(x[u] & 0xffffffffull);
+        done = (x[u] & SP_INCL) != 0;
+      }
+    }
+    if (publish) sp_st(my, SP_INCL | tag | (unsigned)(excl + tot));
+  }
+  if (digit) goff[d] = gbefore + gincl - gh + excl;
   __syncthreads();
-  for (int e = threadIdx.x; e < nt; e += SP_NT) {
+  for (int e = threadIdx.x; e < nt; e += OS_NT) {
     const uint64_t key = skey[e];
     const int dd = (int)((key >> shift) & (SP_RADIX - 1));
     const long long out = goff[dd] + (e - start[dd]);
@@ -450,9 +480,9 @@ static void sp_pass_one(const uint64_t *Kin, const int32_t *I, const int32_t *J,
                         unsigned long long *status, int *ticket, int64_t ntiles, uint64_t *Kout, void *Vout,
                         int *flag, int spin_limit, long long withhold, cudaStream_t st) {
   constexpr size_t smem = sp_scatter_smem<VB>();
-  fit_per_sm(k_sp_onesweep<FIRST, VB>, SP_NT, smem);  // (sets its shared memory limit)
+  fit_per_sm(k_sp_onesweep<FIRST, VB>, OS_NT, smem);  // (sets its shared memory limit)
   count_launch();
-  k_sp_onesweep<FIRST, VB><<<sp_grid(ntiles), SP_NT, smem, st>>>(Kin, I, J, Vin, nnz, nbj, m, n, pass, ghist,
+  k_sp_onesweep<FIRST, VB><<<sp_grid(ntiles), OS_NT, smem, st>>>(Kin, I, J, Vin, nnz, nbj, m, n, pass, ghist,
                                                                  status, ticket, Kout, Vout, flag, spin_limit,
                                                                  withhold);
 }
