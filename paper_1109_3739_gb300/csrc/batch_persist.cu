@@ -140,7 +140,7 @@ template <class SR>
 __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
   using T = typename SR::val_t;
   using Struct = Semiring<OR_AND, NoVal>;
-  using LC = CtaNumLayout<T, BPC_SLOTS, BPC_CAP, BP_NT>;
+  using LC = CtaNumLayout<T, BPC_SLOTS, BPC_CAP, BP_CH>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item, s_count, s_cnt_b[BP_NBUCK], s_wtmp[33], s_kmin, s_kmax;
   const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
     T *vals = reinterpret_cast<T *>(smem_raw + (size_t)BPC_SLOTS * 4);
     int *ck = reinterpret_cast<int *>(smem_raw + LC::region0);
     T *cv = reinterpret_cast<T *>(smem_raw + LC::region0 + (size_t)BPC_CAP * 4);
-    auto &ex = *reinterpret_cast<CtaExpandSmem<T, nch(BP_NT)> *>(smem_raw + LC::ex_off);
+    auto &ex = *reinterpret_cast<CtaExpandSmem<T, BP_CH> *>(smem_raw + LC::ex_off);
     while (true) {
       if (tid == 0) s_item = atomicAdd(&ctr->num_c, 1);
       __syncthreads();
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
           if constexpr (SR::has_val) vals[s] = SR::identity();
         }
         __syncthreads();
-        cta_products<SR, nch(BP_NT)>(A, B, A.p[r], A.p[r + 1], rec >= 0, lo, hi, ex, tl.wtmp,
+        cta_products<SR, BP_CH>(A, B, A.p[r], A.p[r + 1], rec >= 0, lo, hi, ex, tl.wtmp,
                                          [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, &ctr->kerr); });
         if (HS_G(dbg, cb + done + part <= a.cap, 81, cb + done + part))
           group_sort_emit<CtaGroup, T, SR::has_val>(keys, vals, slots, part, ck, cv, smem_raw, tl.wtmp, &tl.es,
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
 template <class SR> size_t bp_smem() {
   using T = typename SR::val_t;
   const size_t w = (size_t)BP_NW * bp_warp_bytes<T>();
-  const size_t c = CtaNumLayout<T, BPC_SLOTS, BPC_CAP, BP_NT>::bytes;
+  const size_t c = CtaNumLayout<T, BPC_SLOTS, BPC_CAP, BP_CH>::bytes;
   const size_t s = (size_t)BPC_SYM * 4 + sizeof(CtaExpandSmem<NoVal, BP_CH>);
   return std::max(w, std::max(c, s));
 }
