@@ -21,6 +21,7 @@
 // Counts go to cnt[row + 1] so an inclusive scan turns them into row offsets.
 #include "common.cuh"
 #include "internal.h"
+#include "sortrow.cuh"
 
 namespace hs {
 
@@ -123,8 +124,12 @@ __global__ void __launch_bounds__(TINY_WPB * 32, 4) k_sym_tiny_group(SymArgs a) 
 // most 512 products (1024 slots) and, in their own launch, of 513..1024
 // products (2048 slots).  BITS: B's columns fit the table's room as a bitmap
 // (32 columns a slot), which replaces the hash set: one atomic a product
-// instead of hash, probe and compare-and-swap.
+// instead of hash, probe and compare-and-swap.  Without one, rows of at most
+// 64 products sort their columns, two a lane, and count the changes: 21
+// stages without a branch, against probes that the lanes of a warp, and
+// repeated columns among them, wait for one another in.
 constexpr int WARP_WPB = 8;
+constexpr int F_SYM_SORT = 64;
 template <int SLOTS, bool BITS>
 __global__ void __launch_bounds__(WARP_WPB * 32, 4) k_sym_warp(SymArgs a) {
   extern __shared__ __align__(16) int tables[];
@@ -140,23 +145,35 @@ __global__ void __launch_bounds__(WARP_WPB * 32, 4) k_sym_warp(SymArgs a) {
   for (; idx < a.count; idx += step) {
     nx.row(A, a.list, idx + step, a.count);
     const int slots = max(64, min(SLOTS, next_pow2(2 * fr)));
+    const bool sorts = !BITS && SLOTS <= 2 * F_WARP && fr <= F_SYM_SORT;
     if constexpr (BITS) bitmap_clear<WarpGroup>(keys, n);
-    else
+    else if (!sorts)
       for (int s = lane; s < slots; s += 32) keys[s] = EMPTY;
     __syncwarp();
     int cnt = 0;
     const unsigned mask = slots - 1;
     nx.range(A);
     if constexpr (!BITS) fr = nx.r >= 0 ? (int)__ldg(a.f + nx.r) : 0;
-    auto put = [&](int col, NoVal, int) {
+    auto put = [&](int col, NoVal, int p) {
       if constexpr (BITS) {
         if (HS_G(a.A.dbg, col >= 0 && col < n, 33, col)) cnt += bitmap_insert(keys, col);
+      } else if (sorts) {
+        if (HS_G(a.A.dbg, p < F_SYM_SORT, 34, p)) keys[p] = col;
       } else {
         cnt += hash_insert_key(keys, mask, col);
       }
     };
-    if (x.r >= 0) warp_products_of<StructSR>(A, B, x, put);
+    const int got = x.r >= 0 ? warp_products_of<StructSR>(A, B, x, put) : 0;
     nx.entries(A);
+    if (sorts) {
+      __syncwarp();
+      uint32_t k[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) k[i] = 2 * lane + i < got ? (uint32_t)keys[(2 * lane + i) & (F_SYM_SORT - 1)] : 0xffffffffu;
+      warp_bitonic_flat<2>(k);
+      const uint32_t before = __shfl_up_sync(FULL, k[1], 1);
+      cnt = (k[0] != 0xffffffffu && (lane == 0 || k[0] != before)) + (k[1] != 0xffffffffu && k[1] != k[0]);
+    }
     cnt = warp_sum(cnt);
     nx.segments(B);
     if (lane == 0 && x.r >= 0) put_count(a, out_row(a.A, x.r), cnt);

@@ -1,0 +1,114 @@
+"""The kernels that take rows by their size, at the edges of their ranges: rows
+sorted instead of hashed, bitmaps of all columns, and rows whose bitmap is
+handed from the symbolic to the numeric pass.  Integer sums, minima and
+structures: every comparison is exact."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1109_3739_gb300 import inputs as I
+from tests.helpers import assert_bitexact, csr
+
+pytestmark = pytest.mark.gpu
+
+
+def H():
+    from paper_1109_3739_gb300 import hspgemm
+    return hspgemm
+
+
+def operands(n, rows, dt, seed):
+    """A and B, a row of A * B for each list of spans (first, last): an entry of A and a row of B for each span,
+    which holds that stretch of one random order of the columns.  A row's products all differ in column, except
+    where its spans overlap."""
+    order = np.argsort(I.draws(seed, 3, 0, n), kind="stable")
+    pieces, arows = [], []
+    for spans in rows:
+        take = []
+        for a, b in spans:
+            take.append(len(pieces))
+            pieces.append(np.sort(order[a:b]))
+        arows.append(np.array(take, np.int64))
+    bptr = np.concatenate([[0], np.cumsum([len(p) for p in pieces])])
+    aptr = np.concatenate([[0], np.cumsum([len(t) for t in arows])])
+    B = csr(len(pieces), n, bptr, np.concatenate(pieces), I.random_values(int(bptr[-1]), dt, seed, kind="signed"), dt)
+    A = csr(len(arows), len(pieces), aptr, np.concatenate(arows), I.random_values(int(aptr[-1]), dt, seed + 1, kind="signed"),
+            dt)
+    return A, B
+
+
+def product(A, B, what, sr):
+    h = H()
+    ref = oracle.spgemm(sr, A, B)
+    dA, dB = h.DeviceCSR.from_host(A), h.DeviceCSR.from_host(B)
+    assert_bitexact(h.spgemm(sr, dA, dB).to_host(), ref, what)
+    P = h.Plan(sr, dA, dB)
+    if P.C.val is not None:
+        P.C.val.zero_()
+    P.execute()
+    assert_bitexact(P.C.to_host(), ref, f"{what}, plan")
+
+
+def split(f, parts, start=0):
+    cuts = np.linspace(0, f, parts + 1).astype(int) + start
+    return [(int(a), int(b)) for a, b in zip(cuts[:-1], cuts[1:])]
+
+
+KINDS = [("plus_times", "i64"), ("min_plus", "f32"), ("or_and", "bool")]
+
+
+@pytest.mark.parametrize("sr,dt", KINDS)
+def test_rows_counted_by_a_sort(sr, dt):
+    """33 to 512 products over too many columns for a bitmap: up to 64 are sorted, more are hashed."""
+    rows = []
+    for f in (33, 63, 64, 65, 128, 512):
+        for dup in (0, 1, f // 2, f - 1):
+            base = split(f - dup, min(3, f - dup))
+            rows.append(base + ([(0, min(dup, f - dup))] if dup else []) + ([(0, 1)] * (dup - min(dup, f - dup))))
+    product(*operands(300001, rows, dt, 5), f"sorted count {sr}", sr)
+
+
+@pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+def test_structure_by_bitmap(n):
+    """Structure-only rows of 500 to 9000 outputs; over 4096 they are not staged."""
+    rows = [split(c, p) + [(0, min(c, d))] for c in (500, 1025, 2049, 4095, 4096, 4097, 9000) for p, d in ((3, 1), (300, 400))]
+    product(*operands(n, rows, "bool", 6), f"{n} columns", "or_and")
+
+
+@pytest.mark.parametrize("n", [(1 << 19) - 1, 1 << 19, (1 << 19) + 1])
+def test_many_rows_of_the_symbolic_bitmap(n):
+    """Enough rows of more than 4096 products for two CTAs an SM, where half a bitmap holds B's columns."""
+    A, B = operands(n, [split(4100 + 40 * i, 3 + i, 17 * i) + [(17 * i, 17 * i + 9)] for i in range(7)], "i64", 7)
+    many = 100  # the seven rows over and over
+    A = csr(7 * many, B.m, np.concatenate([[0], np.cumsum(np.tile(np.diff(A.rowptr), many))]),
+            np.tile(A.col, many), np.tile(A.val, many), "i64")
+    product(A, B, f"{n} columns", "plus_times")
+
+
+@pytest.mark.parametrize("sr,dt", [("plus_times", "i64"), ("min_plus", "f32"), ("or_and", "bool")])
+@pytest.mark.parametrize("n", [70001, (1 << 17) + 4097, 300001])
+def test_rows_that_leave_their_bitmap(n, sr, dt):
+    """Rows of the units on both sides of an output for every second word of the bitmap, some with fewer products
+    than the bitmap has words, and parts of one and of many segments."""
+    half = (n + 63) // 64
+    words = (n + 31) // 32
+    cs = sorted({max(4097, half - 1), max(4097, half), max(4097, half + 1), max(4097, words), 6000, 20011, n // 2, n})
+    rows = [split(c, 5) + [(1, 40)] * 3 for c in cs]
+    product(*operands(n, rows, dt, 8), f"{n} columns {sr}", sr)
+
+
+@pytest.mark.parametrize("sr,dt", [("plus_times", "i64"), ("min_plus", "i32"), ("min_plus", "f32"), ("or_and", "bool")])
+def test_rows_sorted_as_they_are(sr, dt):
+    """1025 to 4096 outputs with few repeated columns, on both sides of the share and of the capacity, the repeats
+    spread over the row or all of one column, in one round of entries and in several."""
+    rows = []
+    for c in (1025, 1820, 2047, 2048, 2049, 3640, 4000, 4095):
+        for dup in (0, 1, c // 8 - 1, c // 8, c // 8 + 1, 2048 - c, 2049 - c, 4096 - c, 4097 - c):
+            if not 0 <= dup <= c or c + dup > 4097:
+                continue
+            rows.append(split(c, 3) + ([(0, dup)] if dup else []))
+            if dup and dup < 600:
+                rows.append(split(c, 290) + [(7, 8)] * dup)
+    product(*operands(600001, rows, dt, 9), f"few repeats {sr} {dt}", sr)
