@@ -274,11 +274,13 @@ __global__ void __launch_bounds__(NT, 1536 / NT) k_sym_cta(SymArgs a) {
 // slower on R-MAT scale 20).
 constexpr int SH_COLS = BITMAP_COLS;          // columns per chunk (one bitmap)
 constexpr int SH_SEGS = SH_COLS / SEG_W;      // segments per chunk (256)
-constexpr int SH_NT = 1024;                   // threads of the heavy symbolic CTA
-constexpr int SH_WARPS = SH_NT / 32;
-constexpr int SH_PPW = SH_SEGS / 2 / SH_WARPS;  // segment pairs per warp (4)
-constexpr int SH_MINB = 1;                    // CTAs per SM the registers are sized for
-static_assert(SH_PPW * SH_WARPS * 2 == SH_SEGS, "the warps' pairs cover a chunk's segments");
+// Threads of the CTA: 1024, one CTA an SM, for a full bitmap; 512, two CTAs an
+// SM, where B's columns need at most half of it and there are SH_ROWS_HALF rows
+// an SM, so that one row's barriers and claims are filled by the other's
+// products (200,003 columns: the pass 2.37 -> 1.83 ms; with few rows the
+// longest one decides, and 512 threads made a product of 256 columns 27 us
+// slower).
+constexpr int SH_NT = 1024, SH_NT_HALF = 512, SH_COLS_HALF = SH_COLS / 2, SH_ROWS_HALF = 4;
 constexpr int SH_BUF = 384;                   // per-warp list staging entries
 static_assert(SEG_W == 4096, "two segments are 256 words: eight per lane");
 
@@ -297,13 +299,16 @@ struct SymHeavyBit {
   }
 };
 
-struct SymHeavySmem {
+template <int NT> struct SymHeavySmem {
+  static constexpr int WARPS = NT / 32;
+  static constexpr int PPW = SH_SEGS / 2 / WARPS;  // segment pairs per warp
+  static_assert(PPW * WARPS * 2 == SH_SEGS, "the warps' pairs cover a chunk's segments");
   CtaExpandSmem<NoVal, CH> ex;
   int wtmp[33];
   int row;
   long long loff;        // the row's list in the pool, or -1
   int scnt[SH_SEGS + 1];  // new columns per segment of the chunk, then their exclusive scan and total
-  int wbuf[SH_WARPS][SH_BUF];
+  int wbuf[WARPS][SH_BUF];
   alignas(16) unsigned bitmap[SH_COLS / 32];
 };
 
@@ -336,19 +341,22 @@ __device__ __forceinline__ void sh_clear8(unsigned *bitmap, int w0, int words) {
   }
 }
 
-__global__ void __launch_bounds__(SH_NT, SH_MINB) k_sym_heavy(SymArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT, SH_NT / NT) k_sym_heavy(SymArgs a) {
+  using L = SymHeavySmem<NT>;
+  constexpr int SH_PPW = L::PPW;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  auto &sm = *reinterpret_cast<SymHeavySmem *>(smem_raw);
+  auto &sm = *reinterpret_cast<L *>(smem_raw);
   const DevCsr A = dev_a(a.A), B = dev_b(a.B);
   const int64_t n = a.B.n;
   const int nchunk = (int)((n + SH_COLS - 1) / SH_COLS);
-  const int lane = lane_id(), warp = threadIdx.x >> 5, nw = SH_WARPS;
+  const int lane = lane_id(), warp = threadIdx.x >> 5, nw = L::WARPS;
   int *buf = sm.wbuf[warp];
   // the first chunk is the widest: clearing its words once leaves the whole
   // bitmap empty, and every chunk clears the words it read afterwards
   {
     const int words0 = (int)((min(n, (int64_t)SH_COLS) + 31) >> 5);
-    for (int wd = threadIdx.x; wd < words0; wd += SH_NT) sm.bitmap[wd] = 0u;
+    for (int wd = threadIdx.x; wd < words0; wd += NT) sm.bitmap[wd] = 0u;
   }
   while (true) {
     if (threadIdx.x == 0) sm.row = atomicAdd(a.dyn, 1);
@@ -585,13 +593,18 @@ void launch_sym_mid_s(const SymArgs &a, cudaStream_t st) { launch_sym_warp_slots
 void launch_sym_mid(const SymArgs &a, cudaStream_t st) { launch_sym_cta<2 * F_MID, 256>(a, st); }
 void launch_sym_large(const SymArgs &a, cudaStream_t st) { launch_sym_cta<16384, 512>(a, st); }
 
+template <int NT> static void launch_sym_heavy_as(const SymArgs &a, cudaStream_t st) {
+  const int64_t words = (a.B.n + 31) / 32;
+  const size_t bytes = offsetof(SymHeavySmem<NT>, bitmap) +
+                       sizeof(unsigned) * (size_t)(words < SH_COLS / 32 ? (words + 3) & ~(int64_t)3 : SH_COLS / 32);
+  const int fit = fit_per_sm(k_sym_heavy<NT>, NT, bytes);
+  count_launch();
+  k_sym_heavy<NT><<<grid_cap(a.count, 1, fit), NT, bytes, st>>>(a);
+}
 void launch_sym_heavy(const SymArgs &a, cudaStream_t st) {
   if (a.count <= 0) return;
-  const int64_t words = (a.B.n + 31) / 32;
-  const size_t bytes = offsetof(SymHeavySmem, bitmap) +
-                       sizeof(unsigned) * (size_t)(words < SH_COLS / 32 ? words : SH_COLS / 32);
-  count_launch();
-  k_sym_heavy<<<grid_cap(a.count, 1, fit_per_sm(k_sym_heavy, SH_NT, bytes)), SH_NT, bytes, st>>>(a);
+  if (a.B.n <= SH_COLS_HALF && a.count >= SH_ROWS_HALF * sm_count()) launch_sym_heavy_as<SH_NT_HALF>(a, st);
+  else launch_sym_heavy_as<SH_NT>(a, st);
 }
 
 }  // namespace hs
