@@ -321,6 +321,75 @@ __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
   }
 }
 
+// ------------------------------------------- structure only, few columns
+// A row of a structure-only product whose B has at most NB_COLS columns needs
+// neither hash nor sort: its products set bits, the bits are counted word by
+// word, and every thread writes the columns of its run of words in order, by
+// way of shared memory when the row is short enough to leave it in one
+// coalesced piece.  It is bound by the products' shared atomics, one each.
+// (R-MAT of 200,003 vertices: the numeric pass 2.07 -> 1.11 ms against hash,
+// compaction and bucket sort.)
+constexpr int NB_COLS = 1 << 18, NB_NT = 256, NB_CH = 256;
+// words a thread reads out at most; an odd number keeps the lanes on different banks
+constexpr int NB_WPT = NB_COLS / 32 / NB_NT + 1;
+constexpr int NB_OUT = 4096;  // columns staged for coalesced stores
+struct NumBitsSmem {
+  unsigned bits[NB_WPT * NB_NT];
+  CtaExpandSmem<NoVal, NB_CH> ex;
+  int out[NB_OUT];
+  int wtmp[33];
+};
+template <class SR>  // (a template only because the header is included more than once)
+__global__ void __launch_bounds__(NB_NT, 4) k_num_bits(NumArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  NumBitsSmem &sm = *reinterpret_cast<NumBitsSmem *>(smem_raw);
+  const DevCsr A = ndev_a(a.A), B = ndev_b(a.B);
+  const int tid = threadIdx.x, n = (int)a.B.n;
+  const int wpt = (((n + 31) / 32 + NB_NT - 1) / NB_NT) | 1;  // words a thread reads out
+  static_assert(NB_WPT % 2 == 1, "an odd run of words holds the widest bitmap");
+  for (int w = tid; w < wpt * NB_NT; w += NB_NT) sm.bits[w] = 0u;
+  __syncthreads();
+  for (int idx = blockIdx.x; idx < a.count; idx += gridDim.x) {
+    const int r = a.list[idx];
+    if (!HS_G(a.A.dbg, r >= 0 && r < a.A.nslots, 36, r)) continue;  // uniform: every thread skips
+    const int64_t o = nout_row(a.A, r);
+    const int64_t cb = a.Cp[o];
+    const int c = (int)(a.Cp[o + 1] - cb);
+    cta_products<SR, NB_CH>(A, B, A.p[r], A.p[r + 1], false, 0, 0, sm.ex, sm.wtmp, [&](int col, NoVal, int) {
+      if (HS_G(a.A.dbg, col >= 0 && col < n, 33, col)) atomicOr(sm.bits + (col >> 5), 1u << (col & 31));
+    });
+    int cnt = 0;
+    for (int k = 0; k < wpt; ++k) cnt += __popc(sm.bits[tid * wpt + k]);
+    const int incl = warp_incl_scan(cnt);
+    if (lane_id() == 31) sm.wtmp[tid >> 5] = incl;
+    __syncthreads();
+    int at = incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < NB_NT / 32; ++w) {
+      const int x = sm.wtmp[w];
+      at += w < (tid >> 5) ? x : 0;
+      total += x;
+    }
+    const bool ok = total == c;  // (uniform)
+    if (!ok && tid == 0) atomicExch(a.err, 1);
+    const bool staged = c <= NB_OUT;
+    for (int k = 0; k < wpt; ++k) {
+      const int w = tid * wpt + k;
+      unsigned bits = sm.bits[w];
+      sm.bits[w] = 0u;  // empty for the next row
+      for (; bits && ok; bits &= bits - 1) {
+        const int col = (w << 5) + __ffs(bits) - 1;
+        if (staged) sm.out[at++] = col;
+        else a.Cj[cb + at++] = col;
+      }
+    }
+    __syncthreads();
+    if (ok && staged)
+      for (int i = tid; i < c; i += NB_NT) __stcs(a.Cj + cb + i, sm.out[i]);
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------------------ heavy
 // Rows whose output exceeds one shared table.  The row's columns are cut into
 // parts (consecutive 4096-column segments, planned from the symbolic pass's
@@ -1107,6 +1176,15 @@ template <class SR> void launch_numeric_sr(int kind, const NumArgs &a, cudaStrea
   using T = typename SR::val_t;
   if (a.count <= 0) return;
   constexpr int CAPL = cap_large<T>();
+  if constexpr (!SR::has_val) {
+    // every block tier, as long as a bitmap of all columns fits a quarter of an SM
+    if (kind >= 3 && kind <= 6 && a.B.n <= NB_COLS) {
+      const int fit = fit_per_sm(k_num_bits<SR>, NB_NT, sizeof(NumBitsSmem));
+      count_launch();
+      k_num_bits<SR><<<ngrid_cap(a.count, 1, fit), NB_NT, sizeof(NumBitsSmem), st>>>(a);
+      return;
+    }
+  }
   switch (kind) {
     case 0: {
       auto k = a.tiny_group ? k_num_tiny_group<SR> : k_num_tiny<SR>;
