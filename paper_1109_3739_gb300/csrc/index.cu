@@ -240,7 +240,7 @@ __global__ void k_spref_offsets(SprefArgs a, int64_t *Bp) {
 // block up to SR_CTA (buckets in shared memory), and longer ones through a
 // bitmap of B's columns (rank = set bits before p).  Every tuple is read and
 // written once; a radix sort of all (row, p) keys took five passes.
-constexpr int SR_WARP = 256, SR_CTA = 2048;
+constexpr int SR_WARP = 64, SR_CTA = 2048;
 template <typename T> struct SprefRowArgs {
   const int64_t *Bp;
   int64_t nI, nJ;
@@ -654,7 +654,7 @@ __global__ void k_asgn_place(AsgnX x, AsgnArgs a, const int64_t *XB, int64_t *at
 }
 
 // assignment: the entries of A inside the I x J block lose their keep bit.  A
-// warp per row of I; a row of more than ASGN_LONG entries by the whole block.
+// warp per row of I, whole blocks for a row of more than ASGN_LONG entries.
 constexpr int ASGN_LONG = 1024;
 __device__ __forceinline__ void asgn_drop(const AsgnArgs &a, int64_t a0, int64_t a1, int64_t step, int64_t first,
                                           uint32_t *keep) {
@@ -674,23 +674,39 @@ __device__ __forceinline__ void asgn_drop(const AsgnArgs &a, int64_t a0, int64_t
     }
   }
 }
+// A long row by ASGN_PARTS blocks (blockIdx.y): it would hold up one block
+// long after the others are done (a row of 3.5e4 entries: 40 us).
+constexpr int ASGN_PARTS = 8;
 __global__ void __launch_bounds__(256) k_asgn_drop(AsgnArgs a, const int32_t *I, int64_t nI, uint32_t *keep) {
-  __shared__ int s_long[8], s_n;
-  const int w = threadIdx.x >> 5;
-  for (int64_t i0 = (int64_t)blockIdx.x * 8; i0 < nI; i0 += (int64_t)gridDim.x * 8) {
+  __shared__ int s_long[8 * ASGN_PARTS], s_n;
+  const int w = threadIdx.x >> 5, part = blockIdx.y;
+  // this block's rows: 64 at a time; a part takes every eighth of the short
+  // ones and its share of all long ones
+  for (int64_t i0 = (int64_t)blockIdx.x * 64; i0 < nI; i0 += (int64_t)gridDim.x * 64) {
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    const int64_t i = i0 + w;
-    const int r = i < nI ? I[i] : -1;
-    if (r >= 0 && r < a.m) {
-      const int64_t a0 = a.Ap[r], a1 = a.Ap[r + 1];
-      if (HS_G(a.dbg, a0 >= 0 && a0 <= a1 && a1 <= a.nnzA, 3, a1)) {
-        if (a1 - a0 <= ASGN_LONG) asgn_drop(a, a0, a1, 32, lane_id(), keep);
-        else if (lane_id() == 0) s_long[atomicAdd(&s_n, 1)] = r;
+    if (threadIdx.x < 64) {
+      const int64_t i = i0 + threadIdx.x;
+      const int r = i < nI ? I[i] : -1;
+      if (r >= 0 && r < a.m && a.Ap[r + 1] - a.Ap[r] > ASGN_LONG) s_long[atomicAdd(&s_n, 1)] = r;
+    }
+    {
+      const int64_t i = i0 + part * 8 + w;
+      const int r = i < nI ? I[i] : -1;
+      if (r >= 0 && r < a.m) {
+        const int64_t a0 = a.Ap[r], a1 = a.Ap[r + 1];
+        if (HS_G(a.dbg, a0 >= 0 && a0 <= a1 && a1 <= a.nnzA, 3, a1) && a1 - a0 <= ASGN_LONG)
+          asgn_drop(a, a0, a1, 32, lane_id(), keep);
       }
     }
     __syncthreads();
-    for (int k = 0; k < s_n; ++k) asgn_drop(a, a.Ap[s_long[k]], a.Ap[s_long[k] + 1], 256, threadIdx.x, keep);
+    for (int k = 0; k < s_n; ++k) {
+      const int64_t a0 = a.Ap[s_long[k]], a1 = a.Ap[s_long[k] + 1];
+      if (!HS_G(a.dbg, a0 >= 0 && a0 <= a1 && a1 <= a.nnzA, 3, a1)) continue;
+      const int64_t share = ((a1 - a0 + ASGN_PARTS - 1) / ASGN_PARTS + 31) & ~(int64_t)31;
+      const int64_t b0 = a0 + part * share, b1 = min(a1, b0 + share);
+      if (b0 < b1) asgn_drop(a, b0, b1, 256, threadIdx.x, keep);
+    }
     __syncthreads();
   }
 }
@@ -719,6 +735,7 @@ __global__ void k_asgn_offsets(AsgnArgs a, const int64_t *XB, const int64_t *S, 
 // A's kept entries into C, a tile of consecutive entries per block: the
 // entries of X that fall inside the tile are found by two searches of at[]
 constexpr int ASGN_NT = 256, ASGN_PER = 8, ASGN_TILE = ASGN_NT * ASGN_PER;
+template <typename V>  // the values' bits by width (NoVal: none); they are asked for with the columns
 __global__ void __launch_bounds__(ASGN_NT) k_asgn_fill_a(AsgnArgs a, const int64_t *at, int64_t nx, const int64_t *S,
                                                          const uint32_t *keep) {
   __shared__ int64_t s_at[ASGN_TILE];
@@ -727,11 +744,15 @@ __global__ void __launch_bounds__(ASGN_NT) k_asgn_fill_a(AsgnArgs a, const int64
   const int64_t k0 = kept_before(S, keep, min(first, a.nnzA));
   const int64_t q0 = (int64_t)blockIdx.x * ASGN_TILE;
   const int w = threadIdx.x >> 5;
+  constexpr bool HAS_VAL = !std::is_same<V, NoVal>::value;
   int c[ASGN_PER];
+  V v[ASGN_PER];
 #pragma unroll
   for (int u = 0; u < ASGN_PER; ++u) {
     const int64_t q = q0 + u * ASGN_NT + threadIdx.x;
-    c[u] = q >= first && q < last ? a.Aj[q] : 0;
+    const bool in = q >= first && q < last;
+    c[u] = in ? __ldcs(a.Aj + q) : 0;
+    if constexpr (HAS_VAL) v[u] = in ? __ldcs(reinterpret_cast<const V *>(a.Av) + q) : V{};
   }
   if (w < 2) {  // entries of X at or before the tile's first and last entry
     const int64_t key = w == 0 ? q0 : q0 + ASGN_TILE - 1;
@@ -760,7 +781,7 @@ __global__ void __launch_bounds__(ASGN_NT) k_asgn_fill_a(AsgnArgs a, const int64
     const int64_t d = kb + __popc(kw & ((1u << (q & 31)) - 1u)) - k0 + l;
     if (!HS_G(a.dbg, d >= 0 && d < a.nnzC, 86, d)) continue;
     a.Cj[d] = c[u];
-    copy_val(a.Cv, d, a.Av, q, a.vbytes);
+    if constexpr (HAS_VAL) reinterpret_cast<V *>(a.Cv)[d] = v[u];
   }
 }
 __global__ void k_asgn_fill_x(AsgnX x, AsgnArgs a, const int64_t *at, const int64_t *src, const int64_t *S,
@@ -793,7 +814,8 @@ void launch_asgn_keep(const AsgnX &x, const AsgnArgs &a, const int32_t *I, int64
   }
   if (!a.accumulate && nI > 0) {
     count_launch();
-    k_asgn_drop<<<grid1(nI * 32), 256, 0, st>>>(a, I, nI, keep);
+    const int64_t g = (nI + 63) / 64, cap = (int64_t)sm_count() * 2;
+    k_asgn_drop<<<dim3((unsigned)(g < cap ? g : cap), ASGN_PARTS), 256, 0, st>>>(a, I, nI, keep);
   }
   if (nw > 0) {
     count_launch();
@@ -809,7 +831,10 @@ void launch_asgn_fill(const AsgnX &x, const AsgnArgs &a, const int64_t *at, cons
                       const uint32_t *keep, cudaStream_t st) {
   if (a.m > 0 && a.nnzA > 0) {
     count_launch();
-    k_asgn_fill_a<<<(unsigned)((a.nnzA + ASGN_TILE - 1) / ASGN_TILE), ASGN_NT, 0, st>>>(a, at, x.nnz, S, keep);
+    const unsigned g = (unsigned)((a.nnzA + ASGN_TILE - 1) / ASGN_TILE);
+    if (a.vbytes == 8) k_asgn_fill_a<unsigned long long><<<g, ASGN_NT, 0, st>>>(a, at, x.nnz, S, keep);
+    else if (a.vbytes == 4) k_asgn_fill_a<uint32_t><<<g, ASGN_NT, 0, st>>>(a, at, x.nnz, S, keep);
+    else k_asgn_fill_a<NoVal><<<g, ASGN_NT, 0, st>>>(a, at, x.nnz, S, keep);
   }
   if (x.nnz > 0) {
     count_launch();
