@@ -419,11 +419,11 @@ void launch_sp_pass(int vb, const uint64_t *Kin, const int32_t *I, const int32_t
                     int nbj, int64_t m, int64_t n, int pass, const unsigned long long *ghist,
                     unsigned long long *status, int *ticket, int64_t ntiles, uint64_t *Kout, void *Vout, int *flag,
                     int spin_limit, long long withhold, cudaStream_t st);
-void launch_sp_heads(const uint64_t *K, int64_t nnz, int64_t *theads, int64_t ntiles, cudaStream_t st);
+int64_t sp_chunks(int64_t nnz);  // run heads are counted by chunks
+void launch_sp_heads(const uint64_t *K, int64_t nnz, int64_t *theads, cudaStream_t st);
 // op: 0 (+) f64, 1 (+) f32, 2 (+) i64, 3 min f32, 4 min i32, 5 structure only
 void launch_sp_emit(int op, const uint64_t *K, const void *V, int64_t nnz, int nbj, const int64_t *theads_incl,
-                    int64_t ntiles, int32_t *Cidx, void *Cval, int64_t *rowcnt, int64_t *longlist, int *nlong,
-                    cudaStream_t st);
+                    int32_t *Cidx, void *Cval, int64_t *rowcnt, int64_t *longlist, int *nlong, cudaStream_t st);
 void launch_rows_from_pos(const int32_t *pos, int64_t m, int64_t *cnt, cudaStream_t st);
 void launch_fill_from_pos(const int32_t *pos, int64_t m, const int64_t *ptr, int32_t *out, cudaStream_t st);
 void launch_iota_i64(int64_t *p, int64_t n, cudaStream_t st);

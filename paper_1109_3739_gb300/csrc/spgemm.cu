@@ -1162,7 +1162,8 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
   if (passes > sp_max_passes()) return HS_EINTERNAL;
   const int64_t tiles = sp_tiles(nnz);
   const int64_t longcap = sp_long_capacity(nnz);
-  const int64_t scan_n = tiles > m + 1 ? tiles : m + 1;
+  const int64_t chunks = sp_chunks(nnz);
+  const int64_t scan_n = chunks > m + 1 ? chunks : m + 1;
   uint64_t *kbuf[2] = {mem.tmp<uint64_t>((size_t)nnz), mem.tmp<uint64_t>((size_t)nnz)};
   void *vbuf[2] = {nullptr, nullptr};
   if (vb) {
@@ -1172,7 +1173,7 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
   unsigned long long *status = mem.tmp<unsigned long long>((size_t)(tiles << rb));
   unsigned long long *ghist = mem.tmp<unsigned long long>((size_t)passes << rb);
   int *ticket = mem.tmp<int>((size_t)passes);
-  int64_t *theads = mem.tmp<int64_t>((size_t)tiles);
+  int64_t *theads = mem.tmp<int64_t>((size_t)chunks);
   int64_t *scan_tmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(scan_n));
   int64_t *longlist = vb ? mem.tmp<int64_t>((size_t)(2 * longcap)) : nullptr;
   int *flags = mem.tmp<int>(2);  // [0] index out of range, [1] long runs
@@ -1200,11 +1201,11 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
                      kbuf[out], vbuf[out], flags, spin, withhold, st);
       cur = out;
     }
-    launch_sp_heads(kbuf[cur], nnz, theads, tiles, st);
-    launch_scan_i64(theads, tiles, scan_tmp, st);
+    launch_sp_heads(kbuf[cur], nnz, theads, st);
+    launch_scan_i64(theads, chunks, scan_tmp, st);
   }
   if (int e = check_launch()) return e;
-  CK(cudaMemcpyAsync(host, theads + tiles - 1, 8, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(host, theads + chunks - 1, 8, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(host + 1, flags, 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   const int fl = *(int *)(host + 1);
@@ -1217,8 +1218,7 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
   if (!C->idx || (vb && !C->val)) return HS_ENOMEM;
   {
     PhaseTimer t("sparse_emit", st);
-    launch_sp_emit(op, kbuf[cur], vbuf[cur], nnz, nbj, theads, tiles, C->idx, C->val, C->ptr, longlist,
-                   flags + 1, st);
+    launch_sp_emit(op, kbuf[cur], vbuf[cur], nnz, nbj, theads, C->idx, C->val, C->ptr, longlist, flags + 1, st);
     launch_scan_i64(C->ptr, m + 1, scan_tmp, st);
   }
   return check_launch();
