@@ -780,7 +780,8 @@ __global__ void k_plan_parts(RowSet A, const int *list, int count, const int32_t
       // a part must lie inside its row (else pc 0: the numeric kernel rejects the unit)
       const bool fits = HS_G(A.dbg, done + pc <= c, 74, done);
       if (base + p < end)
-        units[base + p] = HeavyUnit{r, s0, s1, fits ? pc : 0, done, pbase + p * nq, 0, 0, cb + done, lb + done};
+        units[base + p] = HeavyUnit{r, s0, s1, fits ? pc : 0, done, pbase + p * nq, 0, 0, cb + done,
+                                    lb + (lb & LIST_BITS ? (long long)s0 * (SEG_W / 32) : done)};
     });
   }
 }

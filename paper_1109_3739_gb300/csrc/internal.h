@@ -44,6 +44,9 @@ constexpr int CAP_MID_S = 1024, CAP_MID = 2048;
 // Column segments recorded for rows that may need column parts: width SEG_W
 // (a multiple of 1024, at most every numeric table's capacity).
 constexpr int SEG_W = 4096;
+// In an entry of loff: the row's room in the pool holds its bitmap over all of
+// B's columns (a word per 32), not its sorted columns.
+constexpr int64_t LIST_BITS = (int64_t)1 << 62;
 constexpr int HV_SPAN_SEGS = 64;      // segments a heavy column part spans at most (2^18 columns)
 constexpr int HU_SPAN_SEGS = 32;      // the same for the parts of the unit kernel (2^17 columns)
 constexpr int BITMAP_COLS = 1 << 20;  // columns covered by the heavy symbolic bitmap
@@ -245,6 +248,7 @@ struct SymArgs {
   unsigned long long *lpool;  // pool cursor (entries handed out)
   int64_t lcap;
   int tiny_group;          // tiny rows several to a warp
+  int64_t bits_min;        // rows of at least this many outputs leave their bitmap instead of a list
 };
 void launch_sym_tiny(const SymArgs &a, cudaStream_t st);
 void launch_sym_warp(const SymArgs &a, cudaStream_t st);
@@ -270,7 +274,7 @@ struct alignas(16) HeavyUnit {
   int32_t npairs;  // A entries with products in the part (the slice's used length)
   int32_t pad;
   int64_t out;     // position in C of the part's first entry (C's row offset + done)
-  int64_t lofs;    // position of the part's first column in the sorted-list pool
+  int64_t lofs;    // position of the part's first column, or with LIST_BITS of its first bitmap word, in the pool
 };
 // outputs a heavy column part holds at most, by value width (the part's
 // values live in shared memory)

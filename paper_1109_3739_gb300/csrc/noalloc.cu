@@ -210,7 +210,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
     NA_CK(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)nhist * nseg, st));
   }
 
-  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, nullptr, nullptr, nullptr, 0, tiny_group};
+  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, nullptr, nullptr, nullptr, 0, tiny_group, INT64_MAX};
   auto sym_bin = [&](int k0, int k1) {
     sa.list = list + key_off[k0];
     sa.count = key_off[k1] - key_off[k0];

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NT, 1) k_num_cta(NumArgs a) {
     cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
                           [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
     const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
-    if (lofs >= 0) {
+    if (lofs >= 0 && !(lofs & LIST_BITS)) {
       // the symbolic pass left the row's sorted columns: no sort, each
       // column's value is looked up in the table
       const int32_t *Lr = a.glist + lofs;
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(HV_NT, 2) k_num_heavy(NumArgs a) {
     const bool cached = nrounds == 1;
     // the row's sorted column list left by the symbolic pass, if any
     const int64_t lofs = (r_ok && a.loff && a.glist) ? a.loff[r] : -1;
-    const int32_t *L = lofs >= 0 ? a.glist + lofs : nullptr;
+    const int32_t *L = lofs >= 0 && !(lofs & LIST_BITS) ? a.glist + lofs : nullptr;
     if (L && tid == 0) prefetch_l2(L, c * 4);  // the row's parts read it in order
     if (cached) {
       const int cnt = (int)(q1 - q0);
@@ -837,6 +837,7 @@ __global__ void __launch_bounds__(HV_NT, 2) k_num_heavy(NumArgs a) {
 constexpr int HU_NT = 256;
 constexpr int HU_WMAX = HU_SPAN_SEGS * SEG_W;
 constexpr int HU_WORDS = HU_WMAX / 32;
+static_assert(HU_WORDS / 256 + 1 <= 32, "a thread's run of words has a bit each");
 constexpr int HU_PB = 256;  // B segments copied per batch
 static_assert(HU_PB == HU_NT, "a segment per thread in the batch's scan");
 // as unit_part_cap(): KB kilobytes of values, at least one segment's SEG_W outputs
@@ -850,7 +851,7 @@ template <typename T, int KB> struct UnitSmem {
   // plus the copy's 32 bytes of alignment room)
   static constexpr size_t VBYTES = ((size_t)CAP * (vbytes<T>() > 4 ? vbytes<T>() : 4) + 32 + 15) & ~(size_t)15;
   alignas(16) unsigned char vals_raw[VBYTES];
-  alignas(16) unsigned bitmap[HU_WORDS];  // all zero at every unit's start
+  alignas(16) unsigned bitmap[HU_WORDS + 8];  // all zero at every unit's start (+ copy room)
   alignas(16) int64_t seg[HU_PB + 4];    // B segments as they were laid out (+ copy room), then their starts
   int excl[HU_PB + 1];                   // their product prefix, then the batch's total
   alignas(16) unsigned char aval_raw[(HU_PB + 4) * (vbytes<T>() > 4 ? 8 : 4) + 16];
@@ -874,7 +875,7 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
   long long *dbg = a.A.dbg;
   if constexpr (SR::has_val)
-    for (int w = tid; w < HU_WORDS; w += HU_NT) sm.bitmap[w] = 0u;
+    for (int w = tid; w < HU_WORDS + 8; w += HU_NT) sm.bitmap[w] = 0u;
   if (tid == 0) sm.unit = atomicAdd(a.udyn, 1);
   __syncthreads();
   while (true) {
@@ -896,12 +897,15 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
       const int lo = u.seg_lo * SEG_W;
       const int hi = (int)min((int64_t)u.seg_hi * SEG_W, n);
       const int pc = u.pc;
-      const int32_t *Lp = a.glist + u.lofs;
+      const bool as_bits = (u.lofs & LIST_BITS) != 0;
+      const int32_t *Lp = a.glist + (u.lofs & ~LIST_BITS);
       const int64_t out = u.out;
       if constexpr (SR::has_val) {
         // the list slice and the first batch of B segments, copied at once
         const int nb0 = u.npairs < HU_PB ? u.npairs : HU_PB;
-        const int lofb = async_copy16(sm.vals_raw, Lp, (int64_t)pc * 4, tid, HU_NT) >> 2;
+        const int words = (hi - lo + 31) >> 5;
+        const int lofb = as_bits ? async_copy16(sm.bitmap, Lp, (int64_t)words * 4, tid, HU_NT) >> 2
+                                 : async_copy16(sm.vals_raw, Lp, (int64_t)pc * 4, tid, HU_NT) >> 2;
         const int sofb = async_copy16(sm.seg, a.pseg + u.poff, (int64_t)nb0 * 8, tid, HU_NT) >> 3;
         int aofb = 0;
         if constexpr (SR::needs_a)
@@ -909,22 +913,67 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
                               (int64_t)nb0 * sizeof(T), tid, HU_NT) / (int)sizeof(T);
         async_copy_wait();
         __syncthreads();
+        unsigned *bitmap = sm.bitmap + (as_bits ? lofb : 0);
+        if (as_bits) {
+          // a thread counts a run of words (an odd number, which keeps the
+          // lanes on different banks), then ranks them and walks their columns
+          // into the values' room, which they leave in one coalesced piece
+          const int wpt = ((words + HU_NT - 1) / HU_NT) | 1;
+          const int wb = min(words, tid * wpt), we = min(words, wb + wpt);
+          int cnt = 0;
+          unsigned full = 0u;  // the run's non-empty words
+#pragma unroll 4
+          for (int k = 0; k < wpt; ++k) {
+            const unsigned b = wb + k < we ? bitmap[wb + k] : 0u;
+            cnt += __popc(b);
+            full |= (unsigned)(b != 0u) << k;
+          }
+          const int incl = warp_incl_scan(cnt);
+          if (lane == 31) sm.wtmp[tid >> 5] = incl;
+          __syncthreads();
+          int at = incl - cnt, total = 0;
+#pragma unroll
+          for (int w = 0; w < HU_NT / 32; ++w) {
+            const int x = sm.wtmp[w];
+            at += w < (tid >> 5) ? x : 0;
+            total += x;
+          }
+          int32_t *cols = reinterpret_cast<int32_t *>(sm.vals_raw);
+          const bool same = total == pc;  // (uniform)
+          if (!same && tid == 0) atomicExch(a.err, 9);
+          unsigned cur = 0u;
+          int c0 = 0;
+          for (int k = 0; k < cnt && same; ++k) {  // a column an iteration; the next non-empty word when one is spent
+            if (cur == 0u) {
+              const int w = wb + __ffs(full) - 1;
+              full &= full - 1;
+              cur = bitmap[w];
+              c0 = lo + (w << 5) - 1;
+              sm.wpre[w] = (uint16_t)(at + k);
+            }
+            cols[at + k] = c0 + __ffs(cur);
+            cur &= cur - 1;
+          }
+          __syncthreads();
+          if (same)
+            for (int i = tid; i < pc; i += HU_NT) __stcs(a.Cj + out + i, cols[i]);
+        }
         // columns out, bits and word ranks in (entry i starts word w when
         // entry i-1 lies in another word)
         const int32_t *Ls = reinterpret_cast<const int32_t *>(sm.vals_raw) + lofb;
-        for (int i = tid; i < pc; i += HU_NT) {
+        for (int i = as_bits ? pc : tid; i < pc; i += HU_NT) {
           const int col = Ls[i];
           __stcs(a.Cj + out + i, col);
           const int xx = col - lo;
           if (!HS_G(dbg, xx >= 0 && xx < hi - lo, 63, col)) continue;
           const int w = xx >> 5;
-          atomicOr(sm.bitmap + w, 1u << (xx & 31));
+          atomicOr(bitmap + w, 1u << (xx & 31));
           if (i == 0 || ((Ls[i - 1] - lo) >> 5) != w) sm.wpre[w] = (uint16_t)i;
         }
         if (tid == 0 && nxt < a.nunits) prefetch_l2(a.units + nxt, sizeof(HeavyUnit));
         __syncthreads();  // the list slice is read: its room becomes the values
         for (int i = tid; i < pc; i += HU_NT) vals[i] = SR::identity();
-        HeavyAdd<SR> add_val{sm.bitmap, sm.wpre, vals, lo, (unsigned)(hi - lo), pc, a.err, dbg};
+        HeavyAdd<SR> add_val{bitmap, sm.wpre, vals, lo, (unsigned)(hi - lo), pc, a.err, dbg};
         for (int pb = 0; pb < u.npairs; pb += HU_PB) {
           const int nb = min(HU_PB, u.npairs - pb);
           int so = sofb, ao = aofb;
@@ -960,8 +1009,8 @@ __global__ void __launch_bounds__(HU_NT, (KB > 16 || vbytes<typename SR::val_t>(
         __syncthreads();
         // values in column order; the part's bitmap words cleared for the next unit
         for (int i = tid; i < pc; i += HU_NT) __stcs(Cv + out + i, vals[i]);
-        const int words = (hi - lo + 31) >> 5;
-        for (int w = tid; w < words; w += HU_NT) sm.bitmap[w] = 0u;
+        const int used = words + (as_bits ? 8 : 0);
+        for (int w = tid; w < used; w += HU_NT) sm.bitmap[w] = 0u;
       } else {
         // structure only: the list slice is the part's columns
         for (int i = tid; i < pc; i += HU_NT) __stcs(a.Cj + out + i, __ldg(Lp + i));

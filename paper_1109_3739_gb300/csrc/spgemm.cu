@@ -681,7 +681,19 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   };
 
   // ---- symbolic
-  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, glist, loff, &sb->lpool, lcap, tiny_group};
+  // Rows whose values will be added up by units, and with an output for every
+  // second bitmap word or more, leave the bitmap: writing and reading 128 KB
+  // (2^20 columns) costs no more bytes than the list of 16,384 outputs or
+  // more, the units need the bits anyway, and the columns are walked out of
+  // them where five CTAs share an SM instead of one (R-MAT scale 20: the
+  // symbolic rows 23.7 -> 20.4 ms, the units 32.5 -> 33.6 ms; twice or a third of
+  // this line measured the same).  Without values
+  // the units only copy the list.
+  const int64_t half_words = (n + 63) / 64;
+  const int64_t bits_min = !vb ? INT64_MAX
+                               : (half_words > bins.num_heavy_from + 1 ? half_words : (int64_t)bins.num_heavy_from + 1);
+  SymArgs sa{rs, rb, f, nullptr, 0, Cp, hslot, hist, nseg, &sb->dyn[0], &sb->err, glist, loff, &sb->lpool, lcap, tiny_group,
+             bits_min};
   {
     struct SymBin {
       const char *name;

@@ -372,6 +372,7 @@ __global__ void __launch_bounds__(NT, SH_NT / NT) k_sym_heavy(SymArgs a) {
     int32_t *lst = nullptr;  // the row's list, once its room is taken (first chunk)
     const int64_t lmax = r_ok ? min(a.f[r], n) : 0;  // the list's room: min(f, n) entries bound its output
     int64_t written = 0;  // columns of the earlier chunks
+    bool as_bits = false;
     for (int ch = 0; ch < (r_ok ? nchunk : 0); ++ch) {
       const int lo = ch * SH_COLS;
       const int hi = (int)min((int64_t)lo + SH_COLS, n);
@@ -433,6 +434,21 @@ __global__ void __launch_bounds__(NT, SH_NT / NT) k_sym_heavy(SymArgs a) {
       }
       __syncthreads();
       const int ctotal = sm.scnt[SH_SEGS];
+      // a row that is dense enough leaves its bitmap as it is, if its room in the pool holds it
+      as_bits = lst && nchunk == 1 && ctotal >= a.bits_min && lmax >= words;
+      if (as_bits) {
+        for (int w0 = threadIdx.x; w0 < words; w0 += 4 * NT) {
+          unsigned x[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[u] = w0 + u * NT < words ? sm.bitmap[w0 + u * NT] : 0u;
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (w0 + u * NT < words) {
+              __stcs(lst + w0 + u * NT, (int32_t)x[u]);
+              sm.bitmap[w0 + u * NT] = 0u;
+            }
+        }
+      }
       // list: the same pairs, read again (a row that found no room in the
       // pool only clears them)
       if (!lst && a.glist) {
@@ -442,7 +458,7 @@ __global__ void __launch_bounds__(NT, SH_NT / NT) k_sym_heavy(SymArgs a) {
           if (g < nsc) sh_clear8(sm.bitmap, g * (SEG_W / 32) + 8 * lane, words);
         }
       }
-      if (lst) {
+      if (lst && !as_bits) {
 #pragma unroll
         for (int i = 0; i < SH_PPW; ++i) {
           const int g = 2 * (warp + nw * i);
@@ -529,7 +545,7 @@ __global__ void __launch_bounds__(NT, SH_NT / NT) k_sym_heavy(SymArgs a) {
     }
     if (threadIdx.x == 0 && r_ok) {
       put_count(a, out_row(a.A, r), written);
-      if (a.loff) a.loff[r] = lst ? sm.loff : -1;
+      if (a.loff) a.loff[r] = lst ? sm.loff | (as_bits ? LIST_BITS : 0) : -1;
     }
     __syncthreads();
   }
