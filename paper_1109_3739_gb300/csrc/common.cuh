@@ -1039,16 +1039,19 @@ __device__ __forceinline__ void hash_insert_val(int *keys, T *vals, unsigned mas
 // ----------------------------------------------------------- sorted emit
 // Shared-memory layout used by group_sort_emit (all offsets in bytes):
 //   ck[cap] int32 | cv[cap] T           (compacted entries, arbitrary order)
-//   work: bcnt[nb] int32 | order[c] int32 | sk[c] int32 | sv[c] T
+//   work: bcnt[nb] int32 | sk[c] int32 | sv[c] T
 // `work` may alias the hash table (it is free once compacted).
 //
 // Steps: (1) every occupied slot of the table is appended to ck/cv, and the
 // key range [kmin, kmax] is found; (2) keys are distributed over nb buckets
 // by the monotone map b = (key-kmin)*nb/(kmax-kmin+1); a histogram and an
-// exclusive scan give every bucket its start; (3) entry e's final position
-// is its bucket's start plus the number of keys in the same bucket that are
-// smaller (keys are distinct), so the row leaves in ascending column order;
-// (4) the sorted row is written to global memory with coalesced stores.
+// exclusive scan give every bucket its start, and the entries are put into
+// their buckets; (3) an entry's final position is its bucket's start plus the
+// number of keys in the bucket that are smaller (keys are distinct).  Rows of
+// 2048..4096 entries spent half of their time on (3) when it ran over the
+// unsorted entries, with ids in the buckets and the sorted row gathered in
+// shared memory, every lane through a loop of its own length: R-MAT scale 20,
+// these rows 5.04 -> 4.35 ms, those of 1024..2048 entries 2.56 -> 2.20 ms.
 struct EmitScratch {
   int kmin, kmax, count;
 };
@@ -1061,7 +1064,7 @@ __host__ __device__ __forceinline__ int emit_buckets(int c) {
 }
 // bytes of the `work` region for c entries with values of `vbytes` bytes
 __host__ __device__ __forceinline__ size_t emit_work_bytes(int c, int vbytes) {
-  return ((((size_t)(emit_buckets(c) + 2 * c) * 4 + 7) & ~(size_t)7)) + (size_t)c * vbytes;
+  return ((((size_t)(emit_buckets(c) + c) * 4 + 7) & ~(size_t)7)) + (size_t)c * vbytes;
 }
 
 template <class G, typename T, bool HAS_VAL>
@@ -1086,27 +1089,39 @@ __device__ void group_sort_emit(const int *keys, const T *vals, int slots, int c
     const int nw = G::nwarps(), w = G::warp();
     const int per = ((slots + nw - 1) / nw + 31) & ~31;
     const int s0 = min(slots, w * per), s1 = min(slots, s0 + per);
+    constexpr int CU = 4;  // slots per lane per step: their reads overlap
     int n = 0;
-    for (int sb = s0; sb < s1; sb += 32) n += __popc(__ballot_sync(FULL, sb + lane < s1 && keys[sb + lane] != EMPTY));
+    for (int sb = s0; sb < s1; sb += 32 * CU) {
+      int k[CU];
+#pragma unroll
+      for (int u = 0; u < CU; ++u) k[u] = sb + 32 * u + lane < s1 ? keys[sb + 32 * u + lane] : EMPTY;
+#pragma unroll
+      for (int u = 0; u < CU; ++u) n += k[u] != EMPTY;
+    }
+    n = warp_sum(n);
     int base = 0;
     if (lane == 0 && n) base = atomicAdd(&es->count, n);
     base = __shfl_sync(FULL, base, 0);
     int lmin = 0x7fffffff, lmax = -1;
-    for (int sb = s0; sb < s1; sb += 32) {
-      const int sl = sb + lane;
-      const int k = sl < s1 ? keys[sl] : EMPTY;
-      const bool occ = k != EMPTY;
-      const unsigned m = __ballot_sync(FULL, occ);
-      if (occ) {
-        const int at = base + __popc(m & ((1u << lane) - 1));
-        if (at < c) {
-          ck[at] = k;
-          if constexpr (HAS_VAL) cv[at] = vals[sl];
+    for (int sb = s0; sb < s1; sb += 32 * CU) {
+      int k[CU];
+#pragma unroll
+      for (int u = 0; u < CU; ++u) k[u] = sb + 32 * u + lane < s1 ? keys[sb + 32 * u + lane] : EMPTY;
+#pragma unroll
+      for (int u = 0; u < CU; ++u) {
+        const bool occ = k[u] != EMPTY;
+        const unsigned m = __ballot_sync(FULL, occ);
+        if (occ) {
+          const int at = base + __popc(m & ((1u << lane) - 1));
+          if (at < c) {
+            ck[at] = k[u];
+            if constexpr (HAS_VAL) cv[at] = vals[sb + 32 * u + lane];
+          }
+          lmin = min(lmin, k[u]);
+          lmax = max(lmax, k[u]);
         }
-        lmin = min(lmin, k);
-        lmax = max(lmax, k);
+        base += __popc(m);
       }
-      base += __popc(m);
     }
     lmin = warp_min(lmin);
     lmax = warp_max(lmax);
@@ -1131,9 +1146,8 @@ __device__ void group_sort_emit(const int *keys, const T *vals, int slots, int c
   // (2) buckets
   const int nb = emit_buckets(c);
   int *bcnt = reinterpret_cast<int *>(work);
-  int *order = bcnt + nb;
-  int *sk = order + c;
-  T *sv = reinterpret_cast<T *>(reinterpret_cast<char *>(work) + (((size_t)(nb + 2 * c) * 4 + 7) & ~(size_t)7));
+  int *sk = bcnt + nb;
+  T *sv = reinterpret_cast<T *>(reinterpret_cast<char *>(work) + (((size_t)(nb + c) * 4 + 7) & ~(size_t)7));
   const int kmin = es->kmin;
   const uint64_t range = (uint64_t)(es->kmax - kmin) + 1;
   // monotone bucket map b = floor((key-kmin) * scale / 2^32), scale = floor(nb*2^32/range) < 2^32*nb/range
@@ -1147,58 +1161,66 @@ __device__ void group_sort_emit(const int *keys, const T *vals, int slots, int c
   }
   G::sync();
   group_excl_scan<G>(bcnt, nb, wtmp);
-  // scatter entry ids into their buckets (arbitrary order inside a bucket);
-  // bcnt[b] advances to the bucket's end, so the start is bcnt[b] - size
+  // the entries into their buckets (arbitrary order inside a bucket); bcnt[b]
+  // advances to the bucket's end
   for (int e0 = r; e0 < c; e0 += EU * gs) {
-    int b[EU], at[EU];
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      const int e = e0 + u * gs;
-      b[u] = e < c ? bucket(ck[e]) : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      at[u] = -1;
-      if (b[u] >= 0 && HS_G(dbg, b[u] < nb, 22, b[u])) at[u] = atomicAdd(bcnt + b[u], 1);
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u)
-      if (at[u] >= 0 && HS_G(dbg, at[u] < c, 23, at[u])) order[at[u]] = e0 + u * gs;
-  }
-  G::sync();
-  // (3) rank inside the bucket: bucket b spans [end(b-1), end(b))
-  for (int e0 = r; e0 < c; e0 += EU * gs) {
-    int key[EU], bs[EU], be[EU], rank[EU];
-    T v[EU];
+    int key[EU], at[EU];
 #pragma unroll
     for (int u = 0; u < EU; ++u) {
       const int e = e0 + u * gs;
       key[u] = e < c ? ck[e] : 0;
-      if constexpr (HAS_VAL) v[u] = e < c ? cv[e] : T{};
     }
 #pragma unroll
     for (int u = 0; u < EU; ++u) {
-      const int b = e0 + u * gs < c ? bucket(key[u]) : 0;
-      bs[u] = b ? bcnt[b - 1] : 0;
-      be[u] = e0 + u * gs < c ? bcnt[b] : 0;
-      rank[u] = bs[u];
+      at[u] = -1;
+      const int b = e0 + u * gs < c ? bucket(key[u]) : -1;
+      if (b >= 0 && HS_G(dbg, b < nb, 22, b)) at[u] = atomicAdd(bcnt + b, 1);
     }
 #pragma unroll
     for (int u = 0; u < EU; ++u)
-      for (int t = bs[u]; t < be[u]; ++t)
-        if (HS_G(dbg, t >= 0 && t < c && order[t] >= 0 && order[t] < c, 24, t)) rank[u] += ck[order[t]] < key[u];
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      if (e0 + u * gs >= c || !HS_G(dbg, rank[u] >= 0 && rank[u] < c, 25, rank[u])) continue;
-      sk[rank[u]] = key[u];
-      if constexpr (HAS_VAL) sv[rank[u]] = v[u];
-    }
+      if (at[u] >= 0 && HS_G(dbg, at[u] < c, 23, at[u])) {
+        sk[at[u]] = key[u];
+        if constexpr (HAS_VAL) sv[at[u]] = cv[e0 + u * gs];
+      }
   }
   G::sync();
-  // (4) coalesced stores, evict-first: C is not read again here, B is
-  for (int e = r; e < c; e += gs) {
-    __stcs(out_j + e, sk[e]);
-    if constexpr (HAS_VAL) __stcs(out_v + e, sv[e]);
+  // (3) position i's entry goes out at its bucket's start plus the number of
+  // smaller keys in the bucket, a place or two from i: the lanes read the same
+  // few words and their stores (evict-first: C is not read again here, B is)
+  // fall into the same lines
+  for (int w0 = r - lane; w0 < c; w0 += EU * gs) {  // (whole warps)
+    int key[EU], bs[EU], len[EU], rank[EU];
+    T v[EU];
+    int most = 0;
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      const int i = w0 + lane + u * gs;
+      key[u] = i < c ? sk[i] : kmin;
+      if constexpr (HAS_VAL) v[u] = i < c ? sv[i] : T{};
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      const int b = bucket(key[u]);
+      bs[u] = b ? bcnt[b - 1] : 0;
+      len[u] = w0 + lane + u * gs < c ? bcnt[b] - bs[u] : 0;
+      if (!HS_G(dbg, bs[u] >= 0 && bs[u] + len[u] <= c, 24, bs[u])) len[u] = 0;
+      rank[u] = bs[u];
+      most = max(most, len[u]);
+    }
+    // every lane as many steps as the warp's largest bucket asks for: loops of
+    // their own lengths left the lanes one behind the other
+    most = warp_max(most);
+    for (int t = 0; t < most; ++t) {
+#pragma unroll
+      for (int u = 0; u < EU; ++u) rank[u] += t < len[u] && sk[bs[u] + t] < key[u];
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      if (len[u] > 0) {
+        __stcs(out_j + rank[u], key[u]);
+        if constexpr (HAS_VAL) __stcs(out_v + rank[u], v[u]);
+      }
+    }
   }
   G::sync();
 }
