@@ -250,6 +250,12 @@ template <class V> struct two_stage<V, std::void_t<decltype(V::kTwoStage)>> : st
 template <typename T> __device__ __forceinline__ T shfl_val(T x, int src) { return __shfl_sync(FULL, x, src); }
 template <> __device__ __forceinline__ NoVal shfl_val<NoVal>(NoVal x, int) { return x; }
 
+// Visitors that want a product's index in its row: batch() is told how many
+// products of the round come before those of the next warp_expand, round() how
+// many the round had.
+template <class V, class = void> struct flat_visit : std::false_type {};
+template <class V> struct flat_visit<V, std::enable_if_t<V::kFlat>> : std::true_type {};
+
 // Visit the products of up to 32 B-row segments (one per lane: start s,
 // length len, left value a).  Segments of at least 32 products are walked by
 // the whole warp, one segment at a time, with consecutive lanes on
@@ -850,6 +856,10 @@ __device__ __forceinline__ void cta_expand_staged(const DevCsr &B, const int64_t
     int64_t s = 0;
     int len = 0;
     T a{};
+    if constexpr (flat_visit<std::decay_t<Visit>>::value) {  // products of the round before this batch
+      const int64_t ahead = pb - (excl[eb] - ebase + (int64_t)K * eb + K);
+      visit.batch(excl[eb] - ebase + (int)min(max(ahead, (int64_t)0), (int64_t)(excl[eb + 1] - excl[eb])));
+    }
     if (e < n) {
       const int64_t x0 = excl[e] - ebase + (int64_t)K * e + K, x1 = excl[e + 1] - ebase + (int64_t)K * (e + 1);
       const int64_t cb = max(x0, pb), ce = min(x1, pe);
@@ -974,6 +984,7 @@ __device__ __forceinline__ void cta_products(const DevCsr &A, const DevCsr &B, i
     // only the staged entries are scanned (a short row costs what it holds)
     const int total = group_excl_scan<CtaGroup>(sm.excl, n + 1, wtmp);
     cta_expand_staged<SR, U, 32>(B, sm.sbeg, sm.excl, sm.aval, n, total, visit);
+    if constexpr (flat_visit<std::decay_t<Visit>>::value) visit.round(total);
     __syncthreads();
   }
 }
@@ -1067,11 +1078,99 @@ __host__ __device__ __forceinline__ size_t emit_work_bytes(int c, int vbytes) {
   return ((((size_t)(emit_buckets(c) + c) * 4 + 7) & ~(size_t)7)) + (size_t)c * vbytes;
 }
 
+// Steps (2) and (3): out(place, key, value) for the c entries of ck/cv.  DUPS:
+// keys may be equal, and then keep some order among themselves; out may write
+// to ck/cv, which are not read any more.
+template <class G, typename T, bool HAS_VAL, bool DUPS, class Out>
+__device__ __forceinline__ void group_bucket_sort(const int *ck, const T *cv, int c, int kmin, int kmax, void *work,
+                                                  int *wtmp, long long *dbg, Out &&out) {
+  constexpr int EU = 4;  // entries per thread per step: their shared-memory chains overlap
+  const int gs = G::size(), r = G::rank(), lane = lane_id();
+  const int nb = emit_buckets(c);
+  int *bcnt = reinterpret_cast<int *>(work);
+  int *sk = bcnt + nb;
+  T *sv = reinterpret_cast<T *>(reinterpret_cast<char *>(work) + (((size_t)(nb + c) * 4 + 7) & ~(size_t)7));
+  const uint64_t range = (uint64_t)(kmax - kmin) + 1;
+  // monotone bucket map b = floor((key-kmin) * scale / 2^32), scale = floor(nb*2^32/range) < 2^32*nb/range
+  const uint64_t scale = (((uint64_t)nb) << 32) / range;
+  auto bucket = [&](int key) { return (int)(((uint64_t)(unsigned)(key - kmin) * scale) >> 32); };
+  for (int b = r; b < nb; b += gs) bcnt[b] = 0;
+  G::sync();
+  for (int e = r; e < c; e += gs) {
+    const int b = bucket(ck[e]);
+    if (HS_G(dbg, b >= 0 && b < nb, 21, b)) atomicAdd(bcnt + b, 1);
+  }
+  G::sync();
+  group_excl_scan<G>(bcnt, nb, wtmp);
+  // the entries into their buckets (arbitrary order inside a bucket); bcnt[b]
+  // advances to the bucket's end
+  for (int e0 = r; e0 < c; e0 += EU * gs) {
+    int key[EU], at[EU];
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      const int e = e0 + u * gs;
+      key[u] = e < c ? ck[e] : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      at[u] = -1;
+      const int b = e0 + u * gs < c ? bucket(key[u]) : -1;
+      if (b >= 0 && HS_G(dbg, b < nb, 22, b)) at[u] = atomicAdd(bcnt + b, 1);
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u)
+      if (at[u] >= 0 && HS_G(dbg, at[u] < c, 23, at[u])) {
+        sk[at[u]] = key[u];
+        if constexpr (HAS_VAL) sv[at[u]] = cv[e0 + u * gs];
+      }
+  }
+  G::sync();
+  // (3) position i's entry goes out at its bucket's start plus the number of
+  // smaller keys in the bucket, a place or two from i: the lanes read the same
+  // few words and their stores (evict-first: C is not read again here, B is)
+  // fall into the same lines
+  for (int w0 = r - lane; w0 < c; w0 += EU * gs) {  // (whole warps)
+    int key[EU], bs[EU], len[EU], rank[EU];
+    T v[EU];
+    int most = 0;
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      const int i = w0 + lane + u * gs;
+      key[u] = i < c ? sk[i] : kmin;
+      if constexpr (HAS_VAL) v[u] = i < c ? sv[i] : T{};
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      const int b = bucket(key[u]);
+      bs[u] = b ? bcnt[b - 1] : 0;
+      len[u] = w0 + lane + u * gs < c ? bcnt[b] - bs[u] : 0;
+      if (!HS_G(dbg, bs[u] >= 0 && bs[u] + len[u] <= c, 24, bs[u])) len[u] = 0;
+      rank[u] = bs[u];
+      most = max(most, len[u]);
+    }
+    // every lane as many steps as the warp's largest bucket asks for: loops of
+    // their own lengths left the lanes one behind the other
+    most = warp_max(most);
+    for (int t = 0; t < most; ++t) {
+#pragma unroll
+      for (int u = 0; u < EU; ++u) {
+        const int k = t < len[u] ? sk[bs[u] + t] : 0x7fffffff;
+        rank[u] += k < key[u] || (DUPS && k == key[u] && bs[u] + t < w0 + lane + u * gs);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < EU; ++u) {
+      if (len[u] > 0) {
+        out(rank[u], key[u], v[u]);
+      }
+    }
+  }
+}
+
 template <class G, typename T, bool HAS_VAL>
 __device__ void group_sort_emit(const int *keys, const T *vals, int slots, int c, int *ck, T *cv,
                                 void *work, int *wtmp, EmitScratch *es, int32_t *out_j, T *out_v,
                                 int *err, int cap, long long *dbg, bool unsorted = false) {
-  constexpr int EU = 4;  // entries per thread per step: their shared-memory chains overlap
   const int gs = G::size(), r = G::rank(), lane = lane_id();
   if (!HS_G(dbg, c >= 0 && c <= cap, 20, c)) {
     if (r == 0) atomicExch(err, 8);
@@ -1143,85 +1242,10 @@ __device__ void group_sort_emit(const int *keys, const T *vals, int slots, int c
     }
     return;
   }
-  // (2) buckets
-  const int nb = emit_buckets(c);
-  int *bcnt = reinterpret_cast<int *>(work);
-  int *sk = bcnt + nb;
-  T *sv = reinterpret_cast<T *>(reinterpret_cast<char *>(work) + (((size_t)(nb + c) * 4 + 7) & ~(size_t)7));
-  const int kmin = es->kmin;
-  const uint64_t range = (uint64_t)(es->kmax - kmin) + 1;
-  // monotone bucket map b = floor((key-kmin) * scale / 2^32), scale = floor(nb*2^32/range) < 2^32*nb/range
-  const uint64_t scale = (((uint64_t)nb) << 32) / range;
-  auto bucket = [&](int key) { return (int)(((uint64_t)(unsigned)(key - kmin) * scale) >> 32); };
-  for (int b = r; b < nb; b += gs) bcnt[b] = 0;
-  G::sync();
-  for (int e = r; e < c; e += gs) {
-    const int b = bucket(ck[e]);
-    if (HS_G(dbg, b >= 0 && b < nb, 21, b)) atomicAdd(bcnt + b, 1);
-  }
-  G::sync();
-  group_excl_scan<G>(bcnt, nb, wtmp);
-  // the entries into their buckets (arbitrary order inside a bucket); bcnt[b]
-  // advances to the bucket's end
-  for (int e0 = r; e0 < c; e0 += EU * gs) {
-    int key[EU], at[EU];
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      const int e = e0 + u * gs;
-      key[u] = e < c ? ck[e] : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      at[u] = -1;
-      const int b = e0 + u * gs < c ? bucket(key[u]) : -1;
-      if (b >= 0 && HS_G(dbg, b < nb, 22, b)) at[u] = atomicAdd(bcnt + b, 1);
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u)
-      if (at[u] >= 0 && HS_G(dbg, at[u] < c, 23, at[u])) {
-        sk[at[u]] = key[u];
-        if constexpr (HAS_VAL) sv[at[u]] = cv[e0 + u * gs];
-      }
-  }
-  G::sync();
-  // (3) position i's entry goes out at its bucket's start plus the number of
-  // smaller keys in the bucket, a place or two from i: the lanes read the same
-  // few words and their stores (evict-first: C is not read again here, B is)
-  // fall into the same lines
-  for (int w0 = r - lane; w0 < c; w0 += EU * gs) {  // (whole warps)
-    int key[EU], bs[EU], len[EU], rank[EU];
-    T v[EU];
-    int most = 0;
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      const int i = w0 + lane + u * gs;
-      key[u] = i < c ? sk[i] : kmin;
-      if constexpr (HAS_VAL) v[u] = i < c ? sv[i] : T{};
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      const int b = bucket(key[u]);
-      bs[u] = b ? bcnt[b - 1] : 0;
-      len[u] = w0 + lane + u * gs < c ? bcnt[b] - bs[u] : 0;
-      if (!HS_G(dbg, bs[u] >= 0 && bs[u] + len[u] <= c, 24, bs[u])) len[u] = 0;
-      rank[u] = bs[u];
-      most = max(most, len[u]);
-    }
-    // every lane as many steps as the warp's largest bucket asks for: loops of
-    // their own lengths left the lanes one behind the other
-    most = warp_max(most);
-    for (int t = 0; t < most; ++t) {
-#pragma unroll
-      for (int u = 0; u < EU; ++u) rank[u] += t < len[u] && sk[bs[u] + t] < key[u];
-    }
-#pragma unroll
-    for (int u = 0; u < EU; ++u) {
-      if (len[u] > 0) {
-        __stcs(out_j + rank[u], key[u]);
-        if constexpr (HAS_VAL) __stcs(out_v + rank[u], v[u]);
-      }
-    }
-  }
+  group_bucket_sort<G, T, HAS_VAL, false>(ck, cv, c, es->kmin, es->kmax, work, wtmp, dbg, [&](int at, int k, T v) {
+    __stcs(out_j + at, k);
+    if constexpr (HAS_VAL) __stcs(out_v + at, v);
+  });
   G::sync();
 }
 

@@ -246,6 +246,17 @@ __global__ void __launch_bounds__(NWARP_WPB * 32, 4) k_num_warp(NumArgs a) {
 // 2048 outputs: 3.15 against 2.56 ms).
 constexpr int num_ch(int cap, int nt) { return cap <= CAP_MID_S || nt >= 1024 ? 1024 : 256; }
 
+// Rows of the block tiers with few repeated columns (at most one product in
+// FLAT_DUP beyond the outputs) are sorted as they are: no table to clear, to
+// probe and to read out, where every product would meet an empty slot (R-MAT
+// scale 20, rows of 2048..4096 outputs 4.35 -> 3.28 ms, 1024..2048 2.20 -> 1.83
+// ms).  Repeats cost steps of the ranking, as many as a column has products;
+// the share bounds them (allowing as many repeats as outputs measured the same
+// here).  The kernel of the smallest rows keeps its table: its registers leave
+// room for three CTAs, and it was slower this way (frontier of 256 columns: 173
+// against 204 us).
+constexpr int FLAT_DUP = 8;
+
 template <typename T, int SLOTS, int CAP, int CH> struct CtaNumLayout {
   static constexpr size_t table_bytes = (size_t)SLOTS * (4 + vbytes<T>());
   static constexpr size_t work_bytes =
@@ -263,6 +274,106 @@ template <typename T, int SLOTS, int CAP, int CH> struct CtaNumLayout {
   };
   static constexpr size_t bytes = tail_off + sizeof(Tail);
 };
+
+// The products of a row one after another, and their range of columns.
+template <typename T, bool HAS_VAL> struct FlatProducts {
+  static constexpr bool kFlat = true;
+  int *ck;
+  T *cv;
+  int cap;
+  int row0, at0;  // products of the earlier rounds, products before the batch
+  int kmin, kmax;
+  __device__ __forceinline__ void batch(int before) { at0 = row0 + before; }
+  __device__ __forceinline__ void round(int total) { row0 += total; }
+  __device__ __forceinline__ void operator()(int col, T v, int p) {
+    const int at = at0 + p;
+    if (at >= cap) return;
+    ck[at] = col;
+    if constexpr (HAS_VAL) cv[at] = v;
+    kmin = min(kmin, col);
+    kmax = max(kmax, col);
+  }
+};
+
+// A row of nf products, c of them with different columns, laid out in ck/cv:
+// sorted by column, the products of a column added up, and the row written.
+template <class SR, typename T>
+__device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val> &fp, int nf, int c, void *work, int *wtmp,
+                                              EmitScratch *es, int32_t *out_j, T *out_v, int *err, long long *dbg) {
+  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, nw = blockDim.x >> 5;
+  if (tid == 0) {
+    es->kmin = 0x7fffffff;
+    es->kmax = -1;
+  }
+  __syncthreads();
+  const int lmin = warp_min(fp.kmin), lmax = warp_max(fp.kmax);
+  if (lane == 0) {
+    atomicMin(&es->kmin, lmin);
+    atomicMax(&es->kmax, lmax);
+  }
+  __syncthreads();
+  if (fp.row0 != nf) {  // (uniform) the products are not as many as the analysis counted
+    if (tid == 0) atomicExch(err, 1);
+    return;
+  }
+  if (nf == c) {
+    group_bucket_sort<CtaGroup, T, SR::has_val, false>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg,
+                                                       [&](int at, int k, T v) {
+                                                         __stcs(out_j + at, k);
+                                                         if constexpr (SR::has_val) __stcs(out_v + at, v);
+                                                       });
+    return;
+  }
+  int *sk = fp.ck;
+  T *sv = fp.cv;
+  group_bucket_sort<CtaGroup, T, SR::has_val, true>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg,
+                                                    [&](int at, int k, T v) {
+                                                      sk[at] = k;
+                                                      if constexpr (SR::has_val) sv[at] = v;
+                                                    });
+  __syncthreads();
+  // a warp's run of entries: its columns are counted, then written behind
+  // those of the warps before it
+  const int per = ((nf + nw - 1) / nw + 31) & ~31;
+  const int e0 = min(nf, warp * per), e1 = min(nf, e0 + per);
+  int heads = 0;
+  for (int eb = e0; eb < e1; eb += 32) {
+    const int e = eb + lane;
+    heads += __popc(__ballot_sync(FULL, e < e1 && (e == 0 || sk[e] != sk[e - 1])));
+  }
+  if (lane == 0) wtmp[warp] = heads;
+  __syncthreads();
+  int at = 0, total = 0;
+  for (int w = 0; w < nw; ++w) {
+    const int x = wtmp[w];
+    at += w < warp ? x : 0;
+    total += x;
+  }
+  if (total != c) {  // (uniform) structure disagrees with the symbolic count
+    if (tid == 0) atomicExch(err, 1);
+  } else {
+    for (int eb = e0; eb < e1; eb += 32) {
+      const int e = eb + lane;
+      const int k = e < e1 ? sk[e] : -1;
+      const bool head = e < e1 && (e == 0 || k != sk[e - 1]);
+      const unsigned m = __ballot_sync(FULL, head);
+      if (head) {
+        const int d = at + __popc(m & ((1u << lane) - 1u));
+        __stcs(out_j + d, k);
+        if constexpr (SR::has_val) {
+          // a selector takes the first; a sum starts from the identity, as the table's slots do
+          T acc = sv[e];
+          if constexpr (SR::needs_a && SR::needs_b) {
+            acc = SR::add(SR::identity(), acc);
+            for (int q = e + 1; q < nf && sk[q] == k; ++q) acc = SR::add(acc, sv[q]);
+          }
+          __stcs(out_v + d, acc);
+        }
+      }
+      at += __popc(m);
+    }
+  }
+}
 
 // CTAs an SM that shared memory has room for; the registers are held to them
 // (rows of 2048..4096 outputs with one CTA of 512 threads an SM instead of two:
@@ -289,6 +400,19 @@ __global__ void __launch_bounds__(NT, num_cta_min<typename SR::val_t, CAP, NT>()
     const int64_t o = nout_row(a.A, r);
     const int64_t cb = a.Cp[o];
     const int c = (int)(a.Cp[o + 1] - cb);
+    const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
+    const bool listed = lofs >= 0 && !(lofs & LIST_BITS);
+    const int64_t nf = a.f[r];
+    if (CAP > CAP_MID_S && !listed && !a.unsorted && nf <= CAP && nf - c <= c / FLAT_DUP) {
+      FlatProducts<T, SR::has_val> fp{ck, cv, CAP, 0, 0, 0x7fffffff, -1};
+      cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex,
+                                                                           tl.wtmp, fp);
+      if (c > 0)
+        cta_flat_emit<SR, T>(fp, (int)nf, c, smem_raw, tl.wtmp, &tl.es, a.Cj + cb, SR::has_val ? Cv + cb : nullptr, a.err,
+                             a.A.dbg);
+      __syncthreads();
+      continue;
+    }
     const int slots = max(64, min(SLOTS, next_pow2(2 * min(c, CAP))));
     const unsigned mask = slots - 1;
     for (int s = threadIdx.x; s < slots; s += blockDim.x) {
@@ -298,8 +422,7 @@ __global__ void __launch_bounds__(NT, num_cta_min<typename SR::val_t, CAP, NT>()
     __syncthreads();
     cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
                           [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
-    const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
-    if (lofs >= 0 && !(lofs & LIST_BITS)) {
+    if (listed) {
       // the symbolic pass left the row's sorted columns: no sort, each
       // column's value is looked up in the table
       const int32_t *Lr = a.glist + lofs;
