@@ -25,7 +25,9 @@
  *   - All matrix arrays are DEVICE pointers on the current CUDA device.  The
  *     library never modifies its inputs.
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
- *     stream).  Work is stream ordered.  Each product performs two small
+ *     stream).  Work is stream ordered (the kernels of a product's row bins
+ *     may run side by side on streams of the library's own, which start
+ *     behind `stream` and which it waits for).  Each product performs two small
  *     device->host reads of sizes and therefore two host synchronisations
  *     with `stream` (after binning and after the symbolic pass).
  *   - Outputs and temporaries are allocated through `alloc` (see
@@ -137,11 +139,13 @@ int hs_spgemm(int semiring, const hs_mat *A, const hs_mat *B, hs_mat *C,
  * rows/columns).  This is the product R*A*Q with R = sparse(1:len(I), I, 1)
  * and Q = sparse(J, 1:len(J), 1), evaluated without forming R*A: the rows
  * I[t] are gathered, each entry (I[t], c) becomes (t, p) for every p with
- * J[p] == c, and the entries are ordered by a stable radix sort (none when J
- * is strictly increasing).  Values are copied bit for bit.  Index ranges are
- * always checked; with HS_FLAG_VALIDATE, A is checked to be canonical too.
- * At most 2^31-1 entries of B unless J is strictly increasing; three or four
- * host synchronisations with `stream`.  Errors: HS_EINVAL (an index out of
+ * J[p] == c, and every row is sorted by itself; where J repeats an index the
+ * entries are ordered by a stable radix sort instead (where it is strictly
+ * increasing they need no order).  Values are copied bit for bit.  Index
+ * ranges are always checked; with HS_FLAG_VALIDATE, A is checked to be
+ * canonical too.  At most 2^31-1 entries of B unless J is strictly increasing;
+ * two host synchronisations with `stream` when J repeats no index, up to five
+ * otherwise.  Errors: HS_EINVAL (an index out of
  * range, bad shapes, NULL pointers), HS_ENONCANON (with HS_FLAG_VALIDATE),
  * HS_EUNSUPPORTED, HS_ENOMEM, HS_ECUDA. */
 int hs_spref(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ,

@@ -585,7 +585,7 @@ __device__ void combine_val(const AsgnArgs &a, int64_t di, int64_t ai, int64_t x
 
 // The merge runs over entries, not rows, so a hub row costs what its entries
 // cost (assigning 20,000 edges into a 16M-entry graph: 6.62 of 7.20 ms with one
-// lane walking each touched row, 0.23 of 0.30 ms so; its 270 MB of A and C
+// lane walking each touched row, 0.19 of 0.27 ms so; its 270 MB of A and C
 // take 0.04 ms at the copy rate).  X = R*B*Q as the
 // entries of B moved to row I[i] and column J[c], in (row, column) order:
 // entry t of X goes in front of A's entry at[t] (the first of its row whose

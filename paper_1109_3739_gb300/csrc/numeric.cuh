@@ -11,7 +11,10 @@
 //   warp  (f <= 512)       one warp; private shared hash table of <= 1024
 //                          slots, then sorted emission;
 //   mid   (c <= 2048)      one CTA of 256; shared hash table of 2c slots;
-//   large (c <= CAP)       one CTA of 1024; shared hash table of 2c slots;
+//   large (c <= CAP)       one CTA of 512 or 1024; the same.  In both, rows
+//                          with few repeated columns are sorted as they are
+//                          and structure-only rows over few columns go
+//                          through a bitmap;
 //   heavy (c > CAP)        one CTA of 512 per row (two per SM), rows handed
 //                          out largest first; column parts accumulated with
 //                          a bitmap + rank-indexed value array (see

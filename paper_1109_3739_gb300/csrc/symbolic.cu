@@ -5,17 +5,19 @@
 // counted by the accumulator its bin selects.
 //   tiny  (f <= 32)    several rows to a warp, one product per lane, equal
 //                      columns of a row found with __match_any_sync;
-//   warp  (f <= 512)   one warp, private shared-memory hash set;
-//   mid   (f <= 1024, and f <= 4096)
-//                      one CTA, shared hash set of 2f slots (at most 2048,
-//                      and 8192: the smaller tier keeps more CTAs per SM);
+//   warp  (f <= 1024)  one warp, private shared-memory hash set; or a bitmap
+//                      of B's columns where they fit its room, else, for at
+//                      most 64 products, a sort in registers;
+//   mid   (f <= 4096)  one CTA, shared hash set of 2f slots (at most 8192) or
+//                      a bitmap;
 //   large (f <= min(16384, cap_large), so f <= 8192)
 //                      one CTA, shared hash set of up to 16384 slots;
 //   heavy (larger f)   one CTA, a bitmap over 2^20 columns (occupancy SPA in
 //                      shared memory), rows handed out largest first.  The
 //                      bitmap is read out in column order, so the kernel also
-//                      writes the row's sorted column list for the numeric
-//                      pass, which then only has to place values.
+//                      writes the row's sorted column list (a dense row's
+//                      bitmap) for the numeric pass, which then only has to
+//                      place values.
 // Rows with more than cap_large products also get per-column-segment counts
 // (4096-column segments) from which the numeric pass plans its column parts.
 // Counts go to cnt[row + 1] so an inclusive scan turns them into row offsets.

@@ -112,3 +112,47 @@ def test_rows_sorted_as_they_are(sr, dt):
             if dup and dup < 600:
                 rows.append(split(c, 290) + [(7, 8)] * dup)
     product(*operands(600001, rows, dt, 9), f"few repeats {sr} {dt}", sr)
+
+
+@pytest.mark.parametrize("sr,dt", KINDS)
+def test_hub_rows_beside_short_ones(sr, dt):
+    """Rows of thousands of entries of A (few outputs, and units whose segments are laid out by blocks), B rows of
+    thousands of entries, short rows of every bin, in one product and in a captured replay of its plan."""
+    import torch
+    n = 100003
+    rows = [split(4500, 4500) + [(0, 3)] * 600, split(9000, 1500) + [(5, 2600)], split(20000, 3) + [(0, 2049)] * 4,
+            split(4096, 4096), split(4097, 4097)]
+    for f in (0, 1, 20, 32, 33, 100, 200, 400, 700, 1500, 3000, 4500, 9000):
+        rows += [split(f, min(f, 4)) + ([(0, f // 2)] if f > 1 else [])] * 3 if f else [[]]
+    A, B = operands(n, rows, dt, 10)
+    product(A, B, f"hubs {sr}", sr)
+    if dt == "bool":
+        return
+    h = H()
+    P = h.Plan(sr, h.DeviceCSR.from_host(A), h.DeviceCSR.from_host(B))
+    P.execute()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        P.execute()
+    P.C.val.zero_()
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert_bitexact(P.C.to_host(), oracle.spgemm(sr, A, B), f"hubs {sr}, captured")
+
+
+def test_millions_of_empty_rows():
+    """More rows than one pass of the scan's tiles, almost all empty, with long gaps inside a tile of entries."""
+    m, k, n = 8_500_001, 64, 1000
+    at = np.unique(np.concatenate([np.arange(0, 40), [20000, 20001, 60000, 4_000_000], m - 1 - np.arange(3),
+                                   (I.draws(4, 9, 0, 500) % np.uint64(m)).astype(np.int64)]))
+    lens = 1 + np.arange(len(at)) % 40
+    rowptr = np.zeros(m + 1, np.int64)
+    rowptr[at + 1] = lens
+    rowptr = np.cumsum(rowptr)
+    cols = np.concatenate([np.sort(I.random_unique_sequence(k, int(c), 70 + i)) for i, c in enumerate(lens)])
+    A = csr(m, k, rowptr, cols, I.random_values(len(cols), "i64", 11, kind="signed"), "i64")
+    B = csr(k, n, np.arange(k + 1) * 5, np.concatenate([np.sort(I.random_unique_sequence(n, 5, 80 + i)) for i in range(k)]),
+            I.random_values(5 * k, "i64", 12, kind="signed"), "i64")
+    product(A, B, "empty rows", "plus_times")
