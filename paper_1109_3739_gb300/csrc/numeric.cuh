@@ -298,6 +298,14 @@ template <typename T, bool HAS_VAL> struct FlatProducts {
   }
 };
 
+// A column's sum before its second product: a selector takes the first one, a
+// sum starts from the identity, as the table's slots do (so a NaN does not win a
+// minimum, and -0 becomes 0).
+template <class SR, typename T> __device__ __forceinline__ T first_of(T v) {
+  if constexpr (SR::needs_a && SR::needs_b) return SR::add(SR::identity(), v);
+  return v;
+}
+
 // A row of nf products, c of them with different columns, laid out in ck/cv:
 // sorted by column, the products of a column added up, and the row written.
 template <class SR, typename T>
@@ -323,7 +331,7 @@ __device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val>
     group_bucket_sort<CtaGroup, T, SR::has_val, false>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg,
                                                        [&](int at, int k, T v) {
                                                          __stcs(out_j + at, k);
-                                                         if constexpr (SR::has_val) __stcs(out_v + at, v);
+                                                         if constexpr (SR::has_val) __stcs(out_v + at, first_of<SR>(v));
                                                        });
     return;
   }
@@ -364,12 +372,8 @@ __device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val>
         const int d = at + __popc(m & ((1u << lane) - 1u));
         __stcs(out_j + d, k);
         if constexpr (SR::has_val) {
-          // a selector takes the first; a sum starts from the identity, as the table's slots do
-          T acc = sv[e];
-          if constexpr (SR::needs_a && SR::needs_b) {
-            acc = SR::add(SR::identity(), acc);
-            for (int q = e + 1; q < nf && sk[q] == k; ++q) acc = SR::add(acc, sv[q]);
-          }
+          T acc = first_of<SR>(sv[e]);
+          for (int q = e + 1; q < nf && sk[q] == k; ++q) acc = SR::add(acc, sv[q]);
           __stcs(out_v + d, acc);
         }
       }

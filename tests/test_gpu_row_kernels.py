@@ -156,3 +156,21 @@ def test_millions_of_empty_rows():
     B = csr(k, n, np.arange(k + 1) * 5, np.concatenate([np.sort(I.random_unique_sequence(n, 5, 80 + i)) for i in range(k)]),
             I.random_values(5 * k, "i64", 12, kind="signed"), "i64")
     product(A, B, "empty rows", "plus_times")
+
+
+@pytest.mark.parametrize("c,dup", [(1500, 0), (1500, 100), (3500, 0), (3500, 300)])
+def test_sorted_rows_treat_special_values_as_the_table_does(c, dup):
+    """(min,+) with infinities and NaNs: a row that is sorted as it is against the same row in the table (the
+    unsorted output keeps it)."""
+    h = H()
+    A, B = operands(600001, [split(c, 3) + ([(0, dup)] if dup else [])] * 3, "f32", 13)
+    B.val[::7], B.val[1::11], B.val[2::13], B.val[3::17] = np.nan, np.inf, -np.inf, -0.0
+    A.val[1] = np.inf
+    dA, dB = h.DeviceCSR.from_host(A), h.DeviceCSR.from_host(B)
+    got = h.spgemm("min_plus", dA, dB).to_host()
+    raw = h.spgemm("min_plus", dA, dB, sorted_rows=False).to_host()
+    assert np.array_equal(got.rowptr, raw.rowptr)
+    for a, b in zip(got.rowptr[:-1], got.rowptr[1:]):
+        order = np.argsort(raw.col[a:b])
+        assert np.array_equal(got.col[a:b], raw.col[a:b][order])
+        assert np.array_equal(got.val[a:b], raw.val[a:b][order], equal_nan=True)
