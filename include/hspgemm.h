@@ -26,8 +26,10 @@
  *     library never modifies its inputs.
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *     stream).  Work is stream ordered (the kernels of a product's row bins
- *     may run side by side on streams of the library's own, which start
- *     behind `stream` and which it waits for).  Each product performs two small
+ *     may run side by side on streams of the library's own, of `stream`'s
+ *     priority, which start behind `stream` and which it waits for; work of
+ *     different `stream`s does not wait for one another through them, as long
+ *     as a host thread uses no more than eight).  Each product performs two small
  *     device->host reads of sizes and therefore two host synchronisations
  *     with `stream` (after binning and after the symbolic pass).
  *   - Outputs and temporaries are allocated through `alloc` (see
@@ -293,9 +295,13 @@ int hs_get_tuning(hs_tuning *t);
  * same column ids, so C->ptr and C->idx, and A's and B's ptr/idx/ids arrays,
  * must stay allocated and unchanged while the plan is used.  A_val (B_val) may
  * be NULL where the semiring ignores that operand's values.  The call only
- * enqueues kernels (and one 4-byte memset) on `stream`: it allocates nothing
- * and never waits for the GPU, so it can be captured in a CUDA graph and
- * replayed.  Executions of one plan must not overlap (they share its scratch).
+ * enqueues kernels (and one 8-byte memset) on `stream` and on streams that the
+ * plan made for itself at its creation, which start behind `stream` and which
+ * it waits for: it allocates nothing and never waits for the GPU, so it can be
+ * captured in a CUDA graph and replayed.  On a stream of another priority than
+ * the plan was created on, or while an execution of the plan is part of a
+ * capture that `stream` takes no part in, everything goes to `stream`.
+ * Executions of one plan must not overlap (they share its scratch).
  * Device-side checks raised during executes are reported by hs_plan_status,
  * which synchronises with `stream`: HS_OK or HS_EINTERNAL.
  *

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "../../include/hspgemm.h"
+#include "fan.h"
 #include "internal.h"
 
 namespace hs {
@@ -215,97 +216,49 @@ static void *pinned(size_t bytes) {
   return bytes <= 8192 ? t_pin.p : nullptr;
 }
 
-// Streams beside the caller's, for bins that run at the same time: a few per
-// host thread and device, made on first use and destroyed with the thread.
-// They never outlive a call's work: every call that used one lets the caller's
-// stream wait for it before it returns.
-constexpr int FAN_SIDES = 3, FAN_DEVICES = 64;
-struct SideStreams {
-  struct Dev {
-    cudaStream_t s[FAN_SIDES];
-    cudaEvent_t fork, join[FAN_SIDES];
-    bool ok;
+// the runtime as fan.h wants it: a failed call leaves no error behind
+struct FanCuda {
+  using Stream = cudaStream_t;
+  using Event = cudaEvent_t;
+  struct Capture {
+    bool active;
+    unsigned long long id;
   };
-  Dev *dev[FAN_DEVICES] = {nullptr};
-  ~SideStreams() {
-    for (Dev *d : dev) {
-      if (!d) continue;
-      for (int i = 0; i < FAN_SIDES; ++i) {
-        if (d->s[i]) cudaStreamDestroy(d->s[i]);
-        if (d->join[i]) cudaEventDestroy(d->join[i]);
-      }
-      if (d->fork) cudaEventDestroy(d->fork);
-      delete d;
-    }
+  static bool good(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
   }
-  Dev *get() {
-    int id = 0;
-    if (cudaGetDevice(&id) != cudaSuccess || id < 0 || id >= FAN_DEVICES) return nullptr;
-    if (!dev[id]) {
-      Dev *d = new (std::nothrow) Dev();
-      if (!d) return nullptr;
-      d->ok = cudaEventCreateWithFlags(&d->fork, cudaEventDisableTiming) == cudaSuccess;
-      for (int i = 0; i < FAN_SIDES; ++i)
-        d->ok = d->ok && cudaStreamCreateWithFlags(&d->s[i], cudaStreamNonBlocking) == cudaSuccess &&
-                cudaEventCreateWithFlags(&d->join[i], cudaEventDisableTiming) == cudaSuccess;
-      cudaGetLastError();
-      dev[id] = d;
-    }
-    return dev[id]->ok ? dev[id] : nullptr;
+  static bool device(int *d) { return good(cudaGetDevice(d)); }
+  static bool priority(Stream s, int *p) { return good(cudaStreamGetPriority(s, p)); }
+  static bool capture(Stream s, Capture *c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    c->id = 0;
+    if (!good(cudaStreamGetCaptureInfo(s, &st, &c->id)) || st == cudaStreamCaptureStatusInvalidated) return false;
+    c->active = st == cudaStreamCaptureStatusActive;
+    return true;
   }
+  static bool create(Event *e) { return good(cudaEventCreateWithFlags(e, cudaEventDisableTiming)); }
+  static bool create(Stream *s, int priority) {
+    return good(cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, priority));
+  }
+  static void destroy(Event e) { good(cudaEventDestroy(e)); }
+  static void destroy(Stream s) { good(cudaStreamDestroy(s)); }
+  static bool record(Event e, Stream s) { return good(cudaEventRecord(e, s)); }
+  static bool wait(Stream s, Event e) { return good(cudaStreamWaitEvent(s, e, 0)); }
+  static void synchronize(Stream s) { good(cudaStreamSynchronize(s)); }
 };
-static thread_local SideStreams t_sides;
+using Fan = FanOf<FanCuda>;
+static thread_local SidePool<FanCuda> t_sides;
 
 // The bins of a pass over four streams: the caller's (group 0) and three
 // beside it.  Bins of one pass work on different rows, and the larger ones end
 // in tails of a few blocks (a row of very many entries or products), which the
 // others fill (a contraction's two products 2.44 -> 1.76 ms, a narrow frontier
-// product 1.43 -> 0.93 ms, a batch of random products 6.44 -> 6.15 ms).  All of
-// a pass's work starts after what the caller's stream holds and the caller's
-// stream goes on after all of it, so nothing else changes (stream capture
-// included).  In a product of more than FAN_PRODUCTS products the tails are
-// nothing and the bins only take each other's cache (6.0e9 products: 72.4
-// against 72.2 ms; 6e8: 4.6 against 4.8 ms): its bins run one by one.
+// product 1.43 -> 0.93 ms, a batch of random products 6.44 -> 6.15 ms).  In a
+// product of more than FAN_PRODUCTS products the tails are nothing and the
+// bins only take each other's cache (6.0e9 products: 72.4 against 72.2 ms;
+// 6e8: 4.6 against 4.8 ms): its bins run one by one.
 constexpr unsigned long long FAN_PRODUCTS = 1ull << 31;
-struct Fan {
-  cudaStream_t main;
-  SideStreams::Dev *d = nullptr;
-  bool used[FAN_SIDES] = {false};
-  bool failed = false;
-  // groups: bit g set when group g has work; with one group nothing is forked
-  Fan(cudaStream_t st, unsigned groups) : main(st) {
-    if ((groups & (groups - 1)) == 0) return;
-    d = t_sides.get();
-    if (d && cudaEventRecord(d->fork, main) != cudaSuccess) {
-      cudaGetLastError();
-      d = nullptr;
-    }
-  }
-  cudaStream_t stream(int group) {
-    if (!d || group == 0) return main;
-    const int i = group - 1;
-    if (!used[i]) {
-      if (cudaStreamWaitEvent(d->s[i], d->fork, 0) != cudaSuccess) failed = true;
-      used[i] = true;
-    }
-    return d->s[i];
-  }
-  int join() {
-    for (int i = 0; i < FAN_SIDES; ++i) {
-      if (!used[i]) continue;
-      used[i] = false;
-      if (cudaEventRecord(d->join[i], d->s[i]) != cudaSuccess || cudaStreamWaitEvent(main, d->join[i], 0) != cudaSuccess)
-        failed = true;
-    }
-    if (!failed) return HS_OK;
-    // the side streams' work must end before the caller's buffers are touched again
-    if (d)
-      for (int i = 0; i < FAN_SIDES; ++i) cudaStreamSynchronize(d->s[i]);
-    cudaGetLastError();
-    return HS_ECUDA;
-  }
-  ~Fan() { join(); }
-};
 // numeric kinds: heavy rows, large, mid, and the rows of a warp
 static int num_group(int kind) { return kind == NUM_KINDS - 1 ? 1 : kind == 5 || kind == 6 ? 2 : kind == 3 || kind == 4 ? 3 : 0; }
 
@@ -479,6 +432,15 @@ struct hs_plan {
   hs_allocator al{};
   bool has_al = false;
   bool side_by_side = false;  // the bins run beside each other (hs::Fan)
+  unsigned groups() const {
+    unsigned g = 0;
+    for (int kind = 0; kind < hs::NUM_KINDS; ++kind)
+      if (side_by_side && count[kind] > 0) g |= 1u << hs::num_group(kind);
+    return g;
+  }
+  // streams of the plan's own, so that plans on different streams of a thread
+  // stay independent and an execution makes none (it may be captured)
+  std::unique_ptr<hs::SideSet<hs::FanCuda>> sides;
   std::vector<hs::Mem::Blk> blocks;
 };
 
@@ -712,7 +674,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     for (const SymBin &x : bins_)
       if (side_by_side && key_off[x.k1] > key_off[x.k0]) groups |= 1u << x.group;
     PhaseTimer t("symbolic", st);
-    Fan fan(st, groups);
+    Fan fan(st, groups, groups & (groups - 1) ? t_sides.of(st) : nullptr);
     for (const SymBin &x : bins_) {
       sa.list = list + key_off[x.k0];
       sa.count = key_off[x.k1] - key_off[x.k0];
@@ -724,7 +686,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
       }
       if (int e = phase_check(x.name, bst, sb->dbg)) return e;
     }
-    if (int e = fan.join()) return e;
+    if (!fan.join()) return HS_ECUDA;
   }
 
   // ---- offsets and numeric bins
@@ -826,7 +788,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   }
   if (nheavy > 0) alloc_bci();  // (every allocation before the streams part: they are ordered on the caller's)
   std::unique_ptr<PhaseTimer> t_num(new PhaseTimer("numeric", st));
-  Fan fan(st, groups);
+  Fan fan(st, groups, groups & (groups - 1) ? t_sides.of(st) : nullptr);
   // heavy bin: the B segment index, and the units' B segments
   const cudaStream_t hst = nheavy > 0 ? fan.stream(num_group(NUM_KINDS - 1)) : st;
   if (bci) {
@@ -874,7 +836,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     }
     if (int e = phase_check(names[kind], bst, sb->dbg)) return e;
   }
-  if (int e = fan.join()) return e;
+  if (!fan.join()) return HS_ECUDA;
   t_num.reset();
   if (flags & HS_FLAG_VALIDATE) {
     CK(cudaMemcpyAsync(hb, sb, sizeof(SmallBlock), cudaMemcpyDeviceToHost, st));
@@ -1410,6 +1372,10 @@ int hs_plan_create(int semiring, const hs_mat *A, const hs_mat *B, hs_mat *C, hs
     P->al = *al;
     P->has_al = true;
   }
+  if (const unsigned g = P->groups(); g & (g - 1)) {
+    P->sides.reset(new (std::nothrow) SideSet<FanCuda>());
+    if (P->sides && !P->sides->make((cudaStream_t)stream)) P->sides.reset();  // (the bins then run one by one)
+  }
   *plan = P;
   return HS_OK;
 }
@@ -1428,10 +1394,7 @@ int hs_plan_execute(const hs_plan *P, const void *A_val, const void *B_val, void
   na.B.v = B_val;
   na.Cv = C_val;
   CK(cudaMemsetAsync(P->dyn, 0, 2 * sizeof(int), st));  // the heavy rows' and units' counters
-  unsigned groups = 0;
-  for (int kind = 0; kind < NUM_KINDS; ++kind)
-    if (P->side_by_side && P->count[kind] > 0) groups |= 1u << num_group(kind);
-  Fan fan(st, groups);
+  Fan fan(st, P->groups(), P->sides.get());
   // the heavy units' B segments carry A's values: laid out again from the new ones
   if (na.units && na.pseg && na.nunits > 0)
     launch_build_pairs(na.A, na.B, const_cast<HeavyUnit *>(na.units), na.nunits, na.bci_id, na.bci, na.nseg,
@@ -1444,7 +1407,7 @@ int hs_plan_execute(const hs_plan *P, const void *A_val, const void *B_val, void
     na.count = P->count[kind];
     if (!launch_num(P->sr, P->out_dt, kind, na, fan.stream(num_group(kind)))) return HS_EINVAL;
   }
-  if (int e = fan.join()) return e;
+  if (!fan.join()) return HS_ECUDA;
   return check_launch();
 }
 
