@@ -6,8 +6,8 @@
 // sorted afterwards.  Here the warp lays the row's products (column, value)
 // out in shared memory in product order, sorts packed keys
 // (column - kmin) << PB | product index in registers with Batcher's bitonic
-// network (32*K keys, K per lane), and folds runs of equal columns with a
-// segmented scan over the sorted order: Algorithm 1's row-wise accumulation
+// network (32*K keys, K per lane), and folds runs of equal columns in the
+// sorted order: Algorithm 1's row-wise accumulation
 // done as expand, sort, compress.  The row leaves in ascending column order,
 // its values summed (or minimised, or-ed) with the semiring's add.  A row
 // whose column span does not fit the packed key sorts 64-bit keys
@@ -39,7 +39,6 @@ template <class SR> __device__ __forceinline__ typename SR::val_t sr_identity() 
 }
 
 template <typename T> __device__ __forceinline__ T shfl_up_val(T x, int d) { return __shfl_up_sync(FULL, x, d); }
-template <> __device__ __forceinline__ NoVal shfl_up_val<NoVal>(NoVal x, int) { return x; }
 template <typename T> __device__ __forceinline__ T shfl_down_val(T x, int d) { return __shfl_down_sync(FULL, x, d); }
 template <> __device__ __forceinline__ NoVal shfl_down_val<NoVal>(NoVal x, int) { return x; }
 
@@ -163,10 +162,67 @@ __device__ __forceinline__ int sort_expand(const DevCsr &A, const DevCsr &B, con
   return got;
 }
 
+// The runs of more than four equal columns among a row's F sorted keys (column
+// - kmn) << pb | product index: a segmented scan of each round of 32 in which
+// one begins (a bit of long_in) or goes on, written from the run's last
+// element at its rank (lane i of `before`: columns before round i).
+template <class SR>
+__device__ __forceinline__ void sum_long_runs(int F, int pb, int c, int kmn, unsigned long_in, int before,
+                                           const int *s_col, const typename SR::val_t *s_val, int32_t *out_j,
+                                           typename SR::val_t *out_v, long long *dbg) {
+  using T = typename SR::val_t;
+  const int lane = lane_id();
+  const unsigned le = 0xffffffffu >> (31 - lane), at = (1u << pb) - 1u;
+  auto key_at = [&](int e) { return e < F ? (uint32_t)s_col[sr_pad(e)] : 0xffffffffu; };  // (no element's column)
+  bool open = false;  // a long run reaches into the round
+  T carry = SR::identity();
+  for (int i = 0; i * 32 < F; ++i) {
+    if (!open && !((long_in >> i) & 1u)) continue;
+    const int e = i * 32 + lane;
+    const uint32_t kk = key_at(e);
+    const bool valid = e < F;
+    const bool head = valid && (e == 0 || (key_at(e - 1) >> pb) != (kk >> pb));
+    const bool tail = valid && (key_at(e + 1) >> pb) != (kk >> pb);
+    const unsigned hm = __ballot_sync(FULL, head);
+    const unsigned lm = __ballot_sync(FULL, head && (key_at(e + 4) >> pb) == (kk >> pb));
+    T x = valid ? s_val[kk & at] : SR::identity();
+    bool fl = head;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const T y = shfl_up_val<T>(x, d);
+      const bool g = __shfl_up_sync(FULL, (int)fl, d) != 0;
+      if (lane >= d) {
+        if (!fl) x = SR::add(y, x);
+        fl = fl || g;
+      }
+    }
+    if (!fl && valid) x = SR::add(carry, x);  // continues the run that came in
+    carry = shfl_val<T>(x, 31);
+    const unsigned upto = hm & le;
+    const bool in_long = upto ? (lm >> (31 - __clz(upto))) & 1u : open;
+    const int pos = __shfl_sync(FULL, before, i) + __popc(upto) - 1;
+    if (in_long && tail && HS_G(dbg, pos >= 0 && pos < c, 91, pos)) {
+      __stcs(out_j + pos, (int)(kk >> pb) + kmn);
+      __stcs(out_v + pos, x);
+    }
+    open = __shfl_sync(FULL, (int)(in_long && !tail), 31) != 0;
+  }
+}
+
+// for the kernel of several register widths, which holds one copy of it (a
+// copy per width cost it 1.3 %; the call costs the kernels of one width 1 %)
+template <class SR>
+__device__ __noinline__ void sum_long_runs_call(int F, int pb, int c, int kmn, unsigned long_in, int before,
+                                                const int *s_col, const typename SR::val_t *s_val, int32_t *out_j,
+                                                typename SR::val_t *out_v, long long *dbg) {
+  sum_long_runs<SR>(F, pb, c, kmn, long_in, before, s_col, s_val, out_j, out_v, dbg);
+}
+
 // Sort and fold a row whose F products (F <= 32*K) sort_expand laid out,
 // writing its c outputs at out_j / out_v.  An output count other than c
-// sets *err (the structure disagrees with the symbolic pass).
-template <class SR, int K, bool WIDE>
+// sets *err (the structure disagrees with the symbolic pass).  MANY: the
+// kernel holds this function for several K.
+template <class SR, int K, bool WIDE, bool MANY = false>
 __device__ __forceinline__ void sort_finish(int F, int c, int kmn, int kmx, int *s_col,
                                             const typename SR::val_t *s_val, int32_t *out_j,
                                             typename SR::val_t *out_v, int *err, long long *dbg) {
@@ -191,40 +247,64 @@ __device__ __forceinline__ void sort_finish(int F, int c, int kmn, int kmx, int 
     for (int i = 0; i < K; ++i) s_col[sr_pad(lane * K + i)] = (int)key[i];
     __syncwarp();
     // 3. runs of equal columns, 32 elements a round (lane l takes element
-    // 32*i + l): the lane at a run's head walks the run in sorted (so product)
-    // order and writes its sum at the run's rank among the row's columns.
-    // These rows hardly repeat a column, so a walk is a step or none; a
-    // segmented scan of every round took five shuffle-and-add steps of two
-    // words each whatever the runs.
+    // 32*i + l), at the run's rank among the row's columns.  Most runs are one
+    // or a few elements long: their head adds them up.  Runs of more than four
+    // are left to a segmented scan of the rounds that they touch.
+    // (A head that walked any run kept the warp waiting for the longest one,
+    // and the sum's error grew with the run's length: half of a row's 256 /
+    // 512 / 1024 products on one column took 246 / 468 / 1039 us a numeric
+    // pass, 201 / 370 / 788 now; a scan of every round takes five shuffle-and-add
+    // steps of two words each whatever the runs: 146 / 255 / 512 us without
+    // repeats, 116 / 200 / 403 this way.)
     const unsigned le = 0xffffffffu >> (31 - lane);  // lanes <= this one
-    int outb = 0;
-    uint32_t last = 0;  // the previous round's last key
+    auto key_at = [&](int e) { return e < F ? (uint32_t)s_col[sr_pad(e)] : 0xffffffffu; };  // (no element's column)
+    int outb = 0, before = 0;  // columns so far; lane i: before round i
+    unsigned long_in = 0;      // rounds in which a long run of this lane begins
+    uint32_t last = 0;         // the previous round's last key
     for (int i = 0; i * 32 < F; ++i) {
       const int e = i * 32 + lane;
       const bool valid = e < F;
-      const uint32_t kk = valid ? (uint32_t)s_col[sr_pad(e)] : 0xffffffffu;
+      const uint32_t kk = key_at(e);
       uint32_t kp = __shfl_up_sync(FULL, kk, 1);
       if (lane == 0) kp = last;
       last = __shfl_sync(FULL, kk, 31);
       const bool head = valid && (e == 0 || (kk >> PB) != (kp >> PB));
       const unsigned hm = __ballot_sync(FULL, head);
       const int pos = outb + __popc(hm & le) - 1;
+      if (lane == i) before = outb;
       if (head) {
         T v{};
+        bool more = false;
         if constexpr (SR::has_val) {
           v = s_val[kk & (N - 1)];
-          for (int j = e + 1; j < F; ++j) {
-            const uint32_t kj = (uint32_t)s_col[sr_pad(j)];
-            if ((kj >> PB) != (kk >> PB)) break;
-            v = SR::add(v, s_val[kj & (N - 1)]);
+          const uint32_t k1 = key_at(e + 1);
+          if ((k1 >> PB) == (kk >> PB)) {  // (nested: a loop of up to three steps took 1 % longer)
+            v = SR::add(v, s_val[k1 & (N - 1)]);
+            const uint32_t k2 = key_at(e + 2);
+            if ((k2 >> PB) == (kk >> PB)) {
+              v = SR::add(v, s_val[k2 & (N - 1)]);
+              const uint32_t k3 = key_at(e + 3);
+              if ((k3 >> PB) == (kk >> PB)) {
+                v = SR::add(v, s_val[k3 & (N - 1)]);
+                more = (key_at(e + 4) >> PB) == (kk >> PB);
+              }
+            }
           }
         }
-        if (HS_G(dbg, pos >= 0 && pos < c, 91, pos)) {
+        if (more) long_in |= 1u << i;
+        else if (HS_G(dbg, pos >= 0 && pos < c, 91, pos)) {
           __stcs(out_j + pos, (int)(kk >> PB) + kmn);
           if constexpr (SR::has_val) __stcs(out_v + pos, v);
         }
       }
       outb += __popc(hm);
+    }
+    if constexpr (SR::has_val) {
+      long_in = __reduce_or_sync(FULL, long_in);
+      if (long_in) {
+        if constexpr (MANY) sum_long_runs_call<SR>(F, PB, c, kmn, long_in, before, s_col, s_val, out_j, out_v, dbg);
+        else sum_long_runs<SR>(F, PB, c, kmn, long_in, before, s_col, s_val, out_j, out_v, dbg);
+      }
     }
     if (outb != c && lane == 0) atomicExch(err, 13);
     return;
