@@ -1080,10 +1080,13 @@ __host__ __device__ __forceinline__ size_t emit_work_bytes(int c, int vbytes) {
 
 // Steps (2) and (3): out(place, key, value) for the c entries of ck/cv.  DUPS:
 // keys may be equal, and then keep some order among themselves; out may write
-// to ck/cv, which are not read any more.
+// to ck/cv, which are not read any more.  Step (3) takes as many steps as a
+// bucket has entries: with DUPS, a row whose largest bucket holds more than
+// `limit` is left as it is and false returned (*most: zeroed before).
 template <class G, typename T, bool HAS_VAL, bool DUPS, class Out>
-__device__ __forceinline__ void group_bucket_sort(const int *ck, const T *cv, int c, int kmin, int kmax, void *work,
-                                                  int *wtmp, long long *dbg, Out &&out) {
+__device__ __forceinline__ bool group_bucket_sort(const int *ck, const T *cv, int c, int kmin, int kmax, void *work,
+                                                  int *wtmp, long long *dbg, Out &&out, int *most_shared = nullptr,
+                                                  int limit = 0) {
   constexpr int EU = 4;  // entries per thread per step: their shared-memory chains overlap
   const int gs = G::size(), r = G::rank(), lane = lane_id();
   const int nb = emit_buckets(c);
@@ -1101,6 +1104,14 @@ __device__ __forceinline__ void group_bucket_sort(const int *ck, const T *cv, in
     if (HS_G(dbg, b >= 0 && b < nb, 21, b)) atomicAdd(bcnt + b, 1);
   }
   G::sync();
+  if constexpr (DUPS) {
+    int n = 0;
+    for (int b = r; b < nb; b += gs) n = max(n, bcnt[b]);
+    n = warp_max(n);
+    if (lane == 0 && n > limit) atomicMax(most_shared, n);
+    G::sync();
+    if (*most_shared > limit) return false;
+  }
   group_excl_scan<G>(bcnt, nb, wtmp);
   // the entries into their buckets (arbitrary order inside a bucket); bcnt[b]
   // advances to the bucket's end
@@ -1165,6 +1176,7 @@ __device__ __forceinline__ void group_bucket_sort(const int *ck, const T *cv, in
       }
     }
   }
+  return true;
 }
 
 template <class G, typename T, bool HAS_VAL>

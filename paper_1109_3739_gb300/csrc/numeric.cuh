@@ -255,10 +255,15 @@ constexpr int num_ch(int cap, int nt) { return cap <= CAP_MID_S || nt >= 1024 ? 
 // scale 20, rows of 2048..4096 outputs 4.35 -> 3.28 ms, 1024..2048 2.20 -> 1.83
 // ms).  Repeats cost steps of the ranking, as many as a column has products;
 // the share bounds them (allowing as many repeats as outputs measured the same
-// here).  The kernel of the smallest rows keeps its table: its registers leave
+// here), and rows with more than FLAT_RUN products of one column (or of one
+// bucket) go from their layout to the table (8000 rows of 2300 / 3500 outputs,
+// f32, with 255 / 388 products of one column: 2.12 / 3.47 ms sorted as they
+// are, 0.87 / 1.12 so, 1.00 / 1.45 in the table from the start; with 32: 0.59 /
+// 0.67, 0.64 / 0.80, 0.65 / 0.87).  The kernel of the smallest rows keeps its table: its registers leave
 // room for three CTAs, and it was slower this way (frontier of 256 columns: 173
 // against 204 us).
 constexpr int FLAT_DUP = 8;
+constexpr int FLAT_RUN = 32;
 
 template <typename T, int SLOTS, int CAP, int CH> struct CtaNumLayout {
   static constexpr size_t table_bytes = (size_t)SLOTS * (4 + vbytes<T>());
@@ -308,13 +313,16 @@ template <class SR, typename T> __device__ __forceinline__ T first_of(T v) {
 
 // A row of nf products, c of them with different columns, laid out in ck/cv:
 // sorted by column, the products of a column added up, and the row written.
+// False (in every thread): more than FLAT_RUN products lie in one bucket, and
+// ck/cv are as they were.
 template <class SR, typename T>
-__device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val> &fp, int nf, int c, void *work, int *wtmp,
+__device__ __forceinline__ bool cta_flat_emit(const FlatProducts<T, SR::has_val> &fp, int nf, int c, void *work, int *wtmp,
                                               EmitScratch *es, int32_t *out_j, T *out_v, int *err, long long *dbg) {
   const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, nw = blockDim.x >> 5;
   if (tid == 0) {
     es->kmin = 0x7fffffff;
     es->kmax = -1;
+    es->count = 0;
   }
   __syncthreads();
   const int lmin = warp_min(fp.kmin), lmax = warp_max(fp.kmax);
@@ -325,7 +333,7 @@ __device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val>
   __syncthreads();
   if (fp.row0 != nf) {  // (uniform) the products are not as many as the analysis counted
     if (tid == 0) atomicExch(err, 1);
-    return;
+    return true;
   }
   if (nf == c) {
     group_bucket_sort<CtaGroup, T, SR::has_val, false>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg,
@@ -333,15 +341,17 @@ __device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val>
                                                          __stcs(out_j + at, k);
                                                          if constexpr (SR::has_val) __stcs(out_v + at, first_of<SR>(v));
                                                        });
-    return;
+    return true;
   }
   int *sk = fp.ck;
   T *sv = fp.cv;
-  group_bucket_sort<CtaGroup, T, SR::has_val, true>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg,
-                                                    [&](int at, int k, T v) {
-                                                      sk[at] = k;
-                                                      if constexpr (SR::has_val) sv[at] = v;
-                                                    });
+  const auto put = [&](int at, int k, T v) {
+    sk[at] = k;
+    if constexpr (SR::has_val) sv[at] = v;
+  };
+  if (!group_bucket_sort<CtaGroup, T, SR::has_val, true>(fp.ck, fp.cv, nf, es->kmin, es->kmax, work, wtmp, dbg, put,
+                                                         &es->count, FLAT_RUN))
+    return false;
   __syncthreads();
   // a warp's run of entries: its columns are counted, then written behind
   // those of the warps before it
@@ -380,6 +390,7 @@ __device__ __forceinline__ void cta_flat_emit(const FlatProducts<T, SR::has_val>
       at += __popc(m);
     }
   }
+  return true;
 }
 
 // CTAs an SM that shared memory has room for; the registers are held to them
@@ -410,15 +421,16 @@ __global__ void __launch_bounds__(NT, num_cta_min<typename SR::val_t, CAP, NT>()
     const int64_t lofs = (a.loff && a.glist) ? a.loff[r] : -1;
     const bool listed = lofs >= 0 && !(lofs & LIST_BITS);
     const int64_t nf = a.f[r];
+    bool laid = false;  // (uniform) the products lie in ck/cv
     if (CAP > CAP_MID_S && !listed && !a.unsorted && nf <= CAP && nf - c <= c / FLAT_DUP) {
       FlatProducts<T, SR::has_val> fp{ck, cv, CAP, 0, 0, 0x7fffffff, -1};
       cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex,
                                                                            tl.wtmp, fp);
       if (c > 0)
-        cta_flat_emit<SR, T>(fp, (int)nf, c, smem_raw, tl.wtmp, &tl.es, a.Cj + cb, SR::has_val ? Cv + cb : nullptr, a.err,
-                             a.A.dbg);
+        laid = !cta_flat_emit<SR, T>(fp, (int)nf, c, smem_raw, tl.wtmp, &tl.es, a.Cj + cb,
+                                     SR::has_val ? Cv + cb : nullptr, a.err, a.A.dbg);
       __syncthreads();
-      continue;
+      if (!laid) continue;
     }
     const int slots = max(64, min(SLOTS, next_pow2(2 * min(c, CAP))));
     const unsigned mask = slots - 1;
@@ -427,8 +439,15 @@ __global__ void __launch_bounds__(NT, num_cta_min<typename SR::val_t, CAP, NT>()
       if constexpr (SR::has_val) vals[s] = SR::identity();
     }
     __syncthreads();
-    cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
-                          [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
+    if (laid) {
+      for (int e = threadIdx.x; e < (int)nf; e += blockDim.x)
+        hash_insert_val<SR>(keys, vals, mask, ck[e], SR::has_val ? cv[e] : T{}, a.err);
+      __syncthreads();
+    } else {
+      cta_products<SR, num_ch(CAP, NT), 2, num_ch(CAP, NT) / NT >= 4 ? 4 : 1>(
+          A, B, A.p[r], A.p[r + 1], false, 0, 0, ex, tl.wtmp,
+          [&](int col, T v, int) { hash_insert_val<SR>(keys, vals, mask, col, v, a.err); });
+    }
     if (listed) {
       // the symbolic pass left the row's sorted columns: no sort, each
       // column's value is looked up in the table

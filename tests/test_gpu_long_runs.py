@@ -96,3 +96,25 @@ def test_sums_of_a_long_run_stay_accurate(f):
             assert np.count_nonzero(v == 1.0) >= f - r
 
     every_way("plus_times", A, B, check)
+
+
+@pytest.mark.parametrize("sr,dt", [("plus_times", "i64"), ("min_plus", "f32"), ("or_and", "bool")])
+def test_block_rows_with_a_repeated_column(sr, dt):
+    """Rows of 1100 to 3600 outputs with 31 to 34 products, an eighth of the outputs and a few columns of each:
+    sorted as they are up to 32 products a column, handed to the table beyond; and all of a row's columns but one
+    in one bucket of its sort."""
+    rows = []
+    for c in (1100, 1820, 2300, 3600):
+        rows += [[r] + [1] * (c - 1) for r in (2, 31, 32, 33, 34, c // 9)]
+        rows += [[r] * (c // 10 // r) + [1] * (c - c // 10 // r) for r in (16, 32, 33)] + [[20, 2, 33] + [1] * (c - 3)]
+    A, B = rows_of_runs(rows, dt, 63)
+    h = H()
+    for n, far in ((N, 0), (1 << 24, (1 << 24) - N)):  # (far: the greatest column moved away from the others)
+        B2 = csr(B.m, n, B.rowptr, np.where(B.col == B.col.max(), B.col + far, B.col), B.val, dt)
+        ref = oracle.spgemm(sr, A, B2)
+        dA, dB = h.DeviceCSR.from_host(A), h.DeviceCSR.from_host(B2)
+        assert_bitexact(h.spgemm(sr, dA, dB).to_host(), ref, f"spgemm {n}")
+        P = h.Plan(sr, dA, dB)
+        P.execute()
+        P.status()
+        assert_bitexact(P.C.to_host(), ref, f"plan {n}")
