@@ -141,13 +141,14 @@ int hs_spgemm(int semiring, const hs_mat *A, const hs_mat *B, hs_mat *C,
  * rows/columns).  This is the product R*A*Q with R = sparse(1:len(I), I, 1)
  * and Q = sparse(J, 1:len(J), 1), evaluated without forming R*A: the rows
  * I[t] are gathered, each entry (I[t], c) becomes (t, p) for every p with
- * J[p] == c, and every row is sorted by itself; where J repeats an index the
- * entries are ordered by a stable radix sort instead (where it is strictly
- * increasing they need no order).  Values are copied bit for bit.  Index
+ * J[p] == c, and every row is sorted by itself; where J repeats an index, or
+ * has more than 2^20 entries and enough rows of B more than 2048, the entries
+ * are ordered by a stable radix sort instead (where J is strictly increasing
+ * they need no order).  Values are copied bit for bit.  Index
  * ranges are always checked; with HS_FLAG_VALIDATE, A is checked to be
  * canonical too.  At most 2^31-1 entries of B unless J is strictly increasing;
- * two host synchronisations with `stream` when J repeats no index, up to five
- * otherwise.  Errors: HS_EINVAL (an index out of
+ * two host synchronisations with `stream` when J repeats no index (three with
+ * the radix sort), up to five otherwise.  Errors: HS_EINVAL (an index out of
  * range, bad shapes, NULL pointers), HS_ENONCANON (with HS_FLAG_VALIDATE),
  * HS_EUNSUPPORTED, HS_ENOMEM, HS_ECUDA. */
 int hs_spref(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ,

@@ -226,11 +226,45 @@ __global__ void __launch_bounds__(256) k_spref_emit(SprefArgs a, int32_t *Bj, vo
     copy_val(Bv, d, a.V, g, a.vb);
   }
 }
-__global__ void k_spref_offsets(SprefArgs a, int64_t *Bp) {
+// B's row offsets, the number of kept entries (longs[2]), and the rows that
+// the bitmap kernel below would take (longs[0]) with their entries (longs[1])
+__device__ __forceinline__ int64_t spref_kept(const SprefArgs &a, int64_t g) {
+  const int64_t w = g >> 5;
+  const int b = (int)(g & 31);
+  return (w ? a.S[w - 1] : 0) + (b ? __popc(a.keep[w] & ((1u << b) - 1u)) : 0);
+}
+__global__ void k_spref_offsets(SprefArgs a, int64_t *Bp, unsigned long long *longs) {
   GRID_STRIDE(t, a.nI + 1) {
-    const int64_t g = a.G[t], w = g >> 5;
-    const int b = (int)(g & 31);
-    Bp[t] = (w ? a.S[w - 1] : 0) + (b ? __popc(a.keep[w] & ((1u << b) - 1u)) : 0);
+    const int64_t g = a.G[t], b = spref_kept(a, g);
+    Bp[t] = b;
+    if (t == a.nI) {
+      longs[2] = (unsigned long long)b;
+    } else if (a.G[t + 1] - g > SR_CTA) {
+      const int64_t c = spref_kept(a, a.G[t + 1]) - b;
+      if (c > SR_CTA) {
+        atomicAdd(longs, 1ull);
+        atomicAdd(longs + 1, (unsigned long long)c);
+      }
+    }
+  }
+}
+// ti[d] = the row of B that kept entry d lies in
+__global__ void k_spref_row_ids(const int64_t *Bp, int64_t nI, int64_t ntup, int32_t *ti) {
+  __shared__ int64_t s_row[2];
+  const int64_t d0 = (int64_t)blockIdx.x * SG_TILE, d1 = min(d0 + SG_TILE, ntup);
+  if (threadIdx.x < 64) {
+    const int64_t r = warp_upper_bound(Bp, nI + 1, threadIdx.x < 32 ? d0 : d1 - 1) - 1;
+    if (lane_id() == 0) s_row[threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
+  for (int64_t d = d0 + threadIdx.x; d < d1; d += SG_NT) {
+    int64_t l = s_row[0], h = s_row[1] + 1;  // last row that starts at or before d
+    while (h - l > 1) {
+      const int64_t mid = (l + h) >> 1;
+      if (Bp[mid] <= d) l = mid;
+      else h = mid;
+    }
+    ti[d] = (int32_t)l;
   }
 }
 
@@ -239,8 +273,11 @@ __global__ void k_spref_offsets(SprefArgs a, int64_t *Bp) {
 // lanes a row of at most 8, a warp up to SR_WARP (ranks counted directly), a
 // block up to SR_CTA (buckets in shared memory), and longer ones through a
 // bitmap of B's columns (rank = set bits before p).  Every tuple is read and
-// written once; a radix sort of all (row, p) keys took five passes.
-constexpr int SR_WARP = 64, SR_CTA = 2048;
+// written once; a radix sort of all (row, p) keys took five passes.  Only the
+// bitmap's cost grows with B's width, a sweep and two reads of the row for
+// every 2^20 columns: spref_by_radix (internal.h) says when the radix sort is
+// taken after all.
+constexpr int SR_WARP = 64;
 template <typename T> struct SprefRowArgs {
   const int64_t *Bp;
   int64_t nI, nJ;
@@ -407,9 +444,16 @@ void launch_spref_gather(const SprefArgs &a, cudaStream_t st) {
   count_launch();
   k_spref_gather<<<(unsigned)((a.total + SG_TILE - 1) / SG_TILE), SG_NT, 0, st>>>(a);
 }
-void launch_spref_emit(const SprefArgs &a, int64_t *Bp, int32_t *Bj, void *Bv, cudaStream_t st) {
+void launch_spref_offsets(const SprefArgs &a, int64_t *Bp, unsigned long long *longs, cudaStream_t st) {
   count_launch();
-  k_spref_offsets<<<grid1(a.nI + 1), 256, 0, st>>>(a, Bp);
+  k_spref_offsets<<<grid1(a.nI + 1), 256, 0, st>>>(a, Bp, longs);
+}
+void launch_spref_row_ids(const int64_t *Bp, int64_t nI, int64_t ntup, int32_t *ti, cudaStream_t st) {
+  if (ntup <= 0) return;
+  count_launch();
+  k_spref_row_ids<<<(unsigned)((ntup + SG_TILE - 1) / SG_TILE), SG_NT, 0, st>>>(Bp, nI, ntup, ti);
+}
+void launch_spref_emit(const SprefArgs &a, int32_t *Bj, void *Bv, cudaStream_t st) {
   if (a.total <= 0) return;
   count_launch();
   k_spref_emit<<<grid1(a.total), 256, 0, st>>>(a, Bj, Bv);

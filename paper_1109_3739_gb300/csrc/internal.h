@@ -398,8 +398,30 @@ struct SprefArgs {
   uint32_t *keep;      // a bit per gathered entry
   int64_t *S;          // kept entries per word, then their inclusive scan
 };
+constexpr int SR_CTA = 2048;  // longest row that a block sorts in shared memory
+// Whether all tuples go through the radix sort because of the rows above SR_CTA
+// (`rows` of them with `entries` tuples), which a block of the bitmap kernel,
+// one an SM, takes one by one: 7.2 us and 0.39 ns an entry for every 2^20
+// columns of B, measured on rows of 3000 to 200,000 entries over 2^20 to 2^25
+// columns; the radix sort 60 us and 0.01 ns a tuple and pass (4e6 to 5e7
+// tuples).  20,000 rows of 2500 entries over 2^20 / 2^22 / 2^25 columns: 2.7 /
+// 6.3 / 39.4 ms for the call by bitmaps, 4.3 / 4.3 / 5.7 ms by the radix sort;
+// one row of 200,000 beside 4e6 tuples: 0.59 / 0.85 / 3.9 and 0.68 / 0.70 /
+// 1.4 ms; the rule takes the smaller in all of 24 such cases.
+inline bool spref_by_radix(int64_t rows, int64_t entries, int64_t ntup, int64_t nI, int64_t nJ) {
+  constexpr int64_t SMS = 152;
+  const int64_t chunks = (nJ + BITMAP_COLS - 1) / BITMAP_COLS;
+  if (rows <= 0 || chunks <= 1) return false;
+  int bits = 0;
+  for (int64_t x = nI - 1; x > 0; x >>= 1) ++bits;
+  for (int64_t x = nJ - 1; x > 0; x >>= 1) ++bits;
+  const double a_row = (double)chunks * (7200.0 + 0.39 * (double)entries / (double)rows);
+  return (double)((rows + SMS - 1) / SMS) * a_row > 60000.0 + 0.01 * (double)ntup * ((bits + 7) / 8);
+}
 void launch_spref_gather(const SprefArgs &a, cudaStream_t st);
-void launch_spref_emit(const SprefArgs &a, int64_t *Bp, int32_t *Bj, void *Bv, cudaStream_t st);
+void launch_spref_offsets(const SprefArgs &a, int64_t *Bp, unsigned long long *longs, cudaStream_t st);
+void launch_spref_row_ids(const int64_t *Bp, int64_t nI, int64_t ntup, int32_t *ti, cudaStream_t st);
+void launch_spref_emit(const SprefArgs &a, int32_t *Bj, void *Bv, cudaStream_t st);
 void launch_spref_rows(int vb, const int64_t *Bp, int64_t nI, int64_t nJ, const int32_t *P, const void *V, int32_t *Bj,
                        void *Bv, int64_t lmax, int *count, int32_t *list, long long *dbg, cudaStream_t st);
 void launch_row_starts(const int64_t *G, int64_t nI, int64_t total, int64_t *inc, cudaStream_t st);

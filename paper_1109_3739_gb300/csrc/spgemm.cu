@@ -921,7 +921,8 @@ static int sparse_impl(const int32_t *I, const int32_t *J, const void *V, int64_
 // tuple or none, the tuples lie row by row, and only the rows are sorted (not
 // even those when J is increasing); two host synchronisations.  When J
 // repeats indices the tuples are ordered by (t, p) with the radix sort of
-// sparse(); five host synchronisations.
+// sparse(); five host synchronisations.  So they are, with three, where many
+// long rows meet a wide J (spref_by_radix).
 static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ, hs_mat *Bout,
                       Mem &mem, Mem &outmem, uint32_t flags) {
   cudaStream_t st = mem.st;
@@ -936,7 +937,7 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     int flag[2];
     int count[5];
     int pad;
-    unsigned long long lmax, qmax;
+    unsigned long long lmax, qmax, longs[3];
     int64_t total;
     long long dbg[2];
   };
@@ -968,24 +969,30 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
   const bool repeats = fl & 2, increasing = !(fl & 4);
   const int64_t total = hb->total, lmax = (int64_t)hb->lmax;
 
-  auto out = [&](int64_t nnz) {
+  auto out_ptr = [&]() {
     memset(Bout, 0, sizeof(*Bout));
     Bout->fmt = HS_CSR;
     Bout->dtype = A->dtype;
     Bout->m = nI;
     Bout->n = nJ;
-    Bout->nnz = nnz;
     Bout->ptr = (int64_t *)outmem.raw(sizeof(int64_t) * (size_t)(nI + 1));
+    return Bout->ptr != nullptr;
+  };
+  auto out = [&](int64_t nnz) {
+    Bout->nnz = nnz;
     Bout->idx = (int32_t *)outmem.raw(sizeof(int32_t) * (size_t)(nnz > 0 ? nnz : 1));
     Bout->val = vb ? outmem.raw((size_t)vb * (size_t)(nnz > 0 ? nnz : 1)) : nullptr;
-    return Bout->ptr && Bout->idx && (!vb || Bout->val);
+    return Bout->idx && (!vb || Bout->val);
   };
   auto empty_out = [&]() -> int {
-    if (!out(0)) return HS_ENOMEM;
+    if (!out_ptr() || !out(0)) return HS_ENOMEM;
     CK(cudaMemsetAsync(Bout->ptr, 0, sizeof(int64_t) * (size_t)(nI + 1), st));
     return check_launch();
   };
   if (total == 0 || nJ == 0) return empty_out();
+  // every (t, p) occurs once, so the combining operation of the radix sort
+  // never acts: values are copied bit for bit whatever the operation
+  const int sr = A->dtype == HS_BOOL ? HS_OR_AND : A->dtype == HS_I32 ? HS_MIN_PLUS : HS_PLUS_TIMES;
 
   if (!repeats) {
     const int64_t nw = (total + 31) / 32;
@@ -996,30 +1003,49 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     int64_t *stmp = mem.tmp<int64_t>((size_t)scan_tmp_elems(nw));
     if (mem.failed) return HS_ENOMEM;
     const SprefArgs a{A->ptr, A->idx, A->val, vb, I, nI, n, G, total, pos, P, V, keep, S};
+    // B's offsets are needed now only where spref_by_radix may say yes
+    const bool look = !increasing && lmax > SR_CTA && nJ > BITMAP_COLS;
     {
       PhaseTimer t("spref_gather", st);
       launch_spref_gather(a, st);
       launch_scan_i64(S, nw, stmp, st);
+      if (look) {
+        if (!out_ptr()) return HS_ENOMEM;
+        launch_spref_offsets(a, Bout->ptr, sb->longs, st);
+      }
     }
+    if (look) CK(cudaMemcpyAsync(hb->longs, sb->longs, sizeof(sb->longs), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(&hb->total, S + nw - 1, 8, cudaMemcpyDeviceToHost, st));
     if (int e = check_launch()) return e;
     CK(cudaStreamSynchronize(st));
     const int64_t ntup = hb->total;
-    if (ntup == 0) return empty_out();
+    if (ntup == 0 && !look) return empty_out();
     if (!increasing && ntup > 0x7fffffffLL) return HS_EUNSUPPORTED;
-    if (!out(ntup)) return HS_ENOMEM;
-    PhaseTimer t("spref_emit", st);
+    const bool radix = look && spref_by_radix((int64_t)hb->longs[0], (int64_t)hb->longs[1], ntup, nI, nJ);
+    if (!look && !out_ptr()) return HS_ENOMEM;
+    if (!radix && !out(ntup)) return HS_ENOMEM;
+    if (ntup == 0) return check_launch();  // (the offsets are all zero)
+    std::unique_ptr<PhaseTimer> t(new PhaseTimer("spref_emit", st));
+    if (!look) launch_spref_offsets(a, Bout->ptr, sb->longs, st);
     if (increasing) {
-      launch_spref_emit(a, Bout->ptr, Bout->idx, Bout->val, st);
+      launch_spref_emit(a, Bout->idx, Bout->val, st);
       return check_launch();
     }
     int32_t *tp = mem.tmp<int32_t>((size_t)ntup);
     void *tv = vb ? (void *)mem.tmp<char>((size_t)vb * (size_t)ntup) : nullptr;
-    int32_t *list = mem.tmp<int32_t>((size_t)(2 * nI));
+    int32_t *list = mem.tmp<int32_t>((size_t)(radix ? ntup : 2 * nI));  // (radix: the tuples' rows)
     if (mem.failed) return HS_ENOMEM;
-    launch_spref_emit(a, Bout->ptr, tp, tv, st);
-    launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
-    return check_launch();
+    launch_spref_emit(a, tp, tv, st);
+    if (!radix) {
+      launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
+      return check_launch();
+    }
+    launch_spref_row_ids(Bout->ptr, nI, ntup, list, st);
+    t.reset();
+    outmem.release(Bout->ptr, sizeof(int64_t) * (size_t)(nI + 1));
+    Bout->ptr = nullptr;
+    if (int e = check_launch()) return e;
+    return sparse_impl(list, tp, tv, ntup, nI, nJ, A->dtype, sr, Bout, mem, outmem, flags);
   }
 
   // Q = sparse(J, 1:len(J), 1, n, len(J)): row k holds every p with J[p] == k,
@@ -1082,9 +1108,6 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     launch_gather_fill(ga, W, ti, pj, tv, st);
   }
   if (int e = check_launch()) return e;
-  // every (t, p) occurs once, so the combining operation never acts: values
-  // are copied bit for bit whatever the operation
-  const int sr = A->dtype == HS_BOOL ? HS_OR_AND : A->dtype == HS_I32 ? HS_MIN_PLUS : HS_PLUS_TIMES;
   return sparse_impl(ti, pj, tv, ntup, nI, nJ, A->dtype, sr, Bout, mem, outmem, flags);
 }
 
