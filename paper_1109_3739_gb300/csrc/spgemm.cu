@@ -139,8 +139,14 @@ struct Mem {
       const size_t room = ((bytes ? bytes : 1) + 255) & ~(size_t)255;
       if (room > chunk_left) {
         chunk_left = 0;
+        const bool before = failed;
         chunk = (char *)raw(CHUNK);
-        if (!chunk) return nullptr;
+        if (!chunk) {  // an allocator of small blocks, or too little memory left: the block alone
+          failed = before;
+          T *p = (T *)raw(bytes);
+          if (p) scratch.push_back({p, bytes});
+          return p;
+        }
         scratch.push_back({chunk, CHUNK});
         chunk_left = CHUNK;
       }
