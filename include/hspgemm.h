@@ -369,8 +369,8 @@ int hs_batch_plan_phase_ms(hs_batch_plan *plan, double *ms, void *stream);
  * C->ptr (A->m + 1 int64), C->idx (capacity int32) and, for typed results,
  * C->val (capacity values) already allocated on the device.  The call fills
  * C->ptr, C->idx, C->val and sets C's shape, dtype and nnz.  Temporaries come
- * from one fixed device array of HS_NOALLOC_SCRATCH_MAX bytes inside the
- * library, which every GPU that loads the library holds until the process
+ * from one fixed device array of HS_NOALLOC_SCRATCH_MAX bytes (and 4 KB of
+ * counters) inside the library, which every GPU that loads the library holds until the process
  * exits; host-side readbacks use ordinary host memory.
  *   - HS_ESCRATCH: the product needs more scratch than the maximum (roughly
  *     16 bytes per row of A, plus 4 bytes per 4096 columns for every row of

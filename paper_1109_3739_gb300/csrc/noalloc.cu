@@ -25,8 +25,9 @@
 namespace hs {
 
 // the fixed scratch: every GPU that loads the library holds it until exit
-constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)HS_NOALLOC_SCRATCH_MAX;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
+// (with the counters, of fixed size, behind the temporaries)
+constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)HS_NOALLOC_SCRATCH_MAX, NOALLOC_COUNTER_BYTES = 4096;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_COUNTER_BYTES];
 
 // In host code g_noalloc_scratch names a host-side stand-in, not device
 // memory: its device address is looked up once per device (with that device
@@ -87,6 +88,8 @@ struct NaBlock {  // device counters, read back to host memory
   long long nnz;
   long long dbg[2];
 };
+
+static_assert(sizeof(NaBlock) <= NOALLOC_COUNTER_BYTES, "the counters fit behind the scratch");
 
 static int cuda_fail(cudaError_t e) {
   (void)e;
@@ -176,7 +179,7 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   void *sp = nullptr;
   if (int e = noalloc_scratch(&sp)) return e;
   Arena ar{reinterpret_cast<unsigned char *>(sp), NOALLOC_SCRATCH_BYTES};
-  NaBlock *sb = ar.take<NaBlock>(1);
+  NaBlock *sb = reinterpret_cast<NaBlock *>(ar.base + NOALLOC_SCRATCH_BYTES);
   int64_t *f = ar.take<int64_t>(nslots);
   int *list = ar.take<int>(nslots);
   int32_t *hslot = ar.take<int32_t>(nslots);
