@@ -51,6 +51,8 @@ template <class R> struct SideSet {
 // for each of the caller's streams, so that work of two streams is not queued
 // behind each other; with more streams than sets the one used longest ago is
 // taken over, which costs its two streams their independence and nothing else.
+// A set from here serves the stream it was asked for: device and priority are
+// looked at, and a call that waits for the GPU takes part in no capture.
 template <class R> struct SidePool {
   static constexpr int MOST = 8;
   struct Entry {
@@ -103,9 +105,10 @@ template <class R> struct FanOf {
   Stream main;
   SideSet<R> *d = nullptr;
   bool used[FAN_SIDES] = {false};
-  // groups: bit g set when group g has work; with one group nothing is forked
-  FanOf(Stream st, unsigned groups, SideSet<R> *set) : main(st) {
-    if ((groups & (groups - 1)) == 0 || !set || !set->serves(main)) return;
+  // groups: bit g set when group g has work; with one group nothing is forked.
+  // serves: known to hold for the set.
+  FanOf(Stream st, unsigned groups, SideSet<R> *set, bool serves = false) : main(st) {
+    if ((groups & (groups - 1)) == 0 || !set || !(serves || set->serves(main))) return;
     if (R::record(set->fork, main)) d = set;
   }
   FanOf(const FanOf &) = delete;

@@ -553,6 +553,11 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   const int nhist = hb->nhist;
   const int tiny_group = tiny_group_pays(key_off[KEY_TINY + 1] - key_off[KEY_TINY], hb->stats[4]);
   const bool side_by_side = hb->stats[0] <= FAN_PRODUCTS;
+  SideSet<FanCuda> *sides = nullptr;
+  auto sides_for = [&](unsigned groups) {
+    if (!sides && (groups & (groups - 1))) sides = t_sides.of(st);
+    return sides;
+  };
   const int pair_long = hb->stats[2] > (unsigned long long)PAIR_LONG;  // (read before hb is copied to again)
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
 
@@ -680,7 +685,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     for (const SymBin &x : bins_)
       if (side_by_side && key_off[x.k1] > key_off[x.k0]) groups |= 1u << x.group;
     PhaseTimer t("symbolic", st);
-    Fan fan(st, groups, groups & (groups - 1) ? t_sides.of(st) : nullptr);
+    Fan fan(st, groups, sides_for(groups), true);
     for (const SymBin &x : bins_) {
       sa.list = list + key_off[x.k0];
       sa.count = key_off[x.k1] - key_off[x.k0];
@@ -794,7 +799,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   }
   if (nheavy > 0) alloc_bci();  // (every allocation before the streams part: they are ordered on the caller's)
   std::unique_ptr<PhaseTimer> t_num(new PhaseTimer("numeric", st));
-  Fan fan(st, groups, groups & (groups - 1) ? t_sides.of(st) : nullptr);
+  Fan fan(st, groups, sides_for(groups), true);
   // heavy bin: the B segment index, and the units' B segments
   const cudaStream_t hst = nheavy > 0 ? fan.stream(num_group(NUM_KINDS - 1)) : st;
   if (bci) {
