@@ -703,11 +703,15 @@ def time_device(fn, steps, warmup, flush, stream):
     return statistics.median(ts), (h.launch_count() - l0) // max(1, steps), out
 
 
-def bin_rows(t, f, cnt, cap_large=8192):
+HUB_ENTRIES, HUB_LEVELS, HUB_ROWS = 4096, 6, 304  # as the library's (checked by a test)
+
+
+def bin_rows(t, f, cnt, cap_large=8192, entries=None):
     """Masks over A's rows of every symbolic and numeric bin, as the library bins
     a product with 4-byte values whose B is too wide for the dense accumulator:
     the tuning values clamped as the library clamps them, then the row keys taken
-    in the library's order (f: products per row, cnt: outputs per row)."""
+    in the library's order (f: products per row, cnt: outputs per row), then the
+    hub rows moved (entries: A's entries per row; None: no hub rows)."""
     def clamp(x, lo, hi):
         return min(max(int(x), lo), hi)
     ws = clamp(t["warp_s_max"], 32, 128)
@@ -754,6 +758,18 @@ def bin_rows(t, f, cnt, cap_large=8192):
     take("numeric_large_s", cnt <= ls)
     take("numeric_large", cnt <= cap_large)
     out["numeric_heavy"] = heavy | rest
+    if entries is not None:
+        # rows of many entries outside the tiny and heavy bins, by levels of four times the entries: the levels
+        # from the lowest one that at most HUB_ROWS rows reach
+        entries = np.asarray(entries, dtype=np.int64)
+        always = out["numeric_large_s"] & (entries > HUB_ENTRIES)
+        level = sum((entries > HUB_ENTRIES << 2 * i).astype(np.int64) for i in range(HUB_LEVELS)) - 1
+        level[(cnt <= 0) | out["numeric_tiny"] | out["numeric_heavy"] | out["numeric_large"] | always] = -1
+        first = next((i for i in range(HUB_LEVELS) if np.count_nonzero(level >= i) <= HUB_ROWS), HUB_LEVELS)
+        hub = (level >= first) | always
+        for name in [k for k in out if k.startswith("numeric_")]:
+            out[name] = out[name] & ~hub
+        out["numeric_large"] = out["numeric_large"] | hub
     return out
 
 
@@ -1021,7 +1037,7 @@ def main():
     cnt = np.diff(c_rowptr)
     deg = np.diff(A.rowptr)
     t = h.get_tuning()  # the thresholds in force
-    in_bin = bin_rows(t, f, cnt)[dom]
+    in_bin = bin_rows(t, f, cnt, entries=deg)[dom]
     vb = 4
     b_bytes = (A.m + 1) * 8 + A.nnz * (4 + vb)
     a_bytes = int(in_bin.sum()) * 8 + int(deg[in_bin].sum()) * (4 + vb)

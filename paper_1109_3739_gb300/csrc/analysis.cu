@@ -105,10 +105,33 @@ __device__ __forceinline__ bool last_block(int *ticket, int *s_flag) {
   __threadfence();
   return true;
 }
-// one warp: exclusive scan of the NKEYS counters into offsets and cursors
-__device__ __forceinline__ void key_offsets(const int *cnt, int *off, int *cur) {
+// one warp: exclusive scan of the NKEYS counters into offsets and cursors;
+// with `hub`, which hub rows are moved, and the counts with them there
+__device__ __forceinline__ void key_offsets(const int *cnt, int *off, int *cur, HubRows *hub = nullptr) {
+  static_assert(HUB_KEYS <= 32, "a key per lane");
   const int lane = lane_id();
-  const int a = __ldcg(cnt + 2 * lane), b = __ldcg(cnt + 2 * lane + 1);
+  int a = __ldcg(cnt + 2 * lane), b = __ldcg(cnt + 2 * lane + 1);
+  if (hub) {  // (uniform)
+    int rows[HUB_LEVELS], mine[HUB_LEVELS];  // of all keys, of key KEY_TINY + 1 + lane
+    const int any = __ldcg(&hub->any);
+#pragma unroll
+    for (int l = 0; l < HUB_LEVELS; ++l) rows[l] = mine[l] = lane < HUB_KEYS ? __ldcg(&hub->n[l][lane]) : 0;
+    if (any) {  // (else `from` stays zero: no row reaches a level)
+#pragma unroll
+      for (int l = 0; l < HUB_LEVELS; ++l) rows[l] = warp_sum(rows[l]);
+      const int from = hub_from(rows);
+      if (lane == 0) hub->from = from;
+      int moved = 0;
+#pragma unroll
+      for (int l = 0; l < HUB_LEVELS; ++l) moved += l >= from ? mine[l] : 0;
+      const int all = warp_sum(moved);
+      // (lanes from HUB_KEYS on hold none)
+      a -= __shfl_sync(FULL, moved, (2 * lane - KEY_TINY - 1) & 31) * (2 * lane > KEY_TINY && 2 * lane < KEY_SPA);
+      b -= __shfl_sync(FULL, moved, (2 * lane - KEY_TINY) & 31) * (2 * lane + 1 > KEY_TINY && 2 * lane + 1 < KEY_SPA);
+      a += 2 * lane == KEY_LARGE ? all : 0;
+      b += 2 * lane + 1 == KEY_LARGE ? all : 0;
+    }
+  }
   const int incl = warp_incl_scan(a + b);
   const int ex = incl - a - b;
   off[2 * lane] = ex;
@@ -475,8 +498,14 @@ __global__ void __launch_bounds__(TL_NT) k_num_count(RowSet A, const int64_t *f,
     const int64_t n = r < A.m ? cnt[r + 1] : 0;
     sum += n;
     if (r < A.nslots) {
-      const int key = hub_key(num_key(f[r], A.ids ? raw_count(A, cnt, r) : n, bins), A.p[r + 1] - A.p[r]);
+      const int64_t entries = A.p[r + 1] - A.p[r];
+      const int key = row_key(f[r], A.ids ? raw_count(A, cnt, r) : n, entries, bins);
       if (key) atomicAdd(hist + key, 1);
+      const int level = hub_level(key, entries);
+      if (level >= 0) {  // (few: a row for every 4096 entries at most)
+        atomicAdd(&c.hub->n[level][key - KEY_TINY - 1], 1);
+        c.hub->any = 1;
+      }
     }
   }
   sum = warp_sum(sum);
@@ -490,7 +519,7 @@ __global__ void __launch_bounds__(TL_NT) k_num_count(RowSet A, const int64_t *f,
   for (int i = threadIdx.x; i < NKEYS; i += TL_NT)
     if (hist[i]) atomicAdd(c.cnt + i, hist[i]);
   if (!last_block(c.ticket, &s_last)) return;
-  if (threadIdx.x < 32) key_offsets(c.cnt, c.off, c.cur);
+  if (threadIdx.x < 32) key_offsets(c.cnt, c.off, c.cur, c.hub);
   // exclusive scan of the tile sums, in place
   long long run = 0;
   for (int64_t b = 0; b < tiles; b += TL_TILE) {
@@ -513,10 +542,11 @@ __global__ void __launch_bounds__(TL_NT) k_num_count(RowSet A, const int64_t *f,
 }
 template <bool LISTS>
 __global__ void __launch_bounds__(TL_NT) k_num_offsets(RowSet A, const int64_t *f, int64_t *cnt, BinCfg bins,
-                                                       int *key_cur, const int64_t *tsum, int *list) {
+                                                       BinCounters c, const int64_t *tsum, int *list) {
   __shared__ int s_cnt[NKEYS];
   __shared__ long long s_tot[64];
   if (threadIdx.x < NKEYS) s_cnt[threadIdx.x] = 0;
+  const int from = c.hub->from;
   const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
   long long v[TL_PER];
   int key[TL_PER];
@@ -526,7 +556,10 @@ __global__ void __launch_bounds__(TL_NT) k_num_offsets(RowSet A, const int64_t *
     v[u] = r < A.m ? cnt[r + 1] : 0;
     key[u] = 0;
     if constexpr (LISTS)
-      if (r < A.nslots) key[u] = hub_key(num_key(f[r], v[u], bins), A.p[r + 1] - A.p[r]);
+      if (r < A.nslots) {
+        const int64_t entries = A.p[r + 1] - A.p[r];
+        key[u] = hub_key(row_key(f[r], v[u], entries, bins), entries, from);
+      }
   }
   tile_scan(v, s_tot);
   const int64_t base = tsum[blockIdx.x];
@@ -535,21 +568,23 @@ __global__ void __launch_bounds__(TL_NT) k_num_offsets(RowSet A, const int64_t *
     const int64_t r = r0 + u * TL_NT + threadIdx.x;
     if (r < A.m) cnt[r + 1] = base + v[u];
   }
-  if constexpr (LISTS) append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
+  if constexpr (LISTS) append_tile(key, r0, s_cnt, c.cur, list, A.nslots, A.dbg);
 }
 __global__ void __launch_bounds__(TL_NT) k_num_lists(RowSet A, const int64_t *f, const int64_t *cnt, BinCfg bins,
-                                                     int *key_cur, int *list) {
+                                                     BinCounters c, int *list) {
   __shared__ int s_cnt[NKEYS];
   if (threadIdx.x < NKEYS) s_cnt[threadIdx.x] = 0;
+  const int from = c.hub->from;
   __syncthreads();
   const int64_t r0 = (int64_t)blockIdx.x * TL_TILE;
   int key[TL_PER];
 #pragma unroll
   for (int u = 0; u < TL_PER; ++u) {
     const int64_t r = r0 + u * TL_NT + threadIdx.x;
-    key[u] = r < A.nslots ? hub_key(num_key(f[r], raw_count(A, cnt, r), bins), A.p[r + 1] - A.p[r]) : 0;
+    const int64_t entries = r < A.nslots ? A.p[r + 1] - A.p[r] : 0;
+    key[u] = r < A.nslots ? hub_key(row_key(f[r], raw_count(A, cnt, r), entries, bins), entries, from) : 0;
   }
-  append_tile(key, r0, s_cnt, key_cur, list, A.nslots, A.dbg);
+  append_tile(key, r0, s_cnt, c.cur, list, A.nslots, A.dbg);
 }
 void launch_num_bins(const RowSet &A, const int64_t *f, int64_t *cnt, const BinCfg &bins, const BinCounters &c,
                      int64_t *tsum, long long *nnz, int *list, cudaStream_t st) {
@@ -560,12 +595,12 @@ void launch_num_bins(const RowSet &A, const int64_t *f, int64_t *cnt, const BinC
   k_num_count<<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c, tsum, tiles, nnz);
   if (A.ids) {
     count_launch();
-    k_num_lists<<<(unsigned)((A.nslots + TL_TILE - 1) / TL_TILE), TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, list);
+    k_num_lists<<<(unsigned)((A.nslots + TL_TILE - 1) / TL_TILE), TL_NT, 0, st>>>(A, f, cnt, bins, c, list);
     count_launch();
-    k_num_offsets<false><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, tsum, list);
+    k_num_offsets<false><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c, tsum, list);
   } else {
     count_launch();
-    k_num_offsets<true><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c.cur, tsum, list);
+    k_num_offsets<true><<<(unsigned)tiles, TL_NT, 0, st>>>(A, f, cnt, bins, c, tsum, list);
   }
 }
 

@@ -126,14 +126,44 @@ __host__ __device__ inline int num_key(int64_t f, int64_t c, const BinCfg &b) {
 inline bool tiny_group_pays(int64_t rows, unsigned long long products) {
   return rows >= 65536 && products <= 8ull * (unsigned long long)rows;
 }
-// A row whose key is a warp's or a small block's, but which has more than
-// HUB_ENTRIES entries of A, goes to the kernel of 1024 threads: its time is
-// not its products' but the rounds of entries that are looked up (3.5e4
-// entries with one product each: 0.52 ms as the last row of the kernel of 256
-// threads, 137 rounds of 3.8 us, whatever else ran beside it).
+// Hub rows: rows whose key is a warp's or a small block's, but which have many
+// entries of A, go to the kernel of 1024 threads, which looks up four times as
+// many at once (1 / 30 rows of 5000 entries with a product each, 256 columns:
+// 55 / 53 us a numeric pass, 78 / 76 in the kernel of 256 threads; of 40,000:
+// 253 / 234 and 463 / 407).  But it runs one block an SM, so many rows wait for
+// one another (300 / 1000 / 3000 rows of 5000 over 300 columns: 87 / 223 / 587
+// us, 83 / 144 / 322 in the other kernel; over 1400 columns, f32: 88 / 227 / 597
+// and 117 / 220 / 512): the rows are counted by levels of four times the
+// entries, and only those above the lowest level that at most HUB_ROWS rows, two
+// an SM, exceed are moved.  The kernels of more than 1024 outputs with 8-byte
+// values hold three rows an SM and lose however many there are (over 1400
+// columns, f64: 99 / 261 / 693 moved, 123 / 381 / 919 not): hub_always.
 constexpr int64_t HUB_ENTRIES = 4096;
-__host__ __device__ inline int hub_key(int key, int64_t entries) {
-  return entries > HUB_ENTRIES && key > KEY_TINY && key < KEY_SPA ? KEY_LARGE : key;
+constexpr int HUB_LEVELS = 6, HUB_ROWS = 304, HUB_KEYS = KEY_SPA - KEY_TINY - 1;
+__host__ __device__ inline bool hub_always(int key, const BinCfg &b) {
+  return key == KEY_LARGE_S || (key == KEY_MID && b.cap_large <= CAP_MID * 2);
+}
+// a row's key before its hub level is looked at
+__host__ __device__ inline int row_key(int64_t f, int64_t c, int64_t entries, const BinCfg &b) {
+  const int key = num_key(f, c, b);
+  return entries > HUB_ENTRIES && hub_always(key, b) ? KEY_LARGE : key;
+}
+// the highest level that a row with such a key exceeds, -1 if none (without a
+// branch, as the key functions)
+__host__ __device__ inline int hub_level(int key, int64_t entries) {
+  int l = -1;
+#pragma unroll
+  for (int i = 0; i < HUB_LEVELS; ++i) l += entries > HUB_ENTRIES << 2 * i;
+  return (key > KEY_TINY) & (key < KEY_SPA) & (key != KEY_LARGE) ? l : -1;
+}
+// the lowest level moved (HUB_LEVELS: none), given the rows of each level
+__host__ __device__ inline int hub_from(const int (&rows)[HUB_LEVELS]) {
+  int n = 0, from = HUB_LEVELS;
+  for (int l = HUB_LEVELS - 1; l >= 0 && (n += rows[l]) <= HUB_ROWS; --l) from = l;
+  return from;
+}
+__host__ __device__ inline int hub_key(int key, int64_t entries, int from) {
+  return hub_level(key, entries) >= from ? KEY_LARGE : key;
 }
 // the default thresholds for a value width, clamped tuning values otherwise
 BinCfg bin_config(int value_bytes);
@@ -188,11 +218,18 @@ template <class K> inline int fit_per_sm(K kernel, int threads, size_t smem) {
 
 // --------------------------------------------------------------- launchers
 // analysis.cu
+// hub rows by level and by the key that they would have (zeroed before each
+// binning), and the lowest level that is moved
+struct HubRows {
+  int n[HUB_LEVELS][HUB_KEYS];
+  int any, from;
+};
 // a binning's device counters: rows per key, the keys' list offsets and write
 // cursors, and a ticket that finds the last block (counts and ticket zeroed
 // before each binning)
 struct BinCounters {
   int *cnt, *off, *cur, *ticket;
+  HubRows *hub;  // numeric binning only
 };
 // products per row (f zeroed before) and the A entries with an empty B row;
 // then the rows' symbolic keys, their offsets, and stats[0] total flops, [1]

@@ -87,6 +87,7 @@ struct NaBlock {  // device counters, read back to host memory
   unsigned long long stats[5];
   long long nnz;
   long long dbg[2];
+  HubRows hub;
 };
 
 static_assert(sizeof(NaBlock) <= NOALLOC_COUNTER_BYTES, "the counters fit behind the scratch");
@@ -192,8 +193,8 @@ static int spgemm_noalloc_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat 
   RightOp rb{B->ptr, B->idx, B->val, n, B->m, B->nnz, sb->dbg};
   NA_CK(cudaMemsetAsync(sb, 0, sizeof(NaBlock), st));
   NA_CK(cudaMemsetAsync(f, 0, sizeof(int64_t) * (size_t)nslots, st));
-  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0]};
-  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1]};
+  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0], nullptr};
+  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1], &sb->hub};
   launch_flops(rs, rb, f, &sb->zeros, st);
   launch_row_keys(rs, f, nullptr, sym_c, sb->stats, bins, n, st);
   launch_scatter_sym(rs, f, sb->key_cur, list, hslot, &sb->nhist, bins, st);

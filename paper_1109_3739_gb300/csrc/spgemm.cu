@@ -321,6 +321,7 @@ struct SmallBlock {  // device counters, read back in one copy
   unsigned long long lpool;  // heavy rows' column lists: pool entries handed out
   int bci_cnt;               // B segment index rows handed out
   int pad2;
+  HubRows hub;
   long long nunits;          // numeric heavy units (column parts of rows with lists)
   long long npcap;           // their room in the pair arrays
   long long nnz;
@@ -529,8 +530,8 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   SmallBlock *hb = (SmallBlock *)pinned(sizeof(SmallBlock));
   if (!hb) return HS_ECUDA;
   CK(cudaMemsetAsync(zeroed, 0, sb_bytes + sizeof(int64_t) * (size_t)nslots, st));
-  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0]};
-  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1]};
+  const BinCounters sym_c{sb->key_cnt[0], sb->key_off, sb->key_cur, &sb->ticket[0], nullptr};
+  const BinCounters num_c{sb->key_cnt[1], sb->key_off, sb->key_cur, &sb->ticket[1], &sb->hub};
   {
     PhaseTimer t("analysis", st);
     if (flags & HS_FLAG_VALIDATE) {

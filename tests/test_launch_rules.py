@@ -44,3 +44,27 @@ def test_spref_leaves_the_bitmap_where_b_is_wide(tmp_path):
       for (int64_t len : {2049, 20000})
         CHECK(!spref_by_radix(r, r * len, 2 * r * len, 200000, n) ||
               spref_by_radix(r, r * len, 2 * r * len, 200000, n * 2));""")
+
+
+def test_hub_rows_are_moved_while_they_are_few(tmp_path):
+    """Rows of many entries of A take the kernel of 1024 threads, a block an SM, only as long as at most HUB_ROWS of
+    them do: the longest ones where there are more."""
+    run(tmp_path, r"""
+  const int none[HUB_LEVELS] = {0}, few[HUB_LEVELS] = {3, 2, 1}, many[HUB_LEVELS] = {3000}, mixed[HUB_LEVELS] = {500, 100, 30, 5};
+  const int edge[HUB_LEVELS] = {HUB_ROWS}, over[HUB_LEVELS] = {HUB_ROWS + 1}, all[HUB_LEVELS] = {9, 9, 9, 9, 9, 1000};
+  CHECK(hub_from(none) == 0 && hub_from(few) == 0 && hub_from(edge) == 0);
+  CHECK(hub_from(many) == 1 && hub_from(over) == 1);   // none of those: their level is 0
+  CHECK(hub_from(mixed) == 1 && hub_from(all) == HUB_LEVELS);
+  CHECK(hub_level(KEY_MID, HUB_ENTRIES) < 0 && hub_level(KEY_MID, HUB_ENTRIES + 1) == 0);
+  CHECK(hub_level(KEY_MID, 4 * HUB_ENTRIES) == 0 && hub_level(KEY_MID, 4 * HUB_ENTRIES + 1) == 1);
+  CHECK(hub_level(KEY_MID, 1LL << 40) == HUB_LEVELS - 1);
+  for (int key : {0, KEY_TINY, KEY_LARGE, KEY_SPA, KEY_HEAVY, NKEYS - 1}) CHECK(hub_key(key, 1 << 20, 0) == key);
+  BinCfg narrow{}, wide{};
+  narrow.cap_large = 8192;
+  wide.cap_large = 4096;
+  CHECK(!hub_always(KEY_MID, narrow) && hub_always(KEY_MID, wide) && !hub_always(KEY_MID_S, wide) && hub_always(KEY_LARGE_S, narrow));
+  for (int key = KEY_TINY + 1; key < KEY_SPA; ++key) {
+    if (key == KEY_LARGE) continue;
+    CHECK(hub_key(key, 5000, 0) == KEY_LARGE && hub_key(key, 5000, 1) == key && hub_key(key, 4096, 0) == key);
+    CHECK(hub_key(key, 20000, 1) == KEY_LARGE && hub_key(key, 1LL << 40, HUB_LEVELS) == key);
+  }""")
