@@ -842,11 +842,30 @@ void launch_plan_parts(const RowSet &A, const int *list, int count, const int32_
 // row's units, and scanned the products of its segments, which the unit
 // kernel now does as it copies them.  The searches of many units run at
 // once, so their latency is hidden here instead of sitting on the numeric
-// kernel's path.  A row with more than PAIR_LONG entries of A is left to
+// kernel's path.  A row with more than long_from entries of A is left to
 // k_build_pairs_long: a block per unit, four entries per thread at a time
 // (the few units of a product with 1e5-entry rows of A would keep one warp
 // each busy long after the others are done).
-constexpr int PAIR_NT = 256, PAIR_U = 4, PAIR_GROUP = 8;
+constexpr int PAIR_NT = 256, PAIR_U = 4, PAIR_GROUP = 8, PAIR_LONG = 1024, PAIR_SHARE = 2;
+// consecutive units per warp: as few as leave no warp of the GPU a second group
+static int64_t pair_warps() { return (int64_t)sm_count() * 40; }
+static int pair_group(int64_t nunits) {
+  const int64_t g = (nunits + pair_warps() - 1) / pair_warps();
+  return (int)(g < 1 ? 1 : (g > PAIR_GROUP ? PAIR_GROUP : g));
+}
+// A row is long when a warp's group of its units is more than PAIR_SHARE times
+// the warp's share of the whole layout (`entries`, summed over the units): rows
+// that are all long keep every warp as busy as blocks do, and are gone through
+// once for several units (3000 rows of 5000 / 10,000 entries, eight units each:
+// a numeric pass 1.39 / 2.63 ms, by blocks 1.77 / 3.28, the warps in one and a
+// third rounds of smaller groups 1.74 / 3.49; R-MAT scale 20, whose rows have up
+// to 23,000 entries: the layout 4.6 -> 2.5 ms, the product 67.9 -> 65.8 ms).  At
+// four times the share, 300 such rows took 377 / 704 us, by blocks 207 / 360.
+int64_t pair_long_from(int64_t nunits, int64_t entries, int64_t longest) {
+  const int64_t share = PAIR_SHARE * (entries / (pair_warps() * pair_group(nunits)));
+  const int64_t from = share > PAIR_LONG ? share : PAIR_LONG;
+  return longest > from ? from : INT64_MAX;
+}
 template <int AB> struct PairVal {
   using T = typename std::conditional<AB == 8, unsigned long long, unsigned>::type;
 };
@@ -884,7 +903,7 @@ __device__ __forceinline__ int64_t pair_end(const RightOp &B, int64_t base, int6
 template <int AB>
 __global__ void __launch_bounds__(PAIR_NT) k_build_pairs(RowSet A, RightOp B, HeavyUnit *units, int64_t nunits,
                                                          const int32_t *bci_id, const int32_t *bci, int nseg,
-                                                         int64_t *pseg, void *paval, int group) {
+                                                         int64_t *pseg, void *paval, int group, int64_t long_from) {
   using VT = typename PairVal<AB>::T;
   const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -909,7 +928,7 @@ __global__ void __launch_bounds__(PAIR_NT) k_build_pairs(RowSet A, RightOp B, He
       const int run = __ffs(~same) - 1;  // consecutive units of row r (group <= 8, so ~same is not 0)
       const int j1 = j0 + run;
       const int64_t q0 = r >= 0 ? A.p[r] : 0, q1 = r >= 0 ? A.p[r + 1] : 0;
-      if (q1 - q0 <= PAIR_LONG) {
+      if (q1 - q0 <= long_from) {
         const int lo0 = __shfl_sync(FULL, slo, j0);
         for (int64_t qb = q0; qb < q1; qb += 32) {
           const int64_t q = qb + lane;
@@ -955,7 +974,7 @@ __global__ void __launch_bounds__(PAIR_NT) k_build_pairs(RowSet A, RightOp B, He
 template <int AB>
 __global__ void __launch_bounds__(PAIR_NT) k_build_pairs_long(RowSet A, RightOp B, HeavyUnit *units, int64_t nunits,
                                                               const int32_t *bci_id, const int32_t *bci, int nseg,
-                                                              int64_t *pseg, void *paval) {
+                                                              int64_t *pseg, void *paval, int64_t long_from) {
   using VT = typename PairVal<AB>::T;
   constexpr int NW = PAIR_NT / 32;
   __shared__ int s_long[PAIR_NT], s_n;
@@ -970,7 +989,7 @@ __global__ void __launch_bounds__(PAIR_NT) k_build_pairs_long(RowSet A, RightOp 
     const int64_t mine = (v0 + threadIdx.x) * gridDim.x + blockIdx.x;
     if (mine < nunits) {
       const HeavyUnit u = units[mine];
-      if (unit_ok(A, u, nseg, mine) && A.p[u.row + 1] - A.p[u.row] > PAIR_LONG)
+      if (unit_ok(A, u, nseg, mine) && A.p[u.row + 1] - A.p[u.row] > long_from)
         s_long[atomicAdd(&s_n, 1)] = threadIdx.x;
     }
     __syncthreads();
@@ -1025,22 +1044,19 @@ __global__ void __launch_bounds__(PAIR_NT) k_build_pairs_long(RowSet A, RightOp 
 }
 
 void launch_build_pairs(const RowSet &A, const RightOp &B, HeavyUnit *units, int64_t nunits, const int32_t *bci_id,
-                        const int32_t *bci, int nseg, int a_bytes, int has_long, int64_t *pseg, void *paval,
+                        const int32_t *bci, int nseg, int a_bytes, int64_t long_from, int64_t *pseg, void *paval,
                         cudaStream_t st) {
   if (nunits <= 0) return;
-  // consecutive units per warp: as many as leave every resident warp a group
-  const int64_t warps = (int64_t)sm_count() * 40;
-  int group = (int)(nunits / warps);
-  group = group < 1 ? 1 : (group > PAIR_GROUP ? PAIR_GROUP : group);
+  const int group = pair_group(nunits);
   const int g = grid_for((nunits + group - 1) / group, PAIR_NT / 32, 16);
   const int gl = grid_for(nunits, 1, 4);
 #define HS_PAIRS(AB)                                                                                              \
   do {                                                                                                            \
     count_launch();                                                                                               \
-    k_build_pairs<AB><<<g, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval, group);         \
-    if (has_long) {                                                                                               \
+    k_build_pairs<AB><<<g, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval, group, long_from); \
+    if (long_from < INT64_MAX) {                                                                                             \
       count_launch();                                                                                             \
-      k_build_pairs_long<AB><<<gl, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval);        \
+      k_build_pairs_long<AB><<<gl, PAIR_NT, 0, st>>>(A, B, units, nunits, bci_id, bci, nseg, pseg, paval, long_from); \
     }                                                                                                             \
   } while (0)
   if (a_bytes == 8) HS_PAIRS(8);

@@ -337,15 +337,16 @@ void launch_plan_parts(const RowSet &A, const int *list, int count, const int32_
 // entries inside the part's columns, (segment start and length in one word,
 // the entry's value when the semiring reads it), compacted into the unit's
 // slice; sets npairs.  A part spans at most 2^17 columns, so a length fits 24
-// bits.  a_bytes: width of A's values to copy (0: none); has_long: some row
-// of A holds more than PAIR_LONG entries.
-constexpr int PAIR_LONG = 1024;
+// bits.  a_bytes: width of A's values to copy (0: none).  Rows of A with more
+// than long_from entries are laid out by a block per unit (pair_long_from;
+// INT64_MAX: there are none).
+int64_t pair_long_from(int64_t nunits, int64_t entries, int64_t longest);
 __host__ __device__ constexpr int64_t pair_pack(int64_t start, int len) { return start << 24 | (int64_t)len; }
 __host__ __device__ constexpr int64_t pair_start(int64_t x) { return x >> 24; }
 __host__ __device__ constexpr int pair_len(int64_t x) { return (int)(x & 0xffffff); }
 static_assert(HU_SPAN_SEGS * SEG_W < (1 << 24), "a segment's length fits its word");
 void launch_build_pairs(const RowSet &A, const RightOp &B, HeavyUnit *units, int64_t nunits, const int32_t *bci_id,
-                        const int32_t *bci, int nseg, int a_bytes, int has_long, int64_t *pseg, void *paval,
+                        const int32_t *bci, int nseg, int a_bytes, int64_t long_from, int64_t *pseg, void *paval,
                         cudaStream_t st);
 
 // numeric_*.cu
@@ -376,7 +377,7 @@ struct NumArgs {
   int lists_partial;      // with units: some heavy rows have no list (the row kernel takes them)
   const int64_t *pseg;    // units' B segments (launch_build_pairs)
   const void *paval;
-  int pair_long;          // some row of A holds more than PAIR_LONG entries
+  int64_t pair_long;      // entries from which a row's pairs are laid out by blocks
   int pair_abytes;        // width of the left values the pairs carry (0: none)
   int unit_kb;            // the units' value capacity in KB (16 or 32): which unit kernel runs
   int tiny_group;         // tiny rows several to a warp

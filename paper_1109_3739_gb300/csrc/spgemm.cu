@@ -559,7 +559,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
     if (!sides && (groups & (groups - 1))) sides = t_sides.of(st);
     return sides;
   };
-  const int pair_long = hb->stats[2] > (unsigned long long)PAIR_LONG;  // (read before hb is copied to again)
+  const int64_t longest = (int64_t)hb->stats[2];  // (read before hb is copied to again)
   const int nseg = (int)((n + SEG_W - 1) / SEG_W);
 
   // A entries whose B row is empty make no products.  When they are most of
@@ -767,6 +767,7 @@ static int spgemm_impl(int sr, const hs_mat *A, const hs_mat *B, hs_mat *C, Mem 
   void *paval = nullptr;
   const int64_t nunits = pcnt ? hb->nunits : 0;
   const int64_t npcap = pcnt ? hb->npcap : 0;
+  const int64_t pair_long = pair_long_from(nunits, npcap, longest);
   const int nheavy = key_off[NKEYS] - key_off[KEY_HEAVY];
   const int a_bytes = (sr == HS_PLUS_TIMES || sr == HS_MIN_PLUS || sr == HS_SELECT1ST) ? vb : 0;
   if (nheavy > 0 && nunits > 0) {
