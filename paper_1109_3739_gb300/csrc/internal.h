@@ -120,11 +120,13 @@ __host__ __device__ inline int num_key(int64_t f, int64_t c, const BinCfg &b) {
   return c <= 0 ? 0 : k;
 }
 // Tiny rows (at most 32 products) are taken several to a warp when they are
-// many and small: below 8 products on average a warp holds four rows or more;
-// a list that gives every warp of the GPU but a few rows is a matter of
-// latency, which the kernel for single rows hides better.
+// many and small.  1,000,000 rows of 2 / 8 / 16 products by the call: 1059 /
+// 1233 / 1355 us one by one, 335 / 519 / 886 together, and of 20 / 25 products
+// 1572 / 1509 and 1720 / 1607, so the line lies at 16; 131,072 rows of 2 / 16 /
+// 20: 274 / 300 / 324 and 216 / 254 / 358; from 65,536 rows down a warp has but a
+// few and both are equal (32,768 rows of 2 to 25: 192..208 and 186..205).
 inline bool tiny_group_pays(int64_t rows, unsigned long long products) {
-  return rows >= 65536 && products <= 8ull * (unsigned long long)rows;
+  return rows >= 65536 && products <= 16ull * (unsigned long long)rows;
 }
 // Hub rows: rows whose key is a warp's or a small block's, but which have many
 // entries of A, go to the kernel of 1024 threads, which looks up four times as
