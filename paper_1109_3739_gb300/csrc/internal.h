@@ -50,6 +50,13 @@ constexpr int64_t LIST_BITS = (int64_t)1 << 62;
 constexpr int HV_SPAN_SEGS = 64;      // segments a heavy column part spans at most (2^18 columns)
 constexpr int HU_SPAN_SEGS = 32;      // the same for the parts of the unit kernel (2^17 columns)
 constexpr int BITMAP_COLS = 1 << 20;  // columns covered by the heavy symbolic bitmap
+// Words of that bitmap that a launch has room for, B having n columns: one of
+// four sizes, not one a width, because kernel_fit keeps an answer for each.
+inline int64_t sym_bitmap_words(int64_t n) {
+  int64_t words = BITMAP_COLS / 256;
+  while (words < BITMAP_COLS / 32 && words * 32 < n) words *= 2;
+  return words;
+}
 constexpr int SEG_SMEM = 1024;        // segment counters kept in shared memory when nseg <= this
 
 __host__ __device__ inline int floor_log2_u64(uint64_t x) {

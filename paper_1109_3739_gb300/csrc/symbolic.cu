@@ -612,9 +612,7 @@ void launch_sym_mid(const SymArgs &a, cudaStream_t st) { launch_sym_cta<2 * F_MI
 void launch_sym_large(const SymArgs &a, cudaStream_t st) { launch_sym_cta<16384, 512>(a, st); }
 
 template <int NT> static void launch_sym_heavy_as(const SymArgs &a, cudaStream_t st) {
-  const int64_t words = (a.B.n + 31) / 32;
-  const size_t bytes = offsetof(SymHeavySmem<NT>, bitmap) +
-                       sizeof(unsigned) * (size_t)(words < SH_COLS / 32 ? (words + 3) & ~(int64_t)3 : SH_COLS / 32);
+  const size_t bytes = offsetof(SymHeavySmem<NT>, bitmap) + sizeof(unsigned) * (size_t)sym_bitmap_words(a.B.n);
   const int fit = fit_per_sm(k_sym_heavy<NT>, NT, bytes);
   count_launch();
   k_sym_heavy<NT><<<grid_cap(a.count, 1, fit), NT, bytes, st>>>(a);

@@ -68,3 +68,16 @@ def test_hub_rows_are_moved_while_they_are_few(tmp_path):
     CHECK(hub_key(key, 5000, 0) == KEY_LARGE && hub_key(key, 5000, 1) == key && hub_key(key, 4096, 0) == key);
     CHECK(hub_key(key, 20000, 1) == KEY_LARGE && hub_key(key, 1LL << 40, HUB_LEVELS) == key);
   }""")
+
+
+def test_symbolic_bitmap_sizes_are_few(tmp_path):
+    """The launch sizes of the bitmap kernel hold B's columns and do not follow every width: each is asked of the
+    runtime once and kept."""
+    run(tmp_path, r"""
+  std::set<int64_t> sizes;
+  for (int64_t n = 1; n < 1LL << 31; n += n < 3000000 ? 1 : n / 7) {
+    const int64_t w = sym_bitmap_words(n);
+    CHECK(w * 32 >= (n < BITMAP_COLS ? n : BITMAP_COLS) && w <= BITMAP_COLS / 32);
+    sizes.insert(w);
+  }
+  CHECK(sizes.size() <= 4);""")
