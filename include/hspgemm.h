@@ -148,9 +148,10 @@ int hs_spgemm(int semiring, const hs_mat *A, const hs_mat *B, hs_mat *C,
  * ranges are always checked; with HS_FLAG_VALIDATE, A is checked to be
  * canonical too.  At most 2^31-1 entries of B unless J is strictly increasing;
  * two host synchronisations with `stream` when J repeats no index (three with
- * the radix sort), up to five otherwise.  Errors: HS_EINVAL (an index out of
- * range, bad shapes, NULL pointers), HS_ENONCANON (with HS_FLAG_VALIDATE),
- * HS_EUNSUPPORTED, HS_ENOMEM, HS_ECUDA. */
+ * the radix sort; one more with HS_FLAG_VALIDATE, which reads the row sort's
+ * device-side checks), up to five otherwise.  Errors: HS_EINVAL (an index out
+ * of range, bad shapes, NULL pointers), HS_ENONCANON and HS_EINTERNAL (with
+ * HS_FLAG_VALIDATE), HS_EUNSUPPORTED, HS_ENOMEM, HS_ECUDA. */
 int hs_spref(const hs_mat *A, const int32_t *I, int64_t nI, const int32_t *J, int64_t nJ,
              hs_mat *B, const hs_allocator *al, void *stream, uint32_t flags);
 

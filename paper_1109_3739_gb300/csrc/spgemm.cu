@@ -1051,7 +1051,14 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     launch_spref_emit(a, tp, tv, st);
     if (!radix) {
       launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
-      return check_launch();
+      if (!(flags & HS_FLAG_VALIDATE)) return check_launch();
+      CK(cudaMemcpyAsync(hb, sb, sizeof(Small), cudaMemcpyDeviceToHost, st));  // the row sort's own checks
+      if (int e = check_launch()) return e;
+      CK(cudaStreamSynchronize(st));
+      if (!hb->dbg[0] && !hb->count[4]) return HS_OK;
+      snprintf(t_detail, sizeof(t_detail), "row sort check %d, index check %lld failed at %lld", hb->count[4],
+               (long long)hb->dbg[0], (long long)hb->dbg[1]);
+      return HS_EINTERNAL;
     }
     launch_spref_row_ids(Bout->ptr, nI, ntup, list, st);
     t.reset();
