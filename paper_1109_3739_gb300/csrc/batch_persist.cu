@@ -18,7 +18,7 @@
 //      rows, then adds the totals of the blocks before it);
 //   4. the values, written in ascending column order at the row's offset: a
 //      warp row by sorting its products (128, 256, 512 or 1024 keys) in the warp's
-//      registers and folding equal columns (sort_row), a CTA row in a shared hash table of keys and
+//      registers and folding equal columns (sort_finish), a CTA row in a shared hash table of keys and
 //      values (with more than 2048 outputs column range by column range,
 //      ranges cut from its buckets).
 // No allocation and no host synchronisation happen in an execution, so it

@@ -38,14 +38,6 @@ __device__ __forceinline__ void copy_val(void *dst, int64_t at, const void *src,
 
 __global__ void k_iota_i64(int64_t *p, int64_t n) { GRID_STRIDE(i, n) p[i] = i; }
 
-__global__ void k_fill_i32(int32_t *a, int64_t n, int32_t v) { GRID_STRIDE(i, n) a[i] = v; }
-void launch_fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t st) {
-  if (n > 0) {
-    count_launch();
-    k_fill_i32<<<grid1(n), 256, 0, st>>>(a, n, v);
-  }
-}
-
 __global__ void k_iota_i32(int32_t *p, int64_t n) { GRID_STRIDE(i, n) p[i] = (int32_t)i; }
 void launch_iota_i32(int32_t *p, int64_t n, cudaStream_t st) {
   if (n > 0) {

@@ -409,7 +409,6 @@ void launch_build_Q_fill(const int32_t *J, int64_t nJ, int64_t *Qcur, int32_t *Q
 void launch_sort_short_rows(const int64_t *ptr, int32_t *j, int64_t rows, cudaStream_t st);
 // pos[X[i]] = i for in-range X[i] (bit 1 of flag: out of range; bit 2: repeated)
 void launch_mark_positions(const int32_t *X, int64_t n, int64_t bound, int32_t *pos, int *flag, cudaStream_t st);
-void launch_fill_i32(int32_t *a, int64_t n, int32_t v, cudaStream_t st);
 // SpRef by gathering the selected rows (index.cu)
 struct GatherArgs {
   const int64_t *Ap;

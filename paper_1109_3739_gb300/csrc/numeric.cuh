@@ -1186,7 +1186,7 @@ inline int ngrid_cap(int items, int per_block, int per_sm) {
 }
 // ------------------------------------------------------------- sort tiers
 // Rows with 32 < f <= F_SORT whose output count is close to their product
-// count: one warp per row sorts the row's products (sort_row), one kernel
+// count: one warp per row sorts the row's products (sort_expand, sort_finish), one kernel
 // per register width K (32*K products), so each kernel's code stays small.
 // Only the tiers of at most 32*SORT_WIDE_K products sort 64-bit keys for
 // rows spanning too many columns.

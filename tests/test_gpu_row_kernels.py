@@ -174,3 +174,30 @@ def test_sorted_rows_treat_special_values_as_the_table_does(c, dup):
         order = np.argsort(raw.col[a:b])
         assert np.array_equal(got.col[a:b], raw.col[a:b][order])
         assert np.array_equal(got.val[a:b], raw.val[a:b][order], equal_nan=True)
+
+
+@pytest.mark.parametrize("dt", ["f32", "f64"])
+@pytest.mark.parametrize("c,dup", [(1500, 0), (1500, 100), (3500, 0), (3500, 300)])
+def test_sorted_rows_add_to_the_identity_as_the_table_does(c, dup, dt):
+    """(+,x) with products of -0: a sum starts from 0 in a row that is sorted as it is, as in the table (the unsorted
+    output keeps it), so a lone -0 becomes +0 on both ways, bit for bit."""
+    h = H()
+    A, B = operands(600001, [split(c, 3) + ([(0, dup)] if dup else [])] * 3, dt, 14)
+    A.val[:] = 1
+    B.val[::2], B.val[1::7] = -0.0, np.nan
+    dA, dB = h.DeviceCSR.from_host(A), h.DeviceCSR.from_host(B)
+    got = h.spgemm("plus_times", dA, dB).to_host()
+    raw = h.spgemm("plus_times", dA, dB, sorted_rows=False).to_host()
+    assert np.array_equal(got.rowptr, raw.rowptr)
+    zeros = 0
+    for a, b in zip(got.rowptr[:-1], got.rowptr[1:]):
+        order = np.argsort(raw.col[a:b])
+        x, y = got.val[a:b], raw.val[a:b][order]
+        assert np.array_equal(got.col[a:b], raw.col[a:b][order])
+        nan = np.isnan(x)
+        assert np.array_equal(nan, np.isnan(y))
+        # (sums of several terms are formed in an unspecified order: at most 2 here, so the same either way)
+        assert np.array_equal(np.signbit(x[~nan]), np.signbit(y[~nan])) and np.array_equal(x[~nan], y[~nan])
+        zeros += np.count_nonzero(x[~nan] == 0)
+        assert not np.signbit(x[~nan][x[~nan] == 0]).any()
+    assert zeros > c // 4

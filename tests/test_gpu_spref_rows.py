@@ -1,4 +1,4 @@
-"""SpRef's row sort at the edges of its tiers (8 entries: eight lanes; 256: a
+"""SpRef's row sort at the edges of its tiers (8 entries: eight lanes; 64: a
 warp; 2048: a block; beyond: a bitmap of B's columns, in chunks of 2^20), its
 gather at the edges of words and tiles, and the symbolic and numeric warp rows
 at the edges of their sorts.  Values are copied bit for bit; sums of small
