@@ -65,17 +65,17 @@ def peaks():
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch
 # of the dominant kernel: ncu's one-pass counters for k_num_units at R-MAT
-# scale 18 (5.3628 GB per launch, three launches within 0.05 percent), scaled
-# to scale 20 by the ratio of the launch's algorithmic bytes (26.438 / 3.3377
-# GB: the rows of the numeric heavy bin, with the default routing of 4-byte
-# values); the command and counters are summarised under profiles/.  It is
+# scale 18 (4.5714 GB per launch, two launches within 0.01 percent), per byte
+# of the launch's algorithmic bytes there (3.3377 GB: the rows of the numeric
+# heavy bin, with the default routing of 4-byte values), times those of the
+# measured launch; the command and counters are summarised under profiles/.  It is
 # reported only while the device code of that kernel and of the kernels that
 # write its inputs (bins, lists, units, pairs, segment index) still hashes to
 # the value it had when it was taken (comments and blank lines do not count),
 # and only for the part capacity it was taken with; otherwise the field is
 # null until it is measured again.
-MEASURED_TRAFFIC = {"kernel": "numeric_heavy", "scale": 20, "bytes": 5.3626e9 * 26.4383 / 3.33774,
-                    "measured_at_scale": 18, "heavy_part_kb": 16, "csrc_code_sha256_16": "cfcf5a7f65d676f6"}
+MEASURED_TRAFFIC = {"kernel": "numeric_heavy", "scale": 20, "per_algorithmic_byte": 4.5714e9 / 3.33774e9,
+                    "measured_at_scale": 18, "heavy_part_kb": 16, "csrc_code_sha256_16": "4994dc6b48ec86e7"}
 KERNEL_SOURCES = ("analysis.cu", "common.cuh", "internal.h", "numeric.cuh", "numeric_pt.cu", "symbolic.cu")
 
 
@@ -1049,8 +1049,9 @@ def main():
     achieved = alg_bytes / (dom_ms / 1000.0) / 1e9
     mt = MEASURED_TRAFFIC
     part_kb = h.get_tuning().get("heavy_part_kb", 16)  # the setting the timed steps ran with
-    traffic = mt["bytes"] if (dom == mt["kernel"] and args.scale == mt["scale"] and part_kb == mt["heavy_part_kb"]
-                              and csrc_hash() == mt["csrc_code_sha256_16"]) else None
+    known = (dom == mt["kernel"] and args.scale == mt["scale"] and part_kb == mt["heavy_part_kb"]
+             and csrc_hash() == mt["csrc_code_sha256_16"])
+    traffic = alg_bytes * mt["per_algorithmic_byte"] if known else None
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm, "unit": "GB/s",
                 "frac": achieved / hbm, "traffic": traffic, "peak_kind": peak_kind,
                 "alg_bytes_per_launch": alg_bytes, "ms_per_launch": dom_ms}
