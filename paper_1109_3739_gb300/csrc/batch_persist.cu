@@ -437,13 +437,13 @@ __global__ void __launch_bounds__(BP_NT, 3) k_batch_persist(BpArgs a) {
       } else if (HS_G(dbg, cb + c <= a.cap, 81, cb + c)) {
         T *out_v = SR::has_val ? Cv + cb : nullptr;
         if (g == 0)
-          sort_finish<SR, BPW_FS / 64, true, true>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
+          sort_finish<SR, BPW_FS / 64, true, sizeof(T) == 4>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
         else if (g == 1)
-          sort_finish<SR, BPW_FS / 32, true, true>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
+          sort_finish<SR, BPW_FS / 32, true, sizeof(T) == 4>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
         else if (g == 2)
-          sort_finish<SR, 2 * BPW_FS / 32, false, true>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
+          sort_finish<SR, 2 * BPW_FS / 32, false, sizeof(T) == 4>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
         else
-          sort_finish<SR, BPW_F / 32, false, true>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
+          sort_finish<SR, BPW_F / 32, false, sizeof(T) == 4>(fr, c, kmn, kmx, s_col, s_val, a.Cj + cb, out_v, &ctr->kerr, dbg);
       }
       __syncwarp();
     }
