@@ -159,9 +159,13 @@ struct Mem {
     if (p) scratch.push_back({p, bytes});
     return p;
   }
-  ~Mem() {
-    for (auto &b : scratch) release(b.p, b.n);
+  // the temporaries taken since scratch.size() was n
+  void release_from(size_t n) {
+    for (size_t i = n; i < scratch.size(); ++i) release(scratch[i].p, scratch[i].n);
+    scratch.resize(n);
+    chunk_left = 0;  // (the shared block may be one of them)
   }
+  ~Mem() { release_from(0); }
 };
 
 // A pool of the library's own for calls that allocate and free the same large
@@ -1046,26 +1050,41 @@ static int spref_impl(const hs_mat *A, const int32_t *I, int64_t nI, const int32
     }
     int32_t *tp = mem.tmp<int32_t>((size_t)ntup);
     void *tv = vb ? (void *)mem.tmp<char>((size_t)vb * (size_t)ntup) : nullptr;
-    int32_t *list = mem.tmp<int32_t>((size_t)(radix ? ntup : 2 * nI));  // (radix: the tuples' rows)
     if (mem.failed) return HS_ENOMEM;
     launch_spref_emit(a, tp, tv, st);
-    if (!radix) {
-      launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
-      if (!(flags & HS_FLAG_VALIDATE)) return check_launch();
-      CK(cudaMemcpyAsync(hb, sb, sizeof(Small), cudaMemcpyDeviceToHost, st));  // the row sort's own checks
-      if (int e = check_launch()) return e;
-      CK(cudaStreamSynchronize(st));
-      if (!hb->dbg[0] && !hb->count[4]) return HS_OK;
-      snprintf(t_detail, sizeof(t_detail), "row sort check %d, index check %lld failed at %lld", hb->count[4],
-               (long long)hb->dbg[0], (long long)hb->dbg[1]);
-      return HS_EINTERNAL;
+    if (radix) {
+      const size_t kept = mem.scratch.size();
+      int32_t *ti = mem.tmp<int32_t>((size_t)ntup);
+      hs_mat sorted;
+      memset(&sorted, 0, sizeof(sorted));
+      int e = HS_ENOMEM;
+      if (ti) {
+        launch_spref_row_ids(Bout->ptr, nI, ntup, ti, st);
+        t.reset();
+        if (int e2 = check_launch()) return e2;
+        e = sparse_impl(ti, tp, tv, ntup, nI, nJ, A->dtype, sr, &sorted, mem, outmem, flags);
+      }
+      if (e != HS_ENOMEM) {
+        free_mat(Bout, outmem);
+        *Bout = sorted;
+        return e;
+      }
+      free_mat(&sorted, outmem);  // no room for it: the bitmaps need less
+      mem.release_from(kept);
+      mem.failed = outmem.failed = false;
+      if (!out(ntup)) return HS_ENOMEM;
     }
-    launch_spref_row_ids(Bout->ptr, nI, ntup, list, st);
-    t.reset();
-    outmem.release(Bout->ptr, sizeof(int64_t) * (size_t)(nI + 1));
-    Bout->ptr = nullptr;
+    int32_t *list = mem.tmp<int32_t>((size_t)(2 * nI));
+    if (mem.failed) return HS_ENOMEM;
+    launch_spref_rows(vb, Bout->ptr, nI, nJ, tp, tv, Bout->idx, Bout->val, lmax, sb->count, list, sb->dbg, st);
+    if (!(flags & HS_FLAG_VALIDATE)) return check_launch();
+    CK(cudaMemcpyAsync(hb, sb, sizeof(Small), cudaMemcpyDeviceToHost, st));  // the row sort's own checks
     if (int e = check_launch()) return e;
-    return sparse_impl(list, tp, tv, ntup, nI, nJ, A->dtype, sr, Bout, mem, outmem, flags);
+    CK(cudaStreamSynchronize(st));
+    if (!hb->dbg[0] && !hb->count[4]) return HS_OK;
+    snprintf(t_detail, sizeof(t_detail), "row sort check %d, index check %lld failed at %lld", hb->count[4],
+             (long long)hb->dbg[0], (long long)hb->dbg[1]);
+    return HS_EINTERNAL;
   }
 
   // Q = sparse(J, 1:len(J), 1, n, len(J)): row k holds every p with J[p] == k,

@@ -41,3 +41,25 @@ def test_long_rows_of_a_wide_matrix(count, dt):
         ref = oracle.spref(A, Iv, Jv)
         assert_bitexact(h.spref(d, Iv, Jv).to_host(), ref, f"{count} {dt}")
         assert_bitexact(h.spref(d, Iv, Jv, validate=True).to_host(), ref, f"{count} {dt}, checked")
+
+
+def test_long_rows_of_a_wide_matrix_when_allocations_fail():
+    """Every allocation of the radix route in turn: HS_ENOMEM with nothing left, or the bitmaps take over."""
+    import ctypes
+
+    import torch
+    from paper_1109_3739_gb300 import hspgemm as h
+    from tests.test_gpu_failure import _host, _sweep
+    A = long_rows(400, "i32")
+    d, Jv = h.DeviceCSR.from_host(A), order()
+    Iv = np.arange(A.m, dtype=np.int32)[::-1].copy()
+    dI, dJ, a, ref = torch.from_numpy(Iv).cuda(), torch.from_numpy(Jv).cuda(), d.desc(), oracle.spref(A, Iv, Jv)
+
+    def run(al):
+        c = h.hs_mat()
+        st = h.library().hs_spref(ctypes.byref(a), dI.data_ptr(), len(Iv), dJ.data_ptr(), len(Jv), ctypes.byref(c),
+                                  ctypes.byref(al.struct), None, 0)
+        return st, c
+
+    allocations, nomem, taken_over = _sweep(h, run, lambda c, al: assert_bitexact(_host(h, c, al), ref, "after a failure"))
+    assert allocations >= 12 and nomem >= 3 and taken_over >= 5
